@@ -21,7 +21,14 @@
 //   * scalars every lane needs (event time, block, buffer cursors, ordinals) are kept replicated in
 //     registers and updated identically by all lanes.
 // The next event is a warp-wide argmin over every lane's earliest source (three redux.sync on the bit
-// pattern of the positive doubles plus the source id, which encodes the tie order).  Decisions that look
+// pattern of the positive doubles plus the source id, which encodes the tie order).  Up to 128 GPUs a lane looks at all
+// of its GPUs (unrolled rows); beyond, iteration ends come from a calendar (Sim::load_bucket) or, where an event comes with
+// many local ends, from a scan of all rows.
+//
+// What bounds these kernels is the chain of dependent instructions of each replication and, with a dozen warps per SM at
+// different places of the round loop, instruction fetch: a version of the calendar kernel with 153 KB of code ran 26 % slower
+// than the same algorithm without the parts that made it grow (N = 512).  So rare work exists once (one abandonment handler, draws
+// out of line, loops not unrolled), and the compiled loops are 55-100 KB where they were 80-240.  Decisions that look
 // at all GPUs (least-loaded / k-th eligible GPU) are evaluated by the owners and reduced the same way.
 //
 // All clock arithmetic is IEEE double, one rounding per operation, never contracted (the file is also
@@ -40,12 +47,14 @@ constexpr int NBIN = 1024;
 constexpr unsigned FULL = 0xffffffffu;
 constexpr uint32_t NONE32 = 0xffffffffu;
 constexpr int TOUCH_CAP = 48;
+constexpr uint32_t CAL_FREE = 16;        // free lanes from which the calendar loads another bucket
 
 // Compile-time specialisation of the run kernel.  With F_GENERIC every mode is read from the parameters at
 // run time; otherwise the set bits say which features the instance contains and everything else is
 // compiled out.  SPL > 0 fixes the number of simulated GPUs per lane (N <= 32 SPL) so the per-GPU loops unroll.
 constexpr uint32_t F_GENERIC = 1, F_ABANDON = 2, F_SLI = 4, F_KAPPA = 8, F_HIST = 16, F_BLOCKS = 32, F_RANDOM = 64,
-                   F_OCC = 128, F_SLOTS = 256, F_MW = 512, F_FCFS = 1024, F_SLIG = 2048, F_IMM = 4096;
+                   F_OCC = 128, F_SLOTS = 256, F_MW = 512, F_FCFS = 1024, F_SLIG = 2048, F_IMM = 4096, F_SCAN = 8192;
+// F_SCAN (run-time row count): rounds read all GPUs instead of working from the calendar of iteration ends.
 // F_MW: several warps per replication.  Warp 0 (the master) runs the round loop and every event handler; the
 // other warps (helpers) wait at a block barrier for commands and take their share of the per-GPU work of a
 // round: rows r = warp, warp + W, ... of the candidate scan and of the local iteration ends / retirements.
@@ -59,7 +68,7 @@ constexpr uint32_t SRC_BLOCK = 0, SRC_ARRIVAL = 1, SRC_ABP = 9, SRC_ABD0 = 17, S
 
 enum { STREAM_ARRIVAL = 0, STREAM_ABANDON_P = 1, STREAM_ABANDON_D0 = 2, STREAM_ABANDON_D1 = 3,
        STREAM_PLACEMENT = 4, STREAM_SLI = 5, STREAM_SELECT0 = 6, STREAM_SELECT1 = 7 };
-enum { WANT_SOLO = 0, WANT_MIX = 1, WANT_PREFILL = 2 };
+enum { WANT_SOLO = 1, WANT_MIX = 2, WANT_PREFILL = 4 };
 enum { ERR_NONE = 0, ERR_INTERNAL = 1 };
 
 struct AbClock { double acc, lvl, t_last, t_ab; unsigned long long m; };
@@ -94,7 +103,7 @@ static_assert(sizeof(ClassState) % 8 == 0 && (sizeof(ClassState) * MAXI) % 16 ==
 static_assert(sizeof(RepHeader) % 16 == 0 && offsetof(RepHeader, cs) % 16 == 0, "RepHeader layout");
 
 struct SlotRec { double tpf; uint32_t pk; uint32_t pad; };  // request in a decode slot: prefill end time, packed lengths/class/group
-constexpr int STAGE_CAP = 64;                                 // finished-request records waiting for their accounting
+constexpr int STAGE_CAP = 64, ROW_STAGE_CAP = 32;              // finished-request records waiting for their accounting (stamps on chip / in global memory)
 // Accounting of finished requests, one block per warp (merged into the class records at kernel exit)
 struct WarpClassStats { double sYm_out, sYs_out, sum_tpot; unsigned long long tok_in, tok_out; uint32_t done_mixed, done_solo; };
 struct ADraw { double E; uint32_t pk; uint32_t pad; };     // one arrival draw: unit exponential (divided by the rate already when there is one block) and packed lengths
@@ -152,6 +161,8 @@ struct Params {
     uint32_t tarr_global;        // pf_tarr lives in tarr_g instead of shared memory
     double *tarr_g;              // [R][N]
     uint32_t *pfjob_g;           // [R][N] packed request in prefill, with tarr_g
+    double cal_inv_w;            // calendar of iteration ends (run-time row count, one warp): buckets per second
+    uint32_t cal_nbk, cal_K;     // buckets (a power of two, at most 256); buckets that the shortest iteration lasts at least
     LanePar lane;
 };
 
@@ -183,6 +194,19 @@ __device__ __forceinline__ void draw(const Params &p, uint32_t rep, uint32_t str
     const unsigned long long grep = p.rep_offset + rep;
     philox((uint32_t)index, (uint32_t)(index >> 32), stream, (uint32_t)grep, (uint32_t)p.seed,
            (uint32_t)(p.seed >> 32), w0, w1, w2, w3);
+}
+// The same out of line, for rare draws: the kernels' round loops are about as large as the instruction cache.
+__device__ __noinline__ uint4 draw_words(unsigned long long seed, uint32_t global_rep, uint32_t stream, unsigned long long index)
+{
+    uint4 w;
+    philox((uint32_t)index, (uint32_t)(index >> 32), stream, global_rep, (uint32_t)seed, (uint32_t)(seed >> 32), w.x, w.y, w.z, w.w);
+    return w;
+}
+__device__ __forceinline__ void draw_rare(const Params &p, uint32_t rep, uint32_t stream, unsigned long long index,
+                                          uint32_t &w0, uint32_t &w1, uint32_t &w2, uint32_t &w3)
+{
+    const uint4 w = draw_words(p.seed, (uint32_t)(p.rep_offset + rep), stream, index);
+    w0 = w.x; w1 = w.y; w2 = w.z; w3 = w.w;
 }
 
 // uniform on (0,1]: (top 53 bits of w0:w1, plus one) / 2^53
@@ -327,6 +351,10 @@ __device__ __noinline__ ADraw make_draw(unsigned long long seed, unsigned long l
 
 template <int SPL, uint32_t F>
 struct Sim {
+    // One warp and a run-time row count: iteration ends come from a calendar (load_bucket) instead of a scan of all GPUs,
+    // except in the F_SCAN instances.
+    static constexpr bool CAL = SPL == 0 && !(F & (F_MW | F_SCAN));
+    static constexpr bool STAGED = !(F & F_MW);      // one warp: finished requests are accounted 32 at a time
     __device__ __forceinline__ bool f_abandon() const { return (F & F_GENERIC) ? p.any_theta != 0 : (F & F_ABANDON) != 0; }
     __device__ __forceinline__ bool f_sli() const { return (F & F_GENERIC) ? (p.router == 1 || p.router == 2) : (F & F_SLI) != 0; }
     __device__ __forceinline__ bool f_slig() const { return (F & F_GENERIC) ? p.router == 2 : false; }
@@ -345,7 +373,7 @@ struct Sim {
     int warp, nwarps;            // position in the block (F_MW); 0 / 1 otherwise
     MwCmd *cmd;
     MwRes *res;
-    WarpClassStats *wcs;         // [nwarps][MAXI]
+    WarpClassStats *wcs;         // [nwarps][I]
     // shared memory (lane-owned entries)
     double *tnext, *pf_tarr;               // pf_tarr: arrival time of the request in prefill (shared memory, or global memory on large clusters)
     uint32_t *it, *nfin, *pfjob, *K, *Kpend;
@@ -353,9 +381,9 @@ struct Sim {
     uint16_t *ndec, *nact, *pfcur;
     uint16_t *sfin16;            // [Npad][B]  low 16 bits of each slot's finish iteration (f_slots)
     uint32_t *socc;              // [Npad][ceil(B/32)]  slot occupancy bits; bits past B are set for good
+    uint8_t *bkt;                // [GPUs rounded up to 128] calendar bucket of the GPU's iteration end, 255 when idle (CAL)
+    uint16_t *picked;            // [32] GPUs of the bucket being loaded (CAL)
     uint32_t *touch;
-    double *gate_xi, *gate_dq;
-    uint32_t *gate_ok;
     ClassState *cs;
     // global memory of this replication
     uint32_t *s_fin;
@@ -376,7 +404,19 @@ struct Sim {
     uint32_t need_start;         // per lane: rows of own GPUs touched by the current event
     unsigned long long place_ord, events, rounds, sel_ord0, sel_ord1;
     bool drain_dirty, gate_dirty, touch_all;
+    bool direct;                 // a request has just finished its prefill and its pool's buffer is empty: class and lengths, pool,
+    uint32_t d_pk, d_pool, d_gpu;   // and the GPU it has to decode on (NONE32: the router chooses)
     bool force_nonlocal;         // treat the next event, whatever it is, as non-local (it must end with a dispatch)
+    // calendar: last bucket loaded, bucket of T_end, the pending iteration end that this lane holds (GPU, time)
+    unsigned long long cur, cur_end, held_t;
+    uint32_t held_g;
+    bool held, crowded;          // crowded: the current bucket holds more ends than lanes
+    unsigned long long low;      // no pending event lies in an earlier bucket
+    unsigned long long left_t;   // crowded: earliest pending end of the bucket that no lane holds (time, source)
+    uint32_t left_s;
+    // smallest keys among this lane's GPUs (g mod 32 = lane), see choose(): decode target (solo-first, or solo GPUs only under
+    // the SLI-aware routers), mixed decode target (SLI-aware routers), prefill target; lanes whose keys are out of date
+    uint32_t best_dec, best_mix, best_pf, dirty_dec, dirty_pf;
     // per-lane partial sums
     unsigned long long it_mixed, it_solo;
     double busy_mixed, busy_solo;
@@ -398,6 +438,8 @@ struct Sim {
         blk = b;
         const BlockPar &bp = p.blocks[b];
         M = bp.M;
+        best_dec = best_mix = best_pf = NONE32;
+        dirty_dec = dirty_pf = FULL;
         b_xstar = 0.0; b_nx = 0.0; b_nq = 0.0; b_ps = 0.0;
         if (lane < (int)p.I) {
             b_xstar = bp.xstar[lane]; b_nx = bp.nx[lane]; b_nq = bp.nq[lane]; b_ps = bp.ps[lane];
@@ -413,7 +455,7 @@ struct Sim {
 
     __device__ __forceinline__ void refill(uint32_t i)
     {
-        const unsigned long long base = __shfl_sync(FULL, cs[lane & 7].adraw, i);
+        const unsigned long long base = cs[i].adraw;        // (only I class records exist: every lane reads record i)
         // with a single block the class's rate never changes and the division E / Lambda is done here, 32 at a time
         const double Lam1 = f_blocks() ? 0.0 : __dmul_rn((double)p.N, p.blocks[0].rate[i]);
         aring[i * 32 + lane] = make_draw(p.seed, p.rep_offset + rep, i, p.I, base + (unsigned long long)lane,
@@ -492,20 +534,13 @@ struct Sim {
         schedule_from(ta);
     }
 
-    // warp-wide path: an arrival while some prefill slot is idle (the gate may admit it at once)
-    __device__ void on_arrival(uint32_t i)
-    {
-        if (lane == (int)i) arrival_local();
-        gate_dirty = true;
-    }
-
     __device__ uint32_t count_idle_pf()
     {
         // per-lane count over the lane's rows (branch-free), one warp-wide sum
         uint32_t cnt = 0;
-#pragma unroll 4
+#pragma unroll 1
         for (uint32_t k = 0; k < n_rows(); ++k)
-            cnt += eligible((k << 5) + (uint32_t)lane, WANT_PREFILL) ? 1u : 0u;
+            cnt += key_of((k << 5) + (uint32_t)lane, WANT_PREFILL) != NONE32 ? 1u : 0u;
         return __reduce_add_sync(FULL, cnt);
     }
 
@@ -514,6 +549,7 @@ struct Sim {
     __device__ void ring_remove(QEntry *ring, uint32_t head, uint32_t n, uint32_t pos)
     {
         const uint32_t cap = p.qcap;
+#pragma unroll 1
         for (uint32_t k = pos; k + 1 < n; k += 32) {
             const uint32_t j = k + (uint32_t)lane;
             QEntry e;
@@ -531,127 +567,146 @@ struct Sim {
         }
     }
 
-    __device__ void on_abandon_p(uint32_t i)
+    // A class-i request leaves the prefill queue (which = 0) or the decode buffer of pool which - 1.  One body for the three:
+    // the size of the round loop is what the instruction cache has to hold.
+    __device__ void on_abandon(uint32_t which, uint32_t i)
     {
-        const uint32_t Q = __shfl_sync(FULL, cs[lane & 7].pq_n, i);
-        const uint32_t head = __shfl_sync(FULL, cs[lane & 7].pq_head, i);
-        const unsigned long long m = __shfl_sync(FULL, cs[lane & 7].abp.m, i);
+        const ClassState &ci = cs[i];
+        const AbClock &ai = which == 0 ? ci.abp : (which == 1 ? ci.abd0 : ci.abd1);
+        const uint32_t Q = which == 0 ? ci.pq_n : (which == 1 ? ci.Qd0 : ci.Qd1);
+        const unsigned long long m = ai.m;
         uint32_t w0, w1, w2, w3;
-        draw(p, rep, (STREAM_ABANDON_P << 8) | i, m, w0, w1, w2, w3);
-        const uint32_t rank = __umulhi(w2, Q);       // uniformly chosen waiting job, in FCFS rank
-        cp_async_wait_all();
-        __syncwarp();
-        ring_remove(pq + (size_t)i * p.qcap, head, Q, rank);
-        if (lane == (int)i) {
-            ClassState &c = cs[i];
-            if (Q > 1) pqh[i] = pq[(size_t)i * p.qcap + head];     // the head may have changed
-            area_touch(c.aQp, Q, t);
-            c.pq_n = Q - 1;
-            c.abandoned_p++;
-            AbClock &a = c.abp;
-            a.m = m + 1; a.acc = 0.0; a.lvl = -qlog(u53(w0, w1)); a.t_last = t;
-            a.t_ab = (Q - 1 > 0) ? __dadd_rn(t, __ddiv_rn(a.lvl, __dmul_rn(p.cls[i].theta, (double)(Q - 1)))) : dinf();
-        }
-    }
-
-    __device__ void on_abandon_d(uint32_t pool, uint32_t i)
-    {
-        const uint32_t Q = __shfl_sync(FULL, pool ? cs[lane & 7].Qd1 : cs[lane & 7].Qd0, i);
-        const unsigned long long m = __shfl_sync(FULL, pool ? cs[lane & 7].abd1.m : cs[lane & 7].abd0.m, i);
-        uint32_t w0, w1, w2, w3;
-        draw(p, rep, ((pool ? STREAM_ABANDON_D1 : STREAM_ABANDON_D0) << 8) | i, m, w0, w1, w2, w3);
-        uint32_t rank = __umulhi(w2, Q);
-        QEntry *ring = dq + (size_t)pool * p.qcap;
-        const uint32_t head = pool ? dq_head1 : dq_head0, n = pool ? dq_n1 : dq_n0;
-        // position of the rank-th class-i entry in buffer order
-        uint32_t pos = NONE32;
-        for (uint32_t k = 0; k < n && pos == NONE32; k += 32) {
-            const uint32_t j = k + (uint32_t)lane;
-            bool mine = false;
-            if (j < n) {
-                uint32_t src = head + j; if (src >= p.qcap) src -= p.qcap;
-                mine = ring[src].cls == i;
+        draw_rare(p, rep, ((STREAM_ABANDON_P + which) << 8) | i, m, w0, w1, w2, w3);
+        uint32_t rank = __umulhi(w2, Q), pos = rank;       // uniformly chosen waiting request, in FCFS rank
+        QEntry *ring = pq + (size_t)i * p.qcap;
+        uint32_t head = ci.pq_head, n = Q;
+        if (which == 0) {
+            cp_async_wait_all();
+        } else {
+            // position of the rank-th class-i entry in buffer order
+            ring = dq + (size_t)(which - 1u) * p.qcap;
+            head = which == 2 ? dq_head1 : dq_head0;
+            n = which == 2 ? dq_n1 : dq_n0;
+            pos = NONE32;
+#pragma unroll 1
+            for (uint32_t k = 0; k < n && pos == NONE32; k += 32) {
+                const uint32_t j = k + (uint32_t)lane;
+                bool mine = false;
+                if (j < n) {
+                    uint32_t src = head + j; if (src >= p.qcap) src -= p.qcap;
+                    mine = ring[src].cls == i;
+                }
+                const uint32_t b = __ballot_sync(FULL, mine);
+                const uint32_t c = (uint32_t)__popc(b);
+                if (rank < c) pos = k + (uint32_t)__fns(b, 0, (int)rank + 1);
+                else rank -= c;
             }
-            const uint32_t b = __ballot_sync(FULL, mine);
-            const uint32_t c = (uint32_t)__popc(b);
-            if (rank < c) pos = k + (uint32_t)__fns(b, 0, (int)rank + 1);
-            else rank -= c;
+            if (pos == NONE32) { err = ERR_INTERNAL; return; }
+            if (which == 2) dq_n1--; else dq_n0--;
         }
-        if (pos == NONE32) { err = ERR_INTERNAL; return; }
+        __syncwarp();
         ring_remove(ring, head, n, pos);
-        if (pool) dq_n1--; else dq_n0--;
         if (lane == (int)i) {
             ClassState &c = cs[i];
-            area_touch(c.aQd, c.Qd0 + c.Qd1, t);
-            if (pool) c.Qd1 = Q - 1; else c.Qd0 = Q - 1;
-            c.abandoned_d++;
-            AbClock &a = pool ? c.abd1 : c.abd0;
+            AbClock &a = which == 0 ? c.abp : (which == 1 ? c.abd0 : c.abd1);
+            if (which == 0) {
+                if (Q > 1) pqh[i] = ring[head];     // the head may have changed
+                area_touch(c.aQp, Q, t);
+                c.pq_n = Q - 1;
+                c.abandoned_p++;
+            } else {
+                area_touch(c.aQd, c.Qd0 + c.Qd1, t);
+                if (which == 2) c.Qd1 = Q - 1; else c.Qd0 = Q - 1;
+                c.abandoned_d++;
+            }
             a.m = m + 1; a.acc = 0.0; a.lvl = -qlog(u53(w0, w1)); a.t_last = t;
             a.t_ab = (Q - 1 > 0) ? __dadd_rn(t, __ddiv_rn(a.lvl, __dmul_rn(p.cls[i].theta, (double)(Q - 1)))) : dinf();
         }
     }
 
     // --- GPU choice ----------------------------------------------------------------------------
-    __device__ __forceinline__ bool eligible(uint32_t g, int want) const
+    // --- least-loaded choice on large clusters (CAL) ------------------------------------------------------
+    // Every lane keeps the smallest key of its own GPUs (its column), so a choice is one reduction over the lanes instead of
+    // a pass over all N/32 rows; columns in which something changed since are looked up again by the whole warp, one row
+    // per lane, when a choice needs them.
+    __device__ __forceinline__ void gpu_changed(uint32_t g) { if (CAL) { dirty_dec |= 1u << (g & 31u); dirty_pf |= 1u << (g & 31u); } }
+
+    // key of GPU g for the wanted tiers: solo GPUs first, then decodes held, then index; NONE32 when it is not eligible
+    __device__ __forceinline__ uint32_t key_of(uint32_t g, uint32_t tiers) const
     {
         // g is always inside the padded arrays; every field is read first so that calls over rows overlap
-        const uint32_t nd = ndec[g];
-        const bool pf = pfrem[g] != 0;
+        const uint32_t nd = ndec[g], pf = pfrem[g];
         const bool mix = g < M;
-        const uint32_t cap = (mix || pf) ? p.B - 1 : p.B;   // a mixed GPU keeps one slot for prefill
-        const bool ok = want == WANT_PREFILL ? (mix && !pf && nd <= p.B - 1)
-                                             : ((want == WANT_MIX) == mix && nd < cap);
-        return ok && g < p.N;
+        const uint32_t cap = (mix || pf != 0) ? p.B - 1 : p.B;   // a mixed GPU keeps one slot for prefill
+        const bool ok = tiers == WANT_PREFILL ? (mix && pf == 0 && nd <= p.B - 1) : ((tiers & (mix ? WANT_MIX : WANT_SOLO)) != 0 && nd < cap);
+        return (ok && g < p.N) ? ((mix ? 0x40000000u : 0u) | (nd << 16) | g) : NONE32;
     }
 
-    // uniformly at random among the eligible GPUs (k-th in index order) or least loaded, lowest index
-    // Solo-first target of a decode under least-loaded placement in one reduction: key = tier, load, index.
-    __device__ __forceinline__ uint32_t choose_solo_first()
-    {
-        uint32_t best = NONE32;
-#pragma unroll 4
-        for (uint32_t k = 0; k < n_rows(); ++k) {
-            const uint32_t g = (k << 5) + (uint32_t)lane;
-            const uint32_t nd = ndec[g];
-            const bool mix = g < M;
-            const uint32_t cap = (mix || pfrem[g] != 0) ? p.B - 1 : p.B;
-            const uint32_t key = (mix ? 0x40000000u : 0u) | (nd << 16) | g;
-            best = min(best, (nd < cap && g < p.N) ? key : NONE32);
-        }
-        best = __reduce_min_sync(FULL, best);
-        return best == NONE32 ? NONE32 : (best & 0xffffu);
-    }
-
-    __device__ uint32_t choose_server(int want)
+    // Least loaded (lowest index on ties) or uniformly random among the eligible GPUs of the first tier that has one
+    __device__ __forceinline__ uint32_t choose(uint32_t tiers)
     {
         const uint32_t rows = n_rows();
         if (!f_random()) {
             uint32_t best = NONE32;
+            if (CAL) {
+                const bool pf = tiers == WANT_PREFILL;
+                uint32_t dirty = pf ? dirty_pf : dirty_dec;
+                if (__popc(dirty) > 6) {
+                    uint32_t a = NONE32, b = NONE32;       // every lane over its own rows
+#pragma unroll 2
+                    for (uint32_t k = 0; k < rows; ++k) {
+                        a = min(a, key_of((k << 5) + (uint32_t)lane, pf ? WANT_PREFILL : (f_sli() ? WANT_SOLO : (WANT_SOLO | WANT_MIX))));
+                        if (f_sli() && !pf) b = min(b, key_of((k << 5) + (uint32_t)lane, WANT_MIX));
+                    }
+                    if (pf) best_pf = a; else { best_dec = a; best_mix = b; }
+                    dirty = 0;
+                }
+#pragma unroll 1
+                for (; dirty; dirty &= dirty - 1u) {
+                    const uint32_t col = (uint32_t)__ffs((int)dirty) - 1u;
+                    uint32_t a = NONE32, b = NONE32;
+#pragma unroll 1
+                    for (uint32_t k = (uint32_t)lane; k < rows; k += 32u) {
+                        a = min(a, key_of((k << 5) + col, pf ? WANT_PREFILL : (f_sli() ? WANT_SOLO : (WANT_SOLO | WANT_MIX))));
+                        if (f_sli() && !pf) b = min(b, key_of((k << 5) + col, WANT_MIX));
+                    }
+                    a = __reduce_min_sync(FULL, a);
+                    if (f_sli()) b = __reduce_min_sync(FULL, b);
+                    if (lane == (int)col) { if (pf) best_pf = a; else { best_dec = a; best_mix = b; } }
+                }
+                if (pf) dirty_pf = 0; else dirty_dec = 0;
+                best = pf ? best_pf : ((f_sli() && tiers == WANT_MIX) ? best_mix : best_dec);
+            } else {
 #pragma unroll 4
-            for (uint32_t k = 0; k < rows; ++k) {
-                const uint32_t g = (k << 5) + (uint32_t)lane;
-                best = min(best, eligible(g, want) ? (((uint32_t)ndec[g] << 16) | g) : NONE32);
+                for (uint32_t k = 0; k < rows; ++k) best = min(best, key_of((k << 5) + (uint32_t)lane, tiers));
             }
             best = __reduce_min_sync(FULL, best);
             return best == NONE32 ? NONE32 : (best & 0xffffu);
         }
-        uint32_t cnt = 0;
-        for (uint32_t k = 0; k < rows; ++k)
-            cnt += (uint32_t)__popc(__ballot_sync(FULL, eligible((k << 5) + (uint32_t)lane, want)));
-        if (cnt == 0) return NONE32;
-        uint32_t idx = 0;
-        if (cnt > 1) {
-            uint32_t w0, w1, w2, w3;
-            draw(p, rep, STREAM_PLACEMENT << 8, place_ord++, w0, w1, w2, w3);
-            idx = __umulhi(w0, cnt);
+#pragma unroll(SPL > 0 && !(F & F_GENERIC) ? 3 : 1)
+        for (uint32_t tier = WANT_SOLO; tier <= WANT_PREFILL; tier <<= 1) {
+            if (!(tiers & tier)) continue;
+            uint32_t cnt = 0;
+#pragma unroll(SPL > 0 ? SPL : 4)
+            for (uint32_t k = 0; k < rows; ++k)
+                cnt += (uint32_t)__popc(__ballot_sync(FULL, key_of((k << 5) + (uint32_t)lane, tier) != NONE32));
+            if (cnt == 0) continue;
+            uint32_t idx = 0;
+            if (cnt > 1) {
+                uint32_t w0, w1, w2, w3;
+                draw(p, rep, STREAM_PLACEMENT << 8, place_ord++, w0, w1, w2, w3);
+                idx = __umulhi(w0, cnt);
+            }
+#pragma unroll(SPL > 0 ? SPL : 4)
+            for (uint32_t k = 0; k < rows; ++k) {
+                const uint32_t b = __ballot_sync(FULL, key_of((k << 5) + (uint32_t)lane, tier) != NONE32);
+                const uint32_t c = (uint32_t)__popc(b);
+                if (idx < c) return (k << 5) + (uint32_t)__fns(b, 0, (int)idx + 1);
+                idx -= c;
+            }
+            err = ERR_INTERNAL;
+            return NONE32;
         }
-        for (uint32_t k = 0; k < rows; ++k) {
-            const uint32_t b = __ballot_sync(FULL, eligible((k << 5) + (uint32_t)lane, want));
-            const uint32_t c = (uint32_t)__popc(b);
-            if (idx < c) return (k << 5) + (uint32_t)__fns(b, 0, (int)idx + 1);
-            idx -= c;
-        }
-        err = ERR_INTERNAL;
         return NONE32;
     }
 
@@ -677,8 +732,8 @@ struct Sim {
         if (nonempty > 1) {
             if (!(Wsum > 0.0)) return 0;
             uint32_t w0, w1, w2, w3;
-            if (pool) draw(p, rep, STREAM_SELECT1 << 8, sel_ord1++, w0, w1, w2, w3);
-            else      draw(p, rep, STREAM_SELECT0 << 8, sel_ord0++, w0, w1, w2, w3);
+            if (pool) draw_rare(p, rep, STREAM_SELECT1 << 8, sel_ord1++, w0, w1, w2, w3);
+            else      draw_rare(p, rep, STREAM_SELECT0 << 8, sel_ord0++, w0, w1, w2, w3);
             const double x = __dmul_rn(u53(w0, w1), Wsum);
             double cum = 0.0;
             uint32_t chosen = NONE32, last = NONE32;
@@ -707,22 +762,22 @@ struct Sim {
         return 0;
     }
 
-    // entry pos (0 = head) of the pool's buffer goes to GPU g
-    __device__ void place_decode(uint32_t pool, uint32_t g, uint32_t pos = 0)
+    // Entry pos (0 = head) leaves the pool's buffer to be placed.
+    __device__ __forceinline__ QEntry take_buffered(uint32_t pool, uint32_t pos)
     {
         const uint32_t head = pool ? dq_head1 : dq_head0;
         QEntry *ring = dq + (size_t)pool * p.qcap;
         uint32_t src = head + pos; if (src >= p.qcap) src -= p.qcap;
         const QEntry e = ring[src];
-        if (pos == 0) {
-            if (pool) dq_head1 = (head + 1 == p.qcap) ? 0 : head + 1;
-            else      dq_head0 = (head + 1 == p.qcap) ? 0 : head + 1;
+        if (!f_slig() || pos == 0) {
+            const uint32_t next = (head + 1 == p.qcap) ? 0 : head + 1;
+            if (pool) dq_head1 = next; else dq_head0 = next;
         } else {
             __syncwarp();
             ring_remove(ring, head, pool ? dq_n1 : dq_n0, pos);
         }
         if (pool) dq_n1--; else dq_n0--;
-        place_job(pool, g, e.cls, job_P(e.pk), job_D(e.pk), e.t, true);
+        return e;
     }
 
     // A request of class i whose prefill ended at tpf starts decoding on GPU g.  from_buffer: it waited in
@@ -772,6 +827,7 @@ struct Sim {
             nfin[g] = min(nfin[g], fin);
             if (f_kappa()) Kpend[g] += P;
         }
+        gpu_changed(g);
         touch_server(g);
     }
 
@@ -799,22 +855,34 @@ struct Sim {
             key = __reduce_min_sync(FULL, key);
             return key == NONE32 ? NONE32 : (key & 0xffu);
         }
+        // Occupancy gate: argmin of xi_i = (X_i - n x*_i)/x*_i over the class lanes, ties to the largest Q_p,i - n q*_p,i, then
+        // to the lowest class.  Doubles are compared through their bits (order_key), so a minimum is two reductions.
+        unsigned long long xi = ~0ull;
+        bool ok = false;
         if (lane < (int)p.I) {
             const ClassState &c = cs[lane];
-            gate_ok[lane] = (c.pq_n > 0 && b_xstar > 0.0) ? 1u : 0u;
-            gate_xi[lane] = __ddiv_rn(__dsub_rn((double)c.X, b_nx), b_xstar);   // xi_i = (X_i - n x*_i)/x*_i
-            gate_dq[lane] = __dsub_rn((double)c.pq_n, b_nq);                     // Q_p,i - n q*_p,i
+            ok = c.pq_n > 0 && b_xstar > 0.0;
+            if (ok) xi = order_key(__ddiv_rn(__dsub_rn((double)c.X, b_nx), b_xstar));
         }
-        __syncwarp();
-        uint32_t best = NONE32;
-        double bxi = 0.0, bdq = 0.0;
-        for (uint32_t i = 0; i < p.I; ++i) {
-            if (!gate_ok[i]) continue;
-            const double xi = gate_xi[i], dqv = gate_dq[i];
-            if (best == NONE32 || xi < bxi || (xi == bxi && dqv > bdq)) { best = i; bxi = xi; bdq = dqv; }
+        const uint32_t xh = (uint32_t)(xi >> 32), mh = __reduce_min_sync(FULL, xh);
+        const uint32_t ml = __reduce_min_sync(FULL, xh == mh ? (uint32_t)xi : NONE32);
+        ok = ok && xh == mh && (uint32_t)xi == ml;
+        uint32_t tie = __ballot_sync(FULL, ok);
+        if (tie & (tie - 1u)) {
+            unsigned long long dq = 0ull;
+            if (ok) dq = order_key(__dsub_rn((double)cs[lane].pq_n, b_nq));
+            const uint32_t dh = (uint32_t)(dq >> 32), Mh = __reduce_max_sync(FULL, dh);
+            const uint32_t Ml = __reduce_max_sync(FULL, dh == Mh ? (uint32_t)dq : 0u);
+            tie = __ballot_sync(FULL, ok && dh == Mh && (uint32_t)dq == Ml);
         }
-        __syncwarp();
-        return best;
+        return tie ? (uint32_t)__ffs((int)tie) - 1u : NONE32;
+    }
+
+    // unsigned integers that order as the doubles do (adding zero makes the two zeros one)
+    static __device__ __forceinline__ unsigned long long order_key(double x)
+    {
+        const long long b = __double_as_longlong(__dadd_rn(x, 0.0));
+        return (unsigned long long)b ^ (b < 0 ? ~0ull : 0x8000000000000000ull);
     }
 
     __device__ void admit(uint32_t i, uint32_t g)
@@ -848,6 +916,7 @@ struct Sim {
             pfrem[g] = (uint16_t)job_P(e.pk);
             pf_tarr[g] = e.t;
         }
+        gpu_changed(g);
         touch_server(g);
     }
 
@@ -871,58 +940,48 @@ struct Sim {
             if (f_kappa()) { K[g] = Kg; Kpend[g] = 0; }
             pfcur[g] = (uint16_t)pc;
             nact[g] = (uint16_t)(nd | fl);
-            tnext[g] = __dadd_rn(ts, tau);
+            const double te = __dadd_rn(ts, tau);
+            tnext[g] = te;
+            if (CAL) bkt[g] = bucket_id(te);
         }
     }
-    __device__ __forceinline__ void start_if_needed(uint32_t g) { start_at(g, t); }
 
     __device__ void dispatch()
     {
         __syncwarp();   // queue entries and GPU state written by the event handler are visible to every lane
-        // decode routing: buffered jobs first (FCFS), solo GPUs before mixed ones
-        if (drain_dirty && (dq_n0 | dq_n1)) {
-            if (!f_sli()) {
-                while (dq_n0 > 0) {
-                    uint32_t g;
-                    if (!f_random()) {
-                        g = choose_solo_first();
-                    } else {
-                        g = choose_server(WANT_SOLO);
-                        if (g == NONE32) g = choose_server(WANT_MIX);
-                    }
-                    if (g == NONE32) break;
-                    place_decode(0, g);
-                    __syncwarp();
-                }
-            } else {
-                while (dq_n0 > 0) {
-                    const uint32_t g = choose_server(WANT_SOLO);
-                    if (g == NONE32) break;
-                    place_decode(0, g, f_slig() ? select_in_pool(0) : 0u);
-                    __syncwarp();
-                }
-                while (dq_n1 > 0) {
-                    const uint32_t g = choose_server(WANT_MIX);
-                    if (g == NONE32) break;
-                    place_decode(1, g, f_slig() ? select_in_pool(1) : 0u);
-                    __syncwarp();
-                }
-            }
+        // the request that has just finished its prefill: it passes through its pool's empty buffer
+        if (direct) {
+            uint32_t g = d_gpu;
+            if (g == NONE32) g = f_sli() ? choose(d_pool ? WANT_MIX : WANT_SOLO) : choose(WANT_SOLO | WANT_MIX);
+            if (g != NONE32) place_job(d_pool, g, job_cls(d_pk), job_P(d_pk), job_D(d_pk), t, false);
+            else enqueue_decode();
+            direct = false;
+            __syncwarp();
         }
-        drain_dirty = false;
-        // prefill gate on mixed GPUs whose prefill slot is idle
-        if (gate_dirty) {
+        // decode routing of buffered requests: FCFS, solo GPUs before mixed ones, or pool by pool
+        uint32_t pool = drain_dirty ? 0u : 2u;       // buffer being drained; 2: none left
+        while (pool < 2u) {
+            if (pool == 0 && dq_n0 == 0) pool = f_sli() ? 1u : 2u;
+            if (pool == 1 && dq_n1 == 0) pool = 2u;
+            if (pool == 2u) break;
+            const uint32_t g = f_sli() ? choose(pool ? WANT_MIX : WANT_SOLO) : choose(WANT_SOLO | WANT_MIX);
+            if (g == NONE32) { pool = (pool == 0 && f_sli()) ? 1u : 2u; continue; }
+            const QEntry e = take_buffered(pool, f_slig() ? select_in_pool(pool) : 0u);
+            place_job(pool, g, e.cls, job_P(e.pk), job_D(e.pk), e.t, true);
+            __syncwarp();
+        }
+        // prefill gate on mixed GPUs whose prefill slot is idle; a single idle slot whose GPU is known needs no search (and
+        // draws nothing: one candidate)
+        if (gate_dirty)
             while (n_idle_pf > 0) {
-                if (!__any_sync(FULL, lane < (int)p.I && cs[lane & 7].pq_n > 0)) break;      // nobody waits
-                const uint32_t i = gate_class();
-                if (i == NONE32) break;
-                // a single idle slot whose GPU is known needs no search (and draws nothing: one candidate)
-                const uint32_t g = (n_idle_pf == 1 && idle_hint != NONE32) ? idle_hint : choose_server(WANT_PREFILL);
+                const uint32_t cls = gate_class();
+                if (cls == NONE32) break;
+                const uint32_t g = (n_idle_pf == 1 && idle_hint != NONE32) ? idle_hint : choose(WANT_PREFILL);
                 if (g == NONE32) break;
-                admit(i, g);
+                admit(cls, g);
                 __syncwarp();
             }
-        }
+        drain_dirty = false;
         gate_dirty = false;
         // start the next iteration on every GPU that was touched and is between iterations
         __syncwarp();
@@ -932,14 +991,11 @@ struct Sim {
             for (uint32_t k = 0; k < (uint32_t)(SPL > 0 ? SPL : 1); ++k)
                 start_at((k << 5) + (uint32_t)lane, t, ((need_start >> k) & 1u) != 0);
             need_start = 0;
-        } else if (touch_all) {
-            for (uint32_t k = 0; k < n_rows(); ++k) {
-                const uint32_t g = (k << 5) + (uint32_t)lane;
-                if (g < p.N) start_if_needed(g);
-            }
         } else {
-            // one lane per touched GPU (a GPU noted twice is started by two lanes with the same result)
-            for (uint32_t k = (uint32_t)lane; k < n_touch; k += 32u) start_if_needed(touch[k]);
+            // one lane per touched GPU (a GPU noted twice is started by two lanes with the same result), or all GPUs
+            const uint32_t n = touch_all ? p.N : n_touch;
+#pragma unroll 1
+            for (uint32_t k = (uint32_t)lane; k < n; k += 32u) start_at(touch_all ? k : touch[k], t);
         }
         n_touch = 0;
         touch_all = false;
@@ -952,7 +1008,7 @@ struct Sim {
     {
         const uint32_t i = job_cls(pk), P = job_P(pk), D = job_D(pk);
         if (lane == (int)i) {
-            WarpClassStats &c = wcs[warp * MAXI + (int)i];
+            WarpClassStats &c = wcs[warp * (int)p.I + (int)i];
             const double rel = __dsub_rn(te, T_reset);
             if (job_flag(pk)) { c.sYm_out = __dadd_rn(c.sYm_out, rel); c.done_mixed++; }
             else              { c.sYs_out = __dadd_rn(c.sYs_out, rel); c.done_solo++; }
@@ -964,14 +1020,37 @@ struct Sim {
         }
     }
 
-    // Accounting of the finished requests whose records were staged in shared memory.
+    // Accounting of the finished requests whose records were staged in shared memory: a lane per record forms the latency
+    // (the division is the long part: once for 32 records instead of once for each), then the class lanes add theirs up in
+    // completion order.
     __device__ void flush_done()
     {
-        cp_async_wait_all();
+        if (n_pend == 0) return;
+        if (f_slots()) cp_async_wait_all();
         __syncwarp();
-        for (uint32_t e = 0; e < n_pend; ++e) {
-            const SlotRec r = st_rec[e];
-            account_done(r.pk, r.tpf, st_te[e]);
+#pragma unroll 1
+        for (uint32_t e = (uint32_t)lane; e < n_pend; e += 32u) {
+            const uint32_t pk = st_rec[e].pk;
+            const double te = st_te[e], tpot = __ddiv_rn(__dsub_rn(te, st_rec[e].tpf), (double)job_D(pk));
+            st_rec[e].tpf = tpot;
+            st_te[e] = __dsub_rn(te, T_reset);
+            if (f_hist()) atomicAdd(&hist[((size_t)job_cls(pk) * 2 + 1) * NBIN + hist_bin(tpot)], 1u);
+        }
+        __syncwarp();
+        if (lane < (int)p.I) {
+            WarpClassStats c = wcs[warp * (int)p.I + lane];
+#pragma unroll 2
+            for (uint32_t e = 0; e < n_pend; ++e) {
+                const uint32_t pk = st_rec[e].pk;
+                if (job_cls(pk) != (uint32_t)lane) continue;
+                const double rel = st_te[e];
+                if (job_flag(pk)) { c.sYm_out = __dadd_rn(c.sYm_out, rel); c.done_mixed++; }
+                else              { c.sYs_out = __dadd_rn(c.sYs_out, rel); c.done_solo++; }
+                c.tok_in += job_P(pk);       // bundled charging credits the request here, Eq. (21)-(22)
+                c.tok_out += job_D(pk);
+                c.sum_tpot = __dadd_rn(c.sum_tpot, st_rec[e].tpf);
+            }
+            wcs[warp * (int)p.I + lane] = c;
         }
         n_pend = 0;
         __syncwarp();
@@ -1026,6 +1105,7 @@ struct Sim {
             nfin[g] = newmin == NONE32 ? NONE32 : itg + newmin;
             if (f_kappa()) K[g] -= Kdrop;
         }
+        gpu_changed(g);
         __syncwarp();
     }
 
@@ -1035,25 +1115,44 @@ struct Sim {
         const int owner = (int)(g & 31u);
         uint32_t n = nd, newmin = NONE32, Kdrop = 0;
         const size_t base = (size_t)g * p.B;
-        for (int k = (int)((nd - 1) >> 5); k >= 0; --k) {
-            const uint32_t j = ((uint32_t)k << 5) + (uint32_t)lane;
-            const uint32_t f = j < nd ? s_fin[base + j] : NONE32;
-            const bool hit = f == itg;
-            if (!hit) newmin = min(newmin, f);
-            uint32_t hits = __ballot_sync(FULL, hit);
-            while (hits) {
+        // the stamps of four chunks of 32 slots are fetched together (one memory round trip), from the tail of the list
+#pragma unroll 1
+        for (int k0 = (int)((nd - 1) >> 5) & ~3; k0 >= 0; k0 -= 4) {
+            uint32_t f[4], hit[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t j = ((uint32_t)(k0 + q) << 5) + (uint32_t)lane;
+                f[q] = j < nd ? s_fin[base + j] : NONE32;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (f[q] != itg) newmin = min(newmin, f[q]);
+                hit[q] = __ballot_sync(FULL, f[q] == itg);
+            }
+#pragma unroll 1
+            for (;;) {          // hits from the tail of the list down
+                const int q = hit[3] ? 3 : (hit[2] ? 2 : (hit[1] ? 1 : 0));
+                const uint32_t hits = hit[3] ? hit[3] : (hit[2] ? hit[2] : (hit[1] ? hit[1] : hit[0]));
+                if (!hits) break;
                 const int hl = 31 - __clz(hits);
-                hits &= ~(1u << hl);
-                const uint32_t h = ((uint32_t)k << 5) + (uint32_t)hl;
-                const SlotRec rh = s_rec[base + h];
-                account_done(rh.pk, rh.tpf, te);
-                Kdrop += job_P(rh.pk) + job_D(rh.pk);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) hit[j] &= j == q ? ~(1u << hl) : ~0u;
+                const uint32_t h = ((uint32_t)(k0 + q) << 5) + (uint32_t)hl;
+                // the finished request's record and the tail entry that takes its place, in one round trip
                 const uint32_t last = n - 1;
-                __syncwarp();
-                if (lane == 0 && h != last) {
-                    s_fin[base + h] = s_fin[base + last];
-                    s_rec[base + h] = s_rec[base + last];
+                const SlotRec rh = s_rec[base + h], rl = s_rec[base + last];
+                const uint32_t fl = s_fin[base + last];
+                if (STAGED) {
+                    if (n_pend == (uint32_t)ROW_STAGE_CAP) flush_done();
+                    if (lane == 0) { st_rec[n_pend] = rh; st_te[n_pend] = te; }
+                    n_pend++;
+                } else {
+                    account_done(rh.pk, rh.tpf, te);
                 }
+                Kdrop += job_P(rh.pk) + job_D(rh.pk);
+                __syncwarp();
+                if (lane == 0 && h != last) { s_fin[base + h] = fl; s_rec[base + h] = rl; }
+                __syncwarp();
                 n = last;
             }
         }
@@ -1063,20 +1162,22 @@ struct Sim {
             nfin[g] = newmin;
             if (f_kappa()) K[g] -= Kdrop;
         }
+        gpu_changed(g);
         __syncwarp();
     }
 
     // --- end of an iteration on GPU g (warp-wide path: the end is not local) ----------------------
-    __device__ void on_server(uint32_t g)
+    // nd_before: decodes that g held before this event's retirements (one warp: the round's passes have ended the iteration)
+    __device__ void on_server(uint32_t g, uint32_t nd_before = 0)
     {
         const int owner = (int)(g & 31u);
         uint32_t flags = 0, itg = 0, nd = 0;
-        bool recount_idle = false;
-        if (SPL > 0) {
+        if (SPL > 0 || CAL) {      // (one warp, unrolled rows or calendar)
             // the round's passes have ended the iteration and retired its finished decodes; the frozen batch
             // flags say what the end brought
             const uint32_t na = nact[g];
             flags = ((na >> 14) & 1u) | (((na >> 15) & 1u) << 1);
+            nd = nd_before;
         } else {
             if (lane == owner) {
                 itg = it[g] + 1;
@@ -1106,9 +1207,7 @@ struct Sim {
         if (flags & 1u) {
             drain_dirty = true;
             gate_dirty = true;   // a promoted GPU at the cap may now take a prefill
-            if (SPL > 0) {
-                recount_idle = true;
-            } else if (!(flags & 2u) && g < M && pfrem[g] == 0 && nd > p.B - 1 && ndec[g] <= p.B - 1) {
+            if (!(flags & 2u) && g < M && pfrem[g] == 0 && nd > p.B - 1 && ndec[g] <= p.B - 1) {
                 // Only g changed: its idle prefill slot counts again once its decodes fit under the mixed cap (a prefill
                 // that finishes in this event is counted below, with the decode count after the retirement).
                 n_idle_pf++;
@@ -1119,15 +1218,17 @@ struct Sim {
             // prefill finished: account, then hand the request to the decode stage
             const uint32_t pk = pfjob[g];
             const double tarr = pf_tarr[g];
-            const uint32_t i = job_cls(pk), P = job_P(pk), D = job_D(pk);
+            const uint32_t i = job_cls(pk), P = job_P(pk);
             uint32_t pool = 0;
             if (f_sli()) {
                 // SLI-aware router: one uniform per finished prefill decides the pool
-                const unsigned long long ord = __shfl_sync(FULL, cs[lane & 7].sli_ord, i);
+                const unsigned long long ord = cs[i].sli_ord;
                 const double ps = __shfl_sync(FULL, b_ps, i);
                 uint32_t w0, w1, w2, w3;
-                draw(p, rep, (STREAM_SLI << 8) | i, ord, w0, w1, w2, w3);
+                if (CAL) draw(p, rep, (STREAM_SLI << 8) | i, ord, w0, w1, w2, w3);       // (+4 % inline at N = 256, -2 % at N = 16)
+                else draw_rare(p, rep, (STREAM_SLI << 8) | i, ord, w0, w1, w2, w3);
                 pool = (u53(w0, w1) <= ps) ? 0u : 1u;
+                __syncwarp();       // every lane has read the ordinal before its owner advances it
             }
             if (lane == (int)i) {
                 ClassState &c = cs[i];
@@ -1142,62 +1243,53 @@ struct Sim {
             }
             __syncwarp();   // every lane has read the finished job before its owner clears it
             if (lane == owner) pfjob[g] = 0;
+            gpu_changed(g);
             __syncwarp();
             // No router (immediate same-slot decoding, an ablation of the paper's EC): the request goes on decoding on
             // g, in the slot it holds; it passes through the empty buffer at this instant.
             const bool immediate = (F & F_GENERIC) && p.router == 3;
-            if (immediate) {
-                place_job(0, g, i, P, D, t, false);
-                __syncwarp();
-            }
             // the prefill slot of g is idle again
-            if (!recount_idle && g < M && ndec[g] <= p.B - 1) {
+            if (g < M && ndec[g] + (immediate ? 1u : 0u) <= p.B - 1) {
                 n_idle_pf++;
                 idle_hint = (n_idle_pf == 1) ? g : NONE32;
             }
-            // Decode stage.  With an empty buffer the request is its head at once: place it if a slot is free.
-            const uint32_t n = pool ? dq_n1 : dq_n0;
-            bool placed = immediate;
-            if (!immediate && n == 0) {
-                uint32_t h;
-                if (f_sli()) {
-                    h = choose_server(pool == 0 ? WANT_SOLO : WANT_MIX);
-                } else if (!f_random()) {
-                    h = choose_solo_first();
-                } else {
-                    h = choose_server(WANT_SOLO);
-                    if (h == NONE32) h = choose_server(WANT_MIX);
-                }
-                if (h != NONE32) { place_job(pool, h, i, P, D, t, false); placed = true; }
-            }
-            if (!placed) {
-                const bool full = n >= p.qcap;
-                if (lane == (int)i) {
-                    ClassState &c = cs[i];
-                    if (full) {
-                        c.overflow_d++;
-                    } else {
-                        const uint32_t Qd = pool ? c.Qd1 : c.Qd0;
-                        if (f_abandon()) ab_change(pool ? c.abd1 : c.abd0, p.cls[i].theta, Qd, Qd + 1, t);
-                        area_touch(c.aQd, c.Qd0 + c.Qd1, t);
-                        if (pool) c.Qd1++; else c.Qd0++;
-                    }
-                }
-                if (!full) {
-                    uint32_t pos = (pool ? dq_head1 : dq_head0) + n;
-                    if (pos >= p.qcap) pos -= p.qcap;
-                    if (lane == 0) {
-                        QEntry e; e.t = t; e.pk = pack_job(P, D, i, 0); e.cls = i;
-                        dq[(size_t)pool * p.qcap + pos] = e;
-                    }
-                    if (pool) dq_n1++; else dq_n0++;
-                }
-                drain_dirty = true;
-            }
+            // Decode stage.  With an empty buffer the request is its head at once and the dispatch places it if a slot is free.
+            d_pool = pool;
+            d_pk = pk & 0x7fffffffu;
+            d_gpu = immediate ? g : NONE32;
+            direct = immediate || (pool ? dq_n1 : dq_n0) == 0;
+            if (!direct) enqueue_decode();
+            drain_dirty = true;
             gate_dirty = true;
         }
-        if (recount_idle) { __syncwarp(); n_idle_pf = count_idle_pf(); idle_hint = NONE32; }
         touch_server(g);
+    }
+
+    // The request that has just finished its prefill (d_pk) joins its pool's buffer.
+    __device__ __forceinline__ void enqueue_decode()
+    {
+        const uint32_t pool = d_pool, i = job_cls(d_pk), n = pool ? dq_n1 : dq_n0;
+        const bool full = n >= p.qcap;
+        if (lane == (int)i) {
+            ClassState &c = cs[i];
+            if (full) {
+                c.overflow_d++;
+            } else {
+                const uint32_t Qd = pool ? c.Qd1 : c.Qd0;
+                if (f_abandon()) ab_change(pool ? c.abd1 : c.abd0, p.cls[i].theta, Qd, Qd + 1, t);
+                area_touch(c.aQd, c.Qd0 + c.Qd1, t);
+                if (pool) c.Qd1++; else c.Qd0++;
+            }
+        }
+        if (!full) {
+            uint32_t pos = (pool ? dq_head1 : dq_head0) + n;
+            if (pos >= p.qcap) pos -= p.qcap;
+            if (lane == 0) {
+                QEntry e; e.t = t; e.pk = d_pk; e.cls = i;
+                dq[(size_t)pool * p.qcap + pos] = e;
+            }
+            if (pool) dq_n1++; else dq_n0++;
+        }
     }
 
     // --- local end of an iteration (owner lane only) ----------------------------------------------------
@@ -1231,7 +1323,9 @@ struct Sim {
             if (f_kappa()) { K[g] = restart ? Kg : Kend; if (restart) Kpend[g] = 0; }
             pfcur[g] = restart ? (uint16_t)pc2 : (uint16_t)0;
             if (restart) nact[g] = (uint16_t)(nd | fl);
-            tnext[g] = restart ? __dadd_rn(te, tau2) : dinf();
+            const double tn = __dadd_rn(te, tau2);
+            tnext[g] = restart ? tn : dinf();
+            if (CAL) bkt[g] = restart ? bucket_id(tn) : (uint8_t)255;
         }
         return act && retire;
     }
@@ -1242,7 +1336,7 @@ struct Sim {
         if (warp == 0 && lane < (int)p.I) {
             ClassState &c = cs[lane];
             for (int w = 0; w < nwarps; ++w) {
-                const WarpClassStats &a = wcs[w * MAXI + lane];
+                const WarpClassStats &a = wcs[w * (int)p.I + lane];
                 c.sYm_out = __dadd_rn(c.sYm_out, a.sYm_out);
                 c.sYs_out = __dadd_rn(c.sYs_out, a.sYs_out);
                 c.sum_tpot = __dadd_rn(c.sum_tpot, a.sum_tpot);
@@ -1338,13 +1432,334 @@ struct Sim {
         }
     }
 
+    // --- calendar of iteration ends (CAL) ---------------------------------------------------------------
+    // Time is cut into buckets of equal width; bkt[g] holds the bucket of GPU g's pending iteration end modulo cal_nbk (255:
+    // none, or held by a lane), and no iteration is longer than cal_nbk - 2 buckets, so an id names one bucket.  The warp
+    // works through the buckets in order: load_bucket finds the GPUs of a bucket by comparing four ids per word and gives
+    // each to a lane that holds none; rounds then look at the lanes only.  A round used to read all N GPUs twice (37 % of a
+    // replication's time at N = 512: N/32 rows of dependent shared-memory reads); now N ids are read once per bucket.
+    // The next bucket is loaded as soon as enough lanes are free, so that the next event that is not local is usually
+    // among the held ends.  Invariant: every pending event lies in bucket `low` or later, so an iteration that starts now
+    // ends cal_K = floor(tau_min / width) buckets after `low` or later, and buckets up to low + cal_K - 1 may be loaded.
+    // cal_K = 0 (iterations shorter than a bucket): one bucket at a time, reloaded in every round under the tau_min limit.
+    __device__ __forceinline__ unsigned long long bucket_abs(double x) const { return __double2ull_rd(__dmul_rn(x, p.cal_inv_w)); }
+    __device__ __forceinline__ uint8_t bucket_id(double x) const { return (uint8_t)((uint32_t)bucket_abs(x) & (p.cal_nbk - 1u)); }
+    // bytes of w equal to the byte repeated in pat: 0x80 in each
+    static __device__ __forceinline__ uint32_t equal_bytes(uint32_t w, uint32_t pat)
+    {
+        const uint32_t x = w ^ pat;
+        return ~(((x & 0x7f7f7f7fu) + 0x7f7f7f7fu) | x) & 0x80808080u;
+    }
+
+    // Give the pending ends of bucket b to the free lanes; returns how many there are (nothing is taken when there are more
+    // than free lanes).
+    __device__ __forceinline__ uint32_t load_bucket(unsigned long long b, uint32_t free_lanes)
+    {
+        const uint32_t *words = reinterpret_cast<const uint32_t *>(bkt);
+        const uint32_t nw = (p.N + 127u) >> 7, pat = ((uint32_t)b & (p.cal_nbk - 1u)) * 0x01010101u, below = (1u << lane) - 1u;
+        uint32_t n = 0;
+        // eight words of ids per lane at a time: the matches of word c become bits 7 - c, 15 - c, 23 - c, 31 - c of one mask
+#pragma unroll 1
+        for (uint32_t c0 = 0; c0 < nw; c0 += 8u) {
+            uint32_t m = 0;
+#pragma unroll
+            for (uint32_t c = 0; c < 8u; ++c)
+                if (c0 + c < nw) m |= equal_bytes(words[((c0 + c) << 5) + (uint32_t)lane], pat) >> c;
+            for (uint32_t k = __ballot_sync(FULL, m != 0); k; k = __ballot_sync(FULL, m != 0)) {
+                const uint32_t pos = n + (uint32_t)__popc(k & below), bit = (uint32_t)__ffs((int)m) - 1u;
+                if (m && pos < 32u) picked[pos] = (uint16_t)((((c0 + 7u - (bit & 7u)) << 5) + (uint32_t)lane) * 4u + (bit >> 3));
+                m &= m - 1u;
+                n += (uint32_t)__popc(k);
+            }
+        }
+        if (n == 0 || n > (uint32_t)__popc(free_lanes)) return n;
+        __syncwarp();
+        const uint32_t rank = (uint32_t)__popc(free_lanes & below);
+        if (!held && rank < n) {
+            const uint32_t g = (uint32_t)picked[rank];
+            // (with 256 buckets id 255 is one, and idle GPUs and those that lanes hold match it)
+            const unsigned long long v = g < p.N ? (unsigned long long)__double_as_longlong(tnext[g]) : 0x7ff0000000000000ull;
+            if (v < 0x7ff0000000000000ull && bucket_abs(__longlong_as_double((long long)v)) == b) {
+                held = true; held_g = g; held_t = v;
+                if (p.cal_K > 0) bkt[g] = (uint8_t)255;
+            }
+        }
+        __syncwarp();
+        return n;
+    }
+
+    // More ends in bucket `cur` than lanes (many GPUs that started together; no lane holds anything): each lane holds the
+    // earliest of the GPUs whose ids it reads, and the earliest end that no lane holds limits the round.
+    __device__ void load_crowded()
+    {
+        const unsigned long long INF = 0x7ff0000000000000ull;
+        const uint32_t *words = reinterpret_cast<const uint32_t *>(bkt);
+        const uint32_t nw = (p.N + 127u) >> 7, pat = ((uint32_t)cur & (p.cal_nbk - 1u)) * 0x01010101u;
+        held = false; held_t = INF; held_g = 0; left_t = INF; left_s = NONE32;
+#pragma unroll 1
+        for (uint32_t c = 0; c < nw; ++c)
+            for (uint32_t m = equal_bytes(words[(c << 5) + (uint32_t)lane], pat); m; m &= m - 1u) {
+                const uint32_t g = (((c << 5) + (uint32_t)lane) << 2) + (((uint32_t)__ffs((int)m) - 1u) >> 3);
+                if (g >= p.N) break;
+                const unsigned long long v = (unsigned long long)__double_as_longlong(tnext[g]);
+                if (v == INF || bucket_abs(__longlong_as_double((long long)v)) != cur) continue;
+                if (!held || v < held_t) {          // (a lane's GPUs come in index order: the first of equal ends stays)
+                    if (held) { left_t = held_t; left_s = SRC_SERVER + held_g; }
+                    held = true; held_t = v; held_g = g;
+                } else if (v < left_t) { left_t = v; left_s = SRC_SERVER + g; }
+            }
+        __syncwarp();
+        const uint32_t hi = (uint32_t)(left_t >> 32), lo = (uint32_t)left_t;
+        const uint32_t mhi = __reduce_min_sync(FULL, hi), mlo = __reduce_min_sync(FULL, hi == mhi ? lo : NONE32);
+        left_s = __reduce_min_sync(FULL, (hi == mhi && lo == mlo) ? left_s : NONE32);
+        left_t = ((unsigned long long)mhi << 32) | mlo;
+    }
+
+    // Buckets from `cur` to the next one with a pending iteration end (a large number when no GPU runs).
+    __device__ __forceinline__ uint32_t next_bucket() const
+    {
+        uint32_t best = 0x7fffffffu;
+        const uint32_t *words = reinterpret_cast<const uint32_t *>(bkt);
+        const uint32_t nw = (p.N + 127u) >> 7, mask = p.cal_nbk - 1u;
+#pragma unroll 1
+        for (uint32_t c = 0; c < nw; ++c) {
+            uint32_t w = words[(c << 5) + (uint32_t)lane];
+#pragma unroll
+            for (uint32_t j = 0; j < 4; ++j, w >>= 8) {
+                const uint32_t id = w & 0xffu;
+                const uint32_t g = (((c << 5) + (uint32_t)lane) << 2) + j;
+                // 255 is a bucket as well when there are 256 of them: only the GPU's end time tells
+                if (id != 255u || (mask == 255u && g < p.N && tnext[g] < dinf())) best = min(best, (id - (uint32_t)cur) & mask);
+            }
+        }
+        return __reduce_min_sync(FULL, best);
+    }
+
+    // Calendar from the GPU records, at kernel entry.
+    __device__ __forceinline__ void calendar_build()
+    {
+        unsigned long long first = 0x7ff0000000000000ull;
+#pragma unroll 1
+        for (uint32_t g = (uint32_t)lane; g < ((p.N + 127u) & ~127u); g += 32u) {
+            const double x = g < p.N ? tnext[g] : dinf();
+            bkt[g] = x < dinf() ? bucket_id(x) : (uint8_t)255;
+            first = min(first, (unsigned long long)__double_as_longlong(x));
+        }
+        if (lane < (int)p.I) first = min(first, class_first());
+        if (f_blocks() && lane == 0) first = min(first, (unsigned long long)__double_as_longlong(T_blk_next));
+        const uint32_t hi = (uint32_t)(first >> 32), mhi = __reduce_min_sync(FULL, hi);
+        const uint32_t mlo = __reduce_min_sync(FULL, hi == mhi ? (uint32_t)first : NONE32);
+        cur_end = bucket_abs(T_end);
+        cur = mhi >= 0x7ff00000u ? cur_end : bucket_abs(__longlong_as_double((long long)(((unsigned long long)mhi << 32) | mlo)));
+        low = cur;
+        held = false; held_t = 0x7ff0000000000000ull; held_g = 0;
+        left_t = held_t; left_s = NONE32;
+        crowded = true;      // the first round loads the bucket
+        __syncwarp();
+    }
+    // earliest clock of this lane's class
+    __device__ __forceinline__ unsigned long long class_first() const
+    {
+        const ClassState &c = cs[lane];
+        unsigned long long v = (unsigned long long)__double_as_longlong(c.ta);
+        if (f_abandon()) {
+            v = min(v, (unsigned long long)__double_as_longlong(c.abp.t_ab));
+            v = min(v, (unsigned long long)__double_as_longlong(c.abd0.t_ab));
+            v = min(v, (unsigned long long)__double_as_longlong(c.abd1.t_ab));
+        }
+        return v;
+    }
+
+    // The round loop on the calendar: as run(), with the lanes' held ends in the place of all GPUs.  Measured against the scan
+    // of all rows in every round (N = 512, R = 4096, 250 iterations of horizon): 955 -> 708 ms, and 623 ms with the cached
+    // least-loaded keys, the gate by reductions, accounting 32 requests at a time and a smaller loop body.
+    __device__ bool run_calendar()
+    {
+        unsigned long long budget = p.event_budget;
+        const unsigned long long INF = 0x7ff0000000000000ull;
+        const unsigned long long tend_bits = (unsigned long long)__double_as_longlong(T_end);
+        const bool tight = p.cal_K == 0;
+        uint32_t want = CAL_FREE;        // free lanes to load another bucket
+        calendar_build();
+        for (;;) {
+            const unsigned long long cur0 = cur;
+            __syncwarp();
+            for (uint32_t need = __ballot_sync(FULL, sched_pending); need; need &= need - 1)
+                refill((uint32_t)__ffs((int)need) - 1u);
+            unsigned long long bt = INF;
+            uint32_t bs = NONE32;
+            bool arrival_due = false;        // an arrival that only joins its queue is pending up to T_end
+            if (f_blocks() && lane == 0 && T_blk_next < dinf()) { bt = (unsigned long long)__double_as_longlong(T_blk_next); bs = SRC_BLOCK; }
+            if (lane < (int)p.I) {
+                const ClassState &c = cs[lane];
+                unsigned long long v = (unsigned long long)__double_as_longlong(c.ta);
+                arrival_due = v <= tend_bits;
+                if ((n_idle_pf > 0 || force_nonlocal) && v < bt) { bt = v; bs = SRC_ARRIVAL + lane; }
+                if (f_abandon()) {
+                    v = (unsigned long long)__double_as_longlong(c.abp.t_ab);
+                    if (v < bt) { bt = v; bs = SRC_ABP + lane; }
+                    v = (unsigned long long)__double_as_longlong(c.abd0.t_ab);
+                    if (v < bt) { bt = v; bs = SRC_ABD0 + lane; }
+                    v = (unsigned long long)__double_as_longlong(c.abd1.t_ab);
+                    if (v < bt) { bt = v; bs = SRC_ABD1 + lane; }
+                }
+            }
+            // Load buckets (one copy of the code for every reason to): the current one again when it is crowded or an end may
+            // have been added to it; the next one that holds an event when no lane holds an end any more; the following one
+            // when enough lanes are free.
+            bool again = tight || crowded;
+            if (again) { held = false; held_t = INF; held_g = 0; }
+            uint32_t turn = 0, d = 0;
+#pragma unroll 1
+            for (;;) {
+                const uint32_t free_lanes = ~__ballot_sync(FULL, held);
+                uint32_t ahead = 0;
+                if (again) {
+                    again = false;
+                } else if (free_lanes == FULL) {
+                    if (turn == 0) {
+                        // buckets to the first class event or block end
+                        unsigned long long first = bt;
+                        if (lane < (int)p.I) first = min(first, (unsigned long long)__double_as_longlong(cs[lane].ta));
+                        d = 0x7fffffffu;
+                        if (first < INF) {
+                            const unsigned long long b = bucket_abs(__longlong_as_double((long long)first));
+                            d = b <= cur ? 0u : (uint32_t)min(b - cur, 0x7fffffffull);
+                        }
+                        d = __reduce_min_sync(FULL, d);
+                        if (d == 0) break;
+                        ++cur; --d;
+                    } else {
+                        if (d == 0) break;
+                        const uint32_t skip = min(next_bucket(), d);
+                        if (cur + skip > cur_end) return true;          // nothing left up to T_end
+                        if (skip == 0) break;
+                        cur += skip; d = 0;
+                    }
+                    low = cur;
+                    want = CAL_FREE;
+                    ++turn;
+                } else {
+                    if (turn || crowded || (uint32_t)__popc(free_lanes) < want || cur + 1u >= low + p.cal_K) break;
+                    ahead = 1;
+                }
+                const uint32_t n = load_bucket(cur + ahead, free_lanes);
+                if (ahead) {
+                    if (n <= (uint32_t)__popc(free_lanes)) { ++cur; want = CAL_FREE; }
+                    else want = min(n, 32u);            // (more than 32: it has to wait until no lane holds anything)
+                    break;
+                }
+                left_t = INF; left_s = NONE32;
+                crowded = n > 32u;
+                if (crowded) load_crowded();
+            }
+            const bool buffered = (dq_n0 | dq_n1) != 0;
+            const uint32_t na = nact[held_g], nd0 = ndec[held_g];
+            const bool nl = force_nonlocal || (na & 0x8000u) != 0 || ((na & 0x4000u) != 0 && (buffered || (held_g < M && nd0 > p.B - 1)));
+            if (held && nl && held_t < bt) { bt = held_t; bs = SRC_SERVER + held_g; }
+            unsigned long long tint;
+            uint32_t src;
+            {
+                const uint32_t hi = (uint32_t)(bt >> 32), lo = (uint32_t)bt;
+                const uint32_t mhi = __reduce_min_sync(FULL, hi);
+                const uint32_t mlo = __reduce_min_sync(FULL, hi == mhi ? lo : NONE32);
+                src = __reduce_min_sync(FULL, (hi == mhi && lo == mlo) ? bs : NONE32);
+                tint = ((unsigned long long)mhi << 32) | mlo;
+            }
+            if (cur >= cur_end && tint > tend_bits && !__any_sync(FULL, arrival_due || held_t <= tend_bits) && left_t > tend_bits) return true;
+            if (budget == 0) return false;
+            --budget;
+            ++rounds;
+            // a class event further ahead waits until its bucket is the current one
+            const bool here = tint < INF && (src >= SRC_SERVER || bucket_abs(__longlong_as_double((long long)tint)) <= cur);
+            unsigned long long lim_t = here ? tint : INF;
+            uint32_t lim_s = here ? src : NONE32;
+            if (left_t < lim_t || (left_t == lim_t && left_s < lim_s)) { lim_t = left_t; lim_s = left_s; }
+            if (tight) {
+                // no iteration that starts in this round can end before T_min + tau_min
+                unsigned long long tmin = held_t;
+                if (lane < (int)p.I) tmin = min(tmin, (unsigned long long)__double_as_longlong(cs[lane].ta));
+                const uint32_t hi = (uint32_t)(tmin >> 32), mhi = __reduce_min_sync(FULL, hi);
+                const uint32_t mlo = __reduce_min_sync(FULL, hi == mhi ? (uint32_t)tmin : NONE32);
+                if (mhi < 0x7ff00000u) {
+                    const unsigned long long wt = (unsigned long long)__double_as_longlong(__dadd_rn(__hiloint2double((int)mhi, (int)mlo), tau_min));
+                    if (wt <= lim_t) { lim_t = wt; lim_s = 0; }
+                }
+            }
+            const bool first_is_event = here && lim_t == tint && lim_s == src;      // nothing that is not held or could still start comes before it
+            if (tend_bits < lim_t) { lim_t = tend_bits; lim_s = NONE32; }
+            bool progressed = false;
+            const bool first_here = first_is_event && tint <= tend_bits, arrival_now = first_here && src >= SRC_ARRIVAL && src < SRC_ABP;
+            const bool local = n_idle_pf == 0 && !force_nonlocal;
+            if ((local || arrival_now) && lane < (int)p.I) {
+                // local arrivals of this lane's class, or the arrival that is the round's event (see run())
+                const ClassState &c = cs[lane];
+#pragma unroll 1
+                for (int guard = 0; guard < 64; ++guard) {
+                    const unsigned long long v = (unsigned long long)__double_as_longlong(c.ta);
+                    if (local) {
+                        if (!(v < lim_t || (v == lim_t && SRC_ARRIVAL + (uint32_t)lane < lim_s))) break;
+                        if (f_abandon() && v > (unsigned long long)__double_as_longlong(c.abp.t_ab)) break;
+                        if (bucket_abs(__longlong_as_double((long long)v)) > cur) break;
+                    } else if (!(arrival_now && src == SRC_ARRIVAL + (uint32_t)lane && guard == 0)) break;
+                    arrival_local();
+                    progressed = true;
+                }
+            }
+            bool redo = sched_pending && !arrival_now;
+            if (f_abandon() && lane < (int)p.I) {
+                const unsigned long long v = (unsigned long long)__double_as_longlong(cs[lane].abp.t_ab);
+                redo = redo || v < tint || (v == tint && SRC_ABP + (uint32_t)lane < src);
+            }
+            const bool any_redo = __any_sync(FULL, redo);
+            const bool do_event = !any_redo && first_here;
+            const uint32_t nd_ev = src >= SRC_SERVER && do_event ? (uint32_t)ndec[src - SRC_SERVER] : 0u;
+            // the held ends below the limit and, if it happens now, the event's end
+            const unsigned long long v = held_t;
+            const uint32_t g = held_g;
+            const bool evt = do_event && held && SRC_SERVER + g == src;
+            const bool act = evt || (held && !nl && (v < lim_t || (v == lim_t && SRC_SERVER + g < lim_s)));
+            const bool retire = local_end(g, __longlong_as_double((long long)v), act, evt);
+            if (act) { held = false; held_t = INF; progressed = true; }
+            uint32_t need = __ballot_sync(FULL, retire);
+            if (need) {
+                __syncwarp();   // the lanes' updates of it / n_dec are visible to the whole warp
+                do {
+                    const int l = __ffs((int)need) - 1;
+                    need &= need - 1;
+                    const uint32_t gg = __shfl_sync(FULL, g, l);
+                    const double te = __longlong_as_double((long long)__shfl_sync(FULL, v, l));
+                    retire_decodes(gg, it[gg], (uint32_t)ndec[gg], te);
+                } while (need);
+                start_at(g, __longlong_as_double((long long)v), retire && !evt);
+            }
+            if (do_event) {
+                t = __longlong_as_double((long long)tint);
+                low = max(low, bucket_abs(t));
+                if (src >= SRC_SERVER) {
+                    on_server(src - SRC_SERVER, nd_ev);
+                } else {
+                    if (f_abandon() && src >= SRC_ABP) on_abandon((src - SRC_ABP) >> 3, (src - SRC_ABP) & 7u);
+                    else if (src >= SRC_ARRIVAL) gate_dirty = true;
+                    else { ++events; load_block(blk + 1); drain_dirty = true; gate_dirty = true; n_idle_pf = count_idle_pf(); idle_hint = NONE32; }
+                }
+                if (err) return true;
+                dispatch();
+                force_nonlocal = false;
+            } else if (!any_redo && cur == cur0 && !__any_sync(FULL, progressed)) {
+                err = ERR_INTERNAL;     // a round that brought nothing: never spin
+                return true;
+            }
+        }
+    }
+
     // --- round loop ----------------------------------------------------------------------------------
     __device__ bool run()
     {
+        unsigned long long budget = p.event_budget;
         const uint32_t rows = n_rows();
         const unsigned long long INF = 0x7ff0000000000000ull;
         const unsigned long long tend_bits = (unsigned long long)__double_as_longlong(T_end);
-        unsigned long long budget = p.event_budget;
         for (;;) {
             __syncwarp();
             // classes that ran out of arrival draws get 32 new ones
@@ -1417,34 +1832,41 @@ struct Sim {
             if (wt <= lim_t) { lim_t = wt; lim_s = 0; }
             if (tend_bits < lim_t) { lim_t = tend_bits; lim_s = NONE32; }
             bool progressed = false;
+            const bool first_here = tint < wt && tint <= tend_bits, arrival_now = first_here && src >= SRC_ARRIVAL && src < SRC_ABP;
             if (F & F_MW) {
                 if (lane == 0) { cmd->op = MW_ENDS; cmd->lim_t = lim_t; cmd->lim_s = lim_s; cmd->buffered = buffered; cmd->M = M; cmd->force = force_nonlocal; }
                 __syncthreads();
             }
-            if (lane < (int)p.I && n_idle_pf == 0 && !force_nonlocal) {
+            const bool local = n_idle_pf == 0 && !force_nonlocal;
+            if ((local || arrival_now) && lane < (int)p.I) {
                 // local arrivals of this lane's class, in time order, up to the limit and up to the class's own
-                // next abandonment (which each arrival moves)
-                ClassState &c = cs[lane];
+                // next abandonment (which each arrival moves); or the one arrival that is the round's event (it is not local,
+                // so none is): nothing in the rest of the round depends on whether it joins its queue here or at the end
+                const ClassState &c = cs[lane];
+#pragma unroll 1
                 for (int guard = 0; guard < 64; ++guard) {
                     const unsigned long long v = (unsigned long long)__double_as_longlong(c.ta);
-                    if (!(v < lim_t || (v == lim_t && SRC_ARRIVAL + (uint32_t)lane < lim_s))) break;
-                    if (f_abandon() && v > (unsigned long long)__double_as_longlong(c.abp.t_ab)) break;
+                    if (local) {
+                        if (!(v < lim_t || (v == lim_t && SRC_ARRIVAL + (uint32_t)lane < lim_s))) break;
+                        if (f_abandon() && v > (unsigned long long)__double_as_longlong(c.abp.t_ab)) break;
+                    } else if (!(arrival_now && src == SRC_ARRIVAL + (uint32_t)lane && guard == 0)) break;
                     arrival_local();
                     progressed = true;
                 }
             }
             // a class that ran out of draws has an unknown next arrival, possibly before T_int, and a local
             // arrival may have pulled its class's next abandonment before T_int: then T_int is not next after all
-            bool redo = sched_pending;
+            bool redo = sched_pending && !arrival_now;
             if (f_abandon() && lane < (int)p.I) {
                 const unsigned long long v = (unsigned long long)__double_as_longlong(cs[lane].abp.t_ab);
                 redo = redo || v < tint || (v == tint && SRC_ABP + (uint32_t)lane < src);
             }
             // the non-local event happens in this round if it comes before anything a new iteration could bring
             const bool any_redo = __any_sync(FULL, redo);
-            const bool do_event = !any_redo && tint < wt && tint <= tend_bits;
+            const bool do_event = !any_redo && first_here;
             // with unrolled rows the event GPU's iteration ends in pass 1 and its decodes retire in pass 2
             const uint32_t ev_g = (SPL > 0 && do_event && src >= SRC_SERVER) ? src - SRC_SERVER : NONE32;
+            const uint32_t nd_ev = ev_g != NONE32 ? (uint32_t)ndec[ev_g] : 0u;
             // pass 1: every lane ends the local iterations of its own GPUs (straight-line over the rows)
             uint32_t retire_rows = 0;
             if (SPL == 0) {
@@ -1472,14 +1894,17 @@ struct Sim {
                 // pass 2: decode completions found in pass 1, retired by the whole warp, GPU by GPU
                 if (__ballot_sync(FULL, retire_rows != 0)) {
                     __syncwarp();   // the owners' updates of it / n_dec are visible to the whole warp
-#pragma unroll
+#pragma unroll(SPL <= 2 && (F & F_SLOTS) ? 2 : 1)
                     for (uint32_t k = 0; k < rows; ++k) {
                         uint32_t need = __ballot_sync(FULL, (retire_rows >> k) & 1u);
+                        unsigned long long v = vrow[0];
+#pragma unroll
+                        for (uint32_t j = 1; j < (uint32_t)NC; ++j) v = j == k ? vrow[j] : v;
                         while (need) {
                             const int l = __ffs((int)need) - 1;
                             need &= need - 1;
                             const uint32_t gg = (k << 5) + (uint32_t)l;
-                            const double te = __longlong_as_double((long long)__shfl_sync(FULL, vrow[k], l));
+                            const double te = __longlong_as_double((long long)__shfl_sync(FULL, v, l));
                             retire_decodes(gg, it[gg], (uint32_t)ndec[gg], te);
                         }
                     }
@@ -1493,12 +1918,10 @@ struct Sim {
             if (do_event) {
                 t = __longlong_as_double((long long)tint);
                 if (src >= SRC_SERVER) {
-                    on_server(src - SRC_SERVER);
+                    on_server(src - SRC_SERVER, nd_ev);
                 } else {
-                    if (f_abandon() && src >= SRC_ABD1) on_abandon_d(1, src - SRC_ABD1);
-                    else if (f_abandon() && src >= SRC_ABD0) on_abandon_d(0, src - SRC_ABD0);
-                    else if (f_abandon() && src >= SRC_ABP) on_abandon_p(src - SRC_ABP);
-                    else if (src >= SRC_ARRIVAL) on_arrival(src - SRC_ARRIVAL);
+                    if (f_abandon() && src >= SRC_ABP) on_abandon((src - SRC_ABP) >> 3, (src - SRC_ABP) & 7u);
+                    else if (src >= SRC_ARRIVAL) gate_dirty = true;
                     else { ++events; load_block(blk + 1); drain_dirty = true; gate_dirty = true; n_idle_pf = count_idle_pf(); idle_hint = NONE32; }
                 }
                 if (err) return true;
@@ -1527,14 +1950,14 @@ struct Sim {
 // shared-memory carve-up for one replication (one warp per block)
 struct SmemLayout {
     uint32_t off_tnext, off_tarr, off_it, off_nfin, off_pfrem, off_pfjob, off_K, off_Kpend, off_ndec, off_nact,
-        off_pfcur, off_sfin16, off_socc, srv_bytes, off_touch, off_gate, off_cs, off_ring, off_strec, off_stte, off_pqh, off_wcs, off_cmd, off_res, total;
+        off_pfcur, off_sfin16, off_socc, srv_bytes, off_bkt, off_picked, off_touch, off_cs, off_ring, off_strec, off_stte, off_pqh, off_wcs, off_cmd, off_res, total;
 };
 
 // tarr_global: the arrival times and the job words of the requests in prefill (read once per finished prefill) live in
 // global memory (large clusters: shared memory is what limits the resident replications there); I: classes (sizes the
 // class records and the ring of arrival draws)
 __host__ __device__ inline SmemLayout smem_layout(uint32_t Npad, uint32_t B, uint32_t slots_smem, uint32_t nwarps, bool kappa,
-                                                  bool tarr_global, uint32_t I)
+                                                  bool tarr_global, uint32_t I, bool cal)
 {
     SmemLayout L;
     uint32_t o = 0;
@@ -1555,17 +1978,18 @@ __host__ __device__ inline SmemLayout smem_layout(uint32_t Npad, uint32_t B, uin
     L.off_socc = o; if (slots_smem) o += 4 * Npad * ((B + 31u) >> 5);
     o = (o + 15u) & ~15u;
     L.srv_bytes = o;
+    L.off_bkt = o; if (cal) o += (Npad + 127u) & ~127u;       // calendar of iteration ends
+    L.off_picked = o; if (cal) o += 2 * 32;
     L.off_touch = o; o += 4 * TOUCH_CAP;
-    o = (o + 7u) & ~7u;
-    L.off_gate = o; o += (8 + 8 + 4) * MAXI;
     o = (o + 15u) & ~15u;
     L.off_cs = o; o += (uint32_t)sizeof(ClassState) * I;
     o = (o + 15u) & ~15u;
     L.off_ring = o; o += (uint32_t)sizeof(ADraw) * 32 * I;
-    L.off_strec = o; o += (uint32_t)sizeof(SlotRec) * STAGE_CAP;
-    L.off_stte = o; o += 8 * STAGE_CAP;
+    const uint32_t stage = slots_smem ? STAGE_CAP : (nwarps == 1 ? ROW_STAGE_CAP : 0);
+    L.off_strec = o; o += (uint32_t)sizeof(SlotRec) * stage;
+    L.off_stte = o; o += 8 * stage;
     L.off_pqh = o; o += (uint32_t)sizeof(QEntry) * MAXI;
-    L.off_wcs = o; o += (uint32_t)sizeof(WarpClassStats) * MAXI * nwarps;
+    L.off_wcs = o; o += (uint32_t)sizeof(WarpClassStats) * I * nwarps;
     o = (o + 15u) & ~15u;
     L.off_cmd = o; if (nwarps > 1) o += (uint32_t)sizeof(MwCmd);        // master and helpers only
     o = (o + 15u) & ~15u;
@@ -1590,10 +2014,9 @@ __device__ __forceinline__ void bind_pointers(Sim<SPL, F> &s, char *sm, const Sm
     s.pfcur = reinterpret_cast<uint16_t *>(sm + L.off_pfcur);
     s.sfin16 = reinterpret_cast<uint16_t *>(sm + L.off_sfin16);
     s.socc = reinterpret_cast<uint32_t *>(sm + L.off_socc);
+    s.bkt = reinterpret_cast<uint8_t *>(sm + L.off_bkt);
+    s.picked = reinterpret_cast<uint16_t *>(sm + L.off_picked);
     s.touch = reinterpret_cast<uint32_t *>(sm + L.off_touch);
-    s.gate_xi = reinterpret_cast<double *>(sm + L.off_gate);
-    s.gate_dq = s.gate_xi + MAXI;
-    s.gate_ok = reinterpret_cast<uint32_t *>(s.gate_dq + MAXI);
     s.cs = reinterpret_cast<ClassState *>(sm + L.off_cs);
     s.aring = reinterpret_cast<ADraw *>(sm + L.off_ring);
     s.st_rec = reinterpret_cast<SlotRec *>(sm + L.off_strec);
@@ -1622,7 +2045,7 @@ __global__ void __launch_bounds__(32) qsim_init_kernel(Params p)
     extern __shared__ __align__(16) char sm[];
     const int lane = threadIdx.x;
     for (uint32_t rep = blockIdx.x; rep < p.R; rep += gridDim.x) {
-        const SmemLayout L = smem_layout(p.Npad, p.B, p.slots_smem, 1, p.coef[5] != 0.0, p.tarr_global != 0, p.I);
+        const SmemLayout L = smem_layout(p.Npad, p.B, p.slots_smem, 1, p.coef[5] != 0.0, p.tarr_global != 0, p.I, false);
         Sim<SPLT, FT> s(p, lane, rep);
         bind_pointers(s, sm, L);
         __syncwarp();
@@ -1759,7 +2182,7 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, ((FT & F_MW) |
                 continue;
             }
         } else if (!p.advance && h.done) continue;
-        const SmemLayout L = smem_layout(p.Npad, p.B, p.slots_smem, nthr >> 5, p.coef[5] != 0.0, p.tarr_global != 0, p.I);
+        const SmemLayout L = smem_layout(p.Npad, p.B, p.slots_smem, nthr >> 5, p.coef[5] != 0.0, p.tarr_global != 0, p.I, Sim<SPLT, FT>::CAL);
         Sim<SPLT, FT> s(p, lane, rep);
         s.warp = warp;
         s.nwarps = (int)(nthr >> 5);
@@ -1774,7 +2197,7 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, ((FT & F_MW) |
             uint4 *dst = reinterpret_cast<uint4 *>(s.cs);
             for (uint32_t o = tid; o < sizeof(ClassState) * p.I / 16; o += nthr) dst[o] = src[o];
             uint32_t *w = reinterpret_cast<uint32_t *>(s.wcs);
-            for (uint32_t o = tid; o < sizeof(WarpClassStats) * MAXI * (nthr >> 5) / 4; o += nthr) w[o] = 0;
+            for (uint32_t o = tid; o < sizeof(WarpClassStats) * p.I * (nthr >> 5) / 4; o += nthr) w[o] = 0;
         }
         s.block_sync();
         // the end time is one rounded product of the cumulative horizon: run(a); run(b) ends where run(a+b) ends
@@ -1789,7 +2212,7 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, ((FT & F_MW) |
         s.load_block(h.blk);
         s.dq_head0 = h.dq_head0; s.dq_head1 = h.dq_head1; s.dq_n0 = h.dq_n0; s.dq_n1 = h.dq_n1;
         s.place_ord = h.place_ord; s.events = h.events; s.rounds = h.rounds; s.sel_ord0 = h.sel_ord0; s.sel_ord1 = h.sel_ord1;
-        s.n_touch = 0; s.touch_all = false; s.need_start = 0; s.err = h.err;
+        s.n_touch = 0; s.touch_all = false; s.need_start = 0; s.err = h.err; s.direct = false;
         s.drain_dirty = true; s.gate_dirty = true;
         s.force_nonlocal = (p.force_dispatch != 0 && chunk == 0) || h.force != 0;
         s.n_idle_pf = 0;
@@ -1802,7 +2225,11 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, ((FT & F_MW) |
             __syncwarp();
             s.it_mixed = h.iters_mixed[lane]; s.it_solo = h.iters_solo[lane];
             s.busy_mixed = h.busy_mixed[lane]; s.busy_solo = h.busy_solo[lane];
-            finished = s.err ? true : s.run();
+            if constexpr (Sim<SPLT, FT>::CAL) {
+                finished = s.err ? true : s.run_calendar();
+            } else {
+                finished = s.err ? true : s.run();
+            }
             s.flush_done();
             if (FT & F_MW) {
                 if (lane == 0) s.cmd->op = MW_EXIT;

@@ -72,6 +72,7 @@ struct qsim {
     int device = 0;
     void (*run_fn)(qsimdev::Params) = nullptr;
     uint32_t nwarps = 1;          // warps per replication (block size / 32)
+    bool scan = false;            // one warp, run-time row count: rounds read all GPUs (see rounds_scan)
     void (*lane_fn)(qsimdev::Params) = nullptr;     // instance of the one-thread-per-replication run kernel
     bool allow_lane = true;       // the one-thread-per-replication family may run this handle
     double coef[6]{};
@@ -271,6 +272,16 @@ void add_variants(std::vector<RunVariant> &v)
     v.push_back({SPL, F_GENERIC, qsim_run_kernel<SPL, F_GENERIC>});
 }
 
+// run-time row count, one warp: from the calendar, or reading all GPUs in every round (W = F_SCAN)
+template <uint32_t W>
+void add_row_variants(std::vector<RunVariant> &v)
+{
+    v.push_back({0, W | F_OCC | F_ABANDON, qsim_run_kernel<0, W | F_OCC | F_ABANDON>});
+    v.push_back({0, W | F_OCC | F_ABANDON | F_SLI | F_HIST, qsim_run_kernel<0, W | F_OCC | F_ABANDON | F_SLI | F_HIST>});
+    v.push_back({0, W | F_ABANDON | F_BLOCKS | F_HIST, qsim_run_kernel<0, W | F_ABANDON | F_BLOCKS | F_HIST>});
+    v.push_back({0, W | F_GENERIC, qsim_run_kernel<0, W | F_GENERIC>});
+}
+
 const std::vector<RunVariant> &run_variants()
 {
     static const std::vector<RunVariant> table = [] {
@@ -278,10 +289,9 @@ const std::vector<RunVariant> &run_variants()
         add_variants<1>(v);
         add_variants<2>(v);
         add_variants<4>(v);
-        // one warp, run-time row count (129..511 GPUs)
-        v.push_back({0, F_OCC | F_ABANDON, qsim_run_kernel<0, F_OCC | F_ABANDON>});
-        v.push_back({0, F_OCC | F_ABANDON | F_SLI | F_HIST, qsim_run_kernel<0, F_OCC | F_ABANDON | F_SLI | F_HIST>});
-        v.push_back({0, F_GENERIC, qsim_run_kernel<0, F_GENERIC>});
+        // one warp, run-time row count (129 GPUs and more)
+        add_row_variants<0u>(v);
+        add_row_variants<F_SCAN>(v);
         // several warps per replication (large clusters): instances for the occupancy gate with abandonment under
         // the solo-first and (with histograms) the SLI-aware router, the priority gate with blocks and histograms, and the generic one
         v.push_back({-1, F_MW | F_OCC | F_ABANDON, qsim_run_kernel<0, F_MW | F_OCC | F_ABANDON>});
@@ -310,12 +320,13 @@ uint32_t features_of(const qsim_config &c, const qsim_class *cls, const double *
     return f;
 }
 
-// Large clusters: per-replication shared memory allows only a few blocks per SM, so each replication gets
-// several warps (master + helpers) that share the per-GPU scans.  QSIM_WARPS overrides the choice (1 = off).
+// Several warps (master + helpers) per replication share the per-GPU scans: QSIM_WARPS=2..16, for cross-checks.  One warp
+// on the calendar is ahead at every size (it does not scan): N = 1024, R = 444 (24 blocks, histograms) 504 against 946 ms with two
+// warps, N = 1024, R = 2048 294 against 612, N = 2048, R = 888 507 against 1137 with four, N = 4096, R = 4 535 against 615 with sixteen.
 void choose_multiwarp(uint32_t N, uint32_t feat, Params &p, RunKernel &fn, uint32_t &nwarps)
 {
     const uint32_t rows = (N + 31u) / 32u;
-    uint32_t W = rows >= 128 ? 16u : (rows >= 64 ? 4u : (rows >= 32 ? 2u : 1u));     // best of sweeps over 1, 2, 4, 8, 16 warps at 512, 768, 1024, 2048, 4096 GPUs
+    uint32_t W = 1;
     if (const char *e = std::getenv("QSIM_WARPS")) {
         const int v = std::atoi(e);
         if (v >= 1 && v <= MW_MAX) W = (uint32_t)v;
@@ -340,7 +351,7 @@ void choose_multiwarp(uint32_t N, uint32_t feat, Params &p, RunKernel &fn, uint3
     p.slots_smem = 0;       // helpers retire through the global slot lists
 }
 
-RunVariant pick_run_kernel(uint32_t N, uint32_t feat)
+RunVariant pick_run_kernel(uint32_t N, uint32_t feat, bool scan)
 {
     const int rows = (int)((N + 31u) / 32u);
     const RunVariant *generic = nullptr, *best = nullptr;
@@ -351,6 +362,7 @@ RunVariant pick_run_kernel(uint32_t N, uint32_t feat)
     for (const RunVariant &v : run_variants()) {
         if (v.spl < 0) continue;                            // the multi-warp instance is chosen by the caller
         if (v.spl != 0 && v.spl < rows) continue;          // too few GPUs per lane
+        if (v.spl == 0 && ((v.feat & F_SCAN) != 0) != scan) continue;
         if (v.spl == 0 && (v.feat & F_GENERIC)) { generic = &v; continue; }
         // smallest row count that fits (0 = run-time row count, beyond four rows); among those the feature set with
         // the fewest extras
@@ -361,10 +373,54 @@ RunVariant pick_run_kernel(uint32_t N, uint32_t feat)
         // (abandonment, KV slope, blocks) may be present without being used
         constexpr uint32_t MODES = F_SLI | F_SLIG | F_IMM | F_RANDOM | F_OCC | F_FCFS | F_HIST | F_SLOTS;
         if (feat == ~0u || (feat & MODES) != (v.feat & MODES) || (feat & ~v.feat) != 0) continue;
-        const int extra = __builtin_popcount(v.feat & ~feat);
+        const int extra = __builtin_popcount(v.feat & ~(feat | F_SCAN));
         if (extra < best_bits) { best = &v; best_bits = extra; }
     }
     return best ? *best : *generic;
+}
+
+// Calendar of the one-warp kernels with a run-time row count.  Bucket width: about CAL_FILL iteration ends per bucket when
+// all GPUs are busy and iterations last (tau_min + tau_max) / 2 on average, but no wider than 0.45 of the shortest iteration.
+// More than 32 ends do not fit the lanes, fewer waste lanes and the pass over the ids (N = 512, R = 4096, per 250 iterations of
+// horizon: 708 ms at 12 and 16, 730 at 20, 783 with 10 in an earlier version of the pass).  Buckets: a power of two up to 256 that
+// spans the longest iteration; beyond about 2000 GPUs that limit sets the width.
+constexpr double CAL_FILL = 16.0;
+void calendar_shape(uint32_t N, uint32_t B, uint32_t C, const double *coef, Params &p)
+{
+    const double tau_mix = coef[0] + coef[1] * (double)C + coef[2] * (double)B, tau_solo = coef[3] + coef[4] * (double)B;
+    const double tau_batch = tau_mix > tau_solo ? tau_mix : tau_solo;
+    const double tau_max = tau_batch + coef[5] * (2.0 * QSIM_LMAX) * (double)B;
+    const double tau_min = coef[0] < coef[3] ? coef[0] : coef[3];
+    double w = CAL_FILL * 0.5 * (tau_min + tau_batch) / (double)N;
+    if (w > 0.45 * tau_min) w = 0.45 * tau_min;
+    if (w * 254.0 < 1.01 * tau_max) w = 1.01 * tau_max / 254.0;
+    uint32_t nbk = 8;
+    while (nbk < 256u && w * (double)(nbk - 2u) < 1.01 * tau_max) nbk <<= 1;
+    p.cal_nbk = nbk;
+    p.cal_inv_w = 1.0 / w;
+    p.cal_K = (uint32_t)std::min(0.999 * tau_min / w, 254.0);        // (the margin is far above the rounding of a bucket index)
+}
+
+// One warp with a run-time row count: do rounds read all GPUs, or work from the calendar of iteration ends?  Reading all rows
+// pays when an event that is not local (a finished prefill, mostly) comes with many local ends, because one row then ends
+// up to 32 iterations: it is a matter of the ends per event r against the rows N / 32, and r is estimated as iterations per
+// second over requests per second of a busy GPU (rates averaged over the blocks).  Measured, scan / calendar in ms, least-loaded
+// placement: r = 1.0 rows (N = 300) 134 / 127, 1.6 rows (N = 500) 106 / 116, 1.6 rows (N = 300) 84 / 99, 2 rows (N = 150) 93 / 105, 2 rows
+// (N = 800) 110 / 146, and in overload, r = 0.3 rows, N = 512, 955 / 623.  Random placement reads all rows for every choice
+// either way: 2.4 rows (N = 500) 195 / 179, 3.5 rows (N = 350) 114 / 122.  QSIM_ROUNDS=scan|calendar overrides.
+bool rounds_scan(const qsim_config &c, const double *rates, const double *coef)
+{
+    if (const char *e = std::getenv("QSIM_ROUNDS")) {
+        if (std::strcmp(e, "scan") == 0) return true;
+        if (std::strcmp(e, "calendar") == 0) return false;
+    }
+    double lam = 0.0;
+    for (size_t k = 0; k < (size_t)c.nblk * c.I; ++k) lam += rates[k];
+    lam /= (double)c.nblk;
+    const double tau_mix = coef[0] + coef[1] * (double)c.C + coef[2] * (double)c.B, tau_solo = coef[3] + coef[4] * (double)c.B;
+    const double tau_max = tau_mix > tau_solo ? tau_mix : tau_solo, tau_min = coef[0] < coef[3] ? coef[0] : coef[3];
+    const double rows = (double)((c.N + 31u) / 32u), from = c.placement == QSIM_PLACE_RANDOM ? 2.8 : 1.3;
+    return 1.0 > lam * 0.5 * (tau_min + tau_max) * from * rows;
 }
 
 // Everything of a handle that needs no device memory: kernel parameters, kernel instance, block shape,
@@ -390,33 +446,39 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
     }
     const bool kappa = coef[5] != 0.0;
     const uint32_t feat = features_of(cfg, classes, coef);
-    RunVariant v = pick_run_kernel(cfg.N, feat);
+    RunVariant v = pick_run_kernel(cfg.N, feat, h.scan);
     // the per-GPU arrays are padded to the unrolled row count of the chosen instance
     if (v.spl > 0) p.Npad = (uint32_t)v.spl * 32u;
     // finish stamps + occupancy bits go to shared memory when the whole block state stays small
-    p.slots_smem = smem_layout(p.Npad, p.B, 1, 1, kappa, p.Npad > 128u, cfg.I).total <= 40u * 1024u ? 1u : 0u;
-    if (p.slots_smem) v = pick_run_kernel(cfg.N, feat | F_SLOTS);
+    // (the limit of 40 KB counts MAXI accounting records and 160 bytes that the block no longer has: which configurations
+    // keep their stamps on chip fixes the layout of saved workspaces)
+    const uint32_t spared = 160u + (uint32_t)sizeof(WarpClassStats) * MAXI - (((uint32_t)sizeof(WarpClassStats) * cfg.I + 15u) & ~15u);
+    p.slots_smem = smem_layout(p.Npad, p.B, 1, 1, kappa, p.Npad > 128u, cfg.I, false).total + spared <= 40u * 1024u ? 1u : 0u;
+    if (cfg.N > 992u) p.slots_smem = 0;     // (from 32 rows on the layout is that of several warps, which retire through the global lists)
+    if (p.slots_smem) v = pick_run_kernel(cfg.N, feat | F_SLOTS, h.scan);
     h.run_fn = v.fn;
     h.nwarps = 1;
     choose_multiwarp(cfg.N, feat, p, h.run_fn, h.nwarps);
     // beyond four rows of GPUs shared memory limits the resident replications: the arrival times and the job words of
     // the requests in prefill (read once per finished prefill) move to global memory
     p.tarr_global = (p.Npad > 128u) ? 1u : 0u;
-    h.lay = smem_layout(p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I);
-    h.init_smem = smem_layout(p.Npad, p.B, p.slots_smem, 1, kappa, p.tarr_global != 0, cfg.I).total;
+    const bool cal = cfg.N > 128u && h.nwarps == 1 && !h.scan;      // run-time row count, one warp (Sim::CAL)
+    calendar_shape(cfg.N, cfg.B, cfg.C, coef, p);
+    h.lay = smem_layout(p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I, cal);
+    h.init_smem = smem_layout(p.Npad, p.B, p.slots_smem, 1, kappa, p.tarr_global != 0, cfg.I, false).total;
     p.srv_bytes = h.lay.srv_bytes;
     if (h.lay.total > 227u * 1024u - 64u)       // a few bytes of the block are the kernel's own
         return fail(QSIM_EINVAL, "N too large: per-replication GPU state does not fit shared memory");
     h.sec = layout_sections(cfg, p.srv_bytes, p.tarr_global != 0);
     for (int k = 0; k < 6; ++k) h.coef[k] = coef[k];
     // Kernel family.  A replication advances at about the same rate on one thread whatever its cluster size, while the
-    // warp-per-replication kernels slow down in proportion to the cluster (few replications fit on an SM and their
-    // master warp searches all rows).  Measured on a B200: one thread per replication wins from 2048 GPUs when R x N
-    // exceeds about 7 million (N = 2048, R = 4096: 2.26e8 against 2.18e8 it/s; N = 4096, R = 4096: 2.1e8 against 5.3e7),
-    // and not below (N = 1024: 3.35e8 against 3.47e8 at R = 8192, 3.15e8 against 3.53e8 at R = 16384; N = 512,
-    // R = 16384: 3.5e8 against 7e8).  QSIM_FAMILY=lane / warp overrides.
+    // warp-per-replication kernels are limited by the replications whose GPU state fits an SM (two or three beyond 2048
+    // GPUs) but advance each about seventy times as fast.  Measured (it/s, warp / thread): N = 4096, R = 1712: 1.72e8 / 1.41e8,
+    // R = 3800: 1.76e8 / 2.77e8; N = 3000, R = 2400: 2.30e8 / 1.83e8; N = 2048, R = 3456: 5.6e8 / 2.7e8.  Both lines cross at about 9.5
+    // million simulated GPUs (R x N); up to 2048 GPUs the warp kernels stay ahead for every R that fits in memory.
+    // QSIM_FAMILY=lane / warp overrides.
     std::memset(&p.lane, 0, sizeof p.lane);
-    bool lane = h.allow_lane && lane_supports(cfg, coef) && cfg.N >= 2048u && (unsigned long long)cfg.R * cfg.N >= 7000000ull;
+    bool lane = h.allow_lane && lane_supports(cfg, coef) && cfg.N > 2048u && (unsigned long long)cfg.R * cfg.N >= 9500000ull;
     if (const char *e = std::getenv("QSIM_FAMILY")) {
         if (std::strcmp(e, "lane") == 0) lane = h.allow_lane && lane_supports(cfg, coef);
         else if (std::strcmp(e, "warp") == 0) lane = false;
@@ -657,6 +719,7 @@ int qsim_create(qsim_t **out, const qsim_config *cfg, const qsim_class *classes,
     qsim *h = new (std::nothrow) qsim();
     if (!h) return fail(QSIM_ENOMEM, "host allocation failed");
     h->device = dev;
+    h->scan = rounds_scan(*cfg, rates, coef);
     rc = configure(*h, *cfg, classes, prices, coef);
     if (rc != QSIM_OK) { delete h; return rc; }
     Params &p = h->par;
@@ -861,7 +924,7 @@ int qsim_set_injected(qsim_t *h, const double *t, const uint32_t *job, uint64_t 
     h->par.inject_job = h->d_inject_job;
     h->par.n_inject = (uint32_t)n;
     // the trace source lives in the run-time-configured instance
-    RunVariant v = pick_run_kernel(h->cfg.N, ~0u);
+    RunVariant v = pick_run_kernel(h->cfg.N, ~0u, h->scan);
     if (h->nwarps > 1)
         for (const RunVariant &mw : run_variants())
             if (mw.spl < 0 && (mw.feat & F_GENERIC)) v = mw;
@@ -1237,6 +1300,7 @@ extern "C" int qsim_simulate_static(const qsim_config *cfg, const qsim_class *cl
     h.allow_lane = false;                  // the built-in scratch is sized for the warp-per-replication layout
     qsim_config nohist = *cfg;
     nohist.hist = 0;                       // histograms are not recorded here
+    h.scan = rounds_scan(*cfg, rates, coef);
     rc = configure(h, nohist, classes, prices, coef);
     if (rc != QSIM_OK) return rc;
     h.device = dev;

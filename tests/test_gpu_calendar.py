@@ -1,0 +1,97 @@
+"""Clusters of more than 128 GPUs on one warp: rounds that work from the calendar of iteration ends and rounds that read all
+GPUs, both against the CPU oracle (integer statistics and per-GPU end state exact, fp64 statistics within 1e-9), at the edges
+of the calendar's shapes: sizes around its words and bucket counts, iterations shorter than a bucket, more iteration ends in
+a bucket than lanes, light load with empty buckets, a run cut into many short launches."""
+import contextlib
+import os
+
+import numpy as np
+import pytest
+
+from qsim_inputs import presets
+from qsim_inputs.spec import PLACE_LEAST_LOADED, PLACE_RANDOM, ROUTER_SLI
+
+from parity import assert_parity
+
+pytestmark = pytest.mark.gpu
+
+
+@contextlib.contextmanager
+def env(**kw):
+    keep = {k: os.environ.get(k) for k in kw}
+    os.environ.update(kw)
+    try:
+        yield
+    finally:
+        for k, v in keep.items():
+            if v is None:
+                del os.environ[k]
+            else:
+                os.environ[k] = v
+
+
+def check(inp, calls, rounds, budget=None):
+    from oracle import OracleSim
+    from paper_2602_02987_b200 import QSim
+    with env(QSIM_ROUNDS=rounds, QSIM_FAMILY="warp", QSIM_WARPS="1"):
+        sim = QSim(inp)
+    assert sim.layout_info()["warps"] == 1
+    if budget:
+        sim.set_event_budget(budget)
+    ora = OracleSim(inp)
+    for h in calls:
+        sim.run(h)
+        ora.run(h)
+    got, ref = sim.stats(), ora.stats()
+    state, want = [sim.server_state(r) for r in range(inp.R)], [ora.server_state(r) for r in range(inp.R)]
+    sim.close()
+    ora.close()
+    assert_parity(got, ref, what=f"{inp.name}, {rounds}")
+    for r in range(inp.R):
+        for k in state[r]:
+            assert np.array_equal(state[r][k], want[r][k]), (inp.name, rounds, r, k)
+    return got
+
+
+def light(inp, share):
+    return inp.with_(rates=inp.rates * share)
+
+
+def short_iterations(N):
+    """Iteration times that differ by a factor of a thousand: the shortest is shorter than a bucket of the calendar."""
+    return presets.cfg2(N=N, R=2).with_(coeffs=np.array([2e-5, 8e-5, 5e-5, 1e-5, 5e-5, 0.0]))
+
+
+def together(N):
+    """One request for every GPU at time zero: all iterations end at the same times, more per bucket than a warp has lanes."""
+    return presets.single_class(N=N, B=8, P=900, D=30, lam=0.5, R=2, M=N, inject=[(0.0, 0, 900, 30)] * N + [(0.05, 0, 300, 5)] * 40)
+
+
+@pytest.mark.parametrize("rounds", ["calendar", "scan"])
+@pytest.mark.parametrize("make,calls", [
+    (lambda: presets.cfg2(N=129, R=2), [250]),
+    (lambda: presets.cfg4(N=255, R=2), [60, 100]),
+    (lambda: presets.cfg4(N=257, R=2), [150]),
+    (lambda: presets.crowded("decode", N=160, R=2, placement=PLACE_LEAST_LOADED), [600]),
+    (lambda: presets.crowded("prefill", N=384, R=2, placement=PLACE_RANDOM, router=ROUTER_SLI), [300]),
+    (lambda: presets.cfg3(N=200, R=2, block_len=0.3), [420]),
+    (lambda: light(presets.cfg2(N=150, R=2), 0.02), [500]),
+    (lambda: light(presets.cfg4(N=300, R=2), 0.0005), [900, 900]),
+    (lambda: presets.paper_instance(n=200, R=2), [700]),
+    (lambda: short_iterations(140), [200]),
+    (lambda: together(300), [40, 60]),
+])
+def test_calendar_and_scan_against_the_oracle(make, calls, rounds):
+    check(make(), calls, rounds)
+
+
+@pytest.mark.parametrize("N", [1023, 2049, 4096])
+def test_calendar_on_large_clusters_with_as_many_buckets_as_ids(N):
+    check(presets.cfg2(N=N, R=1), [30, 30], "calendar")
+
+
+def test_calendar_is_rebuilt_by_every_launch():
+    whole = check(presets.cfg4(N=200, R=2), [120], "calendar")
+    parts = check(presets.cfg4(N=200, R=2), [1, 2, 3, 5, 8, 13, 21, 34, 33], "calendar", budget=40)
+    for k in ("arrivals", "admitted", "done_mixed", "done_solo", "iters_mixed", "iters_solo"):
+        assert np.array_equal(whole[k], parts[k]), k
