@@ -3,17 +3,22 @@
 // qsim_device.cuh).
 //
 // Requests of a class are exchangeable here, so a replication is a handful of integers per class plus the
-// class order of its decode buffers: one THREAD simulates one replication, and a warp advances 32
-// replications at once.  Every class has seven unit-rate Poisson processes (arrivals, abandonment from the
-// prefill queue, abandonment from each decode buffer, prefill completions, mixed and solo decode
-// completions) that run on the integrated intensities of Eq. (7)-(9): a process with intensity c n(t) keeps
-// the integral acc of c n since its last jump and the exponential level lvl of its next jump, and its jump
-// time is recomputed whenever n changes.  Per event a thread scans its 7 I jump times, applies the jump,
-// lets the policy act (decode buffers into free slots, solo group first; then the prefill gate) and updates
-// the clocks whose counts changed.  All clock arithmetic is single IEEE operations in a fixed order.
-// While a launch runs, a replication's clocks, counts and statistics sit in shared memory (word w of thread t
-// at w * blockDim + t); the four processes that take one request out of one count share one code path, so
-// the threads of a warp diverge only between arrivals, buffer abandonments and that path.
+// class order of its decode buffers: one THREAD simulates one replication.  Every class has seven unit-rate Poisson
+// processes (arrivals, abandonment from the prefill queue, abandonment from each decode buffer, prefill completions,
+// mixed and solo decode completions) that run on the integrated intensities of Eq. (7)-(9): a process with intensity
+// c n(t) keeps the integral acc of c n since its last jump and the exponential level lvl of its next jump, and its jump
+// time is recomputed whenever n changes.  Per event a thread scans its 7 I jump times, applies the jump, lets the policy
+// act (decode buffers into free slots, solo group first; then the prefill gate) and then brings the clocks of the counts
+// that changed up to date.  All clock arithmetic is single IEEE operations in a fixed order.
+// While a launch runs, a replication's clocks and counts sit in shared memory (word w of thread t at w * lanes + t).
+//
+// Bound: the dependent-instruction latency of each thread's chain and the divergence between jump kinds.  So a jump and the
+// policy only change counts (an addition and a bit in a mask); everything a changed count entails - time integral,
+// accumulated hazard, the division that gives the next jump time - is done once per changed count by one piece of code at
+// the end of the event (commit), where it used to be repeated inline at each of a dozen places (83 KB of code, up to six
+// divisions for a finished prefill whose buffer stays empty).  Measured, two-class instance, SLI-aware router, n = 1000: R = 37888,
+// 3 s 41.2 -> 27.3 ms (6.6e9 -> 10.0e9 jumps/s), R = 300, 8 s 104 -> 38 ms.  Changes at the same instant add nothing to an
+// integral, so the values are those of one update after another.
 #pragma once
 
 namespace qsimdev {
@@ -41,7 +46,7 @@ struct CtmcRep {
 struct CtmcClassPar { double lambda, theta, mu_p, mu_m, mu_s, xstar, nx, nq, ps; uint32_t prio, pad; };
 
 struct CtmcParams {
-    uint32_t I, N, M, B, R, qcap, gate, router, init, pad;
+    uint32_t I, N, M, B, R, qcap, gate, router, init, lanes;     // lanes: replications per warp
     unsigned long long seed, rep_offset, event_budget;
     double T_end;
     CtmcClassPar cls[MAXI];
@@ -50,126 +55,112 @@ struct CtmcParams {
     uint32_t *not_done;
 };
 
-// Working copy of one replication in shared memory: 8-byte words, word w of thread t at [w * blockDim + t]
-// (consecutive threads hit consecutive banks).  Only the I classes in use take space: 5 + 47 I words.  The event
-// counters and the time integrals are only ever added to, so they stay in the global record and take
-// fire-and-forget additions (one thread, one address: applied in program order, so the sums are deterministic).
-struct CtmcWords {
-    unsigned long long *base;   // this thread's word 0
-    uint32_t stride, I;
-    enum { W_EVENTS = 0, W_HEAD0 = 1, W_HEAD1 = 2, W_N0 = 3, W_N1 = 4, W_BASE = 5 };
-    __device__ __forceinline__ uint32_t clk(uint32_t k, uint32_t i, uint32_t f) const { return W_BASE + (k * I + i) * 5u + f; }   // f: acc, lvl, t_last, t_fire, m
-    __device__ __forceinline__ uint32_t count(uint32_t c, uint32_t i) const { return W_BASE + 35u * I + c * I + i; }             // c: Qp, X, Qd0, Qd1, Ym, Ys
-    __device__ __forceinline__ uint32_t sli(uint32_t i) const { return W_BASE + 41u * I + i; }
-    __device__ __forceinline__ uint32_t area_t(uint32_t a, uint32_t i) const { return W_BASE + 42u * I + a * I + i; }
-    __host__ __device__ static uint32_t words(uint32_t I) { return 5u + 47u * I; }
-    __device__ __forceinline__ unsigned long long u(uint32_t w) const { return base[(size_t)w * stride]; }
-    __device__ __forceinline__ void su(uint32_t w, unsigned long long v) const { base[(size_t)w * stride] = v; }
-    __device__ __forceinline__ double d(uint32_t w) const { return __longlong_as_double((long long)u(w)); }
-    __device__ __forceinline__ void sd(uint32_t w, double v) const { su(w, (unsigned long long)__double_as_longlong(v)); }
-};
-enum { CQ_QP = 0, CQ_X = 1, CQ_QD0 = 2, CQ_QD1 = 3, CQ_YM = 4, CQ_YS = 5 };
+// Working copy of one replication in shared memory: 39 I 8-byte words, word w of thread t at [w * lanes + t] (consecutive
+// threads hit consecutive banks).  The event counters and the time integrals are only ever added to, so they stay in the
+// global record and take fire-and-forget additions (one thread, one address: applied in program order, so the sums are
+// deterministic).  A count is stored twice in its word: as it is (low half) and as it was when its clock was last brought up
+// to date (high half).  The time of that is also where its integral stands; the two decode buffers share one integral and
+// have one more word for it.
+enum { CQ_QP = 0, CQ_QD0 = 1, CQ_QD1 = 2, CQ_X = 3, CQ_YM = 4, CQ_YS = 5, CQ_N = 6 };       // the count of process k > 0 is k - 1
 
 struct CtmcSim {
     const CtmcParams &p;
-    const CtmcWords W;
-    CtmcRep &G;                 // the record in global memory: counters and integrals are added to in place
-    uint8_t *ring0, *ring1;
+    unsigned long long *const base;   // this thread's word 0
+    const uint32_t stride, I, per_class;      // per_class = ceil(2^16 / I): (e per_class) >> 16 = e / I for e < 56
+    const double *const coef;         // [7 I] intensity per unit of the count (arrivals: per unit time), shared by the block
+    CtmcRep &G;                       // the record in global memory: counters and integrals are added to in place
+    uint8_t *const ring;              // [2][qcap]
     const uint32_t rep;
-    uint32_t totX, totYm, totYs, err;
+    uint32_t totX, totYm, totYs, err, head0, head1, n0, n1;
+    unsigned long long dirty;         // processes whose count changed in this event (bit k I + i)
 
-    __device__ CtmcSim(const CtmcParams &p_, const CtmcWords &W_, CtmcRep &G_, uint32_t rep_)
-        : p(p_), W(W_), G(G_), ring0(p_.rings + (size_t)rep_ * 2 * p_.qcap), ring1(ring0 + p_.qcap), rep(rep_), totX(0), totYm(0), totYs(0), err(0) {}
+    __device__ CtmcSim(const CtmcParams &p_, unsigned long long *base_, uint32_t stride_, const double *coef_, CtmcRep &G_, uint32_t rep_)
+        : p(p_), base(base_), stride(stride_), I(p_.I), per_class((65536u + p_.I - 1u) / p_.I), coef(coef_), G(G_), ring(p_.rings + (size_t)rep_ * 2 * p_.qcap), rep(rep_),
+          totX(0), totYm(0), totYs(0), err(0), head0(0), head1(0), n0(0), n1(0), dirty(0) {}
+
+    __host__ __device__ static uint32_t words(uint32_t I) { return 39u * I; }
+    // word numbers; e = k I + i
+    __device__ __forceinline__ uint32_t w_fire(uint32_t e) const { return e; }                       // 7 I
+    __device__ __forceinline__ uint32_t w_draws(uint32_t e) const { return 7u * I + e; }             // 7 I
+    __device__ __forceinline__ uint32_t w_acc(uint32_t e) const { return 13u * I + e; }              // e >= I: 6 I each
+    __device__ __forceinline__ uint32_t w_lvl(uint32_t e) const { return 19u * I + e; }
+    __device__ __forceinline__ uint32_t w_last(uint32_t e) const { return 25u * I + e; }
+    __device__ __forceinline__ uint32_t w_count(uint32_t e) const { return 31u * I + e; }
+    __device__ __forceinline__ uint32_t w_qd_last(uint32_t i) const { return 38u * I + i; }          // I
+    __device__ __forceinline__ unsigned long long u(uint32_t w) const { return base[w * stride]; }
+    __device__ __forceinline__ void su(uint32_t w, unsigned long long v) const { base[w * stride] = v; }
+    __device__ __forceinline__ double d(uint32_t w) const { return __longlong_as_double((long long)u(w)); }
+    __device__ __forceinline__ void sd(uint32_t w, double v) const { su(w, (unsigned long long)__double_as_longlong(v)); }
 
     __device__ __forceinline__ uint32_t stream_of(uint32_t k, uint32_t i) const
     {
         const uint32_t purpose = k < CK_SP ? k : k + 4u;      // 0..3 as in the iteration-level simulator, then 8, 9, 10
         return (purpose << 8) | i;
     }
-    __device__ __forceinline__ void rnd(uint32_t stream, unsigned long long index, uint32_t &w0, uint32_t &w1, uint32_t &w2, uint32_t &w3) const
+    __device__ __forceinline__ uint4 rnd(uint32_t stream, unsigned long long index) const
     {
-        const unsigned long long grep = p.rep_offset + rep;
-        philox((uint32_t)index, (uint32_t)(index >> 32), stream, (uint32_t)grep, (uint32_t)p.seed, (uint32_t)(p.seed >> 32), w0, w1, w2, w3);
+        return draw_words(p.seed, (uint32_t)(p.rep_offset + rep), stream, index);
     }
-    // intensity of process k of class i per unit of the count it runs on (the arrival process runs on the constant 1)
-    __device__ __forceinline__ double coef(uint32_t k, uint32_t i) const
-    {
-        const CtmcClassPar &c = p.cls[i];
-        return k <= CK_ABD1 ? (k == CK_ARR ? __dmul_rn((double)p.N, c.lambda) : c.theta)
-                            : (k == CK_SP ? c.mu_p : (k == CK_SDM ? c.mu_m : c.mu_s));
-    }
-    __device__ __forceinline__ uint32_t cq(uint32_t c, uint32_t i) const { return (uint32_t)W.u(W.count(c, i)); }
-    __device__ __forceinline__ void touch(uint32_t a, uint32_t i, uint32_t count, double t)
-    {
-        atomicAdd(&G.area[a][i], __dmul_rn((double)count, __dsub_rn(t, W.d(W.area_t(a, i)))));
-        W.sd(W.area_t(a, i), t);
-    }
-    // the count that process k of class i runs on changes from n_old to n_new at time t
-    __device__ void clk_change(uint32_t k, uint32_t i, uint32_t n_old, uint32_t n_new, double t)
-    {
-        const double c = coef(k, i);
-        if (!(c > 0.0)) return;
-        const double acc = __dadd_rn(W.d(W.clk(k, i, 0)), __dmul_rn(__dmul_rn(c, (double)n_old), __dsub_rn(t, W.d(W.clk(k, i, 2)))));
-        W.sd(W.clk(k, i, 0), acc);
-        W.sd(W.clk(k, i, 2), t);
-        double tf = dinf();
-        if (n_new > 0) {
-            double rem = __dsub_rn(W.d(W.clk(k, i, 1)), acc);
-            if (rem < 0.0) rem = 0.0;
-            tf = __dadd_rn(t, __ddiv_rn(rem, __dmul_rn(c, (double)n_new)));
-        }
-        W.sd(W.clk(k, i, 3), tf);
-    }
-    // process k of class i has just jumped at t and its count is now n_new: next level from draw m
-    __device__ void clk_fired(uint32_t k, uint32_t i, uint32_t n_new, double t, uint32_t &w2)
-    {
-        const unsigned long long m = W.u(W.clk(k, i, 4));
-        uint32_t w0, w1, w3;
-        rnd(stream_of(k, i), m, w0, w1, w2, w3);
-        const double lvl = -qlog(u53(w0, w1));
-        W.sd(W.clk(k, i, 1), lvl);
-        W.su(W.clk(k, i, 4), m + 1);
-        W.sd(W.clk(k, i, 0), 0.0);
-        W.sd(W.clk(k, i, 2), t);
-        W.sd(W.clk(k, i, 3), n_new > 0 ? __dadd_rn(t, __ddiv_rn(lvl, __dmul_rn(coef(k, i), (double)n_new))) : dinf());
-    }
-    // setters that keep the time integral and the process that runs on the count in step
-    __device__ void set_count(uint32_t c, uint32_t i, uint32_t v, double t)
-    {
-        // c -> (process, integral): Qp -> (ABP, Q_p), X -> (SP, X), Ym -> (SDM, Y_m), Ys -> (SDS, Y_s)
-        const uint32_t k = c == CQ_QP ? CK_ABP : (c == CQ_X ? CK_SP : (c == CQ_YM ? CK_SDM : CK_SDS));
-        const uint32_t a = c == CQ_QP ? CA_QP : (c == CQ_X ? CA_X : (c == CQ_YM ? CA_YM : CA_YS));
-        const uint32_t old = cq(c, i);
-        clk_change(k, i, old, v, t);
-        touch(a, i, old, t);
-        W.su(W.count(c, i), v);
-        if (c == CQ_X) totX += v - old;
-        if (c == CQ_YM) totYm += v - old;
-        if (c == CQ_YS) totYs += v - old;
-    }
-    __device__ void set_Qd(uint32_t pool, uint32_t i, uint32_t v, double t)
-    {
-        const uint32_t q0 = cq(CQ_QD0, i), q1 = cq(CQ_QD1, i);
-        clk_change(pool ? CK_ABD1 : CK_ABD0, i, pool ? q1 : q0, v, t);
-        touch(CA_QD, i, q0 + q1, t);
-        W.su(W.count(pool ? CQ_QD1 : CQ_QD0, i), v);
-    }
+    __device__ __forceinline__ uint32_t cq(uint32_t c, uint32_t i) const { return (uint32_t)u(w_count((c + 1u) * I + i)); }
     __device__ __forceinline__ void bump(uint32_t i, uint32_t c) { atomicAdd(&G.cnt[i][c], 1ull); }
+    // count c of class i changes by +1 or -1 (the low half of its word; a count is never negative)
+    __device__ __forceinline__ void change(uint32_t c, uint32_t i, int by)
+    {
+        const uint32_t e = (c + 1u) * I + i, w = w_count(e);
+        const unsigned long long v = u(w);
+        su(w, (v & 0xffffffff00000000ull) | (uint32_t)((uint32_t)v + (uint32_t)by));
+        dirty |= 1ull << e;
+    }
+
+    // Bring every changed count's process up to date at time t.  Process `fired` has just jumped: its hazard starts anew.
+    __device__ __forceinline__ void commit(double t, uint32_t fired)
+    {
+#pragma unroll 1
+        for (; dirty; dirty &= dirty - 1ull) {
+            const uint32_t e = (uint32_t)__ffsll((long long)dirty) - 1u;
+            const uint32_t k = (e * per_class) >> 16, i = e - k * I;
+            const unsigned long long v = u(w_count(e));
+            const uint32_t was = (uint32_t)(v >> 32), now = (uint32_t)v;
+            const double dt = __dsub_rn(t, d(w_last(e))), c = coef[e];
+            double part = __dmul_rn((double)was, dt);
+            uint32_t a = k == CK_ABP ? CA_QP : (k == CK_SP ? CA_X : (k == CK_SDM ? CA_YM : CA_YS));
+            if (k == CK_ABD0 || k == CK_ABD1) {
+                a = CA_QD;
+                const uint32_t both = (uint32_t)(u(w_count(CK_ABD0 * I + i)) >> 32) + (uint32_t)(u(w_count(CK_ABD1 * I + i)) >> 32);
+                part = __dmul_rn((double)both, __dsub_rn(t, d(w_qd_last(i))));
+                sd(w_qd_last(i), t);
+            }
+            atomicAdd(&G.area[a][i], part);
+            double acc = 0.0;
+            if (e != fired) acc = __dadd_rn(d(w_acc(e)), __dmul_rn(__dmul_rn(c, (double)was), dt));
+            double tf = dinf();
+            if (now > 0 && c > 0.0) {
+                double rem = __dsub_rn(d(w_lvl(e)), acc);
+                if (rem < 0.0) rem = 0.0;
+                tf = __dadd_rn(t, __ddiv_rn(rem, __dmul_rn(c, (double)now)));
+            }
+            sd(w_acc(e), acc);
+            sd(w_last(e), t);
+            sd(w_fire(e), tf);
+            su(w_count(e), ((unsigned long long)now << 32) | now);
+        }
+    }
 
     // Section 4.1 occupancy gate (xi_i = (X_i - n x*_i)/x*_i, ties to the largest Q_p,i - n q*_p,i) or the
     // Section 5.1.1 priority gate (smallest static rank); ties to the lowest class index
-    __device__ uint32_t gate_class() const
+    __device__ __forceinline__ uint32_t gate_class() const
     {
         uint32_t best = NONE32;
-        if (p.gate == 1) {
-            for (uint32_t i = 0; i < p.I; ++i)
-                if (cq(CQ_QP, i) > 0 && (best == NONE32 || p.cls[i].prio < p.cls[best].prio)) best = i;
-            return best;
-        }
         double bxi = 0.0, bdq = 0.0;
-        for (uint32_t i = 0; i < p.I; ++i) {
+#pragma unroll 1
+        for (uint32_t i = 0; i < I; ++i) {
             const uint32_t Qp = cq(CQ_QP, i);
-            if (Qp == 0 || !(p.cls[i].xstar > 0.0)) continue;
+            if (Qp == 0) continue;
+            if (p.gate == 1) {
+                if (best == NONE32 || p.cls[i].prio < p.cls[best].prio) best = i;
+                continue;
+            }
+            if (!(p.cls[i].xstar > 0.0)) continue;
             const double xi = __ddiv_rn(__dsub_rn((double)cq(CQ_X, i), p.cls[i].nx), p.cls[i].xstar);
             const double dq = __dsub_rn((double)Qp, p.cls[i].nq);
             if (best == NONE32 || xi < bxi || (xi == bxi && dq > bdq)) { best = i; bxi = xi; bdq = dq; }
@@ -177,40 +168,48 @@ struct CtmcSim {
         return best;
     }
 
-    __device__ void dispatch(double t)
+    // tier that takes the head of the pool's buffer now: 0 solo, 1 mixed, 2 none has a free slot
+    __device__ __forceinline__ uint32_t tier_of(uint32_t pool) const
     {
-        const uint32_t cap_s = (p.N - p.M) * p.B, cap_m = p.M * (p.B - 1u);
-        const uint32_t npools = p.router == 1 ? 2u : 1u;
-        for (uint32_t pool = 0; pool < npools; ++pool) {
-            uint8_t *ring = pool ? ring1 : ring0;
-            const uint32_t wn = pool ? CtmcWords::W_N1 : CtmcWords::W_N0, wh = pool ? CtmcWords::W_HEAD1 : CtmcWords::W_HEAD0;
-            uint32_t n = (uint32_t)W.u(wn);
-            while (n > 0) {
-                bool to_solo;
-                if (p.router == 1) {
-                    to_solo = pool == 0;
-                    if (to_solo ? totYs >= cap_s : totYm >= cap_m) break;
-                } else {
-                    if (totYs < cap_s) to_solo = true;
-                    else if (totYm < cap_m) to_solo = false;
-                    else break;
-                }
-                uint32_t head = (uint32_t)W.u(wh);
-                const uint32_t i = ring[head];
-                head = head + 1 == p.qcap ? 0 : head + 1;
-                W.su(wh, head);
-                n -= 1;
-                W.su(wn, n);
-                set_Qd(pool, i, cq(pool ? CQ_QD1 : CQ_QD0, i) - 1, t);
-                set_count(to_solo ? CQ_YS : CQ_YM, i, cq(to_solo ? CQ_YS : CQ_YM, i) + 1, t);
-                bump(i, to_solo ? CC_PLACED_SOLO : CC_PLACED_MIXED);
+        const bool solo = totYs < (p.N - p.M) * p.B, mix = totYm < p.M * (p.B - 1u);
+        if (p.router == 1) return pool ? (mix ? 1u : 2u) : (solo ? 0u : 2u);
+        return solo ? 0u : (mix ? 1u : 2u);
+    }
+    __device__ __forceinline__ void place(uint32_t i, uint32_t tier)
+    {
+        change(tier ? CQ_YM : CQ_YS, i, 1);
+        totYs += tier ? 0u : 1u; totYm += tier ? 1u : 0u;
+        bump(i, tier ? CC_PLACED_MIXED : CC_PLACED_SOLO);
+    }
+
+    // The policy's turn after every event: buffered requests into free decode slots, then the prefill gate.
+    __device__ __forceinline__ void dispatch()
+    {
+        uint32_t pool = 0;
+#pragma unroll 1
+        while (n0 | n1) {
+            if (pool == 0 && n0 == 0) pool = 1;
+            if (pool == 1 && n1 == 0) break;
+            const uint32_t tier = tier_of(pool);
+            if (tier == 2u) {
+                if (pool == 1) break;
+                pool = 1;
+                continue;
             }
+            uint32_t &head = pool ? head1 : head0;
+            const uint32_t i = ring[pool * p.qcap + head];
+            head = head + 1 == p.qcap ? 0 : head + 1;
+            if (pool) --n1; else --n0;
+            change(pool ? CQ_QD1 : CQ_QD0, i, -1);
+            place(i, tier);
         }
+#pragma unroll 1
         while (totX < p.M) {
             const uint32_t i = gate_class();
             if (i == NONE32) break;
-            set_count(CQ_QP, i, cq(CQ_QP, i) - 1, t);
-            set_count(CQ_X, i, cq(CQ_X, i) + 1, t);
+            change(CQ_QP, i, -1);
+            change(CQ_X, i, 1);
+            ++totX;
             bump(i, CC_ADMITTED);
         }
     }
@@ -218,159 +217,153 @@ struct CtmcSim {
     // empty system at t = 0: every process gets its first level, the arrival processes their first jump time
     __device__ void init()
     {
-        for (uint32_t w = 0; w < CtmcWords::words(p.I); ++w) W.su(w, 0ull);
-        for (uint32_t i = 0; i < p.I; ++i) {
+        for (uint32_t w = 0; w < words(I); ++w) su(w, 0ull);
+        for (uint32_t i = 0; i < I; ++i)
             for (uint32_t k = 0; k < CK_N; ++k) {
-                uint32_t w0, w1, w2, w3;
-                rnd(stream_of(k, i), 0, w0, w1, w2, w3);
-                W.sd(W.clk(k, i, 1), -qlog(u53(w0, w1)));
-                W.sd(W.clk(k, i, 3), dinf());
-                W.su(W.clk(k, i, 4), 1ull);
+                const uint32_t e = k * I + i;
+                const uint4 w = rnd(stream_of(k, i), 0);
+                const double lvl = -qlog(u53(w.x, w.y));
+                sd(w_fire(e), (k == CK_ARR && coef[e] > 0.0) ? __dadd_rn(0.0, __ddiv_rn(lvl, coef[e])) : dinf());
+                su(w_draws(e), 1ull);
+                if (k > 0) sd(w_lvl(e), lvl);
             }
-            const double Lam = __dmul_rn((double)p.N, p.cls[i].lambda);
-            if (Lam > 0.0) W.sd(W.clk(CK_ARR, i, 3), __dadd_rn(0.0, __ddiv_rn(W.d(W.clk(CK_ARR, i, 1)), Lam)));
-        }
     }
 
     // events with t <= T_end, at most `budget` of them; returns true when none is left up to T_end
-    __device__ bool run(double T_end, unsigned long long budget)
+    __device__ bool run(double T_end, unsigned long long budget, unsigned long long &events)
     {
-        for (uint32_t i = 0; i < p.I; ++i) { totX += cq(CQ_X, i); totYm += cq(CQ_YM, i); totYs += cq(CQ_YS, i); }
-        unsigned long long events = W.u(CtmcWords::W_EVENTS);
-        bool finished;
+        for (uint32_t i = 0; i < I; ++i) { totX += cq(CQ_X, i); totYm += cq(CQ_YM, i); totYs += cq(CQ_YS, i); }
+        const uint32_t n_proc = CK_N * I;
+        const unsigned long long tend_bits = (unsigned long long)__double_as_longlong(T_end);
         for (;;) {
-            // earliest process; ties by process kind, then class (strict '<' in that scan order)
-            double te = dinf();
-            uint32_t bk = 0, bi = 0;
-#pragma unroll
-            for (uint32_t k = 0; k < CK_N; ++k)
-                for (uint32_t i = 0; i < p.I; ++i) {
-                    const double tf = W.d(W.clk(k, i, 3));
-                    if (tf < te) { te = tf; bk = k; bi = i; }
-                }
-            if (!(te <= T_end)) { finished = true; break; }
-            if (budget == 0) { finished = false; break; }
+            // earliest process; ties by process kind, then class (strict '<' in that scan order; the times are not negative)
+            unsigned long long te = 0x7ff0000000000000ull;
+            uint32_t e = 0;
+#pragma unroll 7
+            for (uint32_t q = 0; q < n_proc; ++q) {
+                const unsigned long long tf = u(w_fire(q));
+                if (tf < te) { te = tf; e = q; }
+            }
+            if (!(te <= tend_bits) || te == 0x7ff0000000000000ull) return true;
+            if (budget == 0) return false;
             --budget;
-            const double t = te;
-            const uint32_t i = bi;
+            const double t = __longlong_as_double((long long)te);
+            const uint32_t k = (e * per_class) >> 16, i = e - k * I;
             ++events;
-            uint32_t w2 = 0;
-            if (bk == CK_ABD0 || bk == CK_ABD1) {
-                const uint32_t pool = bk == CK_ABD1 ? 1u : 0u;
-                const uint32_t Q = cq(pool ? CQ_QD1 : CQ_QD0, i);
-                clk_fired(bk, i, Q - 1, t, w2);
+            // the process's next level
+            const unsigned long long m = u(w_draws(e));
+            su(w_draws(e), m + 1);
+            const uint4 w = rnd(stream_of(k, i), m);
+            const double lvl = -qlog(u53(w.x, w.y));
+            uint32_t c = k - 1u, cc = CC_ABANDONED_D;
+            if (k == CK_ARR) {
+                c = CQ_QP; cc = CC_ARRIVALS;
+                sd(w_fire(e), __dadd_rn(t, __ddiv_rn(lvl, coef[e])));
+            } else {
+                sd(w_lvl(e), lvl);
+                cc = k == CK_ABP ? CC_ABANDONED_P : (k == CK_SP ? CC_PREFILL_DONE : (k == CK_SDM ? CC_DONE_MIXED : (k == CK_SDS ? CC_DONE_SOLO : CC_ABANDONED_D)));
+            }
+            if (k == CK_ABD0 || k == CK_ABD1) {
                 // a uniformly chosen waiting class-i request leaves the pool's buffer; the rest keep their order
-                uint8_t *ring = pool ? ring1 : ring0;
-                const uint32_t wn = pool ? CtmcWords::W_N1 : CtmcWords::W_N0;
-                uint32_t rank = __umulhi(w2, Q), pos = 0;
-                const uint32_t n = (uint32_t)W.u(wn), head = (uint32_t)W.u(pool ? CtmcWords::W_HEAD1 : CtmcWords::W_HEAD0);
+                const uint32_t pool = k == CK_ABD1 ? 1u : 0u;
+                uint8_t *r = ring + pool * p.qcap;
+                uint32_t rank = __umulhi(w.z, cq(c, i)), pos = 0;
+                const uint32_t n = pool ? n1 : n0, head = pool ? head1 : head0;
                 for (pos = 0; pos < n; ++pos) {
                     uint32_t a = head + pos; if (a >= p.qcap) a -= p.qcap;
-                    if (ring[a] != i) continue;
+                    if (r[a] != i) continue;
                     if (rank == 0) break;
                     --rank;
                 }
-                if (pos >= n) { err = ERR_INTERNAL; finished = true; break; }
-                for (uint32_t k = pos; k + 1 < n; ++k) {
-                    uint32_t a = head + k, b = head + k + 1;
+                if (pos >= n) { err = ERR_INTERNAL; return true; }
+                for (uint32_t q = pos; q + 1 < n; ++q) {
+                    uint32_t a = head + q, b = head + q + 1;
                     if (a >= p.qcap) a -= p.qcap;
                     if (b >= p.qcap) b -= p.qcap;
-                    ring[a] = ring[b];
+                    r[a] = r[b];
                 }
-                W.su(wn, n - 1);
-                touch(CA_QD, i, cq(CQ_QD0, i) + cq(CQ_QD1, i), t);
-                W.su(W.count(pool ? CQ_QD1 : CQ_QD0, i), Q - 1);
-                bump(i, CC_ABANDONED_D);
-            } else {
-                // One code path for the five processes that move one request across one count: an arrival adds one to the
-                // prefill queue (and redraws on the constant count 1); abandonment from the prefill queue, prefill
-                // completion and mixed / solo decode completion take one out of the count they run on.
-                const bool arr = bk == CK_ARR;
-                const uint32_t c = (arr || bk == CK_ABP) ? CQ_QP : (bk == CK_SP ? CQ_X : (bk == CK_SDM ? CQ_YM : CQ_YS));
-                const uint32_t a = (arr || bk == CK_ABP) ? CA_QP : (bk == CK_SP ? CA_X : (bk == CK_SDM ? CA_YM : CA_YS));
-                const uint32_t cc = arr ? CC_ARRIVALS : (bk == CK_ABP ? CC_ABANDONED_P : (bk == CK_SP ? CC_PREFILL_DONE : (bk == CK_SDM ? CC_DONE_MIXED : CC_DONE_SOLO)));
-                const uint32_t old = cq(c, i), now = arr ? old + 1 : old - 1;
-                if (arr) clk_change(CK_ABP, i, old, now, t);       // the queue's abandonment process sees the new length
-                touch(a, i, old, t);
-                W.su(W.count(c, i), now);
-                totX -= bk == CK_SP ? 1u : 0u; totYm -= bk == CK_SDM ? 1u : 0u; totYs -= bk == CK_SDS ? 1u : 0u;
-                bump(i, cc);
-                clk_fired(bk, i, arr ? 1u : now, t, w2);
-                if (bk == CK_SP) {
-                    uint32_t pool = 0;
-                    if (p.router == 1) {
-                        // SLI-aware router: one uniform per finished prefill decides the pool (Section 5.2)
-                        const unsigned long long ord = W.u(W.sli(i));
-                        W.su(W.sli(i), ord + 1);
-                        uint32_t w0, w1, w3;
-                        rnd((STREAM_SLI << 8) | i, ord, w0, w1, w2, w3);
-                        pool = u53(w0, w1) <= p.cls[i].ps ? 0u : 1u;
-                    }
-                    const uint32_t wn = pool ? CtmcWords::W_N1 : CtmcWords::W_N0;
-                    const uint32_t n = (uint32_t)W.u(wn);
-                    if (n >= p.qcap) {
-                        bump(i, CC_OVERFLOW_D);
-                    } else {
-                        uint32_t pos = (uint32_t)W.u(pool ? CtmcWords::W_HEAD1 : CtmcWords::W_HEAD0) + n; if (pos >= p.qcap) pos -= p.qcap;
-                        (pool ? ring1 : ring0)[pos] = (uint8_t)i;
-                        W.su(wn, n + 1);
-                        set_Qd(pool, i, cq(pool ? CQ_QD1 : CQ_QD0, i) + 1, t);
-                    }
+                if (pool) --n1; else --n0;
+            }
+            change(c, i, k == CK_ARR ? 1 : -1);
+            bump(i, cc);
+            totX -= k == CK_SP ? 1u : 0u; totYm -= k == CK_SDM ? 1u : 0u; totYs -= k == CK_SDS ? 1u : 0u;
+            if (k == CK_SP) {
+                uint32_t pool = 0;
+                if (p.router == 1) {
+                    // SLI-aware router: one uniform per finished prefill decides the pool (Section 5.2); its ordinal is the
+                    // number of prefills of the class finished before
+                    const uint4 z = rnd((STREAM_SLI << 8) | i, m - 1ull);
+                    pool = u53(z.x, z.y) <= p.cls[i].ps ? 0u : 1u;
+                }
+                const uint32_t n = pool ? n1 : n0, tier = n == 0 ? tier_of(pool) : 2u;
+                if (tier != 2u) {
+                    place(i, tier);          // it passes through its empty buffer at this instant
+                } else if (n >= p.qcap) {
+                    bump(i, CC_OVERFLOW_D);
+                } else {
+                    uint32_t pos = (pool ? head1 : head0) + n; if (pos >= p.qcap) pos -= p.qcap;
+                    ring[pool * p.qcap + pos] = (uint8_t)i;
+                    if (pool) ++n1; else ++n0;
+                    change(pool ? CQ_QD1 : CQ_QD0, i, 1);
                 }
             }
-            dispatch(t);
+            dispatch();
+            commit(t, k == CK_ARR ? NONE32 : e);
         }
-        W.su(CtmcWords::W_EVENTS, events);
-        return finished;
     }
 
     // the record in global memory <-> the working copy
     __device__ void load(const CtmcRep &S)
     {
-        W.su(CtmcWords::W_EVENTS, S.events);
-        W.su(CtmcWords::W_HEAD0, S.head[0]); W.su(CtmcWords::W_HEAD1, S.head[1]); W.su(CtmcWords::W_N0, S.n[0]); W.su(CtmcWords::W_N1, S.n[1]);
-        for (uint32_t i = 0; i < p.I; ++i) {
+        head0 = S.head[0]; head1 = S.head[1]; n0 = S.n[0]; n1 = S.n[1];
+        for (uint32_t i = 0; i < I; ++i) {
+            const uint32_t cnt[CQ_N] = { S.Qp[i], S.Qd[0][i], S.Qd[1][i], S.X[i], S.Ym[i], S.Ys[i] };
             for (uint32_t k = 0; k < CK_N; ++k) {
                 const CtmcClk &q = S.clk[k][i];
-                W.sd(W.clk(k, i, 0), q.acc); W.sd(W.clk(k, i, 1), q.lvl); W.sd(W.clk(k, i, 2), q.t_last); W.sd(W.clk(k, i, 3), q.t_fire);
-                W.su(W.clk(k, i, 4), q.m);
+                const uint32_t e = k * I + i;
+                sd(w_fire(e), q.t_fire);
+                su(w_draws(e), q.m);
+                if (k == 0) continue;
+                sd(w_acc(e), q.acc); sd(w_lvl(e), q.lvl); sd(w_last(e), q.t_last);
+                su(w_count(e), ((unsigned long long)cnt[k - 1] << 32) | cnt[k - 1]);
             }
-            W.su(W.count(CQ_QP, i), S.Qp[i]); W.su(W.count(CQ_X, i), S.X[i]); W.su(W.count(CQ_QD0, i), S.Qd[0][i]);
-            W.su(W.count(CQ_QD1, i), S.Qd[1][i]); W.su(W.count(CQ_YM, i), S.Ym[i]); W.su(W.count(CQ_YS, i), S.Ys[i]);
-            W.su(W.sli(i), S.sli_ord[i]);
-            for (uint32_t a = 0; a < CA_N; ++a) W.sd(W.area_t(a, i), S.area_t[a][i]);
+            sd(w_qd_last(i), S.area_t[CA_QD][i]);
         }
     }
     __device__ void store(CtmcRep &S) const
     {
-        S.events = W.u(CtmcWords::W_EVENTS);
-        S.head[0] = (uint32_t)W.u(CtmcWords::W_HEAD0); S.head[1] = (uint32_t)W.u(CtmcWords::W_HEAD1);
-        S.n[0] = (uint32_t)W.u(CtmcWords::W_N0); S.n[1] = (uint32_t)W.u(CtmcWords::W_N1);
-        for (uint32_t i = 0; i < p.I; ++i) {
+        S.head[0] = head0; S.head[1] = head1; S.n[0] = n0; S.n[1] = n1;
+        for (uint32_t i = 0; i < I; ++i) {
             for (uint32_t k = 0; k < CK_N; ++k) {
                 CtmcClk &q = S.clk[k][i];
-                q.acc = W.d(W.clk(k, i, 0)); q.lvl = W.d(W.clk(k, i, 1)); q.t_last = W.d(W.clk(k, i, 2)); q.t_fire = W.d(W.clk(k, i, 3));
-                q.m = W.u(W.clk(k, i, 4));
+                const uint32_t e = k * I + i;
+                q.t_fire = d(w_fire(e)); q.m = u(w_draws(e));
+                if (k > 0) { q.acc = d(w_acc(e)); q.lvl = d(w_lvl(e)); q.t_last = d(w_last(e)); }
             }
             S.Qp[i] = cq(CQ_QP, i); S.X[i] = cq(CQ_X, i); S.Qd[0][i] = cq(CQ_QD0, i); S.Qd[1][i] = cq(CQ_QD1, i);
             S.Ym[i] = cq(CQ_YM, i); S.Ys[i] = cq(CQ_YS, i);
-            S.sli_ord[i] = W.u(W.sli(i));
-            for (uint32_t a = 0; a < CA_N; ++a) S.area_t[a][i] = W.d(W.area_t(a, i));
+            S.area_t[CA_QP][i] = d(w_last(CK_ABP * I + i)); S.area_t[CA_X][i] = d(w_last(CK_SP * I + i)); S.area_t[CA_QD][i] = d(w_qd_last(i));
+            S.area_t[CA_YM][i] = d(w_last(CK_SDM * I + i)); S.area_t[CA_YS][i] = d(w_last(CK_SDS * I + i));
         }
     }
 };
 
 // One thread per replication.  The replication's record lives in global memory between launches; a launch works on a
 // copy in shared memory.  init != 0: start from the empty system at t = 0 (no events are processed).
-__global__ void __launch_bounds__(64) qsim_ctmc_kernel(CtmcParams p)
+__global__ void __launch_bounds__(32) qsim_ctmc_kernel(CtmcParams p)
 {
     extern __shared__ __align__(16) unsigned long long ctmc_sm[];
-    const uint32_t rep = blockIdx.x * blockDim.x + threadIdx.x;
-    if (rep >= p.R) return;
+    const uint32_t lanes = p.lanes, rep = blockIdx.x * lanes + threadIdx.x;
+    double *coef = reinterpret_cast<double *>(ctmc_sm);      // [7 I], then the threads' words
+    for (uint32_t e = threadIdx.x; e < CK_N * p.I; e += blockDim.x) {
+        const uint32_t k = e / p.I, i = e - k * p.I;
+        const CtmcClassPar &c = p.cls[i];
+        coef[e] = k == CK_ARR ? __dmul_rn((double)p.N, c.lambda) : (k <= CK_ABD1 ? c.theta : (k == CK_SP ? c.mu_p : (k == CK_SDM ? c.mu_m : c.mu_s)));
+    }
+    __syncwarp();
+    if (threadIdx.x >= lanes || rep >= p.R) return;
     CtmcRep &S = p.reps[rep];
-    CtmcWords W;
-    W.base = ctmc_sm + threadIdx.x; W.stride = blockDim.x; W.I = p.I;
-    CtmcSim sim(p, W, S, rep);
+    CtmcSim sim(p, ctmc_sm + CK_N * p.I + threadIdx.x, lanes, coef, S, rep);
     if (p.init) {
         uint32_t *w = reinterpret_cast<uint32_t *>(&S);
         for (uint32_t o = 0; o < sizeof(CtmcRep) / 4; ++o) w[o] = 0;
@@ -381,12 +374,44 @@ __global__ void __launch_bounds__(64) qsim_ctmc_kernel(CtmcParams p)
     }
     if (S.err || (S.done && S.T_end == p.T_end)) return;
     sim.load(S);
-    const bool finished = sim.run(p.T_end, p.event_budget);
+    unsigned long long events = S.events;
+    const bool finished = sim.run(p.T_end, p.event_budget, events);
     sim.store(S);
+    S.events = events;
     S.T_end = p.T_end;
     S.err = sim.err;
     S.done = finished ? 1u : 0u;
     if (!finished) atomicAdd(p.not_done, 1u);
+}
+
+// The public statistics record of every replication, one warp each: counters as they are, time integrals closed at the end
+// time (the host's formula, rounded the same).  first_err: lowest replication that stopped on an internal error.
+// Memory-bound: 3.7 KB read and 1.2 KB written per replication.
+__global__ void __launch_bounds__(128) qsim_ctmc_stats_kernel(const CtmcRep *reps, uint32_t R, uint32_t I, qsim_ctmc_rep_stats *out, uint32_t *first_err)
+{
+    const uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31u;
+    if (r >= R) return;
+    const CtmcRep &S = reps[r];
+    qsim_ctmc_rep_stats &o = out[r];
+    const double T = S.T_end;
+    for (uint32_t w = lane; w < MAXI * CC_N; w += 32u) o.cnt[w / CC_N][w % CC_N] = w < I * CC_N ? S.cnt[w / CC_N][w % CC_N] : 0ull;
+    for (uint32_t w = lane; w < MAXI * CA_N; w += 32u) {
+        const uint32_t i = w / CA_N, a = w % CA_N;
+        uint32_t n = 0;
+        double area = 0.0;
+        if (i < I) {
+            n = a == CA_QP ? S.Qp[i] : (a == CA_X ? S.X[i] : (a == CA_QD ? S.Qd[0][i] + S.Qd[1][i] : (a == CA_YM ? S.Ym[i] : S.Ys[i])));
+            area = __dadd_rn(S.area[a][i], __dmul_rn((double)n, __dsub_rn(T, S.area_t[a][i])));
+        }
+        o.state[i][a] = n;
+        o.area[i][a] = area;
+    }
+    if (lane < MAXI) o.reserved[lane] = 0;
+    if (lane == 0) {
+        o.events = S.events;
+        o.T_elapsed = T;
+        if (S.err) atomicMin(first_err, r);
+    }
 }
 
 }  // namespace qsimdev
@@ -429,14 +454,44 @@ CtmcSections ctmc_sections(const qsim_ctmc_config &c)
     return s;
 }
 
-// one warp per block: many small blocks spread the replications over all SMs; the working copies of a block's
-// replications take 32 (5 + 47 I) 8-byte words of shared memory
-int ctmc_launch_shape(uint32_t I, uint32_t &threads, size_t &smem)
+// One warp per block, its first `lanes` threads run a replication each.  A warp executes every path that any of its threads
+// takes, so few replications are spread over more warps: the largest power of two that still gives CTMC_WARPS warps (fewer
+// replications than that: one per warp).  Measured with the smaller code: n = 1000, R = 300: 104 -> 38 ms (32 -> 1 per warp), n = 50,
+// R = 1000: 5.7 -> 2.3 (1), n = 200, R = 3000: 19.2 -> 11.8 (2), n = 1000, R = 8192: 62.6 -> 51.2 (8).
+constexpr uint32_t CTMC_WARPS = 888;
+int ctmc_launch_shape(const qsim_ctmc_config &c, uint32_t &lanes, size_t &smem)
 {
-    threads = 32;
-    smem = (size_t)threads * CtmcWords::words(I) * 8;
+    lanes = 32;
+    while (lanes > 1u && c.R / lanes < CTMC_WARPS) lanes >>= 1;
+    smem = ((size_t)lanes * CtmcSim::words(c.I) + CK_N * c.I) * 8;
     if (smem > 48u * 1024u)
         CUDA_TRY(cudaFuncSetAttribute(qsim_ctmc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    return QSIM_OK;
+}
+
+// The public records from a copy of the device records: for a device without room for the former.
+int ctmc_stats_on_host(const qsim_ctmc_config &cfg, const char *dev_reps, cudaStream_t st, qsim_ctmc_rep_stats *per_rep)
+{
+    std::vector<CtmcRep> reps(cfg.R);
+    CUDA_TRY(cudaMemcpyAsync(reps.data(), dev_reps, reps.size() * sizeof(CtmcRep), cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaStreamSynchronize(st));
+    for (uint32_t r = 0; r < cfg.R; ++r) {
+        const CtmcRep &S = reps[r];
+        if (S.err) return fail(QSIM_EOVERFLOW, "replication " + std::to_string(r) + " stopped on an internal error");
+        qsim_ctmc_rep_stats &o = per_rep[r];
+        std::memset(&o, 0, sizeof o);
+        const double T = S.T_end;
+        for (uint32_t i = 0; i < cfg.I; ++i) {
+            for (int k = 0; k < CC_N; ++k) o.cnt[i][k] = S.cnt[i][k];
+            const uint32_t state[5] = { S.Qp[i], S.X[i], S.Qd[0][i] + S.Qd[1][i], S.Ym[i], S.Ys[i] };
+            for (int a = 0; a < CA_N; ++a) {
+                o.state[i][a] = state[a];
+                o.area[i][a] = S.area[a][i] + (double)state[a] * (T - S.area_t[a][i]);     // integral up to the end time
+            }
+        }
+        o.events = S.events;
+        o.T_elapsed = T;
+    }
     return QSIM_OK;
 }
 
@@ -482,11 +537,10 @@ int qsim_ctmc_init(const qsim_ctmc_config *cfg, const qsim_ctmc_class *classes, 
     if (rc != QSIM_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     p.init = 1;
-    uint32_t threads = 0;
     size_t smem = 0;
-    rc = ctmc_launch_shape(cfg->I, threads, smem);
+    rc = ctmc_launch_shape(*cfg, p.lanes, smem);
     if (rc != QSIM_OK) return rc;
-    qsim_ctmc_kernel<<<(cfg->R + threads - 1u) / threads, threads, smem, st>>>(p);
+    qsim_ctmc_kernel<<<(cfg->R + p.lanes - 1u) / p.lanes, 32, smem, st>>>(p);
     CUDA_TRY(cudaGetLastError());
     return QSIM_OK;
 }
@@ -501,15 +555,14 @@ int qsim_ctmc_run_until(const qsim_ctmc_config *cfg, const qsim_ctmc_class *clas
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     p.T_end = T_end;
     uint64_t n = 0;
-    uint32_t threads = 0;
     size_t smem = 0;
-    rc = ctmc_launch_shape(cfg->I, threads, smem);
+    rc = ctmc_launch_shape(*cfg, p.lanes, smem);
     if (rc != QSIM_OK) return rc;
     // a replication that used up its per-launch event budget is continued by further launches
     uint32_t flag = 1;
     for (int guard = 0; guard < 100000 && flag != 0; ++guard) {
         CUDA_TRY(cudaMemsetAsync(p.not_done, 0, 4, st));
-        qsim_ctmc_kernel<<<(cfg->R + threads - 1u) / threads, threads, smem, st>>>(p);
+        qsim_ctmc_kernel<<<(cfg->R + p.lanes - 1u) / p.lanes, 32, smem, st>>>(p);
         CUDA_TRY(cudaGetLastError());
         ++n;
         CUDA_TRY(cudaMemcpyAsync(&flag, p.not_done, 4, cudaMemcpyDeviceToHost, st));
@@ -527,26 +580,29 @@ int qsim_ctmc_stats(const qsim_ctmc_config *cfg, const void *dev_workspace, size
     const CtmcSections sec = ctmc_sections(*cfg);
     if (!dev_workspace || bytes < sec.total) return fail(QSIM_EWORKSPACE, "workspace missing or too small");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    std::vector<CtmcRep> reps(cfg->R);
-    CUDA_TRY(cudaMemcpyAsync(reps.data(), static_cast<const char *>(dev_workspace) + sec.reps, reps.size() * sizeof(CtmcRep), cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    for (uint32_t r = 0; r < cfg->R; ++r) {
-        const CtmcRep &S = reps[r];
-        if (S.err) return fail(QSIM_EOVERFLOW, "replication " + std::to_string(r) + " stopped on an internal error");
-        qsim_ctmc_rep_stats &o = per_rep[r];
-        std::memset(&o, 0, sizeof o);
-        const double T = S.T_end;
-        for (uint32_t i = 0; i < cfg->I; ++i) {
-            for (int k = 0; k < CC_N; ++k) o.cnt[i][k] = S.cnt[i][k];
-            const uint32_t state[5] = { S.Qp[i], S.X[i], S.Qd[0][i] + S.Qd[1][i], S.Ym[i], S.Ys[i] };
-            for (int a = 0; a < CA_N; ++a) {
-                o.state[i][a] = state[a];
-                o.area[i][a] = S.area[a][i] + (double)state[a] * (T - S.area_t[a][i]);     // integral up to the end time
-            }
-        }
-        o.events = S.events;
-        o.T_elapsed = T;
+    // the public records are formed on the device: a third of the bytes cross to the host, and nothing is left to do there
+    const size_t out_bytes = (size_t)cfg->R * sizeof(qsim_ctmc_rep_stats);
+    char *scratch = nullptr;
+    if (cudaMallocAsync(reinterpret_cast<void **>(&scratch), out_bytes + 4, st) != cudaSuccess) {
+        cudaGetLastError();
+        return ctmc_stats_on_host(*cfg, static_cast<const char *>(dev_workspace) + sec.reps, st, per_rep);
     }
+    uint32_t first_err = NONE32;
+    cudaError_t e = cudaMemsetAsync(scratch + out_bytes, 0xff, 4, st);
+    if (e == cudaSuccess) {
+        qsim_ctmc_stats_kernel<<<(cfg->R + 3u) / 4u, 128, 0, st>>>(reinterpret_cast<const CtmcRep *>(static_cast<const char *>(dev_workspace) + sec.reps),
+                                                                  cfg->R, cfg->I, reinterpret_cast<qsim_ctmc_rep_stats *>(scratch),
+                                                                  reinterpret_cast<uint32_t *>(scratch + out_bytes));
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&first_err, scratch + out_bytes, 4, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess && first_err == NONE32) e = cudaMemcpyAsync(per_rep, scratch, out_bytes, cudaMemcpyDeviceToHost, st);
+    const cudaError_t ef = cudaFreeAsync(scratch, st);
+    if (e == cudaSuccess) e = ef;
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return fail(QSIM_ECUDA, std::string("qsim_ctmc_stats: ") + cudaGetErrorString(e));
+    if (first_err != NONE32) return fail(QSIM_EOVERFLOW, "replication " + std::to_string(first_err) + " stopped on an internal error");
     return QSIM_OK;
 }
 
