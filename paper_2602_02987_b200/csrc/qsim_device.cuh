@@ -1950,13 +1950,13 @@ struct Sim {
 // shared-memory carve-up for one replication (one warp per block)
 struct SmemLayout {
     uint32_t off_tnext, off_tarr, off_it, off_nfin, off_pfrem, off_pfjob, off_K, off_Kpend, off_ndec, off_nact,
-        off_pfcur, off_sfin16, off_socc, srv_bytes, off_bkt, off_picked, off_touch, off_cs, off_ring, off_strec, off_stte, off_pqh, off_wcs, off_cmd, off_res, total;
+        off_pfcur, off_sfin16, off_socc, img_sfin16, img_socc, srv_bytes, off_bkt, off_picked, off_touch, off_cs, off_ring, off_strec, off_stte, off_pqh, off_wcs, off_cmd, off_res, total;
 };
 
 // tarr_global: the arrival times and the job words of the requests in prefill (read once per finished prefill) live in
 // global memory (large clusters: shared memory is what limits the resident replications there); I: classes (sizes the
 // class records and the ring of arrival draws)
-__host__ __device__ inline SmemLayout smem_layout(uint32_t Npad, uint32_t B, uint32_t slots_smem, uint32_t nwarps, bool kappa,
+__host__ __device__ inline SmemLayout smem_layout(uint32_t N, uint32_t Npad, uint32_t B, uint32_t slots_smem, uint32_t nwarps, bool kappa,
                                                   bool tarr_global, uint32_t I, bool cal)
 {
     SmemLayout L;
@@ -1973,11 +1973,16 @@ __host__ __device__ inline SmemLayout smem_layout(uint32_t Npad, uint32_t B, uin
     L.off_pfcur = o; o += 2 * Npad;
     L.off_pfrem = o; o += 2 * Npad;
     o = (o + 15u) & ~15u;
-    L.off_sfin16 = o; if (slots_smem) o += 2 * Npad * B;
+    // the slot arrays of the image cover the padded GPUs; on chip only the N real ones have any (N = 16, B = 256: 16 KB of shared
+    // memory instead of 24, which is 12 resident replications per SM instead of 9)
+    const uint32_t words = (B + 31u) >> 5;
+    L.img_sfin16 = o;
+    L.img_socc = (o + (slots_smem ? 2 * Npad * B : 0u) + 15u) & ~15u;
+    L.srv_bytes = (L.img_socc + (slots_smem ? 4 * Npad * words : 0u) + 15u) & ~15u;
+    L.off_sfin16 = o; if (slots_smem) o += 2 * N * B;
     o = (o + 15u) & ~15u;
-    L.off_socc = o; if (slots_smem) o += 4 * Npad * ((B + 31u) >> 5);
+    L.off_socc = o; if (slots_smem) o += 4 * N * words;
     o = (o + 15u) & ~15u;
-    L.srv_bytes = o;
     L.off_bkt = o; if (cal) o += (Npad + 127u) & ~127u;       // calendar of iteration ends
     L.off_picked = o; if (cal) o += 2 * 32;
     L.off_touch = o; o += 4 * TOUCH_CAP;
@@ -2045,7 +2050,7 @@ __global__ void __launch_bounds__(32) qsim_init_kernel(Params p)
     extern __shared__ __align__(16) char sm[];
     const int lane = threadIdx.x;
     for (uint32_t rep = blockIdx.x; rep < p.R; rep += gridDim.x) {
-        const SmemLayout L = smem_layout(p.Npad, p.B, p.slots_smem, 1, p.coef[5] != 0.0, p.tarr_global != 0, p.I, false);
+        const SmemLayout L = smem_layout(p.Npad, p.Npad, p.B, p.slots_smem, 1, p.coef[5] != 0.0, p.tarr_global != 0, p.I, false);       // (laid out as the image)
         Sim<SPLT, FT> s(p, lane, rep);
         bind_pointers(s, sm, L);
         __syncwarp();
@@ -2111,16 +2116,39 @@ __device__ __forceinline__ void st_release_u32(uint32_t *a, uint32_t v)
 // Another block is running that chunk, so the wait lasts one chunk at most.
 constexpr uint32_t CHUNK_SPIN_LIMIT = 1u << 28;
 
+// The per-GPU image of a replication between global memory and its place on chip, in 16-byte words (IN: to shared memory).
+template <bool IN>
+__device__ __forceinline__ void copy16(char *sm, char *img, uint32_t bytes, uint32_t tid, uint32_t nthr)
+{
+    for (uint32_t o = tid * 16; o < bytes; o += nthr * 16) {
+        if (IN) *reinterpret_cast<uint4 *>(sm + o) = *reinterpret_cast<const uint4 *>(img + o);
+        else    *reinterpret_cast<uint4 *>(img + o) = *reinterpret_cast<const uint4 *>(sm + o);
+    }
+}
+template <bool IN>
+__device__ __forceinline__ void stage_image(char *sm, char *img, const SmemLayout &L, const Params &p, uint32_t tid, uint32_t nthr)
+{
+    copy16<IN>(sm, img, L.img_sfin16, tid, nthr);
+    if (p.slots_smem) {
+        copy16<IN>(sm + L.off_sfin16, img + L.img_sfin16, 2 * p.N * p.B, tid, nthr);
+        copy16<IN>(sm + L.off_socc, img + L.img_socc, 4 * p.N * ((p.B + 31u) >> 5), tid, nthr);
+    }
+}
+
 // Advance replications to their new end time (or until the per-launch event budget runs out).
 template <int SPLT, uint32_t FT>
 // One-warp instances whose slot records live in global memory need little shared memory, so registers decide how many
 // replications are resident on an SM: they are compiled for at least 12 blocks per SM (at most 168 registers, a few
 // bytes of spills; +16-24 % at N = 64 with thousands of replications).  Instances with the finish stamps on chip are
-// limited by shared memory and keep all the registers they want (the cap cost them 13 %).
+// limited by shared memory and keep all the registers they want (the cap cost them 13 %), but for those of up to 32 GPUs, whose
+// stamps take little (N = 16, R = 8192: 133 -> 98 ms).
 #ifndef QSIM_MIN_BLOCKS
 #define QSIM_MIN_BLOCKS 12
 #endif
-__global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, ((FT & F_MW) || (FT & F_SLOTS)) ? 1 : QSIM_MIN_BLOCKS) qsim_run_kernel(Params p)
+#ifndef QSIM_SLOT_BLOCKS
+#define QSIM_SLOT_BLOCKS 12
+#endif
+__global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, (FT & F_MW) ? 1 : ((FT & F_SLOTS) ? (SPLT == 1 ? QSIM_SLOT_BLOCKS : 1) : QSIM_MIN_BLOCKS)) qsim_run_kernel(Params p)
 {
     extern __shared__ __align__(16) char sm[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -2182,16 +2210,15 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, ((FT & F_MW) |
                 continue;
             }
         } else if (!p.advance && h.done) continue;
-        const SmemLayout L = smem_layout(p.Npad, p.B, p.slots_smem, nthr >> 5, p.coef[5] != 0.0, p.tarr_global != 0, p.I, Sim<SPLT, FT>::CAL);
+        const SmemLayout L = smem_layout(p.N, p.Npad, p.B, p.slots_smem, nthr >> 5, p.coef[5] != 0.0, p.tarr_global != 0, p.I, Sim<SPLT, FT>::CAL);
         Sim<SPLT, FT> s(p, lane, rep);
         s.warp = warp;
         s.nwarps = (int)(nthr >> 5);
         bind_pointers(s, sm, L);
         s.block_sync();
         // stage state: per-GPU arrays (coalesced 16-byte copies) and the class records; clear the per-warp accounting
-        const char *img = p.srv + (size_t)rep * p.srv_bytes;
-        for (uint32_t o = tid * 16; o < L.srv_bytes; o += nthr * 16)
-            *reinterpret_cast<uint4 *>(sm + o) = *reinterpret_cast<const uint4 *>(img + o);
+        char *const img = p.srv + (size_t)rep * p.srv_bytes;
+        stage_image<true>(sm, img, L, p, (uint32_t)tid, nthr);
         {
             const uint4 *src = reinterpret_cast<const uint4 *>(h.cs);
             uint4 *dst = reinterpret_cast<uint4 *>(s.cs);
@@ -2243,9 +2270,7 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, ((FT & F_MW) |
         if (warp == 0 && lane < (int)p.I) s.cs[lane].adraw -= s.ring_n;     // unused arrival draws are produced again next time
         s.block_sync();
         // stage back
-        char *out = p.srv + (size_t)rep * p.srv_bytes;
-        for (uint32_t o = tid * 16; o < L.srv_bytes; o += nthr * 16)
-            *reinterpret_cast<uint4 *>(out + o) = *reinterpret_cast<const uint4 *>(sm + o);
+        stage_image<false>(sm, img, L, p, (uint32_t)tid, nthr);
         {
             uint4 *dst = reinterpret_cast<uint4 *>(h.cs);
             const uint4 *src = reinterpret_cast<const uint4 *>(s.cs);

@@ -453,7 +453,7 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
     // (the limit of 40 KB counts MAXI accounting records and 160 bytes that the block no longer has: which configurations
     // keep their stamps on chip fixes the layout of saved workspaces)
     const uint32_t spared = 160u + (uint32_t)sizeof(WarpClassStats) * MAXI - (((uint32_t)sizeof(WarpClassStats) * cfg.I + 15u) & ~15u);
-    p.slots_smem = smem_layout(p.Npad, p.B, 1, 1, kappa, p.Npad > 128u, cfg.I, false).total + spared <= 40u * 1024u ? 1u : 0u;
+    p.slots_smem = smem_layout(p.Npad, p.Npad, p.B, 1, 1, kappa, p.Npad > 128u, cfg.I, false).total + spared <= 40u * 1024u ? 1u : 0u;
     if (cfg.N > 992u) p.slots_smem = 0;     // (from 32 rows on the layout is that of several warps, which retire through the global lists)
     if (p.slots_smem) v = pick_run_kernel(cfg.N, feat | F_SLOTS, h.scan);
     h.run_fn = v.fn;
@@ -464,8 +464,8 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
     p.tarr_global = (p.Npad > 128u) ? 1u : 0u;
     const bool cal = cfg.N > 128u && h.nwarps == 1 && !h.scan;      // run-time row count, one warp (Sim::CAL)
     calendar_shape(cfg.N, cfg.B, cfg.C, coef, p);
-    h.lay = smem_layout(p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I, cal);
-    h.init_smem = smem_layout(p.Npad, p.B, p.slots_smem, 1, kappa, p.tarr_global != 0, cfg.I, false).total;
+    h.lay = smem_layout(cfg.N, p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I, cal);
+    h.init_smem = smem_layout(p.Npad, p.Npad, p.B, p.slots_smem, 1, kappa, p.tarr_global != 0, cfg.I, false).total;
     p.srv_bytes = h.lay.srv_bytes;
     if (h.lay.total > 227u * 1024u - 64u)       // a few bytes of the block are the kernel's own
         return fail(QSIM_EINVAL, "N too large: per-replication GPU state does not fit shared memory");
