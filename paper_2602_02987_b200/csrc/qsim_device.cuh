@@ -53,7 +53,7 @@ constexpr uint32_t CAL_FREE = 16;        // free lanes from which the calendar l
 // run time; otherwise the set bits say which features the instance contains and everything else is
 // compiled out.  SPL > 0 fixes the number of simulated GPUs per lane (N <= 32 SPL) so the per-GPU loops unroll.
 constexpr uint32_t F_GENERIC = 1, F_ABANDON = 2, F_SLI = 4, F_KAPPA = 8, F_HIST = 16, F_BLOCKS = 32, F_RANDOM = 64,
-                   F_OCC = 128, F_SLOTS = 256, F_MW = 512, F_FCFS = 1024, F_SLIG = 2048, F_IMM = 4096, F_SCAN = 8192;
+                   F_OCC = 128, F_SLOTS = 256, F_MW = 512, F_FCFS = 1024, F_SLIG = 2048, F_IMM = 4096, F_SCAN = 8192, F_INJECT = 16384;
 // F_SCAN (run-time row count): rounds read all GPUs instead of working from the calendar of iteration ends.
 // F_MW: several warps per replication.  Warp 0 (the master) runs the round loop and every event handler; the
 // other warps (helpers) wait at a block barrier for commands and take their share of the per-GPU work of a
@@ -475,7 +475,7 @@ struct Sim {
     __device__ void schedule_from(double t0)
     {
         ClassState &c = cs[lane];
-        if ((F & F_GENERIC) && p.n_inject > 0) {
+        if ((F & (F_GENERIC | F_INJECT)) && p.n_inject > 0) {
             // trace replay: the next entry of this class in the injected list (c.ablk is the read position)
             uint32_t k = c.ablk;
             while (k < p.n_inject && p.inject_job[3 * k] != (uint32_t)lane) ++k;

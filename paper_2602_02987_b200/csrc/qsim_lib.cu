@@ -269,6 +269,9 @@ void add_variants(std::vector<RunVariant> &v)
     v.push_back({SPL, F_OCC | F_ABANDON, qsim_run_kernel<SPL, F_OCC | F_ABANDON>});
     v.push_back({SPL, F_OCC | F_ABANDON | F_SLI | F_HIST, qsim_run_kernel<SPL, F_OCC | F_ABANDON | F_SLI | F_HIST>});
     v.push_back({SPL, F_SLOTS | F_OCC | F_ABANDON | F_SLI | F_HIST, qsim_run_kernel<SPL, F_SLOTS | F_OCC | F_ABANDON | F_SLI | F_HIST>});
+    // priority gate with blocks and histograms (time-varying demand); trace replay with the KV slope and uniform placement
+    v.push_back({SPL, F_ABANDON | F_BLOCKS | F_HIST, qsim_run_kernel<SPL, F_ABANDON | F_BLOCKS | F_HIST>});
+    if (SPL == 1) v.push_back({SPL, F_SLOTS | F_OCC | F_RANDOM | F_KAPPA | F_INJECT, qsim_run_kernel<SPL, F_SLOTS | F_OCC | F_RANDOM | F_KAPPA | F_INJECT>});
     v.push_back({SPL, F_GENERIC, qsim_run_kernel<SPL, F_GENERIC>});
 }
 
@@ -279,6 +282,7 @@ void add_row_variants(std::vector<RunVariant> &v)
     v.push_back({0, W | F_OCC | F_ABANDON, qsim_run_kernel<0, W | F_OCC | F_ABANDON>});
     v.push_back({0, W | F_OCC | F_ABANDON | F_SLI | F_HIST, qsim_run_kernel<0, W | F_OCC | F_ABANDON | F_SLI | F_HIST>});
     v.push_back({0, W | F_ABANDON | F_BLOCKS | F_HIST, qsim_run_kernel<0, W | F_ABANDON | F_BLOCKS | F_HIST>});
+    v.push_back({0, W | F_SLOTS | F_OCC | F_ABANDON | F_RANDOM, qsim_run_kernel<0, W | F_SLOTS | F_OCC | F_ABANDON | F_RANDOM>});
     v.push_back({0, W | F_GENERIC, qsim_run_kernel<0, W | F_GENERIC>});
 }
 
@@ -446,6 +450,7 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
     }
     const bool kappa = coef[5] != 0.0;
     const uint32_t feat = features_of(cfg, classes, coef);
+    h.feat = feat;
     RunVariant v = pick_run_kernel(cfg.N, feat, h.scan);
     // the per-GPU arrays are padded to the unrolled row count of the chosen instance
     if (v.spl > 0) p.Npad = (uint32_t)v.spl * 32u;
@@ -923,8 +928,8 @@ int qsim_set_injected(qsim_t *h, const double *t, const uint32_t *job, uint64_t 
     h->par.inject_t = h->d_inject_t;
     h->par.inject_job = h->d_inject_job;
     h->par.n_inject = (uint32_t)n;
-    // the trace source lives in the run-time-configured instance
-    RunVariant v = pick_run_kernel(h->cfg.N, ~0u, h->scan);
+    // the trace source lives in the instances built for it and in the run-time-configured ones
+    RunVariant v = pick_run_kernel(h->cfg.N, h->feat | F_INJECT | (h->par.slots_smem ? F_SLOTS : 0u), h->scan);
     if (h->nwarps > 1)
         for (const RunVariant &mw : run_variants())
             if (mw.spl < 0 && (mw.feat & F_GENERIC)) v = mw;
