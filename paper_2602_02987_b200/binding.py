@@ -164,18 +164,13 @@ def marshal(inp):
     return cfg, classes, rates, lengths, prices, coeffs, tg
 
 
-def _unpack(per, R, I, T_hist=None):
-    out = {}
-    for n in _COUNTERS:
-        out[n] = np.array([[getattr(per[r].cls[i], n) for i in range(I)] for r in range(R)], np.uint64)
-    for n in _STATE:
-        out[n] = np.array([[getattr(per[r].cls[i], n) for i in range(I)] for r in range(R)], np.uint32)
-    for n in _SUMS:
-        out[n] = np.array([[getattr(per[r].cls[i], n) for i in range(I)] for r in range(R)], np.float64)
-    for n in ("iters_mixed", "iters_solo", "events"):
-        out[n] = np.array([getattr(per[r], n) for r in range(R)], np.uint64)
-    for n in ("busy_mixed", "busy_solo", "T_elapsed"):
-        out[n] = np.array([getattr(per[r], n) for r in range(R)], np.float64)
+def _unpack(per, R, I):
+    """Statistics records (a ctypes array of R of them, or one) -> arrays of their fields, classes beyond I left out."""
+    rec = np.frombuffer(per, dtype=np.dtype(qsim_rep_stats), count=R)
+    cls = rec["cls"][:, :I]
+    out = {n: cls[n].copy() for n in _COUNTERS + _STATE + _SUMS}
+    for n in ("iters_mixed", "iters_solo", "events", "busy_mixed", "busy_solo", "T_elapsed"):
+        out[n] = rec[n].copy()
     return out
 
 
@@ -286,7 +281,7 @@ class QSim:
         if with_totals:
             b, s = C.c_double(), C.c_double()
             _check(self.L.qsim_revenue(self.h, C.byref(tot), C.byref(b), C.byref(s)))
-            out["_totals"] = _unpack((tot,), 1, I)
+            out["_totals"] = _unpack(tot, 1, I)
             out["_revenue_bundled"] = b.value
             out["_revenue_separate"] = s.value
         return out
@@ -333,7 +328,7 @@ def simulate_host(inp, horizon_iters: int, per_rep: bool = True) -> dict:
     _check(L.qsim_simulate(C.byref(cfg), classes, _ptr(rates), _ptr(lengths), _ptr(prices), _ptr(coeffs), tg,
                            int(horizon_iters), C.byref(tot), per))
     out = _unpack(per, inp.R, inp.I) if per_rep else {}
-    out["_totals"] = _unpack((tot,), 1, inp.I)
+    out["_totals"] = _unpack(tot, 1, inp.I)
     return out
 
 
@@ -347,7 +342,7 @@ def simulate_waves(inp, horizon_iters: int, wave: int = 0) -> dict:
     _check(L.qsim_simulate_waves(C.byref(cfg), classes, _ptr(rates), _ptr(lengths), _ptr(prices), _ptr(coeffs), tg,
                                  int(horizon_iters), int(wave), C.byref(tot), per, C.byref(n)))
     out = _unpack(per, inp.R, inp.I)
-    out["_totals"] = _unpack((tot,), 1, inp.I)
+    out["_totals"] = _unpack(tot, 1, inp.I)
     out["_waves"] = int(n.value)
     return out
 
@@ -364,7 +359,7 @@ def simulate_static(inp, horizon_iters: int, stream=None) -> dict:
     _check(L.qsim_simulate_static(C.byref(cfg), classes, _ptr(rates), _ptr(lengths), _ptr(prices), _ptr(coeffs), tg,
                                   int(horizon_iters), C.byref(tot), per, sp))
     out = _unpack(per, inp.R, inp.I)
-    out["_totals"] = _unpack((tot,), 1, inp.I)
+    out["_totals"] = _unpack(tot, 1, inp.I)
     return out
 
 
@@ -413,22 +408,15 @@ class QSimCTMC:
         with torch.cuda.device(self.device):
             _check(self.L.qsim_ctmc_stats(C.byref(self.cfg), C.c_void_p(self.ptr), self.nbytes,
                                           C.c_void_p(self.stream.cuda_stream), per))
-        raw = np.frombuffer(per, dtype=np.uint8).reshape(R, C.sizeof(qsim_ctmc_rep_stats))
-        o_state = 10 * 8 * MAXI
-        o_area = o_state + 5 * 4 * MAXI + 4 * MAXI
-        cnt = raw[:, :o_state].copy().view(np.uint64).reshape(R, MAXI, 10)
-        state = raw[:, o_state:o_state + 5 * 4 * MAXI].copy().view(np.uint32).reshape(R, MAXI, 5)
-        area = raw[:, o_area:o_area + 5 * 8 * MAXI].copy().view(np.float64).reshape(R, MAXI, 5)
-        tail = raw[:, o_area + 5 * 8 * MAXI:].copy()
+        rec = np.frombuffer(per, dtype=np.dtype(qsim_ctmc_rep_stats))
+        # the classes in use first, in one pass over the records, then one array per statistic
+        cnt, state, area = (rec[n][:, :I].copy() for n in ("cnt", "state", "area"))
         out = {}
-        for k, n in enumerate(_CTMC_COUNTERS):
-            out[n] = np.ascontiguousarray(cnt[:, :I, k])
-        for k, n in enumerate(_STATE):
-            out[n] = np.ascontiguousarray(state[:, :I, k])
-        for k, n in enumerate(_CTMC_AREAS):
-            out[n] = np.ascontiguousarray(area[:, :I, k])
-        out["events"] = tail[:, :8].copy().view(np.uint64).reshape(R)
-        out["T_elapsed"] = tail[:, 8:16].copy().view(np.float64).reshape(R)
+        for names, values in ((_CTMC_COUNTERS, cnt), (_STATE, state), (_CTMC_AREAS, area)):
+            for k, n in enumerate(names):
+                out[n] = np.ascontiguousarray(values[:, :, k])
+        out["events"] = rec["events"].copy()
+        out["T_elapsed"] = rec["T_elapsed"].copy()
         # per-GPU revenue rate of every replication under the instance's charging scheme (qsim_ctmc_revenue)
         rate = np.zeros(R, np.float64)
         P = np.ascontiguousarray(self.inp.P, np.float64); D = np.ascontiguousarray(self.inp.D, np.float64)
