@@ -339,7 +339,7 @@ void choose_multiwarp(uint32_t N, uint32_t feat, Params &p, RunKernel &fn, uint3
     const char *force = std::getenv("QSIM_KERNEL");
     const bool generic_only = force && std::strcmp(force, "generic") == 0;
     // mode bits must match exactly, capability bits may be present unused (as in pick_run_kernel)
-    constexpr uint32_t MODES = F_SLI | F_SLIG | F_IMM | F_RANDOM | F_OCC | F_FCFS | F_HIST;
+    constexpr uint32_t MODES = F_SLI | F_SLIG | F_IMM | F_RANDOM | F_OCC | F_FCFS | F_HIST | F_KAPPA;
     const RunVariant *best = nullptr;
     int best_bits = 99;
     for (const RunVariant &v : run_variants()) {
@@ -373,9 +373,9 @@ RunVariant pick_run_kernel(uint32_t N, uint32_t feat, bool scan)
         int spl_fit = rows <= 1 ? 1 : (rows <= 2 ? 2 : (rows <= 4 ? 4 : 0));
         if (v.spl != spl_fit) continue;
         if (v.feat & F_GENERIC) { if (!best) { best = &v; best_bits = 98; } continue; }
-        // mode bits (router, placement, gate, histograms) select code and must match exactly; capability bits
-        // (abandonment, KV slope, blocks) may be present without being used
-        constexpr uint32_t MODES = F_SLI | F_SLIG | F_IMM | F_RANDOM | F_OCC | F_FCFS | F_HIST | F_SLOTS;
+        // mode bits (router, placement, gate, histograms, KV slope: its arrays exist only where the slope is not zero) select
+        // code and must match exactly; capability bits (abandonment, blocks, trace) may be present without being used
+        constexpr uint32_t MODES = F_SLI | F_SLIG | F_IMM | F_RANDOM | F_OCC | F_FCFS | F_HIST | F_SLOTS | F_KAPPA;
         if (feat == ~0u || (feat & MODES) != (v.feat & MODES) || (feat & ~v.feat) != 0) continue;
         const int extra = __builtin_popcount(v.feat & ~(feat | F_SCAN));
         if (extra < best_bits) { best = &v; best_bits = extra; }

@@ -69,3 +69,27 @@ def test_run_until_matches_iteration_horizon_on_the_gpu():
             assert np.allclose(sa[k], sb[k], rtol=1e-12, atol=0), k
         else:
             assert np.array_equal(sa[k], sb[k]), k
+
+
+@pytest.mark.parametrize("theta", [0.0, 0.2])
+@pytest.mark.parametrize("coeffs", [presets.COEFFS_PAPER, presets.COEFFS_PAPER_KV], ids=["no KV slope", "KV slope"])
+@pytest.mark.parametrize("placement", [0, 1])
+@pytest.mark.parametrize("n", [4, 10, 32, 33])
+def test_trace_replay_with_and_without_the_kv_slope(n, placement, coeffs, theta):
+    # the KV bookkeeping has memory only where the slope is not zero: every instance that a replay can get, up to and beyond 32 GPUs
+    from oracle import OracleSim
+    from paper_2602_02987_b200 import QSim
+    inp, Pm, Dm = presets.trace_replay(n=n, R=2, T=25.0, placement=placement, coeffs=coeffs)
+    inp = inp.with_(theta=np.full(inp.I, theta))
+    out = []
+    for cls in (QSim, OracleSim):
+        sim = cls(inp)
+        made = online.run_online(sim, inp, Pm, Dm, 25.0)
+        out.append((made, sim.stats(), [sim.server_state(r) for r in range(inp.R)]))
+        sim.close()
+    (dg, gs, gstate), (do, os_, ostate) = out
+    assert dg == do
+    assert_parity(gs, os_, what=f"trace replay n={n}, placement {placement}, slope {coeffs[5]}, theta {theta}")
+    for a, b in zip(gstate, ostate):
+        for k in a:
+            assert np.array_equal(a[k], b[k]), k
