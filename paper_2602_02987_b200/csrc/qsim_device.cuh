@@ -1257,7 +1257,9 @@ struct Sim {
             d_pool = pool;
             d_pk = pk & 0x7fffffffu;
             d_gpu = immediate ? g : NONE32;
-            direct = immediate || (pool ? dq_n1 : dq_n0) == 0;
+            // (The solo pool is served first; under random placement both pools draw from one sequence, so a request of the
+            // mixed pool waits its turn behind a backlog of the solo pool, which new targets may have made room for.)
+            direct = immediate || ((pool ? dq_n1 : dq_n0) == 0 && !(f_random() && pool == 1u && dq_n0 != 0));
             if (!direct) enqueue_decode();
             drain_dirty = true;
             gate_dirty = true;

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 from qsim_inputs import online, presets
+from qsim_inputs.spec import PLACE_LEAST_LOADED, PLACE_RANDOM, ROUTER_SLI, ROUTER_SLI_GENERAL
 
 from parity import assert_parity
 
@@ -90,6 +91,37 @@ def test_trace_replay_with_and_without_the_kv_slope(n, placement, coeffs, theta)
     (dg, gs, gstate), (do, os_, ostate) = out
     assert dg == do
     assert_parity(gs, os_, what=f"trace replay n={n}, placement {placement}, slope {coeffs[5]}, theta {theta}")
+    for a, b in zip(gstate, ostate):
+        for k in a:
+            assert np.array_equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("placement", [PLACE_LEAST_LOADED, PLACE_RANDOM])
+@pytest.mark.parametrize("router", [ROUTER_SLI, ROUTER_SLI_GENERAL])
+@pytest.mark.parametrize("N", [12, 140])
+def test_smaller_mixed_group_with_a_backlog_in_the_solo_pool(N, router, placement):
+    # New targets turn mixed GPUs into solo ones, so the solo pool's backlog finds slots at the next event; when that event ends a
+    # prefill whose request goes to the empty mixed pool, the solo pool is still served first (both draw from one sequence)
+    from oracle import OracleSim
+    from paper_2602_02987_b200 import QSim
+    # (few first events after a change are such a prefill: many replications and changes)
+    R = 512 if N < 100 else 96
+    inp = presets.crowded("decode", N=N, R=R, placement=placement, router=router)
+    if router == ROUTER_SLI_GENERAL:
+        inp = inp.with_(w_solo=np.array([[0.7, 0.3]]), w_mix=np.array([[0.2, 0.8]]))
+    w = (inp.w_solo[0], inp.w_mix[0]) if router == ROUTER_SLI_GENERAL else (None, None)
+    out = []
+    for cls in (QSim, OracleSim):
+        sim = cls(inp)
+        for k in range(48):
+            M = N // 2 if k % 2 == 0 else N // 4
+            sim.set_targets(M, inp.xstar[0], inp.n_xstar[0], inp.n_qpstar[0], [0.88, 0.88], *w)
+            sim.run(6)
+        out.append((sim.stats(), [sim.server_state(r) for r in range(inp.R)]))
+        sim.close()
+    (gs, gstate), (os_, ostate) = out
+    assert os_["Qd"].sum() > R
+    assert_parity(gs, os_, what=f"target change, N={N}, router {router}, placement {placement}")
     for a, b in zip(gstate, ostate):
         for k in a:
             assert np.array_equal(a[k], b[k]), k
