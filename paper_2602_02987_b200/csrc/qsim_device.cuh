@@ -47,6 +47,7 @@ constexpr int NBIN = 1024;
 constexpr unsigned FULL = 0xffffffffu;
 constexpr uint32_t NONE32 = 0xffffffffu;
 constexpr int TOUCH_CAP = 48;
+constexpr int ARRIVALS_PER_ROUND = 64;    // arrivals of a class that one round takes (a trace may bring any number at one time)
 constexpr uint32_t CAL_FREE = 16;        // free lanes from which the calendar loads another bucket
 
 // Compile-time specialisation of the run kernel.  With F_GENERIC every mode is read from the parameters at
@@ -1693,22 +1694,24 @@ struct Sim {
             bool progressed = false;
             const bool first_here = first_is_event && tint <= tend_bits, arrival_now = first_here && src >= SRC_ARRIVAL && src < SRC_ABP;
             const bool local = n_idle_pf == 0 && !force_nonlocal;
+            bool redo = false;
             if ((local || arrival_now) && lane < (int)p.I) {
                 // local arrivals of this lane's class, or the arrival that is the round's event (see run())
                 const ClassState &c = cs[lane];
 #pragma unroll 1
-                for (int guard = 0; guard < 64; ++guard) {
+                for (int guard = 0;; ++guard) {
                     const unsigned long long v = (unsigned long long)__double_as_longlong(c.ta);
                     if (local) {
                         if (!(v < lim_t || (v == lim_t && SRC_ARRIVAL + (uint32_t)lane < lim_s))) break;
                         if (f_abandon() && v > (unsigned long long)__double_as_longlong(c.abp.t_ab)) break;
                         if (bucket_abs(__longlong_as_double((long long)v)) > cur) break;
                     } else if (!(arrival_now && src == SRC_ARRIVAL + (uint32_t)lane && guard == 0)) break;
+                    if (guard == ARRIVALS_PER_ROUND) { redo = true; break; }
                     arrival_local();
                     progressed = true;
                 }
             }
-            bool redo = sched_pending && !arrival_now;
+            redo = redo || (sched_pending && !arrival_now);
             if (f_abandon() && lane < (int)p.I) {
                 const unsigned long long v = (unsigned long long)__double_as_longlong(cs[lane].abp.t_ab);
                 redo = redo || v < tint || (v == tint && SRC_ABP + (uint32_t)lane < src);
@@ -1840,25 +1843,28 @@ struct Sim {
                 __syncthreads();
             }
             const bool local = n_idle_pf == 0 && !force_nonlocal;
+            bool redo = false;
             if ((local || arrival_now) && lane < (int)p.I) {
                 // local arrivals of this lane's class, in time order, up to the limit and up to the class's own
                 // next abandonment (which each arrival moves); or the one arrival that is the round's event (it is not local,
                 // so none is): nothing in the rest of the round depends on whether it joins its queue here or at the end
                 const ClassState &c = cs[lane];
 #pragma unroll 1
-                for (int guard = 0; guard < 64; ++guard) {
+                for (int guard = 0;; ++guard) {
                     const unsigned long long v = (unsigned long long)__double_as_longlong(c.ta);
                     if (local) {
                         if (!(v < lim_t || (v == lim_t && SRC_ARRIVAL + (uint32_t)lane < lim_s))) break;
                         if (f_abandon() && v > (unsigned long long)__double_as_longlong(c.abp.t_ab)) break;
                     } else if (!(arrival_now && src == SRC_ARRIVAL + (uint32_t)lane && guard == 0)) break;
+                    if (guard == ARRIVALS_PER_ROUND) { redo = true; break; }
                     arrival_local();
                     progressed = true;
                 }
             }
-            // a class that ran out of draws has an unknown next arrival, possibly before T_int, and a local
-            // arrival may have pulled its class's next abandonment before T_int: then T_int is not next after all
-            bool redo = sched_pending && !arrival_now;
+            // a class that ran out of draws has an unknown next arrival, possibly before T_int, one that stopped at the bound of
+            // the loop has a known one, and a local arrival may have pulled its class's next abandonment before T_int: then T_int
+            // is not next after all
+            redo = redo || (sched_pending && !arrival_now);
             if (f_abandon() && lane < (int)p.I) {
                 const unsigned long long v = (unsigned long long)__double_as_longlong(cs[lane].abp.t_ab);
                 redo = redo || v < tint || (v == tint && SRC_ABP + (uint32_t)lane < src);

@@ -125,3 +125,15 @@ def test_smaller_mixed_group_with_a_backlog_in_the_solo_pool(N, router, placemen
     for a, b in zip(gstate, ostate):
         for k in a:
             assert np.array_equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("burst", [64, 65, 200])
+@pytest.mark.parametrize("N,rounds", [(1, "scan"), (40, "scan"), (140, "scan"), (140, "calendar")])
+def test_a_burst_of_arrivals_joins_the_queue_before_the_next_event(N, rounds, burst, monkeypatch):
+    # every GPU holds a prefill, which ends 0.7 ms after the burst (less than the shortest iteration, 5 ms): what finds the queue full is
+    # lost, although the prefills that end next make room
+    monkeypatch.setenv("QSIM_ROUNDS", rounds)
+    inj = [(0.0, 0, 512, 40)] * N + [(0.0195, 0, 900, 25)] * burst + [(0.0196, 0, 500, 10)] * 3
+    inp = presets.single_class(N=N, B=8, P=900, D=25, lam=0.5, theta=0.0, R=2, M=N, inject=inj).with_(qcap=64 if burst == 64 else burst - 1)
+    st = _both(inp, 90)
+    assert int(st["overflow"][0, 0]) == (3 if burst == 64 else 4)
