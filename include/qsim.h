@@ -147,8 +147,10 @@ int qsim_bind(qsim_t *h, void *dev_workspace, size_t bytes, void *cuda_stream);
 /*
  * Checkpoint / resume.  All state of the replications lives in the caller's workspace, so a checkpoint is a copy of
  * its first qsim_workspace_bytes bytes taken between calls (after qsim_run / qsim_run_until has returned), and a
- * resume is: qsim_create with the same arguments, copy the bytes into a [device] workspace, then this call in place of
- * qsim_bind.  Nothing is initialised; the next qsim_run continues where the checkpointed run stopped, with the results
+ * resume is: qsim_create with the same arguments, copy the bytes into a [device] workspace of that size, then this call in
+ * place of qsim_bind.  A state goes on in the kernel family that it was saved by, whichever of the two the new handle would have
+ * got by itself (that is a rule on measured speed; qsim_workspace_bytes tells the size of the adopted one afterwards).
+ * Nothing is initialised; the next qsim_run continues where the checkpointed run stopped, with the results
  * of an uninterrupted sequence of the same calls [the time horizon of Eq. (21)-(23) composes, see qsim_run].  Targets installed with
  * qsim_set_targets are part of the handle, not of the workspace: install them again.  QSIM_ESTATE if the bytes hold
  * no resumable state (some replication stopped on an internal error) or were saved by a handle of another configuration or

@@ -197,7 +197,8 @@ class QSim:
                 _check(self.L.qsim_set_injected(self.h, _ptr(it), _ptr(ij), it.shape[0]))
             nbytes = C.c_size_t()
             _check(self.L.qsim_workspace_bytes(self.h, C.byref(nbytes)))
-            self.workspace_bytes = int(nbytes.value)
+            # (a saved state goes on in the kernel family that it is from, whose workspace may have another size)
+            self.workspace_bytes = int(nbytes.value) if checkpoint is None else checkpoint.numel()
             self.ws = torch.empty(self.workspace_bytes + 256, dtype=torch.uint8, device=self.device)
             base = (self.ws.data_ptr() + 255) & ~255
             self.stream = stream if stream is not None else torch.cuda.current_stream(self.device)
@@ -206,11 +207,12 @@ class QSim:
                 _check(self.L.qsim_bind(self.h, C.c_void_p(base), self.workspace_bytes, C.c_void_p(self.stream.cuda_stream)))
             else:
                 off = base - self.ws.data_ptr()
-                if checkpoint.numel() != self.workspace_bytes:
-                    raise QSimError("checkpoint size does not match this configuration")
                 self.ws[off:off + self.workspace_bytes].copy_(checkpoint)
                 _check(self.L.qsim_bind_restore(self.h, C.c_void_p(base), self.workspace_bytes,
                                                 C.c_void_p(self.stream.cuda_stream)))
+                _check(self.L.qsim_workspace_bytes(self.h, C.byref(nbytes)))
+                if nbytes.value != self.workspace_bytes:
+                    raise QSimError("checkpoint size does not match this configuration")
 
     def checkpoint(self):
         """The workspace bytes (a CPU uint8 tensor) after the work queued so far: pass them to QSim(..., checkpoint=)."""

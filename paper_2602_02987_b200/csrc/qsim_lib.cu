@@ -75,6 +75,7 @@ struct qsim {
     bool scan = false;            // one warp, run-time row count: rounds read all GPUs (see rounds_scan)
     void (*lane_fn)(qsimdev::Params) = nullptr;     // instance of the one-thread-per-replication run kernel
     bool allow_lane = true;       // the one-thread-per-replication family may run this handle
+    int family = -1;              // that family (1) or the warp family (0), whatever the rule says: that of an adopted workspace
     double coef[6]{};
 };
 
@@ -488,6 +489,9 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
         if (std::strcmp(e, "lane") == 0) lane = h.allow_lane && lane_supports(cfg, coef);
         else if (std::strcmp(e, "warp") == 0) lane = false;
     }
+    if (h.family >= 0) lane = h.family == 1 && h.allow_lane && lane_supports(cfg, coef);
+    h.resident_blocks = 0;
+    h.lane_fn = nullptr;
     if (lane) {
         // the smallest instance that contains the configuration's features
         const bool ab = p.any_theta != 0, sli = cfg.router == QSIM_ROUTER_SLI, hist = cfg.hist != 0, blk = cfg.nblk > 1;
@@ -832,21 +836,59 @@ int qsim_bind(qsim_t *h, void *ws, size_t bytes, void *cuda_stream)
     return QSIM_OK;
 }
 
-int qsim_bind_restore(qsim_t *h, void *ws, size_t bytes, void *cuda_stream)
+// Lays the handle out again (another kernel family), keeping the tables that it owns and what the caller has set.
+static int configure_again(qsim_t *h)
+{
+    const uint64_t budget = h->par.event_budget;
+    int rc = configure(*h, h->cfg, h->cls, h->prices, h->coef);
+    if (rc != QSIM_OK) return rc;
+    h->par.event_budget = budget;
+    cudaError_t e = allow_large_smem(reinterpret_cast<const void *>(h->run_fn));
+    if (e == cudaSuccess && h->lane_fn) e = allow_large_smem(reinterpret_cast<const void *>(h->lane_fn));
+    if (e != cudaSuccess) return fail(QSIM_ECUDA, cudaGetErrorString(e));
+    return QSIM_OK;
+}
+
+// Do the bytes come from a handle of the same configuration and layout?  (Waits for the stream.)
+static int adopt_workspace(qsim_t *h, void *ws, size_t bytes, void *cuda_stream)
 {
     int rc = attach_workspace(h, ws, bytes, cuda_stream);
     if (rc != QSIM_OK) return rc;
-    // the bytes must come from a handle of the same configuration and layout
     unsigned long long want[2], got[2] = { 0, 0 };
     workspace_tag(h, want);
     CUDA_TRY(cudaMemcpyAsync(got, reinterpret_cast<char *>(h->par.not_done) + 16, sizeof got, cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    if (got[0] != want[0] || got[1] != want[1])
+        return fail(QSIM_ESTATE, "the workspace was not saved by a handle of this configuration");
+    return QSIM_OK;
+}
+
+int qsim_bind_restore(qsim_t *h, void *ws, size_t bytes, void *cuda_stream)
+{
+    if (h) h->bound = false;       // until the bytes are known to be a state of this configuration
+    int rc = adopt_workspace(h, ws, bytes, cuda_stream);
+    if ((rc == QSIM_ESTATE || rc == QSIM_EWORKSPACE) && ws && h->allow_lane && h->par.n_inject == 0 && lane_supports(h->cfg, h->coef)) {
+        // Which kernel family a new handle gets is a rule on measured speed; a saved state goes on in the family that it is from.
+        const std::string why = g_err;
+        const int keep = h->family;
+        h->family = h->par.lane.on ? 0 : 1;
+        int other = configure_again(h);
+        if (other == QSIM_OK) other = adopt_workspace(h, ws, bytes, cuda_stream);
+        if (other != QSIM_OK) {
+            h->family = keep;
+            const int back = configure_again(h);
+            if (back != QSIM_OK) return back;
+            g_err = why;
+            return rc;
+        }
+        rc = QSIM_OK;
+    }
+    if (rc != QSIM_OK) return rc;
     // the end time reached so far is in every replication's record; a state in which any replication stopped on an
     // internal error cannot be resumed
     std::vector<RepHeader> hdr(h->cfg.R);
     CUDA_TRY(cudaMemcpyAsync(hdr.data(), h->par.hdr, hdr.size() * sizeof(RepHeader), cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
-    if (got[0] != want[0] || got[1] != want[1])
-        return fail(QSIM_ESTATE, "the workspace was not saved by a handle of this configuration");
     for (uint32_t r = 0; r < h->cfg.R; ++r)
         if (hdr[r].err != 0 || !(hdr[r].T_end >= 0.0) || !std::isfinite(hdr[r].T_end))
             return fail(QSIM_ESTATE, "the workspace does not hold a resumable state (replication " + std::to_string(r) + ")");
@@ -907,12 +949,8 @@ int qsim_set_injected(qsim_t *h, const double *t, const uint32_t *job, uint64_t 
     if (h->par.lane.on) {
         // trace replay lives in the warp-per-replication family: lay the handle out again for it
         h->allow_lane = false;
-        int rc = configure(*h, h->cfg, h->cls, h->prices, h->coef);
+        int rc = configure_again(h);
         if (rc != QSIM_OK) return rc;
-        h->par.blocks = h->d_blocks;
-        h->par.lengths = h->d_lengths;
-        cudaError_t e = allow_large_smem(reinterpret_cast<const void *>(h->run_fn));
-        if (e != cudaSuccess) return fail(QSIM_ECUDA, cudaGetErrorString(e));
     }
     for (uint64_t k = 0; k < n; ++k) {
         if (!(t[k] >= 0.0) || !std::isfinite(t[k]) || (k > 0 && t[k] < t[k - 1])) return fail(QSIM_EINVAL, "injected times must be ascending and >= 0");

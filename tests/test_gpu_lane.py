@@ -226,3 +226,35 @@ def test_whole_runs_in_waves_do_not_depend_on_the_wave_size():
     for k in resident["warp"]:
         if not k.startswith("hist"):
             assert np.array_equal(tail[k], resident["warp"][k][200:]), k
+
+
+@pytest.mark.parametrize("saved_by,default", [("lane", "warp"), ("warp", "lane")])
+def test_a_saved_state_goes_on_in_its_own_family(saved_by, default, monkeypatch):
+    # which family a handle gets is a rule that may differ between the handle that saved a state and the one that resumes it
+    from oracle import run_oracle
+    from paper_2602_02987_b200 import QSim, QSimError
+    inp = presets.cfg4(N=24, R=40)
+    warps = {"lane": 0, "warp": 1}
+    monkeypatch.setenv("QSIM_FAMILY", saved_by)
+    sim = QSim(inp)
+    assert sim.layout_info()["warps"] == warps[saved_by]
+    sim.run(300)
+    saved = sim.checkpoint()
+    sim.close()
+    monkeypatch.setenv("QSIM_FAMILY", default)
+    sim = QSim(inp, checkpoint=saved)
+    assert sim.layout_info()["warps"] == warps[saved_by]
+    sim.set_event_budget(50)
+    sim.run(200)
+    assert_parity(sim.stats(), run_oracle(inp, 500), what=f"{saved_by} state resumed")
+    again = sim.checkpoint()                        # and it can be saved and resumed again
+    sim.close()
+    sim = QSim(inp, checkpoint=again)
+    sim.run(100)
+    assert_parity(sim.stats(), run_oracle(inp, 600), what=f"{saved_by} state resumed twice")
+    sim.close()
+    # what neither family can have saved stays refused
+    with pytest.raises(QSimError, match="configuration|too small"):
+        QSim(inp.with_(seed=inp.seed + 1), checkpoint=saved)
+    with pytest.raises(QSimError, match="too small"):
+        QSim(inp, checkpoint=saved[:saved.numel() // 8])
