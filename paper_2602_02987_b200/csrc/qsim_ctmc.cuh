@@ -38,7 +38,7 @@ struct CtmcRep {
     uint32_t err, done;
     CtmcClk clk[CK_N][MAXI];
     uint32_t Qp[MAXI], X[MAXI], Qd[2][MAXI], Ym[MAXI], Ys[MAXI];
-    unsigned long long sli_ord[MAXI];
+    unsigned long long reserved[MAXI];       // (keeps the layout of saved workspaces)
     double area[CA_N][MAXI], area_t[CA_N][MAXI];
     unsigned long long cnt[MAXI][CC_N];
 };
@@ -324,7 +324,11 @@ struct CtmcSim {
                 sd(w_fire(e), q.t_fire);
                 su(w_draws(e), q.m);
                 if (k == 0) continue;
-                sd(w_acc(e), q.acc); sd(w_lvl(e), q.lvl); sd(w_last(e), q.t_last);
+                // the clock and the integral of a count are brought up to date together, but for a clock of intensity zero that an
+                // earlier build saved: that one stood still, so the time is the integral's (the two buffers have w_qd_last for it)
+                const double last = k == CK_ABP ? S.area_t[CA_QP][i] : (k == CK_SP ? S.area_t[CA_X][i] : (k == CK_SDM ? S.area_t[CA_YM][i]
+                                  : (k == CK_SDS ? S.area_t[CA_YS][i] : q.t_last)));
+                sd(w_acc(e), q.acc); sd(w_lvl(e), q.lvl); sd(w_last(e), last);
                 su(w_count(e), ((unsigned long long)cnt[k - 1] << 32) | cnt[k - 1]);
             }
             sd(w_qd_last(i), S.area_t[CA_QD][i]);

@@ -9,6 +9,8 @@ from qsim_inputs.spec import GATE_OCCUPANCY, GATE_PRIORITY, ROUTER_SLI, ROUTER_S
 
 pytestmark = pytest.mark.gpu
 
+RECORD = 3816      # bytes of a replication's record in the workspace
+
 
 def instance(I, R, router, gate, n=12, M=None):
     rng = np.random.default_rng(100 * I + R % 97)
@@ -43,3 +45,29 @@ def test_replications_per_warp_and_class_counts(I, R, router, gate, M):
                 assert np.array_equal(got[k][r], v[0]), (r, k)
             else:
                 assert np.allclose(got[k][r], v[0], rtol=1e-9, atol=1e-300), (r, k)
+
+
+@pytest.mark.parametrize("router", [ROUTER_SOLO_FIRST, ROUTER_SLI])
+def test_a_state_whose_clocks_of_intensity_zero_stood_still(router):
+    # A workspace saved by an earlier build without patience: the abandonment clocks were never brought up to date there, while the
+    # time integrals were.  The record: 40 bytes of scalars, then clocks [7][8] of (acc, lvl, t_last, t_fire, m), 8 bytes each.
+    import torch
+    from paper_2602_02987_b200 import QSimCTMC
+    inp = instance(2, 5, router, GATE_OCCUPANCY).with_(theta=np.zeros(2))
+    got = []
+    for old in (False, True):
+        sim = QSimCTMC(inp)
+        sim.run_until(7.0)
+        if old:
+            first = sim.ptr - sim.ws.data_ptr()
+            rec = sim.ws[first:first + inp.R * RECORD].view(inp.R, RECORD)
+            for k in (1, 2, 3):
+                for i in range(2):
+                    at = 40 + (k * 8 + i) * 40 + 16
+                    rec[:, at:at + 8] = 0
+            torch.cuda.synchronize()
+        sim.run_until(19.0)
+        got.append(sim.stats())
+        sim.close()
+    for k in got[0]:
+        assert np.array_equal(got[0][k], got[1][k]), k
