@@ -1635,9 +1635,21 @@ struct Sim {
                     } else {
                         if (d == 0) break;
                         const uint32_t skip = min(next_bucket(), d);
-                        if (cur + skip > cur_end) return true;          // nothing left up to T_end
-                        if (skip == 0) break;
-                        cur += skip; d = 0;
+                        if (skip >= 0x7ffffffeu) {
+                            // no GPU runs and d is at its cap: go to the first class event or block end, however far it is
+                            unsigned long long first = bt;
+                            if (lane < (int)p.I) first = min(first, (unsigned long long)__double_as_longlong(cs[lane].ta));
+                            const uint32_t hi = (uint32_t)(first >> 32), mhi = __reduce_min_sync(FULL, hi);
+                            const uint32_t mlo = __reduce_min_sync(FULL, hi == mhi ? (uint32_t)first : NONE32);
+                            first = ((unsigned long long)mhi << 32) | mlo;
+                            if (first > tend_bits) return true;
+                            cur = bucket_abs(__longlong_as_double((long long)first));
+                        } else {
+                            if (cur + skip > cur_end) return true;      // nothing left up to T_end
+                            if (skip == 0) break;
+                            cur += skip;
+                        }
+                        d = 0;
                     }
                     low = cur;
                     want = CAL_FREE;

@@ -11,7 +11,7 @@ import pytest
 from qsim_inputs import presets
 from qsim_inputs.spec import PLACE_LEAST_LOADED, PLACE_RANDOM, ROUTER_SLI
 
-from parity import assert_parity
+from parity import F64_KEYS, INT_KEYS, assert_parity
 
 pytestmark = pytest.mark.gpu
 
@@ -95,3 +95,30 @@ def test_calendar_is_rebuilt_by_every_launch():
     parts = check(presets.cfg4(N=200, R=2), [1, 2, 3, 5, 8, 13, 21, 34, 33], "calendar", budget=40)
     for k in ("arrivals", "admitted", "done_mixed", "done_solo", "iters_mixed", "iters_solo"):
         assert np.array_equal(whole[k], parts[k]), k
+
+
+@pytest.mark.parametrize("rounds", ["calendar", "scan"])
+@pytest.mark.parametrize("rate,T", [(0.0, 1e15), (1e-10, 4e8)])
+def test_long_idle_times_are_skipped(rate, T, rounds):
+    # an end time, or a next arrival, more than 2^31 buckets after the last event
+    from oracle import OracleSim
+    from paper_2602_02987_b200 import QSim
+    inp = together(140) if rate == 0.0 else presets.single_class(N=140, B=8, P=900, D=30, lam=rate, R=2, M=140)
+    with env(QSIM_ROUNDS=rounds):
+        sim = QSim(inp)
+    ora = OracleSim(inp)
+    for s in (sim, ora):
+        s.run_until(T)
+    got, ref = sim.stats(), ora.stats()
+    assert sim.round_count() < 10000
+    sim.close()
+    ora.close()
+    assert (got["arrivals"] > 0).all()
+    for k in INT_KEYS:
+        if k in ref:
+            assert np.array_equal(got[k], ref[k]), k
+    # a time integral is the difference of two sums of at most n times, none after the last event, in any order: each of the n
+    # additions of a sum rounds by at most 2^-53 of n times the last event's time
+    n, last = float(got["arrivals"].max()), 4e8 if rate > 0.0 else 10.0
+    for k in F64_KEYS:
+        assert np.allclose(got[k], ref[k], rtol=1e-9, atol=2 * n * n * last * 2.0 ** -53), k
