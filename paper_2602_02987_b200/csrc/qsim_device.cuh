@@ -1226,7 +1226,7 @@ struct Sim {
                 const unsigned long long ord = cs[i].sli_ord;
                 const double ps = __shfl_sync(FULL, b_ps, i);
                 uint32_t w0, w1, w2, w3;
-                if (CAL) draw(p, rep, (STREAM_SLI << 8) | i, ord, w0, w1, w2, w3);       // (+4 % inline at N = 256, -2 % at N = 16)
+                if (SPL == 0 && !(F & F_MW)) draw(p, rep, (STREAM_SLI << 8) | i, ord, w0, w1, w2, w3);       // (+4 % inline at N = 256, -2 % at N = 16)
                 else draw_rare(p, rep, (STREAM_SLI << 8) | i, ord, w0, w1, w2, w3);
                 pool = (u53(w0, w1) <= ps) ? 0u : 1u;
                 __syncwarp();       // every lane has read the ordinal before its owner advances it
