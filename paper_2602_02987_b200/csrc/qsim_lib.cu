@@ -45,6 +45,11 @@ struct Sections {
 
 }  // namespace
 
+struct RoundPlan {
+    bool scan = false;            // one warp, run-time row count: rounds read all GPUs instead of the calendar
+    uint32_t warps = 1;           // warps per replication that share the reading of all GPUs (1: the line above decides)
+};
+
 struct qsim {
     qsim_config cfg{};
     qsim_class cls[QSIM_MAXI]{};
@@ -72,7 +77,7 @@ struct qsim {
     int device = 0;
     void (*run_fn)(qsimdev::Params) = nullptr;
     uint32_t nwarps = 1;          // warps per replication (block size / 32)
-    bool scan = false;            // one warp, run-time row count: rounds read all GPUs (see rounds_scan)
+    RoundPlan plan;               // how the rounds of the warp family find what happens next on a large cluster
     void (*lane_fn)(qsimdev::Params) = nullptr;     // instance of the one-thread-per-replication run kernel
     bool allow_lane = true;       // the one-thread-per-replication family may run this handle
     int family = -1;              // that family (1) or the warp family (0), whatever the rule says: that of an adopted workspace
@@ -325,13 +330,10 @@ uint32_t features_of(const qsim_config &c, const qsim_class *cls, const double *
     return f;
 }
 
-// Several warps (master + helpers) per replication share the per-GPU scans: QSIM_WARPS=2..16, for cross-checks.  One warp
-// on the calendar is ahead at every size (it does not scan): N = 1024, R = 444 (24 blocks, histograms) 504 against 946 ms with two
-// warps, N = 1024, R = 2048 294 against 612, N = 2048, R = 888 507 against 1137 with four, N = 4096, R = 4 535 against 615 with sixteen.
-void choose_multiwarp(uint32_t N, uint32_t feat, Params &p, RunKernel &fn, uint32_t &nwarps)
+// Several warps (master + helpers) per replication share the per-GPU scans where round_plan says so.  QSIM_WARPS=1..16 overrides.
+void choose_multiwarp(uint32_t N, uint32_t feat, uint32_t W, Params &p, RunKernel &fn, uint32_t &nwarps)
 {
     const uint32_t rows = (N + 31u) / 32u;
-    uint32_t W = 1;
     if (const char *e = std::getenv("QSIM_WARPS")) {
         const int v = std::atoi(e);
         if (v >= 1 && v <= MW_MAX) W = (uint32_t)v;
@@ -406,26 +408,51 @@ void calendar_shape(uint32_t N, uint32_t B, uint32_t C, const double *coef, Para
     p.cal_K = (uint32_t)std::min(0.999 * tau_min / w, 254.0);        // (the margin is far above the rounding of a bucket index)
 }
 
-// One warp with a run-time row count: do rounds read all GPUs, or work from the calendar of iteration ends?  Reading all rows
-// pays when an event that is not local (a finished prefill, mostly) comes with many local ends, because one row then ends
+// More than 128 GPUs: do rounds read all GPUs, with how many warps, or work from the calendar of iteration ends?  Reading all
+// rows pays when an event that is not local (a finished prefill, mostly) comes with many local ends, because one row then ends
 // up to 32 iterations: it is a matter of the ends per event r against the rows N / 32, and r is estimated as iterations per
-// second over requests per second of a busy GPU (rates averaged over the blocks).  Measured, scan / calendar in ms, least-loaded
+// second over requests per second of a busy GPU (lambda requests per second and GPU).
+//
+// One warp.  Measured, scan / calendar in ms, least-loaded
 // placement: r = 1.0 rows (N = 300) 134 / 127, 1.6 rows (N = 500) 106 / 116, 1.6 rows (N = 300) 84 / 99, 2 rows (N = 150) 93 / 105, 2 rows
 // (N = 800) 110 / 146, and in overload, r = 0.3 rows, N = 512, 955 / 623.  Random placement reads all rows for every choice
-// either way: 2.4 rows (N = 500) 195 / 179, 3.5 rows (N = 350) 114 / 122.  QSIM_ROUNDS=scan|calendar overrides.
-bool rounds_scan(const qsim_config &c, const double *rates, const double *coef)
+// either way: 2.4 rows (N = 500) 195 / 179, 3.5 rows (N = 350) 114 / 122.  QSIM_ROUNDS=scan|calendar overrides (and means one warp).
+//
+// Several warps, from 32 rows on (two, from 64 rows four, from 128 rows sixteen: the best of sweeps).  The calendar's time hardly
+// depends on the load, being a pass over the ids per bucket, and that of several warps is proportional to the events.  Both sides
+// in ms for 20 iterations of horizon, several warps / calendar, at r = 49, 20, 10, 5 (cfg2 with 0.1, 0.25, 0.5, 0.95 of its load):
+//   N = 1024, R = 888   12 / 21    27 / 24    49 / 32    85 / 43
+//   N = 2048, R = 740   43 / 101   96 / 109   178 / 122  323 / 159
+//   N = 3000, R = 444   75 / 227   171 / 239  323 / 254  592 / 270
+//   N = 4096, R = 592   134 / 474  316 / 489  616 / 518  1143 / 531
+//   N = 4096, R = 148   34 / 237   80 / 245   156 / 258  287 / 266
+// The last two differ because a block of sixteen warps has an SM to itself, and two replications on the calendar share one.  The
+// lines below also hold for the priority gate with blocks (N = 1024, R = 585, r = 21: 55 / 62).  Uniform placement: N = 1024, R = 592, r = 49
+// and 20, 20 / 20 and 45 / 40; N = 2048, R = 444, r = 20 and 10, 90 / 95 and 171 / 140; N = 4096, R = 444, r = 20 and 10, 629 / 769 and 1238 / 1068.
+constexpr uint32_t SMS = 148;
+RoundPlan round_plan(const qsim_config &c, double lambda, const double *coef)
 {
-    if (const char *e = std::getenv("QSIM_ROUNDS")) {
-        if (std::strcmp(e, "scan") == 0) return true;
-        if (std::strcmp(e, "calendar") == 0) return false;
-    }
-    double lam = 0.0;
-    for (size_t k = 0; k < (size_t)c.nblk * c.I; ++k) lam += rates[k];
-    lam /= (double)c.nblk;
+    RoundPlan plan;
+    const char *e = std::getenv("QSIM_ROUNDS");
+    if (e && std::strcmp(e, "scan") == 0) { plan.scan = true; return plan; }
+    if (e && std::strcmp(e, "calendar") == 0) return plan;
     const double tau_mix = coef[0] + coef[1] * (double)c.C + coef[2] * (double)c.B, tau_solo = coef[3] + coef[4] * (double)c.B;
     const double tau_max = tau_mix > tau_solo ? tau_mix : tau_solo, tau_min = coef[0] < coef[3] ? coef[0] : coef[3];
     const double rows = (double)((c.N + 31u) / 32u), from = c.placement == QSIM_PLACE_RANDOM ? 2.8 : 1.3;
-    return 1.0 > lam * 0.5 * (tau_min + tau_max) * from * rows;
+    const double per_end = lambda * 0.5 * (tau_min + tau_max);        // 1 / r
+    plan.scan = 1.0 > per_end * from * rows;
+    if (c.N > 992u) {
+        const double r_from = c.N <= 2016u ? (c.placement == QSIM_PLACE_RANDOM ? 45.0 : 20.5) : (c.N <= 4064u ? 19.0 : (c.R <= SMS ? 6.5 : 14.0));
+        if (1.0 > per_end * r_from) plan.warps = c.N <= 2016u ? 2u : (c.N <= 4064u ? 4u : 16u);
+    }
+    return plan;
+}
+
+double mean_rate(const qsim_config &c, const double *rates)      // requests per second and GPU, averaged over the blocks
+{
+    double lam = 0.0;
+    for (size_t k = 0; k < (size_t)c.nblk * c.I; ++k) lam += rates[k];
+    return lam / (double)c.nblk;
 }
 
 // Everything of a handle that needs no device memory: kernel parameters, kernel instance, block shape,
@@ -452,7 +479,7 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
     const bool kappa = coef[5] != 0.0;
     const uint32_t feat = features_of(cfg, classes, coef);
     h.feat = feat;
-    RunVariant v = pick_run_kernel(cfg.N, feat, h.scan);
+    RunVariant v = pick_run_kernel(cfg.N, feat, h.plan.scan);
     // the per-GPU arrays are padded to the unrolled row count of the chosen instance
     if (v.spl > 0) p.Npad = (uint32_t)v.spl * 32u;
     // finish stamps + occupancy bits go to shared memory when the whole block state stays small
@@ -461,14 +488,14 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
     const uint32_t spared = 160u + (uint32_t)sizeof(WarpClassStats) * MAXI - (((uint32_t)sizeof(WarpClassStats) * cfg.I + 15u) & ~15u);
     p.slots_smem = smem_layout(p.Npad, p.Npad, p.B, 1, 1, kappa, p.Npad > 128u, cfg.I, false).total + spared <= 40u * 1024u ? 1u : 0u;
     if (cfg.N > 992u) p.slots_smem = 0;     // (from 32 rows on the layout is that of several warps, which retire through the global lists)
-    if (p.slots_smem) v = pick_run_kernel(cfg.N, feat | F_SLOTS, h.scan);
+    if (p.slots_smem) v = pick_run_kernel(cfg.N, feat | F_SLOTS, h.plan.scan);
     h.run_fn = v.fn;
     h.nwarps = 1;
-    choose_multiwarp(cfg.N, feat, p, h.run_fn, h.nwarps);
+    choose_multiwarp(cfg.N, feat, h.plan.warps, p, h.run_fn, h.nwarps);
     // beyond four rows of GPUs shared memory limits the resident replications: the arrival times and the job words of
     // the requests in prefill (read once per finished prefill) move to global memory
     p.tarr_global = (p.Npad > 128u) ? 1u : 0u;
-    const bool cal = cfg.N > 128u && h.nwarps == 1 && !h.scan;      // run-time row count, one warp (Sim::CAL)
+    const bool cal = cfg.N > 128u && h.nwarps == 1 && !h.plan.scan;      // run-time row count, one warp (Sim::CAL)
     calendar_shape(cfg.N, cfg.B, cfg.C, coef, p);
     h.lay = smem_layout(cfg.N, p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I, cal);
     h.init_smem = smem_layout(p.Npad, p.Npad, p.B, p.slots_smem, 1, kappa, p.tarr_global != 0, cfg.I, false).total;
@@ -728,7 +755,7 @@ int qsim_create(qsim_t **out, const qsim_config *cfg, const qsim_class *classes,
     qsim *h = new (std::nothrow) qsim();
     if (!h) return fail(QSIM_ENOMEM, "host allocation failed");
     h->device = dev;
-    h->scan = rounds_scan(*cfg, rates, coef);
+    h->plan = round_plan(*cfg, mean_rate(*cfg, rates), coef);
     rc = configure(*h, *cfg, classes, prices, coef);
     if (rc != QSIM_OK) { delete h; return rc; }
     Params &p = h->par;
@@ -966,7 +993,7 @@ int qsim_set_injected(qsim_t *h, const double *t, const uint32_t *job, uint64_t 
     h->par.inject_job = h->d_inject_job;
     h->par.n_inject = (uint32_t)n;
     // the trace source lives in the instances built for it and in the run-time-configured ones
-    RunVariant v = pick_run_kernel(h->cfg.N, h->feat | F_INJECT | (h->par.slots_smem ? F_SLOTS : 0u), h->scan);
+    RunVariant v = pick_run_kernel(h->cfg.N, h->feat | F_INJECT | (h->par.slots_smem ? F_SLOTS : 0u), h->plan.scan);
     if (h->nwarps > 1)
         for (const RunVariant &mw : run_variants())
             if (mw.spl < 0 && (mw.feat & F_GENERIC)) v = mw;
@@ -1341,7 +1368,7 @@ extern "C" int qsim_simulate_static(const qsim_config *cfg, const qsim_class *cl
     h.allow_lane = false;                  // the built-in scratch is sized for the warp-per-replication layout
     qsim_config nohist = *cfg;
     nohist.hist = 0;                       // histograms are not recorded here
-    h.scan = rounds_scan(*cfg, rates, coef);
+    h.plan = round_plan(*cfg, mean_rate(*cfg, rates), coef);
     rc = configure(h, nohist, classes, prices, coef);
     if (rc != QSIM_OK) return rc;
     h.device = dev;

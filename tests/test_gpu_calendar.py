@@ -122,3 +122,23 @@ def test_long_idle_times_are_skipped(rate, T, rounds):
     n, last = float(got["arrivals"].max()), 4e8 if rate > 0.0 else 10.0
     for k in F64_KEYS:
         assert np.allclose(got[k], ref[k], rtol=1e-9, atol=2 * n * n * last * 2.0 ** -53), k
+
+
+@pytest.mark.parametrize("make,load,warps", [
+    (lambda N: presets.cfg2(N=N, R=2), 0.1, {992: 1, 993: 2, 2017: 4, 4096: 16}),
+    (lambda N: presets.cfg3(N=N, R=2, block_len=0.3), 0.1, {1100: 2}),
+    (lambda N: presets.cfg4(N=N, R=2), 0.1, {1100: 2}),
+    (lambda N: presets.cfg2(N=N, R=149), 0.6, {4096: 1}),
+    (lambda N: presets.cfg2(N=N, R=2), 1.0, {1100: 1, 4096: 1}),
+])
+def test_several_warps_on_lightly_loaded_large_clusters(make, load, warps):
+    from oracle import run_oracle
+    from paper_2602_02987_b200 import QSim
+    for N, want in warps.items():
+        inp = light(make(N), load)
+        sim = QSim(inp)
+        assert sim.layout_info()["warps"] == want, N
+        if inp.R == 2:
+            sim.run(60)
+            assert_parity(sim.stats(), run_oracle(inp, 60), what=f"{inp.name}, {want} warps")
+        sim.close()
