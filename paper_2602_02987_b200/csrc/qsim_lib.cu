@@ -973,17 +973,18 @@ int qsim_set_injected(qsim_t *h, const double *t, const uint32_t *job, uint64_t 
     if (!h || !t || !job || n == 0 || n > 0x7fffffffull) return fail(QSIM_EINVAL, "bad injected arrival list");
     if (h->bound) return fail(QSIM_ESTATE, "qsim_set_injected must come before qsim_bind");
     if (h->cfg.nblk != 1) return fail(QSIM_EINVAL, "injected arrivals need nblk == 1");
-    if (h->par.lane.on) {
-        // trace replay lives in the warp-per-replication family: lay the handle out again for it
-        h->allow_lane = false;
-        int rc = configure_again(h);
-        if (rc != QSIM_OK) return rc;
-    }
     for (uint64_t k = 0; k < n; ++k) {
         if (!(t[k] >= 0.0) || !std::isfinite(t[k]) || (k > 0 && t[k] < t[k - 1])) return fail(QSIM_EINVAL, "injected times must be ascending and >= 0");
         if (job[3 * k] >= h->cfg.I || job[3 * k + 1] < 1 || job[3 * k + 1] > QSIM_LMAX || job[3 * k + 2] < 1 || job[3 * k + 2] > QSIM_LMAX)
             return fail(QSIM_EINVAL, "injected job out of range");
     }
+    // Trace replay lives in the warp-per-replication family, and its load is the trace's and not that of the class rates (which a
+    // program may leave at any value): lay the handle out again for both.  N = 1024, 16 replications of a congested trace whose rates
+    // are place-holders: 1326 ms by the rates (rounds that read all GPUs), 792 by the trace; N = 2048, 8: 4275 and 2168.
+    h->allow_lane = false;
+    h->plan = round_plan(h->cfg, t[n - 1] > 0.0 ? (double)n / (t[n - 1] * (double)h->cfg.N) : INFINITY, h->coef);
+    int rc = configure_again(h);
+    if (rc != QSIM_OK) return rc;
     if (h->d_inject_t) { cudaFree(h->d_inject_t); cudaFree(h->d_inject_job); h->d_inject_t = nullptr; h->d_inject_job = nullptr; }
     CUDA_TRY(cudaMalloc(&h->d_inject_t, n * sizeof(double)));
     CUDA_TRY(cudaMalloc(&h->d_inject_job, n * 3 * sizeof(uint32_t)));

@@ -137,3 +137,22 @@ def test_a_burst_of_arrivals_joins_the_queue_before_the_next_event(N, rounds, bu
     inp = presets.single_class(N=N, B=8, P=900, D=25, lam=0.5, theta=0.0, R=2, M=N, inject=inj).with_(qcap=64 if burst == 64 else burst - 1)
     st = _both(inp, 90)
     assert int(st["overflow"][0, 0]) == (3 if burst == 64 else 4)
+
+
+@pytest.mark.parametrize("rate", [0.0, 1e-6, 50.0])
+@pytest.mark.parametrize("N,gap", [(140, 0.0001), (140, 0.5), (1100, 0.0001), (1100, 0.5)])
+def test_rounds_on_large_clusters_follow_the_load_of_the_trace(N, gap, rate):
+    # whatever the class rates say: on the calendar (more shared memory than reading all GPUs) when requests come fast, by reading all
+    # GPUs, from 32 rows on with two warps, when they come slowly
+    from oracle import run_oracle
+    from paper_2602_02987_b200 import QSim
+    inj = [(gap * (k + 1), 0, 300 + k, 20 + k % 7) for k in range(60)]
+    inp = presets.single_class(N=N, B=8, P=900, D=25, lam=0.5, theta=0.0, R=2, M=N // 2, inject=inj).with_(rates=np.array([[rate]]))
+    sim = QSim(inp)
+    plain = QSim(inp.with_(inject_t=None, inject_job=None, rates=np.array([[1.0 / (gap * N)]])))
+    assert sim.layout_info()["warps"] == plain.layout_info()["warps"] == (2 if N > 992 and gap > 0.1 else 1)
+    assert sim.layout_info()["smem_bytes"] == plain.layout_info()["smem_bytes"]
+    plain.close()
+    sim.run(600)
+    assert_parity(sim.stats(), run_oracle(inp, 600), what=f"trace of gap {gap}, N={N}, rates {rate}")
+    sim.close()
