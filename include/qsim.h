@@ -344,7 +344,7 @@ typedef struct {
     double T_elapsed;               /* end time reached */
 } qsim_ctmc_rep_stats;
 
-/* Bytes of device memory the three calls below need for this configuration. */
+/* Bytes of the workspace of the three calls below for this configuration. */
 int qsim_ctmc_workspace_bytes(const qsim_ctmc_config *cfg, size_t *bytes);
 
 /* Empty system at t = 0 in [device] dev_workspace (256-byte aligned, at least qsim_ctmc_workspace_bytes; owned by
@@ -359,7 +359,9 @@ int qsim_ctmc_run_until(const qsim_ctmc_config *cfg, const qsim_ctmc_class *clas
                         void *cuda_stream, double T_end, uint64_t *launches);
 
 /* Copy the statistics of all replications to [host] per_rep[R]; time integrals are closed at the end time.
- * Synchronises the stream.  QSIM_EOVERFLOW if a replication stopped on an internal error. */
+ * Synchronises the stream.  From 768 replications on the records are formed in device memory that the call takes from the
+ * stream's memory pool (sizeof(qsim_ctmc_rep_stats) R bytes) and gives back; without room for them they are formed on the
+ * host.  QSIM_EOVERFLOW if a replication stopped on an internal error. */
 int qsim_ctmc_stats(const qsim_ctmc_config *cfg, const void *dev_workspace, size_t bytes, void *cuda_stream,
                     qsim_ctmc_rep_stats *per_rep);
 

@@ -164,9 +164,12 @@ def marshal(inp):
     return cfg, classes, rates, lengths, prices, coeffs, tg
 
 
+_REP_STATS, _CTMC_REP_STATS = np.dtype(qsim_rep_stats), np.dtype(qsim_ctmc_rep_stats)
+
+
 def _unpack(per, R, I):
     """Statistics records (a ctypes array of R of them, or one) -> arrays of their fields, classes beyond I left out."""
-    rec = np.frombuffer(per, dtype=np.dtype(qsim_rep_stats), count=R)
+    rec = np.frombuffer(per, dtype=_REP_STATS, count=R)
     cls = rec["cls"][:, :I]
     out = {n: cls[n].copy() for n in _COUNTERS + _STATE + _SUMS}
     for n in ("iters_mixed", "iters_solo", "events", "busy_mixed", "busy_solo", "T_elapsed"):
@@ -410,7 +413,7 @@ class QSimCTMC:
         with torch.cuda.device(self.device):
             _check(self.L.qsim_ctmc_stats(C.byref(self.cfg), C.c_void_p(self.ptr), self.nbytes,
                                           C.c_void_p(self.stream.cuda_stream), per))
-        rec = np.frombuffer(per, dtype=np.dtype(qsim_ctmc_rep_stats))
+        rec = np.frombuffer(per, dtype=_CTMC_REP_STATS)
         # the classes in use first, in one pass over the records, then one array per statistic
         cnt, state, area = (rec[n][:, :I].copy() for n in ("cnt", "state", "area"))
         out = {}

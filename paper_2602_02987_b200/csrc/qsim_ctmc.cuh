@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(32) qsim_ctmc_kernel(CtmcParams p)
 
 // The public statistics record of every replication, one warp each: counters as they are, time integrals closed at the end
 // time (the host's formula, rounded the same).  first_err: lowest replication that stopped on an internal error.
-// Memory-bound: 3.7 KB read and 1.2 KB written per replication.
+// Memory-bound: about 190 bytes per class in use read and 1.2 KB written per replication.
 __global__ void __launch_bounds__(128) qsim_ctmc_stats_kernel(const CtmcRep *reps, uint32_t R, uint32_t I, qsim_ctmc_rep_stats *out, uint32_t *first_err)
 {
     const uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31u;
@@ -473,7 +473,10 @@ int ctmc_launch_shape(const qsim_ctmc_config &c, uint32_t &lanes, size_t &smem)
     return QSIM_OK;
 }
 
-// The public records from a copy of the device records: for a device without room for the former.
+// The public records from a copy of the device records (3.8 KB each): for few replications, and for a device without room for the
+// public records.  Forming them on the device means an allocation and its return, 0.45 ms whatever their number; host / device in ms:
+// R = 64 0.12 / 0.53, 256 0.34 / 0.61, 1024 1.09 / 0.95, 4096 4.0 / 1.7.
+constexpr uint32_t CTMC_STATS_ON_DEVICE = 768;
 int ctmc_stats_on_host(const qsim_ctmc_config &cfg, const char *dev_reps, cudaStream_t st, qsim_ctmc_rep_stats *per_rep)
 {
     std::vector<CtmcRep> reps(cfg.R);
@@ -584,6 +587,7 @@ int qsim_ctmc_stats(const qsim_ctmc_config *cfg, const void *dev_workspace, size
     const CtmcSections sec = ctmc_sections(*cfg);
     if (!dev_workspace || bytes < sec.total) return fail(QSIM_EWORKSPACE, "workspace missing or too small");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    if (cfg->R < CTMC_STATS_ON_DEVICE) return ctmc_stats_on_host(*cfg, static_cast<const char *>(dev_workspace) + sec.reps, st, per_rep);
     // the public records are formed on the device: a third of the bytes cross to the host, and nothing is left to do there
     const size_t out_bytes = (size_t)cfg->R * sizeof(qsim_ctmc_rep_stats);
     char *scratch = nullptr;

@@ -71,3 +71,19 @@ def test_a_state_whose_clocks_of_intensity_zero_stood_still(router):
         sim.close()
     for k in got[0]:
         assert np.array_equal(got[0][k], got[1][k]), k
+
+
+@pytest.mark.parametrize("I", [1, 2, 8])
+def test_statistics_formed_on_the_host_and_on_the_device(I):
+    # 767 replications are read out on the host and 768 on the device; a replication does not depend on how many there are
+    from paper_2602_02987_b200 import QSimCTMC
+    got = []
+    for R in (767, 768):
+        sim = QSimCTMC(instance(I, 5, ROUTER_SLI, GATE_OCCUPANCY).with_(R=R))
+        sim.run_until(11.0)
+        got.append(sim.stats())
+        sim.close()
+    assert (got[0]["events"] > 0).all()
+    for k in got[0]:
+        assert got[0][k].shape[0] == 767 and got[1][k].shape[0] == 768
+        assert np.array_equal(got[0][k], got[1][k][:767]), k
