@@ -88,13 +88,15 @@ def test_random_sizes_on_the_benchmark_feature_sets(seed):
 
 
 @pytest.mark.parametrize("recipe,N,B", [("cfg2", 1024, 100), ("cfg4", 2049, 17), ("cfg2", 2049, 33), ("cfg4", 1023, 256)])
-def test_sizes_around_the_warp_count_thresholds(recipe, N, B):
-    # 1024 GPUs = 32 rows (two warps per replication, 1023 still one), 2049 = 65 rows (four warps, last row holds one GPU)
+@pytest.mark.parametrize("several", [False, True])
+def test_sizes_around_the_warp_count_thresholds(recipe, N, B, several, monkeypatch):
+    # 1024 GPUs = 32 rows (two warps per replication under light load), 2049 = 65 rows (four, last row holds one GPU); and one warp
+    monkeypatch.setenv("QSIM_WARPS", ("4" if N > 2016 else "2") if several else "1")
     from oracle import OracleSim
     from paper_2602_02987_b200 import QSim
     inp = getattr(presets, recipe)(N=N, R=2).with_(B=B, seed=N + B)
     H = 150
-    sim = QSim(inp); sim.run(H); got = sim.stats(); gstate = [sim.server_state(r) for r in range(inp.R)]; sim.close()
+    sim = QSim(inp); assert (sim.layout_info()["warps"] > 1) == several; sim.run(H); got = sim.stats(); gstate = [sim.server_state(r) for r in range(inp.R)]; sim.close()
     o = OracleSim(inp); o.run(H); ref = o.stats(); ostate = [o.server_state(r) for r in range(inp.R)]; o.close()
     assert_parity(got, ref, what=f"{inp.name}: N={inp.N} B={inp.B}")
     for a, b in zip(gstate, ostate):

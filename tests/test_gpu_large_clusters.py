@@ -1,4 +1,4 @@
-"""Parity of the several-warps instances (clusters of 512 simulated GPUs and more) with the CPU oracle in steady state:
+"""Parity of the one-warp and several-warps instances on clusters of 512 simulated GPUs and more with the CPU oracle in steady state:
 horizons well past one decode lifetime, so that batches are full, requests finish, wait and abandon under every warp
 count, at the cluster sizes of the benchmark configurations."""
 import os
@@ -58,20 +58,21 @@ def oracle_stats(inp, horizon):
     return st, [out[r][1] for r in range(inp.R)]
 
 
-def check(inp, horizon, **kw):
+def check(inp, horizon, warps=(None,), **kw):
     ref, rstate = oracle_stats(inp, horizon)
-    got, gstate = gpu_stats(inp, horizon, **kw)
-    assert_parity(got, ref, what=f"{inp.name} N={inp.N} {kw}")
-    for a, b in zip(gstate, rstate):
-        for k in a:
-            assert np.array_equal(a[k], b[k]), (inp.name, "GPU state", k)
+    for w in warps:
+        got, gstate = gpu_stats(inp, horizon, warps=w, **kw)
+        assert_parity(got, ref, what=f"{inp.name} N={inp.N} warps={w} {kw}")
+        for a, b in zip(gstate, rstate):
+            for k in a:
+                assert np.array_equal(a[k], b[k]), (inp.name, "GPU state", w, k)
     return ref
 
 
 @pytest.mark.parametrize("N,H", [(1024, 700), (4096, 450)])
 def test_cfg4_steady_state_at_benchmark_cluster_sizes(N, H):
-    # occupancy gate, SLI-aware router, histograms; four (N = 1024) and sixteen (N = 4096) warps per replication in the warp family
-    st = check(presets.cfg4(N=N, R=2), H, chunks=[H // 3, H - H // 3])
+    # occupancy gate, SLI-aware router, histograms; one warp, and the two (N = 1024) and sixteen (N = 4096) of light load
+    st = check(presets.cfg4(N=N, R=2), H, chunks=[H // 3, H - H // 3], warps=(1, 2 if N == 1024 else 16))
     done = st["done_mixed"] + st["done_solo"]
     assert done.sum() > 20 * N and st["abandoned_p"].sum() > 0
     assert st["hist_tpot"].sum() == done.sum()
@@ -81,27 +82,27 @@ def test_cfg3_full_cluster_all_blocks_with_role_changes():
     # priority gate, 24 blocks, per-block targets: M changes at more than two block ends
     inp = presets.cfg3(N=1024, R=2, block_len=0.5)
     assert int((np.diff(inp.M.astype(int)) != 0).sum()) >= 2
-    st = check(inp, inp.meta["horizon_iters"])
+    st = check(inp, inp.meta["horizon_iters"], warps=(1, 2))
     assert st["abandoned_p"].sum() > 0 and (st["done_mixed"] + st["done_solo"]).sum() > 20_000
 
 
 def test_cfg2_full_cluster_with_abandonment():
-    st = check(presets.cfg2(N=512, R=2), 700)
+    st = check(presets.cfg2(N=512, R=2), 700, warps=(1, 2))
     assert st["abandoned_p"].sum() > 0
 
 
 @pytest.mark.parametrize("N,H,placement", [(1100, 1000, PLACE_RANDOM), (2100, 600, PLACE_LEAST_LOADED), (2100, 300, PLACE_RANDOM)])
 def test_decode_backlog_on_large_clusters(N, H, placement):
     # decode slots scarce: thousands of requests wait in the decode buffer and abandon it, every decode completion
-    # frees a slot that the buffer's head takes (solo GPUs first), on both sides of the eight-warp threshold
-    st = check(presets.crowded("decode", N=N, R=2, placement=placement), H)
+    # frees a slot that the buffer's head takes (solo GPUs first), with one warp and with the two and four of light load
+    st = check(presets.crowded("decode", N=N, R=2, placement=placement), H, warps=(1, 2 if N == 1100 else 4))
     assert st["abandoned_d"].sum() > 1000 and st["Qd"].sum() > 1000
     assert st["placed_solo"].sum() > 0 and st["placed_mixed"].sum() > 0
 
 
 def test_prefill_backlog_with_the_sli_router_on_a_large_cluster():
     inp = presets.crowded("prefill", N=1500, R=2, placement=PLACE_LEAST_LOADED, router=ROUTER_SLI)
-    st = check(inp, 800)
+    st = check(inp, 800, warps=(1, 2))
     assert st["abandoned_p"].sum() > 1000
 
 
@@ -110,12 +111,14 @@ def test_every_warp_count_gives_the_same_trajectory(warps):
     # the number of warps per replication is a launch parameter, not part of the method
     for inp, H in ((presets.cfg4(N=640, R=2), 400), (presets.crowded("decode", N=530, R=2), 500),
                    (presets.cfg3(N=512, R=1, block_len=0.25), None)):
-        check(inp, H or inp.meta["horizon_iters"], warps=warps)
+        check(inp, H or inp.meta["horizon_iters"], warps=(warps,))
 
 
-def test_one_warp_instances_agree_on_a_cluster_that_defaults_to_several_warps():
-    inp = presets.cfg2(N=1024, R=2)
-    check(inp, 200, warps=1)
+@pytest.mark.parametrize("N,warps", [(1024, 2), (2049, 4), (4096, 16)])
+def test_one_warp_agrees_on_a_cluster_that_defaults_to_several_warps(N, warps):
+    inp = presets.cfg2(N=N, R=2)
+    inp = inp.with_(rates=inp.rates * 0.1)
+    check(inp, 200, warps=(None, warps, 1))
 
 
 def test_handles_of_different_sizes_share_kernels():

@@ -148,20 +148,22 @@ def test_cfg4_subset_sli_router_constrained_targets():
         check(inp, H)
 
 
-def test_multi_warp_instances_large_clusters():
-    # N >= 512 runs several warps per replication; each specialised instance and the generic one against the oracle
-    import os
+def test_multi_warp_instances_large_clusters(monkeypatch):
+    # several warps per replication; each specialised instance and the generic one against the oracle
+    from paper_2602_02987_b200 import QSim
+    monkeypatch.setenv("QSIM_WARPS", "2")
+    check(presets.cfg2(N=512, R=2), 300)                     # occupancy gate
     inp = presets.cfg3(N=512, R=2, block_len=0.25)          # priority gate, blocks, histograms
     H = inp.meta["horizon_iters"]
     st = check(inp, H)
     assert st["hist_tpot"].sum() == (st["done_mixed"] + st["done_solo"]).sum()
     inp4 = presets.cfg4(N=512, R=2)                          # occupancy gate, SLI router, histograms
     g = check(inp4, 300)
-    os.environ["QSIM_KERNEL"] = "generic"
-    try:
-        g2, _ = gpu_run(inp4, 300)
-    finally:
-        del os.environ["QSIM_KERNEL"]
+    monkeypatch.setenv("QSIM_KERNEL", "generic")
+    g2, _ = gpu_run(inp4, 300)
+    sim = QSim(inp4)
+    assert sim.layout_info()["warps"] == 2
+    sim.close()
     assert_parity(g2, g, what="generic multi-warp instance")
 
 
