@@ -541,7 +541,7 @@ struct Sim {
         uint32_t cnt = 0;
 #pragma unroll 1
         for (uint32_t k = 0; k < n_rows(); ++k)
-            cnt += key_of((k << 5) + (uint32_t)lane, WANT_PREFILL) != NONE32 ? 1u : 0u;
+            cnt += eligible((k << 5) + (uint32_t)lane, WANT_PREFILL) ? 1u : 0u;
         return __reduce_add_sync(FULL, cnt);
     }
 
@@ -632,15 +632,25 @@ struct Sim {
     // per lane, when a choice needs them.
     __device__ __forceinline__ void gpu_changed(uint32_t g) { if (CAL) { dirty_dec |= 1u << (g & 31u); dirty_pf |= 1u << (g & 31u); } }
 
-    // key of GPU g for the wanted tiers: solo GPUs first, then decodes held, then index; NONE32 when it is not eligible
-    __device__ __forceinline__ uint32_t key_of(uint32_t g, uint32_t tiers) const
+    // does GPU g, with nd decodes and prefill state pf, take a request of the wanted tiers?
+    __device__ __forceinline__ bool takes(uint32_t g, uint32_t tiers, uint32_t nd, uint32_t pf) const
     {
-        // g is always inside the padded arrays; every field is read first so that calls over rows overlap
-        const uint32_t nd = ndec[g], pf = pfrem[g];
         const bool mix = g < M;
         const uint32_t cap = (mix || pf != 0) ? p.B - 1 : p.B;   // a mixed GPU keeps one slot for prefill
         const bool ok = tiers == WANT_PREFILL ? (mix && pf == 0 && nd <= p.B - 1) : ((tiers & (mix ? WANT_MIX : WANT_SOLO)) != 0 && nd < cap);
-        return (ok && g < p.N) ? ((mix ? 0x40000000u : 0u) | (nd << 16) | g) : NONE32;
+        return ok && g < p.N;
+    }
+    // (g is always inside the padded arrays; every field is read first so that calls over rows overlap)
+    __device__ __forceinline__ bool eligible(uint32_t g, uint32_t tiers) const
+    {
+        const uint32_t nd = ndec[g], pf = pfrem[g];
+        return takes(g, tiers, nd, pf);
+    }
+    // key of GPU g for the wanted tiers: solo GPUs first, then decodes held, then index; NONE32 when it is not eligible
+    __device__ __forceinline__ uint32_t key_of(uint32_t g, uint32_t tiers) const
+    {
+        const uint32_t nd = ndec[g], pf = pfrem[g];
+        return takes(g, tiers, nd, pf) ? ((g < M ? 0x40000000u : 0u) | (nd << 16) | g) : NONE32;
     }
 
     // Least loaded (lowest index on ties) or uniformly random among the eligible GPUs of the first tier that has one
@@ -690,7 +700,7 @@ struct Sim {
             uint32_t cnt = 0;
 #pragma unroll(SPL > 0 ? SPL : 4)
             for (uint32_t k = 0; k < rows; ++k)
-                cnt += (uint32_t)__popc(__ballot_sync(FULL, key_of((k << 5) + (uint32_t)lane, tier) != NONE32));
+                cnt += (uint32_t)__popc(__ballot_sync(FULL, eligible((k << 5) + (uint32_t)lane, tier)));
             if (cnt == 0) continue;
             uint32_t idx = 0;
             if (cnt > 1) {
@@ -700,7 +710,7 @@ struct Sim {
             }
 #pragma unroll(SPL > 0 ? SPL : 4)
             for (uint32_t k = 0; k < rows; ++k) {
-                const uint32_t b = __ballot_sync(FULL, key_of((k << 5) + (uint32_t)lane, tier) != NONE32);
+                const uint32_t b = __ballot_sync(FULL, eligible((k << 5) + (uint32_t)lane, tier));
                 const uint32_t c = (uint32_t)__popc(b);
                 if (idx < c) return (k << 5) + (uint32_t)__fns(b, 0, (int)idx + 1);
                 idx -= c;
