@@ -541,7 +541,7 @@ struct Sim {
         uint32_t cnt = 0;
 #pragma unroll 1
         for (uint32_t k = 0; k < n_rows(); ++k)
-            cnt += eligible((k << 5) + (uint32_t)lane, WANT_PREFILL) ? 1u : 0u;
+            cnt += key_of((k << 5) + (uint32_t)lane, WANT_PREFILL) != NONE32 ? 1u : 0u;
         return __reduce_add_sync(FULL, cnt);
     }
 
@@ -632,25 +632,28 @@ struct Sim {
     // per lane, when a choice needs them.
     __device__ __forceinline__ void gpu_changed(uint32_t g) { if (CAL) { dirty_dec |= 1u << (g & 31u); dirty_pf |= 1u << (g & 31u); } }
 
-    // does GPU g, with nd decodes and prefill state pf, take a request of the wanted tiers?
-    __device__ __forceinline__ bool takes(uint32_t g, uint32_t tiers, uint32_t nd, uint32_t pf) const
-    {
-        const bool mix = g < M;
-        const uint32_t cap = (mix || pf != 0) ? p.B - 1 : p.B;   // a mixed GPU keeps one slot for prefill
-        const bool ok = tiers == WANT_PREFILL ? (mix && pf == 0 && nd <= p.B - 1) : ((tiers & (mix ? WANT_MIX : WANT_SOLO)) != 0 && nd < cap);
-        return ok && g < p.N;
-    }
-    // (g is always inside the padded arrays; every field is read first so that calls over rows overlap)
-    __device__ __forceinline__ bool eligible(uint32_t g, uint32_t tiers) const
-    {
-        const uint32_t nd = ndec[g], pf = pfrem[g];
-        return takes(g, tiers, nd, pf);
-    }
     // key of GPU g for the wanted tiers: solo GPUs first, then decodes held, then index; NONE32 when it is not eligible
     __device__ __forceinline__ uint32_t key_of(uint32_t g, uint32_t tiers) const
     {
+        // g is always inside the padded arrays; every field is read first so that calls over rows overlap
         const uint32_t nd = ndec[g], pf = pfrem[g];
-        return takes(g, tiers, nd, pf) ? ((g < M ? 0x40000000u : 0u) | (nd << 16) | g) : NONE32;
+        const bool mix = g < M;
+        const uint32_t cap = (mix || pf != 0) ? p.B - 1 : p.B;   // a mixed GPU keeps one slot for prefill
+        const bool ok = tiers == WANT_PREFILL ? (mix && pf == 0 && nd <= p.B - 1) : ((tiers & (mix ? WANT_MIX : WANT_SOLO)) != 0 && nd < cap);
+        return (ok && g < p.N) ? ((mix ? 0x40000000u : 0u) | (nd << 16) | g) : NONE32;
+    }
+    // The GPUs of one tier as a range of indices and a bound on the decodes held, without and with a prefill: what key_of tests,
+    // with the tier's part of it done once for all rows.
+    struct Tier { uint32_t from, to, cap, cap_pf; };
+    __device__ __forceinline__ Tier tier_gpus(uint32_t tier) const
+    {
+        if (tier == WANT_SOLO) return { M, p.N, p.B, p.B - 1u };
+        return { 0u, M, tier == WANT_MIX ? p.B - 1u : p.B, tier == WANT_MIX ? p.B - 1u : 0u };
+    }
+    __device__ __forceinline__ bool in_tier(uint32_t g, const Tier &w) const
+    {
+        const uint32_t nd = ndec[g], pf = pfrem[g];
+        return g >= w.from && g < w.to && nd < (pf != 0 ? w.cap_pf : w.cap);
     }
 
     // Least loaded (lowest index on ties) or uniformly random among the eligible GPUs of the first tier that has one
@@ -697,10 +700,12 @@ struct Sim {
 #pragma unroll(SPL > 0 && !(F & F_GENERIC) ? 3 : 1)
         for (uint32_t tier = WANT_SOLO; tier <= WANT_PREFILL; tier <<= 1) {
             if (!(tiers & tier)) continue;
+            const Tier w = tier_gpus(tier);
+            const uint32_t first = SPL > 0 ? 0u : w.from >> 5, last = SPL > 0 ? rows : (w.to + 31u) >> 5;
             uint32_t cnt = 0;
 #pragma unroll(SPL > 0 ? SPL : 4)
-            for (uint32_t k = 0; k < rows; ++k)
-                cnt += (uint32_t)__popc(__ballot_sync(FULL, eligible((k << 5) + (uint32_t)lane, tier)));
+            for (uint32_t k = first; k < last; ++k)
+                cnt += (uint32_t)__popc(__ballot_sync(FULL, in_tier((k << 5) + (uint32_t)lane, w)));
             if (cnt == 0) continue;
             uint32_t idx = 0;
             if (cnt > 1) {
@@ -709,8 +714,8 @@ struct Sim {
                 idx = __umulhi(w0, cnt);
             }
 #pragma unroll(SPL > 0 ? SPL : 4)
-            for (uint32_t k = 0; k < rows; ++k) {
-                const uint32_t b = __ballot_sync(FULL, eligible((k << 5) + (uint32_t)lane, tier));
+            for (uint32_t k = first; k < last; ++k) {
+                const uint32_t b = __ballot_sync(FULL, in_tier((k << 5) + (uint32_t)lane, w));
                 const uint32_t c = (uint32_t)__popc(b);
                 if (idx < c) return (k << 5) + (uint32_t)__fns(b, 0, (int)idx + 1);
                 idx -= c;

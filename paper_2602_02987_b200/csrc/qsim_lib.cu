@@ -416,8 +416,8 @@ void calendar_shape(uint32_t N, uint32_t B, uint32_t C, const double *coef, Para
 // One warp.  Measured, scan / calendar in ms, least-loaded
 // placement: r = 1.0 rows (N = 300) 134 / 127, 1.6 rows (N = 500) 106 / 116, 1.6 rows (N = 300) 84 / 99, 2 rows (N = 150) 93 / 105, 2 rows
 // (N = 800) 110 / 146, and in overload, r = 0.3 rows, N = 512, 955 / 623.  Random placement (which reads all rows
-// for every choice either way): r = 2.6 rows (N = 600) 18.0 / 24.5, 1.95 rows (N = 300) 35.0 / 42.6, 1.95 rows (N = 150) 26.4 / 30.6, 1.0 rows
-// (N = 150) 46.4 / 42.2, 1.0 rows (N = 300) 65.6 / 65.5, 0.5 rows (N = 600) 77.4 / 75.0.  QSIM_ROUNDS=scan|calendar overrides (and means one warp).
+// for every choice either way): r = 2.6 rows (N = 600) 15.5 / 21.5, 1.95 rows (N = 300) 30.9 / 40.9, 1.95 rows (N = 150) 24.4 / 30.2, 1.0 rows
+// (N = 600) 35.6 / 42.1, 1.0 rows (N = 300) 58.5 / 62.5, 1.0 rows (N = 150) 41.8 / 41.0, 0.5 rows (N = 600) 65.0 / 64.8, 0.5 rows (N = 300) 98 / 85.  QSIM_ROUNDS=scan|calendar overrides (and means one warp).
 //
 // Several warps, from 32 rows on (two, from 64 rows four, from 128 rows sixteen: the best of sweeps).  The calendar's time hardly
 // depends on the load, being a pass over the ids per bucket, and that of several warps is proportional to the events.  Both sides
@@ -439,7 +439,7 @@ RoundPlan round_plan(const qsim_config &c, double lambda, const double *coef)
     if (e && std::strcmp(e, "calendar") == 0) return plan;
     const double tau_mix = coef[0] + coef[1] * (double)c.C + coef[2] * (double)c.B, tau_solo = coef[3] + coef[4] * (double)c.B;
     const double tau_max = tau_mix > tau_solo ? tau_mix : tau_solo, tau_min = coef[0] < coef[3] ? coef[0] : coef[3];
-    const double rows = (double)((c.N + 31u) / 32u), from = 1.3;
+    const double rows = (double)((c.N + 31u) / 32u), from = c.placement == QSIM_PLACE_RANDOM ? 0.9 : 1.3;
     const double per_end = lambda * 0.5 * (tau_min + tau_max);        // 1 / r
     plan.scan = 1.0 > per_end * from * rows;
     if (c.N > 992u) {
