@@ -46,7 +46,10 @@ constexpr int LMAX = 8192;
 constexpr int NBIN = 1024;
 constexpr unsigned FULL = 0xffffffffu;
 constexpr uint32_t NONE32 = 0xffffffffu;
-constexpr int TOUCH_CAP = 48;
+constexpr uint32_t CAL_CHAINS = 2;       // lists per bucket of the calendar (by GPU index, odd or even)
+constexpr uint32_t CAL_NONE = 0xffffu;   // end of a list
+constexpr uint32_t BATCH_MASK = 0x1fffu, BATCH_MIXED = 0x2000u;   // nact: decodes in the batch (B <= 4096), the iteration processes prompt tokens (CAL)
+constexpr unsigned long long BUDGET_MAX = 1ull << 29;    // rounds per launch: per-lane counters of a launch have 32 bits
 constexpr int ARRIVALS_PER_ROUND = 64;    // arrivals of a class that one round takes (a trace may bring any number at one time)
 constexpr uint32_t CAL_FREE = 16;        // free lanes from which the calendar loads another bucket
 
@@ -107,7 +110,8 @@ struct SlotRec { double tpf; uint32_t pk; uint32_t pad; };  // request in a deco
 constexpr int STAGE_CAP = 64, ROW_STAGE_CAP = 32;              // finished-request records waiting for their accounting (stamps on chip / in global memory)
 // Accounting of finished requests, one block per warp (merged into the class records at kernel exit)
 struct WarpClassStats { double sYm_out, sYs_out, sum_tpot; unsigned long long tok_in, tok_out; uint32_t done_mixed, done_solo; };
-struct ADraw { double E; uint32_t pk; uint32_t pad; };     // one arrival draw: unit exponential (divided by the rate already when there is one block) and packed lengths
+struct ClassAim { double xstar, nx, nq, ps, theta; };       // LP targets, share of the solo pool and abandonment rate of a class
+struct ADraw { double E; uint32_t pk; uint32_t pad; };     // one arrival draw: interarrival time (unit exponential over the rate) and packed lengths
 struct QEntry { double t; uint32_t pk; uint32_t cls; };   // 16 bytes: prefill queue (t = arrival) / decode buffer (t = prefill end)
 
 struct ClassPar { double theta; uint32_t P, D, prio, pad; };
@@ -163,7 +167,7 @@ struct Params {
     double *tarr_g;              // [R][N]
     uint32_t *pfjob_g;           // [R][N] packed request in prefill, with tarr_g
     double cal_inv_w;            // calendar of iteration ends (run-time row count, one warp): buckets per second
-    uint32_t cal_nbk, cal_K;     // buckets (a power of two, at most 256); buckets that the shortest iteration lasts at least
+    uint32_t cal_nbk, cal_K;     // buckets (a power of two); buckets that the shortest iteration lasts at least (0: no calendar)
     LanePar lane;
 };
 
@@ -241,6 +245,9 @@ __device__ __forceinline__ double qlog(double x)
     return __dadd_rn(__dmul_rn((double)e, 0.6931471805599453), logm);
 }
 
+// unit exponential from two words, out of line for rare draws
+__device__ __noinline__ double unit_exp(uint32_t w0, uint32_t w1) { return -qlog(u53(w0, w1)); }
+
 // iteration time of a batch with pf prefill tokens, d decodes, K resident KV tokens (Eq. (1)-(3))
 __device__ __forceinline__ double iter_time(const Params &p, uint32_t pf, uint32_t d, uint32_t K, bool kappa = true)
 {
@@ -281,20 +288,29 @@ __device__ __forceinline__ void area_touch(Area &a, uint32_t count, double t)
 }
 
 // Abandonment clock of one (class, queue): integrated hazard acc against the exponential level lvl
-// (random time change, Eq. (8)-(9)); called by the owning class lane before the count changes.
+// (random time change, Eq. (8)-(9)); brought up to date by the owning class lane before the count changes.  The time at
+// which the level is reached with the new count costs a division; Sim::settle_queue forms it where it is next asked for.
+__device__ __forceinline__ void ab_touch(AbClock &c, double theta, uint32_t Q_old, double t)
+{
+    c.acc = __dadd_rn(c.acc, __dmul_rn(__dmul_rn(theta, (double)Q_old), __dsub_rn(t, c.t_last)));
+    c.t_last = t;
+}
+// Next abandonment with Q waiting requests, from the state of the clock at its last change.
+__device__ __forceinline__ double ab_next(const AbClock &c, double theta, uint32_t Q)
+{
+    double rem = __dsub_rn(c.lvl, c.acc);
+    if (rem < 0.0) rem = 0.0;
+    return Q > 0 ? __dadd_rn(c.t_last, __ddiv_rn(rem, __dmul_rn(theta, (double)Q))) : dinf();
+}
+// The two together, where the next time is wanted at once (one thread per replication).
 __device__ __forceinline__ void ab_change(AbClock &c, double theta, uint32_t Q_old, uint32_t Q_new, double t)
 {
     if (!(theta > 0.0)) return;
-    c.acc = __dadd_rn(c.acc, __dmul_rn(__dmul_rn(theta, (double)Q_old), __dsub_rn(t, c.t_last)));
-    c.t_last = t;
-    if (Q_new > 0) {
-        double rem = __dsub_rn(c.lvl, c.acc);
-        if (rem < 0.0) rem = 0.0;
-        c.t_ab = __dadd_rn(t, __ddiv_rn(rem, __dmul_rn(theta, (double)Q_new)));
-    } else {
-        c.t_ab = dinf();
-    }
+    ab_touch(c, theta, Q_old, t);
+    c.t_ab = ab_next(c, theta, Q_new);
 }
+// Out of line for the warp kernels, where it is rarely asked for.
+__device__ __noinline__ double ab_next_call(const AbClock &c, double theta, uint32_t Q) { return ab_next(c, theta, Q); }
 
 // 16-byte asynchronous copy global -> shared (L2 only), and the wait for this thread's copies
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc)
@@ -382,9 +398,10 @@ struct Sim {
     uint16_t *ndec, *nact, *pfcur;
     uint16_t *sfin16;            // [Npad][B]  low 16 bits of each slot's finish iteration (f_slots)
     uint32_t *socc;              // [Npad][ceil(B/32)]  slot occupancy bits; bits past B are set for good
-    uint8_t *bkt;                // [GPUs rounded up to 128] calendar bucket of the GPU's iteration end, 255 when idle (CAL)
+    uint32_t *cal_head;          // [buckets][CAL_CHAINS] first GPU of every list of the calendar (CAL)
+    uint16_t *cal_next;          // [GPUs] the GPU after this one in its list (CAL)
     uint16_t *picked;            // [32] GPUs of the bucket being loaded (CAL)
-    uint32_t *touch;
+    uint32_t *row_key;           // [3][rows] smallest key of every row of 32 GPUs (CAL, see choose())
     ClassState *cs;
     // global memory of this replication
     uint32_t *s_fin;
@@ -394,40 +411,54 @@ struct Sim {
     double *st_te;
     QEntry *pqh;
     uint32_t n_pend;
+    double late_tpf;             // lane 0: record of the request that finished last, on its way from memory (entry n_pend of the staged ones)
+    uint32_t late_pk;
+    bool has_late;
     uint32_t rec_after;          // per lane: record copies committed since this lane's last queue-head copy
     QEntry *pq, *dq;
     uint32_t *hist;
     // replicated scalars
-    double t, T_end, T_blk_next, T_reset, tau_min;
+    double t, T_end, T_blk_next, tau_min;
+    const double *T_reset_at;     // (in shared memory, like all that is not read in every round)
     uint32_t blk, M, dq_head0, dq_head1, dq_n0, dq_n1, n_touch, err;
     uint32_t n_idle_pf;          // mixed GPUs whose prefill slot is idle (and that may take a prefill)
     uint32_t idle_hint;          // when n_idle_pf == 1: that GPU if known, else NONE32
     uint32_t need_start;         // per lane: rows of own GPUs touched by the current event
-    unsigned long long place_ord, events, rounds, sel_ord0, sel_ord1;
+    uint32_t touch_g;            // run-time row count: GPU touched by the current event (lanes below n_touch)
+    uint32_t events, rounds;     // of this launch
+    unsigned long long place_ord, sel_ord0, sel_ord1;
     bool drain_dirty, gate_dirty, touch_all;
-    bool direct;                 // a request has just finished its prefill and its pool's buffer is empty: class and lengths, pool,
-    uint32_t d_pk, d_pool, d_gpu;   // and the GPU it has to decode on (NONE32: the router chooses)
+    bool handed;                 // a request has just finished its prefill: class and lengths, pool, its arrival time, and the
+    uint32_t d_pk, d_pool, d_gpu;   // GPU it has to decode on (NONE32: the router chooses)
+    double d_tarr;
+    bool direct;                 // its pool's buffer is empty: it may pass through
+    uint32_t stale;              // class lane: abandonment clocks (prefill queue, decode buffers) whose next time is out of date
+    uint32_t pools;              // class lane: pools of 32 finished prefills (SLI-aware routers)
+    bool pools_due;              // and whether they have to be drawn
+    unsigned long long place_base;  // placement draws held by the lanes: ordinal of lane 0's, and the word of this lane's
+    uint32_t place_w;
     bool force_nonlocal;         // treat the next event, whatever it is, as non-local (it must end with a dispatch)
-    // calendar: last bucket loaded, bucket of T_end, the pending iteration end that this lane holds (GPU, time)
-    unsigned long long cur, cur_end, held_t;
+    // calendar: last bucket loaded, the pending iteration end that this lane holds (GPU, time)
+    unsigned long long cur, held_t;
     uint32_t held_g;
+    uint32_t held_na;            // its batch word
+    uint32_t held_pk;            // the request whose prefill that end finishes: packed lengths and class, and arrival time
+    double held_tarr;
     bool held, crowded;          // crowded: the current bucket holds more ends than lanes
-    unsigned long long low;      // no pending event lies in an earlier bucket
-    unsigned long long left_t;   // crowded: earliest pending end of the bucket that no lane holds (time, source)
-    uint32_t left_s;
-    // smallest keys among this lane's GPUs (g mod 32 = lane), see choose(): decode target (solo-first, or solo GPUs only under
-    // the SLI-aware routers), mixed decode target (SLI-aware routers), prefill target; lanes whose keys are out of date
-    uint32_t best_dec, best_mix, best_pf, dirty_dec, dirty_pf;
+    uint32_t lead;               // no pending event lies more than this many buckets before `cur`
+    unsigned long long *left;    // crowded: earliest pending end of the bucket that no lane holds (time, source), in shared memory
+    uint32_t dirty_dec, dirty_pf;   // bit k: the keys of row lane + 32 k are out of date (decode / prefill targets)
     // per-lane partial sums
-    unsigned long long it_mixed, it_solo;
+    uint32_t it_mixed, it_solo;
     double busy_mixed, busy_solo;
     // pre-generated arrival draws of this lane's class (ring in shared memory) and a pending scheduling request
-    ADraw *aring;
+    double *aring;
+    uint32_t *aring_pk;
     uint32_t ring_n, ring_pos;
     bool sched_pending;
-    double t0_pending;
-    // block parameters of the current block (lane i holds class i)
-    double b_xstar, b_nx, b_nq, b_ps;
+    uint32_t ring_blk;           // block whose rate the draws are divided by, and its end
+    double ring_end;
+    ClassAim *aim;               // [I] parameters of the classes in the current block
 
     __device__ Sim(const Params &p_, int lane_, uint32_t rep_) : p(p_), lane(lane_), rep(rep_), warp(0), nwarps(1) {}
     __device__ __forceinline__ void block_sync() const { if (F & F_MW) __syncthreads(); else __syncwarp(); }
@@ -439,11 +470,14 @@ struct Sim {
         blk = b;
         const BlockPar &bp = p.blocks[b];
         M = bp.M;
-        best_dec = best_mix = best_pf = NONE32;
-        dirty_dec = dirty_pf = FULL;
-        b_xstar = 0.0; b_nx = 0.0; b_nq = 0.0; b_ps = 0.0;
+        dirty_dec = dirty_pf = 0;
+        if (CAL)
+            for (uint32_t k = 0; ((k << 5) + (uint32_t)lane) < n_rows(); ++k) dirty_dec = dirty_pf |= 1u << k;
+        pools_due = f_sli() && lane < (int)p.I;
         if (lane < (int)p.I) {
-            b_xstar = bp.xstar[lane]; b_nx = bp.nx[lane]; b_nq = bp.nq[lane]; b_ps = bp.ps[lane];
+            ClassAim a;
+            a.xstar = bp.xstar[lane]; a.nx = bp.nx[lane]; a.nq = bp.nq[lane]; a.ps = bp.ps[lane]; a.theta = p.cls[lane].theta;
+            aim[lane] = a;
         }
         T_blk_next = (f_blocks() && b + 1 < p.nblk) ? block_start(b + 1) : dinf();
     }
@@ -456,24 +490,32 @@ struct Sim {
 
     __device__ __forceinline__ void refill(uint32_t i)
     {
+        const double t0 = aring[i * 32];                    // (the ring is empty: where the search for the class's next arrival starts)
         const unsigned long long base = cs[i].adraw;        // (only I class records exist: every lane reads record i)
-        // with a single block the class's rate never changes and the division E / Lambda is done here, 32 at a time
-        const double Lam1 = f_blocks() ? 0.0 : __dmul_rn((double)p.N, p.blocks[0].rate[i]);
-        aring[i * 32 + lane] = make_draw(p.seed, p.rep_offset + rep, i, p.I, base + (unsigned long long)lane,
-                                         p.length_mode == 1 ? p.lengths : nullptr, p.cls[i].P, p.cls[i].D, Lam1);
+        const uint32_t b = f_blocks() ? cs[i].ablk : 0u;
+        // the division E / Lambda is done here, 32 at a time, for the block in which the class's next arrival is looked for
+        const double Lam1 = __dmul_rn((double)p.N, p.blocks[b].rate[i]);
+        __syncwarp();
+        const ADraw d = make_draw(p.seed, p.rep_offset + rep, i, p.I, base + (unsigned long long)lane,
+                                  p.length_mode == 1 ? p.lengths : nullptr, p.cls[i].P, p.cls[i].D, Lam1);
+        aring[i * 32 + lane] = d.E;
+        aring_pk[i * 32 + lane] = d.pk;
         __syncwarp();
         if (lane == (int)i) {
-            cs[i].adraw = base + 32ull;
+            const bool some = Lam1 > 0.0;       // (a class that never arrives asks for draws once, at the start)
+            if (some) cs[i].adraw = base + 32ull;
             ring_pos = 0;
-            ring_n = 32;
-            if (sched_pending) { sched_pending = false; schedule_from(t0_pending); }
+            ring_n = some ? 32u : 0u;
+            ring_blk = b;
+            ring_end = (f_blocks() && b + 1 < p.nblk) ? block_start(b + 1) : dinf();
+            if (sched_pending) { sched_pending = false; schedule_from(t0); }
         }
         __syncwarp();
     }
 
     // Class lane only: next arrival of this lane's class after t0.  A candidate at or past the end of its
     // block is discarded and drawn again from the boundary under the next block's rate (memorylessness).
-    __device__ void schedule_from(double t0)
+    __device__ __forceinline__ void schedule_from(double t0)
     {
         ClassState &c = cs[lane];
         if ((F & (F_GENERIC | F_INJECT)) && p.n_inject > 0) {
@@ -488,51 +530,109 @@ struct Sim {
             }
             return;
         }
-        uint32_t b = c.ablk;
-        for (;;) {
-            const double Lam = __dmul_rn((double)p.N, p.blocks[b].rate[lane]);
-            const bool has_next = f_blocks() && b + 1 < p.nblk;
-            if (!(Lam > 0.0)) {
-                if (!has_next) { c.ta = dinf(); c.ablk = b; return; }
-                ++b; t0 = block_start(b);
-                continue;
-            }
-            if (ring_n == 0) {          // out of draws: the warp refills at the top of the next round
-                sched_pending = true; t0_pending = t0; c.ablk = b; c.ta = dinf();
+        uint32_t b = f_blocks() ? c.ablk : 0u;
+        if (ring_n > 0 && (!f_blocks() || b == ring_blk)) {
+            const double cand = __dadd_rn(t0, aring[lane * 32 + ring_pos]);
+            const uint32_t pk = aring_pk[lane * 32 + ring_pos];
+            ring_pos++; ring_n--;
+            if (!f_blocks() || cand < ring_end) {
+                c.ta = cand; c.nextP = job_P(pk); c.nextD = job_D(pk);
                 return;
             }
-            const ADraw d = aring[lane * 32 + ring_pos];
-            ring_pos++; ring_n--;
-            const double cand = __dadd_rn(t0, f_blocks() ? __ddiv_rn(d.E, Lam) : d.E);
-            if (has_next && cand >= block_start(b + 1)) {
-                ++b; t0 = block_start(b);
-                continue;
-            }
-            c.ta = cand; c.ablk = b; c.nextP = job_P(d.pk); c.nextD = job_D(d.pk);
-            return;
+            ++b; t0 = ring_end;
         }
+        // no draws, or draws divided by the rate of another block: the warp makes new ones at the top of the next round
+        if (f_blocks()) { c.adraw -= ring_n; ring_n = 0; }
+        bool any = p.blocks[b].rate[lane] > 0.0;
+        while (!any && f_blocks() && b + 1 < p.nblk) {
+            ++b; t0 = block_start(b);
+            any = p.blocks[b].rate[lane] > 0.0;
+        }
+        c.ablk = b; c.ta = dinf();
+        sched_pending = any;
+        aring[lane * 32] = t0;
     }
 
     // Class lane only: the arrival scheduled at c.ta happens; nothing outside the class is touched.
-    __device__ void arrival_local()
+    __device__ __forceinline__ void arrival_local()
     {
         const uint32_t i = (uint32_t)lane;
         ClassState &c = cs[i];
         const double ta = c.ta;
-        c.arrivals++;
-        if (c.pq_n >= p.qcap) {
+        const uint32_t n = c.pq_n, head = c.pq_head;
+        QEntry e; e.t = ta; e.pk = pack_job(c.nextP, c.nextD, i, 0); e.cls = i;
+        if (n >= p.qcap) {
             c.overflow++;
         } else {
-            if (f_abandon()) ab_change(c.abp, p.cls[i].theta, c.pq_n, c.pq_n + 1, ta);
-            area_touch(c.aQp, c.pq_n, ta);
-            uint32_t pos = c.pq_head + c.pq_n;
+            if (f_abandon() && aim[lane].theta > 0.0) { ab_touch(c.abp, aim[lane].theta, n, ta); stale |= 1u; }
+            area_touch(c.aQp, n, ta);
+            c.pq_n = n + 1;
+            uint32_t pos = head + n;
             if (pos >= p.qcap) pos -= p.qcap;
-            QEntry e; e.t = ta; e.pk = pack_job(c.nextP, c.nextD, i, 0); e.cls = i;
             pq[(size_t)i * p.qcap + pos] = e;
-            if (c.pq_n == 0) pqh[i] = e;        // it is the head: keep a copy on chip
-            c.pq_n++;
+            if (n == 0) pqh[i] = e;        // it is the head: keep a copy on chip
         }
         schedule_from(ta);
+    }
+
+    // Class lane only: next abandonment times of the clocks whose counts changed (the prefill queue's changes in almost every round).
+    __device__ __forceinline__ void settle_queue()
+    {
+        ClassState &c = cs[lane];
+        if (stale & 1u) c.abp.t_ab = ab_next(c.abp, aim[lane].theta, c.pq_n);
+        stale &= ~1u;
+    }
+    __device__ __forceinline__ void settle_buffers()
+    {
+        ClassState &c = cs[lane];
+#pragma unroll 1
+        for (uint32_t k = 0; k < 2u; ++k) {
+            AbClock &a = k ? c.abd1 : c.abd0;
+            if (stale & (2u << k)) a.t_ab = ab_next_call(a, aim[lane].theta, k ? c.Qd1 : c.Qd0);
+        }
+        stale = 0;
+    }
+    // Class lane only, after local arrivals: may the class's next prefill-queue abandonment come before the source src at time
+    // tint?  Mostly not, which a product shows (the margin of a few ulps covers its roundings and those of the quotient).
+    __device__ __forceinline__ bool abandons_before(unsigned long long tint, uint32_t src)
+    {
+        ClassState &c = cs[lane];
+        if (stale & 1u) {
+            const double ti = __longlong_as_double((long long)tint), dt = __dadd_rn(__dsub_rn(ti, c.abp.t_last), __dmul_rn(ti, 1e-15));
+            if (__dsub_rn(c.abp.lvl, c.abp.acc) > __dmul_rn(__dmul_rn(dt, 1.0 + 1e-14), __dmul_rn(aim[lane].theta, (double)c.pq_n))) return false;
+            c.abp.t_ab = ab_next_call(c.abp, aim[lane].theta, c.pq_n);
+            stale &= ~1u;
+        }
+        const unsigned long long v = (unsigned long long)__double_as_longlong(c.abp.t_ab);
+        return v < tint || (v == tint && SRC_ABP + (uint32_t)lane < src);
+    }
+
+    // SLI-aware router: pools of the next 32 finished prefills of class i (bit k: the mixed pool for ordinals k mod 32), drawn together
+    __device__ __forceinline__ void refill_pools(uint32_t i)
+    {
+        const unsigned long long ord = (cs[i].sli_ord & ~31ull) + (unsigned long long)lane;
+        const double ps = aim[i].ps;
+        uint32_t w0, w1, w2, w3;
+        draw_rare(p, rep, (STREAM_SLI << 8) | i, ord, w0, w1, w2, w3);
+        const uint32_t m = __ballot_sync(FULL, !(u53(w0, w1) <= ps));
+        if (lane == (int)i) { pools = m; pools_due = false; }
+    }
+
+    // Top of a round: classes that ran out of arrival draws or pool draws get 32 new ones; clocks whose counts changed get their
+    // next abandonment time.
+    __device__ __forceinline__ void replenish()
+    {
+        // (a class whose next candidate lies past the end of its block asks again)
+        for (uint32_t need = __ballot_sync(FULL, sched_pending || (f_sli() && pools_due)); need;
+             need = f_blocks() ? __ballot_sync(FULL, sched_pending || (f_sli() && pools_due)) : need & (need - 1u)) {
+            const uint32_t i = (uint32_t)__ffs((int)need) - 1u;
+            if (!f_sli() || __shfl_sync(FULL, (int)sched_pending, (int)i)) refill(i);
+            if (f_sli() && __shfl_sync(FULL, (int)pools_due, (int)i)) refill_pools(i);
+        }
+        if (f_abandon() && lane < (int)p.I) {
+            settle_queue();
+            if (stale) settle_buffers();
+        }
     }
 
     __device__ uint32_t count_idle_pf()
@@ -599,7 +699,8 @@ struct Sim {
                 }
                 const uint32_t b = __ballot_sync(FULL, mine);
                 const uint32_t c = (uint32_t)__popc(b);
-                if (rank < c) pos = k + (uint32_t)__fns(b, 0, (int)rank + 1);
+                // (the lane with `rank` of them before it)
+                if (rank < c) pos = k + (uint32_t)__ffs((int)__ballot_sync(FULL, mine && (uint32_t)__popc(b & ((1u << lane) - 1u)) == rank)) - 1u;
                 else rank -= c;
             }
             if (pos == NONE32) { err = ERR_INTERNAL; return; }
@@ -620,17 +721,21 @@ struct Sim {
                 if (which == 2) c.Qd1 = Q - 1; else c.Qd0 = Q - 1;
                 c.abandoned_d++;
             }
-            a.m = m + 1; a.acc = 0.0; a.lvl = -qlog(u53(w0, w1)); a.t_last = t;
-            a.t_ab = (Q - 1 > 0) ? __dadd_rn(t, __ddiv_rn(a.lvl, __dmul_rn(p.cls[i].theta, (double)(Q - 1)))) : dinf();
+            a.m = m + 1; a.acc = 0.0; a.lvl = unit_exp(w0, w1); a.t_last = t;
+            stale |= 1u << which;
         }
     }
 
     // --- GPU choice ----------------------------------------------------------------------------
     // --- least-loaded choice on large clusters (CAL) ------------------------------------------------------
-    // Every lane keeps the smallest key of its own GPUs (its column), so a choice is one reduction over the lanes instead of
-    // a pass over all N/32 rows; columns in which something changed since are looked up again by the whole warp, one row
-    // per lane, when a choice needs them.
-    __device__ __forceinline__ void gpu_changed(uint32_t g) { if (CAL) { dirty_dec |= 1u << (g & 31u); dirty_pf |= 1u << (g & 31u); } }
+    // The smallest key of every row of 32 GPUs is kept, so a choice looks at N / 32 keys (one per lane up to 1024 GPUs) instead
+    // of all GPUs; rows in which something changed since are looked up again, a GPU per lane, when a choice needs them.
+    __device__ __forceinline__ void decodes_changed(uint32_t g) { if (CAL && lane == (int)((g >> 5) & 31u)) { dirty_dec |= 1u << (g >> 10); dirty_pf |= 1u << (g >> 10); } }
+    __device__ __forceinline__ void prefill_changed(uint32_t g)
+    {
+        // (a solo GPU that still holds a prefill has a slot less for decodes)
+        if (CAL && lane == (int)((g >> 5) & 31u)) { dirty_pf |= 1u << (g >> 10); if (g >= M) dirty_dec |= 1u << (g >> 10); }
+    }
 
     // key of GPU g for the wanted tiers: solo GPUs first, then decodes held, then index; NONE32 when it is not eligible
     __device__ __forceinline__ uint32_t key_of(uint32_t g, uint32_t tiers) const
@@ -663,33 +768,26 @@ struct Sim {
         if (!f_random()) {
             uint32_t best = NONE32;
             if (CAL) {
+                // keys of the solo-first router, or of solo GPUs under the SLI-aware ones; of mixed GPUs under those; of prefill targets
                 const bool pf = tiers == WANT_PREFILL;
-                uint32_t dirty = pf ? dirty_pf : dirty_dec;
-                if (__popc(dirty) > 6) {
-                    uint32_t a = NONE32, b = NONE32;       // every lane over its own rows
-#pragma unroll 2
-                    for (uint32_t k = 0; k < rows; ++k) {
-                        a = min(a, key_of((k << 5) + (uint32_t)lane, pf ? WANT_PREFILL : (f_sli() ? WANT_SOLO : (WANT_SOLO | WANT_MIX))));
-                        if (f_sli() && !pf) b = min(b, key_of((k << 5) + (uint32_t)lane, WANT_MIX));
-                    }
-                    if (pf) best_pf = a; else { best_dec = a; best_mix = b; }
-                    dirty = 0;
-                }
 #pragma unroll 1
-                for (; dirty; dirty &= dirty - 1u) {
-                    const uint32_t col = (uint32_t)__ffs((int)dirty) - 1u;
-                    uint32_t a = NONE32, b = NONE32;
-#pragma unroll 1
-                    for (uint32_t k = (uint32_t)lane; k < rows; k += 32u) {
-                        a = min(a, key_of((k << 5) + col, pf ? WANT_PREFILL : (f_sli() ? WANT_SOLO : (WANT_SOLO | WANT_MIX))));
-                        if (f_sli() && !pf) b = min(b, key_of((k << 5) + col, WANT_MIX));
+                for (uint32_t bits = __ballot_sync(FULL, (pf ? dirty_pf : dirty_dec) != 0); bits; bits = __ballot_sync(FULL, (pf ? dirty_pf : dirty_dec) != 0)) {
+                    const uint32_t l = (uint32_t)__ffs((int)bits) - 1u, m = __shfl_sync(FULL, pf ? dirty_pf : dirty_dec, (int)l);
+                    const uint32_t row = (((uint32_t)__ffs((int)m) - 1u) << 5) + l, g = (row << 5) + (uint32_t)lane;
+                    const uint32_t a = __reduce_min_sync(FULL, key_of(g, pf ? WANT_PREFILL : (f_sli() ? WANT_SOLO : (WANT_SOLO | WANT_MIX))));
+                    if (f_sli() && !pf) {
+                        const uint32_t b = __reduce_min_sync(FULL, key_of(g, WANT_MIX));
+                        if (lane == (int)l) row_key[rows + row] = b;
                     }
-                    a = __reduce_min_sync(FULL, a);
-                    if (f_sli()) b = __reduce_min_sync(FULL, b);
-                    if (lane == (int)col) { if (pf) best_pf = a; else { best_dec = a; best_mix = b; } }
+                    if (lane == (int)l) {
+                        row_key[(pf ? 2u * rows : 0u) + row] = a;
+                        if (pf) dirty_pf &= dirty_pf - 1u; else dirty_dec &= dirty_dec - 1u;
+                    }
                 }
-                if (pf) dirty_pf = 0; else dirty_dec = 0;
-                best = pf ? best_pf : ((f_sli() && tiers == WANT_MIX) ? best_mix : best_dec);
+                // (a lane reads the rows that it has written)
+                const uint32_t *keys = row_key + (pf ? 2u * rows : ((f_sli() && tiers == WANT_MIX) ? rows : 0u));
+#pragma unroll 1
+                for (uint32_t k = (uint32_t)lane; k < rows; k += 32u) best = min(best, keys[k]);
             } else {
 #pragma unroll 4
                 for (uint32_t k = 0; k < rows; ++k) best = min(best, key_of((k << 5) + (uint32_t)lane, tiers));
@@ -708,16 +806,17 @@ struct Sim {
                 cnt += (uint32_t)__popc(__ballot_sync(FULL, in_tier((k << 5) + (uint32_t)lane, w)));
             if (cnt == 0) continue;
             uint32_t idx = 0;
-            if (cnt > 1) {
-                uint32_t w0, w1, w2, w3;
-                draw(p, rep, STREAM_PLACEMENT << 8, place_ord++, w0, w1, w2, w3);
-                idx = __umulhi(w0, cnt);
-            }
+            if (cnt > 1) idx = __umulhi(placement_word(), cnt);
 #pragma unroll(SPL > 0 ? SPL : 4)
             for (uint32_t k = first; k < last; ++k) {
-                const uint32_t b = __ballot_sync(FULL, in_tier((k << 5) + (uint32_t)lane, w));
+                const bool in = in_tier((k << 5) + (uint32_t)lane, w);
+                const uint32_t b = __ballot_sync(FULL, in);
                 const uint32_t c = (uint32_t)__popc(b);
-                if (idx < c) return (k << 5) + (uint32_t)__fns(b, 0, (int)idx + 1);
+                if (idx < c) {
+                    // the lane whose GPU has idx eligible ones before it in the row
+                    const uint32_t at = __ballot_sync(FULL, in && (uint32_t)__popc(b & ((1u << lane) - 1u)) == idx);
+                    return (k << 5) + (uint32_t)__ffs((int)at) - 1u;
+                }
                 idx -= c;
             }
             err = ERR_INTERNAL;
@@ -726,12 +825,26 @@ struct Sim {
         return NONE32;
     }
 
-    // GPU g may have to start an iteration at the end of this event: noted in its owner's row mask
+    // Word of the next placement draw: the warp makes the draws of 32 consecutive ordinals together, one per lane.
+    __device__ __forceinline__ uint32_t placement_word()
+    {
+        const unsigned long long ord = place_ord++;
+        if ((ord & ~31ull) != place_base) {
+            uint32_t w1, w2, w3;
+            place_base = ord & ~31ull;
+            draw_rare(p, rep, STREAM_PLACEMENT << 8, place_base + (unsigned long long)lane, place_w, w1, w2, w3);
+        }
+        return __shfl_sync(FULL, place_w, (int)(ord & 31ull));
+    }
+
+    // GPU g may have to start an iteration at the end of this event: noted in its owner's row mask, or once in a list over the lanes
     __device__ __forceinline__ void touch_server(uint32_t g)
     {
         if (SPL > 0) { if (lane == (int)(g & 31u)) need_start |= 1u << (g >> 5); }
-        else if (n_touch < TOUCH_CAP) { if (lane == 0) touch[n_touch] = g; n_touch++; }
-        else touch_all = true;
+        else if (!__any_sync(FULL, (uint32_t)lane < n_touch && touch_g == g)) {
+            if (n_touch == 32u) touch_all = true;
+            else { if (lane == (int)n_touch) touch_g = g; n_touch++; }
+        }
     }
 
     // --- decode placement ------------------------------------------------------------------------
@@ -796,27 +909,81 @@ struct Sim {
         return e;
     }
 
-    // A request of class i whose prefill ended at tpf starts decoding on GPU g.  from_buffer: it waited in
-    // the pool's buffer; otherwise it passes through the (empty) buffer at this very instant, which
-    // leaves the buffer's count, integral and abandonment clock as one touch at time t would.
-    __device__ void place_job(uint32_t pool, uint32_t g, uint32_t i, uint32_t P, uint32_t D, double tpf, bool from_buffer)
+    // A request leaves for its decode on GPU g.  fresh: it has just finished its prefill (d_pk, arrived at d_tarr) and passes through
+    // its pool's empty buffer at this very instant, which leaves the buffer's count, integral and abandonment clock as one
+    // touch at time t would, or joins the buffer (g = NONE32); else it is an entry of the pool's buffer.
+    // One body for all of that, and its parts - the class lane's and the GPU's - read before they write, so that their reads overlap.
+    __device__ __forceinline__ void place(uint32_t pool, uint32_t g, bool fresh)
     {
-        const bool mixed = g < M;
+        const bool placed = g != NONE32, mixed = placed && g < M;
+        const uint32_t n_buf = pool ? dq_n1 : dq_n0;
+        uint32_t pk = d_pk;
+        double tpf = t;
+        if (!fresh) {
+            const QEntry e = take_buffered(pool, f_slig() ? select_in_pool(pool) : 0u);
+            pk = pack_job(job_P(e.pk), job_D(e.pk), e.cls, 0);
+            tpf = e.t;
+        }
+        const bool full = fresh && !placed && n_buf >= p.qcap;
+        const uint32_t i = job_cls(pk);
+        // the GPU (every lane reads it)
+        const uint32_t gg = placed ? g : 0u;
+        const uint32_t nd = ndec[gg], it0 = it[gg], nf = nfin[gg];
+        const bool running = tnext[gg] < dinf();
         if (lane == (int)i) {
             ClassState &c = cs[i];
-            const uint32_t Qd = pool ? c.Qd1 : c.Qd0;
-            if (f_abandon()) ab_change(pool ? c.abd1 : c.abd0, p.cls[i].theta, Qd, from_buffer ? Qd - 1 : Qd, t);
-            area_touch(c.aQd, c.Qd0 + c.Qd1, t);
-            if (from_buffer) { if (pool) c.Qd1--; else c.Qd0--; }
-            const double rel = __dsub_rn(t, T_reset);
-            if (mixed) { c.sYm_in = __dadd_rn(c.sYm_in, rel); c.Ym++; c.placed_mixed++; }
-            else       { c.sYs_in = __dadd_rn(c.sYs_in, rel); c.Ys++; c.placed_solo++; }
+            const uint32_t Qd0 = c.Qd0, Qd1 = c.Qd1, Qd = pool ? Qd1 : Qd0;
+            if (fresh) {
+                const uint32_t X = c.X;
+                area_touch(c.aX, X, t);
+                c.X = X - 1;
+                c.prefill_done++;
+                c.tok_in_pf += job_P(pk);                  // separate charging credits the prompt here, Eq. (23)
+                const double ttft = __dsub_rn(t, d_tarr);
+                c.sum_ttft = __dadd_rn(c.sum_ttft, ttft);
+                if (f_hist()) atomicAdd(&hist[((size_t)i * 2 + 0) * NBIN + hist_bin(ttft)], 1u);
+                if (f_sli()) {
+                    const unsigned long long ord = c.sli_ord + 1ull;
+                    c.sli_ord = ord;
+                    if ((ord & 31ull) == 0) pools_due = true;
+                }
+            }
+            if (full) {
+                c.overflow_d++;
+            } else if (fresh && placed) {
+                // (nothing accrues on an empty buffer, and its clock starts when it fills)
+                if (Qd0 + Qd1 != 0) area_touch(c.aQd, Qd0 + Qd1, t);
+            } else {
+                const uint32_t Qn = fresh ? Qd + 1u : Qd - 1u;
+                if (f_abandon() && aim[lane].theta > 0.0) {
+                    ab_touch(pool ? c.abd1 : c.abd0, aim[lane].theta, Qd, t);
+                    stale |= pool ? 4u : 2u;
+                }
+                area_touch(c.aQd, Qd0 + Qd1, t);
+                if (pool) c.Qd1 = Qn; else c.Qd0 = Qn;
+            }
+            if (placed) {
+                const double rel = __dsub_rn(t, *T_reset_at);
+                if (mixed) { c.sYm_in = __dadd_rn(c.sYm_in, rel); c.Ym++; }
+                else       { c.sYs_in = __dadd_rn(c.sYs_in, rel); c.Ys++; }
+            }
         }
+        if (!placed) {
+            if (!full) {
+                uint32_t pos = (pool ? dq_head1 : dq_head0) + n_buf;
+                if (pos >= p.qcap) pos -= p.qcap;
+                if (lane == 0) {
+                    QEntry e; e.t = t; e.pk = pk; e.cls = i;
+                    dq[(size_t)pool * p.qcap + pos] = e;
+                }
+                if (pool) dq_n1++; else dq_n0++;
+            }
+            return;
+        }
+        const uint32_t P = job_P(pk), D = job_D(pk);
         if (lane == (int)(g & 31u)) {
-            const uint32_t sl = ndec[g];
-            const bool running = tnext[g] < dinf();
             // joins the iteration that starts next: a running iteration first finishes as it+1
-            const uint32_t fin = it[g] + (running ? 1u : 0u) + D;
+            const uint32_t fin = it0 + (running ? 1u : 0u) + D;
             size_t o;
             if (f_slots()) {
                 // first free slot of the GPU's occupancy words
@@ -834,16 +1001,16 @@ struct Sim {
                 sfin16[g * p.B + slot] = (uint16_t)fin;
                 o = (size_t)g * p.B + slot;
             } else {
-                o = (size_t)g * p.B + sl;
+                o = (size_t)g * p.B + nd;
                 s_fin[o] = fin;
             }
             SlotRec r; r.tpf = tpf; r.pk = pack_job(P, D, i, mixed ? 1u : 0u); r.pad = 0;
             s_rec[o] = r;
-            ndec[g] = (uint16_t)(sl + 1);
-            nfin[g] = min(nfin[g], fin);
+            ndec[g] = (uint16_t)(nd + 1);
+            nfin[g] = min(nf, fin);
             if (f_kappa()) Kpend[g] += P;
         }
-        gpu_changed(g);
+        decodes_changed(g);
         touch_server(g);
     }
 
@@ -877,8 +1044,8 @@ struct Sim {
         bool ok = false;
         if (lane < (int)p.I) {
             const ClassState &c = cs[lane];
-            ok = c.pq_n > 0 && b_xstar > 0.0;
-            if (ok) xi = order_key(__ddiv_rn(__dsub_rn((double)c.X, b_nx), b_xstar));
+            ok = c.pq_n > 0 && aim[lane].xstar > 0.0;
+            if (ok) xi = order_key(__ddiv_rn(__dsub_rn((double)c.X, aim[lane].nx), aim[lane].xstar));
         }
         const uint32_t xh = (uint32_t)(xi >> 32), mh = __reduce_min_sync(FULL, xh);
         const uint32_t ml = __reduce_min_sync(FULL, xh == mh ? (uint32_t)xi : NONE32);
@@ -886,7 +1053,7 @@ struct Sim {
         uint32_t tie = __ballot_sync(FULL, ok);
         if (tie & (tie - 1u)) {
             unsigned long long dq = 0ull;
-            if (ok) dq = order_key(__dsub_rn((double)cs[lane].pq_n, b_nq));
+            if (ok) dq = order_key(__dsub_rn((double)cs[lane].pq_n, aim[lane].nq));
             const uint32_t dh = (uint32_t)(dq >> 32), Mh = __reduce_max_sync(FULL, dh);
             const uint32_t Ml = __reduce_max_sync(FULL, dh == Mh ? (uint32_t)dq : 0u);
             tie = __ballot_sync(FULL, ok && dh == Mh && (uint32_t)dq == Ml);
@@ -915,15 +1082,14 @@ struct Sim {
         __syncwarp();
         if (lane == (int)i) {
             ClassState &c = cs[i];
-            const uint32_t head = c.pq_head;
-            if (f_abandon()) ab_change(c.abp, p.cls[i].theta, c.pq_n, c.pq_n - 1, t);
-            area_touch(c.aQp, c.pq_n, t);
-            c.pq_n--;
-            c.pq_head = (head + 1 == p.qcap) ? 0 : head + 1;
-            if (c.pq_n > 0) { cp_async16(&pqh[i], &pq[(size_t)i * p.qcap + c.pq_head]); cp_async_commit(); rec_after = 0; }
-            area_touch(c.aX, c.X, t);
-            c.X++;
-            c.admitted++;
+            const uint32_t n = c.pq_n, X = c.X, head = c.pq_head, next = (head + 1 == p.qcap) ? 0 : head + 1;
+            if (f_abandon() && aim[lane].theta > 0.0) { ab_touch(c.abp, aim[lane].theta, n, t); stale |= 1u; }
+            area_touch(c.aQp, n, t);
+            area_touch(c.aX, X, t);
+            c.pq_n = n - 1;
+            c.pq_head = next;
+            c.X = X + 1;
+            if (n > 1) { cp_async16(&pqh[i], &pq[(size_t)i * p.qcap + next]); cp_async_commit(); rec_after = 0; }
         }
         n_idle_pf--;
         idle_hint = NONE32;
@@ -932,7 +1098,7 @@ struct Sim {
             pfrem[g] = (uint16_t)job_P(e.pk);
             pf_tarr[g] = e.t;
         }
-        gpu_changed(g);
+        prefill_changed(g);
         touch_server(g);
     }
 
@@ -951,39 +1117,39 @@ struct Sim {
         const uint32_t pc = has_pf ? min(p.C, rem) : 0u;
         uint32_t fl = (nf == it0 + 1u) ? 0x4000u : 0u;
         if (pc > 0 && pc == rem) fl |= 0x8000u;
+        if (CAL && pc > 0) fl |= BATCH_MIXED;
         const double tau = iter_time(p, pc, nd, Kg, f_kappa());
         if (act && tn >= 0x7ff0000000000000ull && (nd > 0 || has_pf)) {
             if (f_kappa()) { K[g] = Kg; Kpend[g] = 0; }
-            pfcur[g] = (uint16_t)pc;
+            if (!CAL) pfcur[g] = (uint16_t)pc;
             nact[g] = (uint16_t)(nd | fl);
             const double te = __dadd_rn(ts, tau);
             tnext[g] = te;
-            if (CAL) bkt[g] = bucket_id(te);
+            if (CAL) file_end(g, te);
         }
     }
 
     __device__ void dispatch()
     {
         __syncwarp();   // queue entries and GPU state written by the event handler are visible to every lane
-        // the request that has just finished its prefill: it passes through its pool's empty buffer
-        if (direct) {
-            uint32_t g = d_gpu;
-            if (g == NONE32) g = f_sli() ? choose(d_pool ? WANT_MIX : WANT_SOLO) : choose(WANT_SOLO | WANT_MIX);
-            if (g != NONE32) place_job(d_pool, g, job_cls(d_pk), job_P(d_pk), job_D(d_pk), t, false);
-            else enqueue_decode();
-            direct = false;
-            __syncwarp();
-        }
-        // decode routing of buffered requests: FCFS, solo GPUs before mixed ones, or pool by pool
+        // decode routing: the request that has just finished its prefill, then the buffered ones, FCFS, solo GPUs before mixed ones,
+        // or pool by pool
         uint32_t pool = drain_dirty ? 0u : 2u;       // buffer being drained; 2: none left
-        while (pool < 2u) {
-            if (pool == 0 && dq_n0 == 0) pool = f_sli() ? 1u : 2u;
-            if (pool == 1 && dq_n1 == 0) pool = 2u;
-            if (pool == 2u) break;
-            const uint32_t g = f_sli() ? choose(pool ? WANT_MIX : WANT_SOLO) : choose(WANT_SOLO | WANT_MIX);
-            if (g == NONE32) { pool = (pool == 0 && f_sli()) ? 1u : 2u; continue; }
-            const QEntry e = take_buffered(pool, f_slig() ? select_in_pool(pool) : 0u);
-            place_job(pool, g, e.cls, job_P(e.pk), job_D(e.pk), e.t, true);
+#pragma unroll 1
+        for (;;) {
+            uint32_t q = d_pool, g = d_gpu;
+            const bool fresh = handed, search = !fresh || (direct && g == NONE32);
+            if (!fresh) {
+                if (pool == 0 && dq_n0 == 0) pool = f_sli() ? 1u : 2u;
+                if (pool == 1 && dq_n1 == 0) pool = 2u;
+                if (pool == 2u) break;
+                q = pool;
+            }
+            if (search) g = choose(f_sli() ? (q ? WANT_MIX : WANT_SOLO) : (WANT_SOLO | WANT_MIX));
+            if (!fresh && g == NONE32) { pool = (pool == 0 && f_sli()) ? 1u : 2u; continue; }
+            if (fresh && search && g == NONE32 && !f_sli()) pool = 2u;       // no GPU has a slot: nothing to drain either
+            place(q, g, fresh);
+            handed = false;
             __syncwarp();
         }
         // prefill gate on mixed GPUs whose prefill slot is idle; a single idle slot whose GPU is known needs no search (and
@@ -1008,10 +1174,10 @@ struct Sim {
                 start_at((k << 5) + (uint32_t)lane, t, ((need_start >> k) & 1u) != 0);
             need_start = 0;
         } else {
-            // one lane per touched GPU (a GPU noted twice is started by two lanes with the same result), or all GPUs
+            // one lane per touched GPU, or all GPUs
             const uint32_t n = touch_all ? p.N : n_touch;
 #pragma unroll 1
-            for (uint32_t k = (uint32_t)lane; k < n; k += 32u) start_at(touch_all ? k : touch[k], t);
+            for (uint32_t k = (uint32_t)lane; k < n; k += 32u) start_at(touch_all ? k : touch_g, t);
         }
         n_touch = 0;
         touch_all = false;
@@ -1025,7 +1191,7 @@ struct Sim {
         const uint32_t i = job_cls(pk), P = job_P(pk), D = job_D(pk);
         if (lane == (int)i) {
             WarpClassStats &c = wcs[warp * (int)p.I + (int)i];
-            const double rel = __dsub_rn(te, T_reset);
+            const double rel = __dsub_rn(te, *T_reset_at);
             if (job_flag(pk)) { c.sYm_out = __dadd_rn(c.sYm_out, rel); c.done_mixed++; }
             else              { c.sYs_out = __dadd_rn(c.sYs_out, rel); c.done_solo++; }
             c.tok_in += P;       // bundled charging credits the request here, Eq. (21)-(22)
@@ -1049,13 +1215,13 @@ struct Sim {
             const uint32_t pk = st_rec[e].pk;
             const double te = st_te[e], tpot = __ddiv_rn(__dsub_rn(te, st_rec[e].tpf), (double)job_D(pk));
             st_rec[e].tpf = tpot;
-            st_te[e] = __dsub_rn(te, T_reset);
+            st_te[e] = __dsub_rn(te, *T_reset_at);
             if (f_hist()) atomicAdd(&hist[((size_t)job_cls(pk) * 2 + 1) * NBIN + hist_bin(tpot)], 1u);
         }
         __syncwarp();
         if (lane < (int)p.I) {
             WarpClassStats c = wcs[warp * (int)p.I + lane];
-#pragma unroll 2
+#pragma unroll 1
             for (uint32_t e = 0; e < n_pend; ++e) {
                 const uint32_t pk = st_rec[e].pk;
                 if (job_cls(pk) != (uint32_t)lane) continue;
@@ -1121,7 +1287,7 @@ struct Sim {
             nfin[g] = newmin == NONE32 ? NONE32 : itg + newmin;
             if (f_kappa()) K[g] -= Kdrop;
         }
-        gpu_changed(g);
+        decodes_changed(g);
         __syncwarp();
     }
 
@@ -1130,45 +1296,54 @@ struct Sim {
         if (f_slots()) { retire_slots(g, itg, nd, te); return; }
         const int owner = (int)(g & 31u);
         uint32_t n = nd, newmin = NONE32, Kdrop = 0;
-        const size_t base = (size_t)g * p.B;
-        // the stamps of four chunks of 32 slots are fetched together (one memory round trip), from the tail of the list
+        uint32_t *fin = s_fin + (size_t)g * p.B;
+        SlotRec *rec = s_rec + (size_t)g * p.B;
+        // The stamps of 128 slots are fetched together, four neighbours per lane, and with them the tail entry that will close the
+        // gap of the first finished request: one memory round trip.  The finished request's own record only feeds the
+        // statistics: with one warp it stays on its way until the next one (`late`).
+        SlotRec rl; rl.tpf = 0.0; rl.pk = 0; rl.pad = 0;
+        uint32_t fl = 0;
+        if (lane == 0) { rl = rec[nd - 1]; fl = fin[nd - 1]; }
 #pragma unroll 1
-        for (int k0 = (int)((nd - 1) >> 5) & ~3; k0 >= 0; k0 -= 4) {
-            uint32_t f[4], hit[4];
+        for (int k0 = (int)((nd - 1u) & ~127u); k0 >= 0; k0 -= 128) {
+            uint32_t f[4], mine = 0;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const uint32_t j = ((uint32_t)(k0 + q) << 5) + (uint32_t)lane;
-                f[q] = j < nd ? s_fin[base + j] : NONE32;
+                const uint32_t j = (uint32_t)(k0 + 4 * lane + q);
+                f[q] = j < nd ? fin[j] : NONE32;
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                if (f[q] != itg) newmin = min(newmin, f[q]);
-                hit[q] = __ballot_sync(FULL, f[q] == itg);
+                if (f[q] == itg) mine |= 1u << q;
+                else newmin = min(newmin, f[q]);
             }
 #pragma unroll 1
-            for (;;) {          // hits from the tail of the list down
-                const int q = hit[3] ? 3 : (hit[2] ? 2 : (hit[1] ? 1 : 0));
-                const uint32_t hits = hit[3] ? hit[3] : (hit[2] ? hit[2] : (hit[1] ? hit[1] : hit[0]));
-                if (!hits) break;
-                const int hl = 31 - __clz(hits);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) hit[j] &= j == q ? ~(1u << hl) : ~0u;
-                const uint32_t h = ((uint32_t)(k0 + q) << 5) + (uint32_t)hl;
-                // the finished request's record and the tail entry that takes its place, in one round trip
-                const uint32_t last = n - 1;
-                const SlotRec rh = s_rec[base + h], rl = s_rec[base + last];
-                const uint32_t fl = s_fin[base + last];
-                if (STAGED) {
+            for (uint32_t any = __ballot_sync(FULL, mine != 0); any; any = __ballot_sync(FULL, mine != 0)) {      // from the tail of the list down
+                const int hl = 31 - __clz((int)any);
+                const int q = 31 - __clz((int)__shfl_sync(FULL, mine, hl));
+                if (lane == hl) mine &= ~(1u << q);
+                const uint32_t h = (uint32_t)(k0 + 4 * hl + q), last = n - 1u;
+                if (STAGED && !f_kappa()) {
+                    stage_late();
                     if (n_pend == (uint32_t)ROW_STAGE_CAP) flush_done();
-                    if (lane == 0) { st_rec[n_pend] = rh; st_te[n_pend] = te; }
-                    n_pend++;
+                    has_late = true;
+                    if (lane == 0) { const SlotRec r = rec[h]; late_tpf = r.tpf; late_pk = r.pk; st_te[n_pend] = te; }
                 } else {
-                    account_done(rh.pk, rh.tpf, te);
+                    const SlotRec rh = rec[h];
+                    if (STAGED) {
+                        if (n_pend == (uint32_t)ROW_STAGE_CAP) flush_done();
+                        if (lane == 0) { st_rec[n_pend] = rh; st_te[n_pend] = te; }
+                        n_pend++;
+                    } else {
+                        account_done(rh.pk, rh.tpf, te);
+                    }
+                    Kdrop += job_P(rh.pk) + job_D(rh.pk);
+                    __syncwarp();
                 }
-                Kdrop += job_P(rh.pk) + job_D(rh.pk);
-                __syncwarp();
-                if (lane == 0 && h != last) { s_fin[base + h] = fl; s_rec[base + h] = rl; }
-                __syncwarp();
+                if (lane == 0) {
+                    if (h != last) { fin[h] = fl; rec[h] = rl; }
+                    if (last > 0) { rl = rec[last - 1]; fl = fin[last - 1]; }      // for the next one, if there is one
+                }
                 n = last;
             }
         }
@@ -1178,27 +1353,36 @@ struct Sim {
             nfin[g] = newmin;
             if (f_kappa()) K[g] -= Kdrop;
         }
-        gpu_changed(g);
+        decodes_changed(g);
         __syncwarp();
+    }
+
+    // The record that was on its way joins the staged ones.
+    __device__ __forceinline__ void stage_late()
+    {
+        if (!has_late) return;
+        if (lane == 0) { SlotRec r; r.tpf = late_tpf; r.pk = late_pk; r.pad = 0; st_rec[n_pend] = r; }
+        n_pend++;
+        has_late = false;
     }
 
     // --- end of an iteration on GPU g (warp-wide path: the end is not local) ----------------------
     // nd_before: decodes that g held before this event's retirements (one warp: the round's passes have ended the iteration)
-    __device__ void on_server(uint32_t g, uint32_t nd_before = 0)
+    // na_ev: its batch word; pk_ev, tarr_ev: the request whose prefill has ended (CAL: it was read when the end was loaded)
+    __device__ __forceinline__ void on_server(uint32_t g, uint32_t nd_before, uint32_t na_ev, uint32_t pk_ev, double tarr_ev)
     {
         const int owner = (int)(g & 31u);
         uint32_t flags = 0, itg = 0, nd = 0;
         if (SPL > 0 || CAL) {      // (one warp, unrolled rows or calendar)
             // the round's passes have ended the iteration and retired its finished decodes; the frozen batch
             // flags say what the end brought
-            const uint32_t na = nact[g];
-            flags = ((na >> 14) & 1u) | (((na >> 15) & 1u) << 1);
+            flags = na_ev >> 14;
             nd = nd_before;
         } else {
             if (lane == owner) {
                 itg = it[g] + 1;
                 it[g] = itg;
-                const uint32_t na = nact[g] & 0x3fffu, pc = pfcur[g], Kg = f_kappa() ? K[g] : 0u;
+                const uint32_t na = nact[g] & BATCH_MASK, pc = pfcur[g], Kg = f_kappa() ? K[g] : 0u;
                 const double tau = iter_time(p, pc, na, Kg, f_kappa());     // duration of the iteration that ends (the chain of its start)
                 if (pc > 0) { it_mixed++; busy_mixed = __dadd_rn(busy_mixed, tau); }
                 else        { it_solo++;  busy_solo = __dadd_rn(busy_solo, tau); }
@@ -1231,41 +1415,21 @@ struct Sim {
             }
         }
         if (flags & 2u) {
-            // prefill finished: account, then hand the request to the decode stage
-            const uint32_t pk = pfjob[g];
-            const double tarr = pf_tarr[g];
-            const uint32_t i = job_cls(pk), P = job_P(pk);
+            // prefill finished: the request goes to the decode stage (place())
+            const uint32_t pk = CAL ? pk_ev : pfjob[g], i = job_cls(pk);
+            d_tarr = CAL ? tarr_ev : pf_tarr[g];
+            const uint32_t nd_now = ndec[g];
             uint32_t pool = 0;
-            if (f_sli()) {
-                // SLI-aware router: one uniform per finished prefill decides the pool
-                const unsigned long long ord = cs[i].sli_ord;
-                const double ps = __shfl_sync(FULL, b_ps, i);
-                uint32_t w0, w1, w2, w3;
-                if (SPL == 0 && !(F & F_MW)) draw(p, rep, (STREAM_SLI << 8) | i, ord, w0, w1, w2, w3);       // (+4 % inline at N = 256, -2 % at N = 16)
-                else draw_rare(p, rep, (STREAM_SLI << 8) | i, ord, w0, w1, w2, w3);
-                pool = (u53(w0, w1) <= ps) ? 0u : 1u;
-                __syncwarp();       // every lane has read the ordinal before its owner advances it
-            }
-            if (lane == (int)i) {
-                ClassState &c = cs[i];
-                area_touch(c.aX, c.X, t);
-                c.X--;
-                c.prefill_done++;
-                c.tok_in_pf += P;                  // separate charging credits the prompt here, Eq. (23)
-                const double ttft = __dsub_rn(t, tarr);
-                c.sum_ttft = __dadd_rn(c.sum_ttft, ttft);
-                if (f_hist()) atomicAdd(&hist[((size_t)i * 2 + 0) * NBIN + hist_bin(ttft)], 1u);
-                if (f_sli()) c.sli_ord++;
-            }
+            // SLI-aware router: one uniform per finished prefill decides the pool
+            if (f_sli()) pool = (__shfl_sync(FULL, pools, (int)i) >> ((uint32_t)cs[i].sli_ord & 31u)) & 1u;
             __syncwarp();   // every lane has read the finished job before its owner clears it
             if (lane == owner) pfjob[g] = 0;
-            gpu_changed(g);
-            __syncwarp();
+            prefill_changed(g);
             // No router (immediate same-slot decoding, an ablation of the paper's EC): the request goes on decoding on
             // g, in the slot it holds; it passes through the empty buffer at this instant.
             const bool immediate = (F & F_GENERIC) && p.router == 3;
             // the prefill slot of g is idle again
-            if (g < M && ndec[g] + (immediate ? 1u : 0u) <= p.B - 1) {
+            if (g < M && nd_now + (immediate ? 1u : 0u) <= p.B - 1) {
                 n_idle_pf++;
                 idle_hint = (n_idle_pf == 1) ? g : NONE32;
             }
@@ -1273,41 +1437,14 @@ struct Sim {
             d_pool = pool;
             d_pk = pk & 0x7fffffffu;
             d_gpu = immediate ? g : NONE32;
+            handed = true;
             // (The solo pool is served first; under random placement both pools draw from one sequence, so a request of the
             // mixed pool waits its turn behind a backlog of the solo pool, which new targets may have made room for.)
             direct = immediate || ((pool ? dq_n1 : dq_n0) == 0 && !(f_random() && pool == 1u && dq_n0 != 0));
-            if (!direct) enqueue_decode();
             drain_dirty = true;
             gate_dirty = true;
         }
         touch_server(g);
-    }
-
-    // The request that has just finished its prefill (d_pk) joins its pool's buffer.
-    __device__ __forceinline__ void enqueue_decode()
-    {
-        const uint32_t pool = d_pool, i = job_cls(d_pk), n = pool ? dq_n1 : dq_n0;
-        const bool full = n >= p.qcap;
-        if (lane == (int)i) {
-            ClassState &c = cs[i];
-            if (full) {
-                c.overflow_d++;
-            } else {
-                const uint32_t Qd = pool ? c.Qd1 : c.Qd0;
-                if (f_abandon()) ab_change(pool ? c.abd1 : c.abd0, p.cls[i].theta, Qd, Qd + 1, t);
-                area_touch(c.aQd, c.Qd0 + c.Qd1, t);
-                if (pool) c.Qd1++; else c.Qd0++;
-            }
-        }
-        if (!full) {
-            uint32_t pos = (pool ? dq_head1 : dq_head0) + n;
-            if (pos >= p.qcap) pos -= p.qcap;
-            if (lane == 0) {
-                QEntry e; e.t = t; e.pk = d_pk; e.cls = i;
-                dq[(size_t)pool * p.qcap + pos] = e;
-            }
-            if (pool) dq_n1++; else dq_n0++;
-        }
     }
 
     // --- local end of an iteration (owner lane only) ----------------------------------------------------
@@ -1318,34 +1455,51 @@ struct Sim {
     __device__ __forceinline__ bool local_end(uint32_t g, double te, bool act = true, bool evt = false)
     {
         // straight-line: all fields are read first and the stores are predicated on `act` (see start_at)
-        const uint32_t it0 = it[g], na_raw = nact[g], pc = pfcur[g], nd = ndec[g], pr = pfrem[g], nf = nfin[g];
+        const uint32_t it0 = it[g], na_raw = nact[g], nd = ndec[g], pr = pfrem[g], nf = nfin[g];
+        const uint32_t pc = CAL ? ((na_raw & BATCH_MIXED) ? min(p.C, pr) : 0u) : (uint32_t)pfcur[g];
         uint32_t K0 = 0, Kp = 0;
         if (f_kappa()) { K0 = K[g]; Kp = Kpend[g]; }
-        const double tau = iter_time(p, pc, na_raw & 0x3fffu, K0, f_kappa());   // duration of the iteration that ends (the chain of its start)
+        const double tau = iter_time(p, pc, na_raw & BATCH_MASK, K0, f_kappa());   // duration of the iteration that ends (the chain of its start)
         const uint32_t itg = it0 + 1u;
         const uint32_t rem = pr - pc;                       // prompt tokens left after this iteration's chunk
         const bool retire = (na_raw & 0x4000u) != 0;        // a decode finished: the GPU waits for retire_decodes
         const bool has_pf = rem != 0;                       // (the end of a prefill is never local: rem > 0 while one runs)
         const bool restart = !retire && !evt && (nd != 0 || has_pf);
         // restart at te with what the GPU holds now (requests placed meanwhile join here)
-        const uint32_t Kend = K0 + (na_raw & 0x3fffu);
+        const uint32_t Kend = K0 + (na_raw & BATCH_MASK);
         const uint32_t Kg = Kend + Kp;
         const uint32_t pc2 = has_pf ? min(p.C, rem) : 0u;
         uint32_t fl = (nf == itg + 1u) ? 0x4000u : 0u;
         if (pc2 > 0 && pc2 == rem) fl |= 0x8000u;
+        if (CAL && pc2 > 0) fl |= BATCH_MIXED;
         const double tau2 = iter_time(p, pc2, nd, Kg, f_kappa());
         if (act) {
             it[g] = itg;
             if (pc > 0) { it_mixed++; busy_mixed = __dadd_rn(busy_mixed, tau); pfrem[g] = (uint16_t)rem; }
             else        { it_solo++;  busy_solo = __dadd_rn(busy_solo, tau); }
             if (f_kappa()) { K[g] = restart ? Kg : Kend; if (restart) Kpend[g] = 0; }
-            pfcur[g] = restart ? (uint16_t)pc2 : (uint16_t)0;
+            if (!CAL) pfcur[g] = restart ? (uint16_t)pc2 : (uint16_t)0;
             if (restart) nact[g] = (uint16_t)(nd | fl);
             const double tn = __dadd_rn(te, tau2);
             tnext[g] = restart ? tn : dinf();
-            if (CAL) bkt[g] = restart ? bucket_id(tn) : (uint8_t)255;
+            if (CAL && restart) file_end(g, tn);
         }
         return act && retire;
+    }
+
+    // Counters that follow from others while a launch runs are kept as their difference from those: every request that arrived is
+    // in the queue or was admitted, left or was turned away; one that was admitted is in prefill or has finished it; one that was
+    // placed decodes or is done.  (Class lanes; `back` at the end of the launch.)
+    __device__ __forceinline__ void derived_counters(bool back)
+    {
+        ClassState &c = cs[lane];
+        const unsigned long long in_prefill = c.X + c.prefill_done, m = c.Ym + c.done_mixed, so = c.Ys + c.done_solo;
+        const unsigned long long admitted = back ? c.admitted + in_prefill : c.admitted;
+        const unsigned long long arrived = c.pq_n + admitted + c.abandoned_p + c.overflow;
+        c.admitted += back ? in_prefill : 0ull - in_prefill;
+        c.arrivals += back ? arrived : 0ull - arrived;
+        c.placed_mixed += back ? m : 0ull - m;
+        c.placed_solo += back ? so : 0ull - so;
     }
 
     // Class lanes of the master: add every warp's accounting of finished requests to the class records.
@@ -1451,105 +1605,98 @@ struct Sim {
     }
 
     // --- calendar of iteration ends (CAL) ---------------------------------------------------------------
-    // Time is cut into buckets of equal width; bkt[g] holds the bucket of GPU g's pending iteration end modulo cal_nbk (255:
-    // none, or held by a lane), and no iteration is longer than cal_nbk - 2 buckets, so an id names one bucket.  The warp
-    // works through the buckets in order: load_bucket finds the GPUs of a bucket by comparing four ids per word and gives
-    // each to a lane that holds none; rounds then look at the lanes only.  A round used to read all N GPUs twice (37 % of a
-    // replication's time at N = 512: N/32 rows of dependent shared-memory reads); now N ids are read once per bucket.
-    // The next bucket is loaded as soon as enough lanes are free, so that the next event that is not local is usually
-    // among the held ends.  Invariant: every pending event lies in bucket `low` or later, so an iteration that starts now
-    // ends cal_K = floor(tau_min / width) buckets after `low` or later, and buckets up to low + cal_K - 1 may be loaded.
-    // cal_K = 0 (iterations shorter than a bucket): one bucket at a time, reloaded in every round under the tau_min limit.
+    // Time is cut into buckets of equal width.  The GPUs whose iterations end in a bucket form CAL_CHAINS linked lists (a new end is
+    // put at the front with one atomic exchange; a lane follows each list), and no iteration is longer than cal_nbk - 2
+    // buckets, so a list holds the ends of one bucket only.  The warp works through the buckets in order: load_bucket gives
+    // the GPUs of a bucket to lanes that hold none; rounds then look at the lanes only.  The next bucket is loaded as soon as
+    // enough lanes are free, so that the next event that is not local is usually among the held ends.  Invariant: every pending
+    // event lies in bucket cur - lead or later, so an iteration that starts now ends cal_K = floor(tau_min / width) >= 1
+    // buckets after that one or later, and the bucket after `cur` may be loaded while lead + 1 < cal_K.
     __device__ __forceinline__ unsigned long long bucket_abs(double x) const { return __double2ull_rd(__dmul_rn(x, p.cal_inv_w)); }
-    __device__ __forceinline__ uint8_t bucket_id(double x) const { return (uint8_t)((uint32_t)bucket_abs(x) & (p.cal_nbk - 1u)); }
-    // bytes of w equal to the byte repeated in pat: 0x80 in each
-    static __device__ __forceinline__ uint32_t equal_bytes(uint32_t w, uint32_t pat)
+    __device__ __forceinline__ void file_end(uint32_t g, double te)
     {
-        const uint32_t x = w ^ pat;
-        return ~(((x & 0x7f7f7f7fu) + 0x7f7f7f7fu) | x) & 0x80808080u;
+        const uint32_t b = (uint32_t)bucket_abs(te) & (p.cal_nbk - 1u);
+        cal_next[g] = (uint16_t)atomicExch(&cal_head[b * CAL_CHAINS + (g & (CAL_CHAINS - 1u))], g);
     }
 
-    // Give the pending ends of bucket b to the free lanes; returns how many there are (nothing is taken when there are more
-    // than free lanes).
-    __device__ __forceinline__ uint32_t load_bucket(unsigned long long b, uint32_t free_lanes)
+    // Give the GPUs whose ends lie in bucket b to the free lanes (mine: this lane's, or NONE32); returns how many there are (nothing
+    // is taken when there are more than free lanes).
+    __device__ __forceinline__ uint32_t load_bucket(unsigned long long b, uint32_t free_lanes, uint32_t &mine)
     {
-        const uint32_t *words = reinterpret_cast<const uint32_t *>(bkt);
-        const uint32_t nw = (p.N + 127u) >> 7, pat = ((uint32_t)b & (p.cal_nbk - 1u)) * 0x01010101u, below = (1u << lane) - 1u;
-        uint32_t n = 0;
-        // eight words of ids per lane at a time: the matches of word c become bits 7 - c, 15 - c, 23 - c, 31 - c of one mask
+        const uint32_t below = (1u << lane) - 1u;
+        uint32_t *head = cal_head + ((uint32_t)b & (p.cal_nbk - 1u)) * CAL_CHAINS + (uint32_t)lane;
+        uint32_t n = 0, g = (uint32_t)lane < CAL_CHAINS ? *head : CAL_NONE;
 #pragma unroll 1
-        for (uint32_t c0 = 0; c0 < nw; c0 += 8u) {
-            uint32_t m = 0;
-#pragma unroll
-            for (uint32_t c = 0; c < 8u; ++c)
-                if (c0 + c < nw) m |= equal_bytes(words[((c0 + c) << 5) + (uint32_t)lane], pat) >> c;
-            for (uint32_t k = __ballot_sync(FULL, m != 0); k; k = __ballot_sync(FULL, m != 0)) {
-                const uint32_t pos = n + (uint32_t)__popc(k & below), bit = (uint32_t)__ffs((int)m) - 1u;
-                if (m && pos < 32u) picked[pos] = (uint16_t)((((c0 + 7u - (bit & 7u)) << 5) + (uint32_t)lane) * 4u + (bit >> 3));
-                m &= m - 1u;
-                n += (uint32_t)__popc(k);
+        for (uint32_t k = __ballot_sync(FULL, g != CAL_NONE); k && n <= 32u; k = __ballot_sync(FULL, g != CAL_NONE)) {
+            const uint32_t pos = n + (uint32_t)__popc(k & below);
+            n += (uint32_t)__popc(k);
+            if (g != CAL_NONE) {
+                if (pos < 32u) picked[pos] = (uint16_t)g;
+                g = cal_next[g];
             }
         }
         if (n == 0 || n > (uint32_t)__popc(free_lanes)) return n;
+        if ((uint32_t)lane < CAL_CHAINS) *head = CAL_NONE;
         __syncwarp();
         const uint32_t rank = (uint32_t)__popc(free_lanes & below);
-        if (!held && rank < n) {
-            const uint32_t g = (uint32_t)picked[rank];
-            // (with 256 buckets id 255 is one, and idle GPUs and those that lanes hold match it)
-            const unsigned long long v = g < p.N ? (unsigned long long)__double_as_longlong(tnext[g]) : 0x7ff0000000000000ull;
-            if (v < 0x7ff0000000000000ull && bucket_abs(__longlong_as_double((long long)v)) == b) {
-                held = true; held_g = g; held_t = v;
-                if (p.cal_K > 0) bkt[g] = (uint8_t)255;
-            }
-        }
+        if (!held && rank < n) mine = (uint32_t)picked[rank];
         __syncwarp();
         return n;
     }
+    // This lane holds GPU g's pending end.  What the end will read from memory is asked for now, rounds before it is needed: the
+    // request whose prefill it finishes; the stamps of the decodes when one of them finishes.
+    __device__ __forceinline__ void hold(uint32_t g)
+    {
+        held = true; held_g = g;
+        held_t = (unsigned long long)__double_as_longlong(tnext[g]);
+        const uint32_t na = nact[g];
+        held_na = na;
+        if (na & 0x8000u) { held_pk = pfjob[g]; held_tarr = pf_tarr[g]; }
+        if ((na & 0x4000u) && !f_slots()) {
+            const uint32_t nd = ndec[g];
+            const char *a = reinterpret_cast<const char *>(s_fin + (size_t)g * p.B);
+#pragma unroll 1
+            for (uint32_t o = 0; o < nd * 4u; o += 128u) asm volatile("prefetch.global.L2 [%0];" :: "l"(a + o));
+            asm volatile("prefetch.global.L2 [%0];" :: "l"(s_rec + (size_t)g * p.B + (nd - 1u)));
+        }
+    }
 
-    // More ends in bucket `cur` than lanes (many GPUs that started together; no lane holds anything): each lane holds the
-    // earliest of the GPUs whose ids it reads, and the earliest end that no lane holds limits the round.
-    __device__ void load_crowded()
+    // More ends in bucket `cur` than lanes (many GPUs that started together), or ends that are in no list: each lane gets the
+    // earliest of its GPUs that ends in the bucket, and the earliest end that no lane holds limits the round.
+    __device__ __forceinline__ uint32_t load_crowded()
     {
         const unsigned long long INF = 0x7ff0000000000000ull;
-        const uint32_t *words = reinterpret_cast<const uint32_t *>(bkt);
-        const uint32_t nw = (p.N + 127u) >> 7, pat = ((uint32_t)cur & (p.cal_nbk - 1u)) * 0x01010101u;
-        held = false; held_t = INF; held_g = 0; left_t = INF; left_s = NONE32;
+        if ((uint32_t)lane < CAL_CHAINS) cal_head[((uint32_t)cur & (p.cal_nbk - 1u)) * CAL_CHAINS + (uint32_t)lane] = CAL_NONE;
+        unsigned long long first = INF;
+        uint32_t mine = NONE32;
+        held = false; held_t = INF; held_g = 0;
+        unsigned long long left_t = INF;
+        uint32_t left_s = NONE32;
 #pragma unroll 1
-        for (uint32_t c = 0; c < nw; ++c)
-            for (uint32_t m = equal_bytes(words[(c << 5) + (uint32_t)lane], pat); m; m &= m - 1u) {
-                const uint32_t g = (((c << 5) + (uint32_t)lane) << 2) + (((uint32_t)__ffs((int)m) - 1u) >> 3);
-                if (g >= p.N) break;
-                const unsigned long long v = (unsigned long long)__double_as_longlong(tnext[g]);
-                if (v == INF || bucket_abs(__longlong_as_double((long long)v)) != cur) continue;
-                if (!held || v < held_t) {          // (a lane's GPUs come in index order: the first of equal ends stays)
-                    if (held) { left_t = held_t; left_s = SRC_SERVER + held_g; }
-                    held = true; held_t = v; held_g = g;
-                } else if (v < left_t) { left_t = v; left_s = SRC_SERVER + g; }
-            }
-        __syncwarp();
+        for (uint32_t g = (uint32_t)lane; g < p.N; g += 32u) {
+            const unsigned long long v = (unsigned long long)__double_as_longlong(tnext[g]);
+            if (v == INF || bucket_abs(__longlong_as_double((long long)v)) != cur) continue;
+            if (v < first) {          // (a lane's GPUs come in index order: the first of equal ends stays)
+                if (first < INF) { left_t = first; left_s = SRC_SERVER + mine; }
+                first = v; mine = g;
+            } else if (v < left_t) { left_t = v; left_s = SRC_SERVER + g; }
+        }
+        crowded = __any_sync(FULL, left_t < INF);
         const uint32_t hi = (uint32_t)(left_t >> 32), lo = (uint32_t)left_t;
         const uint32_t mhi = __reduce_min_sync(FULL, hi), mlo = __reduce_min_sync(FULL, hi == mhi ? lo : NONE32);
         left_s = __reduce_min_sync(FULL, (hi == mhi && lo == mlo) ? left_s : NONE32);
-        left_t = ((unsigned long long)mhi << 32) | mlo;
+        if (lane == 0) { left[0] = ((unsigned long long)mhi << 32) | mlo; left[1] = left_s; }
+        __syncwarp();
+        return mine;
     }
 
     // Buckets from `cur` to the next one with a pending iteration end (a large number when no GPU runs).
     __device__ __forceinline__ uint32_t next_bucket() const
     {
         uint32_t best = 0x7fffffffu;
-        const uint32_t *words = reinterpret_cast<const uint32_t *>(bkt);
-        const uint32_t nw = (p.N + 127u) >> 7, mask = p.cal_nbk - 1u;
 #pragma unroll 1
-        for (uint32_t c = 0; c < nw; ++c) {
-            uint32_t w = words[(c << 5) + (uint32_t)lane];
-#pragma unroll
-            for (uint32_t j = 0; j < 4; ++j, w >>= 8) {
-                const uint32_t id = w & 0xffu;
-                const uint32_t g = (((c << 5) + (uint32_t)lane) << 2) + j;
-                // 255 is a bucket as well when there are 256 of them: only the GPU's end time tells
-                if (id != 255u || (mask == 255u && g < p.N && tnext[g] < dinf())) best = min(best, (id - (uint32_t)cur) & mask);
-            }
-        }
+        for (uint32_t c = (uint32_t)lane; c < p.cal_nbk * CAL_CHAINS; c += 32u)
+            if (cal_head[c] != CAL_NONE) best = min(best, (c / CAL_CHAINS - (uint32_t)cur) & (p.cal_nbk - 1u));
         return __reduce_min_sync(FULL, best);
     }
 
@@ -1558,21 +1705,23 @@ struct Sim {
     {
         unsigned long long first = 0x7ff0000000000000ull;
 #pragma unroll 1
-        for (uint32_t g = (uint32_t)lane; g < ((p.N + 127u) & ~127u); g += 32u) {
-            const double x = g < p.N ? tnext[g] : dinf();
-            bkt[g] = x < dinf() ? bucket_id(x) : (uint8_t)255;
-            first = min(first, (unsigned long long)__double_as_longlong(x));
-        }
+        for (uint32_t c = (uint32_t)lane; c < p.cal_nbk * CAL_CHAINS; c += 32u) cal_head[c] = CAL_NONE;
+#pragma unroll 1
+        for (uint32_t g = (uint32_t)lane; g < p.N; g += 32u) first = min(first, (unsigned long long)__double_as_longlong(tnext[g]));
         if (lane < (int)p.I) first = min(first, class_first());
         if (f_blocks() && lane == 0) first = min(first, (unsigned long long)__double_as_longlong(T_blk_next));
         const uint32_t hi = (uint32_t)(first >> 32), mhi = __reduce_min_sync(FULL, hi);
         const uint32_t mlo = __reduce_min_sync(FULL, hi == mhi ? (uint32_t)first : NONE32);
-        cur_end = bucket_abs(T_end);
-        cur = mhi >= 0x7ff00000u ? cur_end : bucket_abs(__longlong_as_double((long long)(((unsigned long long)mhi << 32) | mlo)));
-        low = cur;
-        held = false; held_t = 0x7ff0000000000000ull; held_g = 0;
-        left_t = held_t; left_s = NONE32;
-        crowded = true;      // the first round loads the bucket
+        cur = mhi >= 0x7ff00000u ? bucket_abs(T_end) : bucket_abs(__longlong_as_double((long long)(((unsigned long long)mhi << 32) | mlo)));
+        lead = 0;
+        held = false; held_t = 0x7ff0000000000000ull; held_g = 0; held_na = 0; held_pk = 0; held_tarr = 0.0;
+        crowded = true;      // the first round finds the ends of this bucket by looking at all GPUs
+        __syncwarp();
+#pragma unroll 1
+        for (uint32_t g = (uint32_t)lane; g < p.N; g += 32u) {
+            const double x = tnext[g];
+            if (x < dinf() && bucket_abs(x) != cur) file_end(g, x);
+        }
         __syncwarp();
     }
     // earliest clock of this lane's class
@@ -1588,22 +1737,23 @@ struct Sim {
         return v;
     }
 
-    // The round loop on the calendar: as run(), with the lanes' held ends in the place of all GPUs.  Measured against the scan
-    // of all rows in every round (N = 512, R = 4096, 250 iterations of horizon): 955 -> 708 ms, and 623 ms with the cached
-    // least-loaded keys, the gate by reductions, accounting 32 requests at a time and a smaller loop body.
+    // The round loop on the calendar: as run(), with the lanes' held ends in the place of all GPUs.
+    // Bound: the chain of dependent instructions of each replication, about 1500 a round, and fetching them.  Measured at N = 512,
+    // R = 4096, 250 iterations of horizon: 955 ms reading all rows in every round, 594 with a byte per GPU that names its bucket
+    // and is searched for every bucket, 563 with lists per bucket, one memory round trip per retirement and no registers
+    // spilled (8 bytes spilled in the loop cost 20 %: the L1 next to 200 KB of shared memory is too small for them).
+    // N = 4096, R = 1712: 698 -> 579 ms.  Cycles a warp waits for instructions, per instruction: 2.5 -> 1.2 of 9.1 -> 8.2.
     __device__ bool run_calendar()
     {
-        unsigned long long budget = p.event_budget;
+        const uint32_t budget = (uint32_t)min(p.event_budget, BUDGET_MAX);
         const unsigned long long INF = 0x7ff0000000000000ull;
         const unsigned long long tend_bits = (unsigned long long)__double_as_longlong(T_end);
-        const bool tight = p.cal_K == 0;
         uint32_t want = CAL_FREE;        // free lanes to load another bucket
         calendar_build();
         for (;;) {
             const unsigned long long cur0 = cur;
             __syncwarp();
-            for (uint32_t need = __ballot_sync(FULL, sched_pending); need; need &= need - 1)
-                refill((uint32_t)__ffs((int)need) - 1u);
+            replenish();
             unsigned long long bt = INF;
             uint32_t bs = NONE32;
             bool arrival_due = false;        // an arrival that only joins its queue is pending up to T_end
@@ -1622,19 +1772,19 @@ struct Sim {
                     if (v < bt) { bt = v; bs = SRC_ABD1 + lane; }
                 }
             }
-            // Load buckets (one copy of the code for every reason to): the current one again when it is crowded or an end may
-            // have been added to it; the next one that holds an event when no lane holds an end any more; the following one
-            // when enough lanes are free.
-            bool again = tight || crowded;
-            if (again) { held = false; held_t = INF; held_g = 0; }
+            // Load buckets (one copy of the code for every reason to): the current one again when it is crowded; the next one that
+            // holds an event when no lane holds an end any more; the following one when enough lanes are free.
+            bool look = crowded;
             uint32_t turn = 0, d = 0;
 #pragma unroll 1
             for (;;) {
                 const uint32_t free_lanes = ~__ballot_sync(FULL, held);
-                uint32_t ahead = 0;
-                if (again) {
-                    again = false;
-                } else if (free_lanes == FULL) {
+                uint32_t ahead = 0, mine = NONE32, n = 0;
+                const bool all = look;
+                look = false;
+                if (all) {
+                    mine = load_crowded();
+                } else if (free_lanes == FULL && !crowded) {
                     if (turn == 0) {
                         // buckets to the first class event or block end
                         unsigned long long first = bt;
@@ -1660,31 +1810,30 @@ struct Sim {
                             if (first > tend_bits) return true;
                             cur = bucket_abs(__longlong_as_double((long long)first));
                         } else {
-                            if (cur + skip > cur_end) return true;      // nothing left up to T_end
+                            if (cur + skip > bucket_abs(T_end)) return true;      // nothing left up to T_end
                             if (skip == 0) break;
                             cur += skip;
                         }
                         d = 0;
                     }
-                    low = cur;
+                    lead = 0;
                     want = CAL_FREE;
                     ++turn;
                 } else {
-                    if (turn || crowded || (uint32_t)__popc(free_lanes) < want || cur + 1u >= low + p.cal_K) break;
+                    if (turn || crowded || (uint32_t)__popc(free_lanes) < want || lead + 1u >= p.cal_K) break;
                     ahead = 1;
                 }
-                const uint32_t n = load_bucket(cur + ahead, free_lanes);
+                if (!all) n = load_bucket(cur + ahead, free_lanes, mine);
+                if (mine != NONE32) hold(mine);
                 if (ahead) {
-                    if (n <= (uint32_t)__popc(free_lanes)) { ++cur; want = CAL_FREE; }
+                    if (n <= (uint32_t)__popc(free_lanes)) { ++cur; ++lead; want = CAL_FREE; }
                     else want = min(n, 32u);            // (more than 32: it has to wait until no lane holds anything)
                     break;
                 }
-                left_t = INF; left_s = NONE32;
-                crowded = n > 32u;
-                if (crowded) load_crowded();
+                look = n > 32u;
             }
             const bool buffered = (dq_n0 | dq_n1) != 0;
-            const uint32_t na = nact[held_g], nd0 = ndec[held_g];
+            const uint32_t na = held_na, nd0 = ndec[held_g];
             const bool nl = force_nonlocal || (na & 0x8000u) != 0 || ((na & 0x4000u) != 0 && (buffered || (held_g < M && nd0 > p.B - 1)));
             if (held && nl && held_t < bt) { bt = held_t; bs = SRC_SERVER + held_g; }
             unsigned long long tint;
@@ -1696,25 +1845,17 @@ struct Sim {
                 src = __reduce_min_sync(FULL, (hi == mhi && lo == mlo) ? bs : NONE32);
                 tint = ((unsigned long long)mhi << 32) | mlo;
             }
-            if (cur >= cur_end && tint > tend_bits && !__any_sync(FULL, arrival_due || held_t <= tend_bits) && left_t > tend_bits) return true;
-            if (budget == 0) return false;
-            --budget;
+            const unsigned long long left_t = crowded ? left[0] : INF;
+            if (tint > tend_bits && left_t > tend_bits && cur >= bucket_abs(T_end) && !__any_sync(FULL, arrival_due || held_t <= tend_bits)) return true;
+            if (rounds == budget) return false;
             ++rounds;
             // a class event further ahead waits until its bucket is the current one
             const bool here = tint < INF && (src >= SRC_SERVER || bucket_abs(__longlong_as_double((long long)tint)) <= cur);
             unsigned long long lim_t = here ? tint : INF;
             uint32_t lim_s = here ? src : NONE32;
-            if (left_t < lim_t || (left_t == lim_t && left_s < lim_s)) { lim_t = left_t; lim_s = left_s; }
-            if (tight) {
-                // no iteration that starts in this round can end before T_min + tau_min
-                unsigned long long tmin = held_t;
-                if (lane < (int)p.I) tmin = min(tmin, (unsigned long long)__double_as_longlong(cs[lane].ta));
-                const uint32_t hi = (uint32_t)(tmin >> 32), mhi = __reduce_min_sync(FULL, hi);
-                const uint32_t mlo = __reduce_min_sync(FULL, hi == mhi ? (uint32_t)tmin : NONE32);
-                if (mhi < 0x7ff00000u) {
-                    const unsigned long long wt = (unsigned long long)__double_as_longlong(__dadd_rn(__hiloint2double((int)mhi, (int)mlo), tau_min));
-                    if (wt <= lim_t) { lim_t = wt; lim_s = 0; }
-                }
+            if (crowded) {
+                const uint32_t left_s = (uint32_t)left[1];
+                if (left_t < lim_t || (left_t == lim_t && left_s < lim_s)) { lim_t = left_t; lim_s = left_s; }
             }
             const bool first_is_event = here && lim_t == tint && lim_s == src;      // nothing that is not held or could still start comes before it
             if (tend_bits < lim_t) { lim_t = tend_bits; lim_s = NONE32; }
@@ -1730,7 +1871,10 @@ struct Sim {
                     const unsigned long long v = (unsigned long long)__double_as_longlong(c.ta);
                     if (local) {
                         if (!(v < lim_t || (v == lim_t && SRC_ARRIVAL + (uint32_t)lane < lim_s))) break;
-                        if (f_abandon() && v > (unsigned long long)__double_as_longlong(c.abp.t_ab)) break;
+                        if (f_abandon()) {
+                            if (stale & 1u) { cs[lane].abp.t_ab = ab_next_call(cs[lane].abp, aim[lane].theta, cs[lane].pq_n); stale &= ~1u; }
+                            if (v > (unsigned long long)__double_as_longlong(c.abp.t_ab)) break;
+                        }
                         if (bucket_abs(__longlong_as_double((long long)v)) > cur) break;
                     } else if (!(arrival_now && src == SRC_ARRIVAL + (uint32_t)lane && guard == 0)) break;
                     if (guard == ARRIVALS_PER_ROUND) { redo = true; break; }
@@ -1739,18 +1883,15 @@ struct Sim {
                 }
             }
             redo = redo || (sched_pending && !arrival_now);
-            if (f_abandon() && lane < (int)p.I) {
-                const unsigned long long v = (unsigned long long)__double_as_longlong(cs[lane].abp.t_ab);
-                redo = redo || v < tint || (v == tint && SRC_ABP + (uint32_t)lane < src);
-            }
+            if (f_abandon() && lane < (int)p.I) redo = redo || abandons_before(tint, src);
             const bool any_redo = __any_sync(FULL, redo);
             const bool do_event = !any_redo && first_here;
-            const uint32_t nd_ev = src >= SRC_SERVER && do_event ? (uint32_t)ndec[src - SRC_SERVER] : 0u;
             // the held ends below the limit and, if it happens now, the event's end
             const unsigned long long v = held_t;
             const uint32_t g = held_g;
             const bool evt = do_event && held && SRC_SERVER + g == src;
             const bool act = evt || (held && !nl && (v < lim_t || (v == lim_t && SRC_SERVER + g < lim_s)));
+            const uint32_t ev_lane = __ballot_sync(FULL, evt);       // the lane that holds the event's end, if it is one
             const bool retire = local_end(g, __longlong_as_double((long long)v), act, evt);
             if (act) { held = false; held_t = INF; progressed = true; }
             uint32_t need = __ballot_sync(FULL, retire);
@@ -1767,9 +1908,10 @@ struct Sim {
             }
             if (do_event) {
                 t = __longlong_as_double((long long)tint);
-                low = max(low, bucket_abs(t));
+                lead = min(lead, (uint32_t)(cur - min(cur, bucket_abs(t))));
                 if (src >= SRC_SERVER) {
-                    on_server(src - SRC_SERVER, nd_ev);
+                    const int l = __ffs((int)ev_lane) - 1;
+                    on_server(src - SRC_SERVER, __shfl_sync(FULL, nd0, l), __shfl_sync(FULL, na, l), __shfl_sync(FULL, held_pk, l), __shfl_sync(FULL, held_tarr, l));
                 } else {
                     if (f_abandon() && src >= SRC_ABP) on_abandon((src - SRC_ABP) >> 3, (src - SRC_ABP) & 7u);
                     else if (src >= SRC_ARRIVAL) gate_dirty = true;
@@ -1788,15 +1930,13 @@ struct Sim {
     // --- round loop ----------------------------------------------------------------------------------
     __device__ bool run()
     {
-        unsigned long long budget = p.event_budget;
+        const uint32_t budget = (uint32_t)min(p.event_budget, BUDGET_MAX);
         const uint32_t rows = n_rows();
         const unsigned long long INF = 0x7ff0000000000000ull;
         const unsigned long long tend_bits = (unsigned long long)__double_as_longlong(T_end);
         for (;;) {
             __syncwarp();
-            // classes that ran out of arrival draws get 32 new ones
-            for (uint32_t need = __ballot_sync(FULL, sched_pending); need; need &= need - 1)
-                refill((uint32_t)__ffs((int)need) - 1u);
+            replenish();
             // next non-local event of this lane (sources scanned in id order with '<' keep the tie order);
             // an arrival is local while no prefill slot is idle: it only joins its class queue
             unsigned long long bt = INF, tmin = INF;
@@ -1851,8 +1991,7 @@ struct Sim {
                 warp_keys(bt, bs, tmin, tint, src, tmin_all);
             }
             if (tint > tend_bits && tmin_all > tend_bits) return true;     // nothing left up to T_end
-            if (budget == 0) return false;
-            --budget;
+            if (rounds == budget) return false;
             ++rounds;
             // no iteration that starts in this round can end before T_min + tau_min
             unsigned long long wt = INF;
@@ -1881,7 +2020,10 @@ struct Sim {
                     const unsigned long long v = (unsigned long long)__double_as_longlong(c.ta);
                     if (local) {
                         if (!(v < lim_t || (v == lim_t && SRC_ARRIVAL + (uint32_t)lane < lim_s))) break;
-                        if (f_abandon() && v > (unsigned long long)__double_as_longlong(c.abp.t_ab)) break;
+                        if (f_abandon()) {
+                            if (stale & 1u) { cs[lane].abp.t_ab = ab_next_call(cs[lane].abp, aim[lane].theta, cs[lane].pq_n); stale &= ~1u; }
+                            if (v > (unsigned long long)__double_as_longlong(c.abp.t_ab)) break;
+                        }
                     } else if (!(arrival_now && src == SRC_ARRIVAL + (uint32_t)lane && guard == 0)) break;
                     if (guard == ARRIVALS_PER_ROUND) { redo = true; break; }
                     arrival_local();
@@ -1892,10 +2034,7 @@ struct Sim {
             // the loop has a known one, and a local arrival may have pulled its class's next abandonment before T_int: then T_int
             // is not next after all
             redo = redo || (sched_pending && !arrival_now);
-            if (f_abandon() && lane < (int)p.I) {
-                const unsigned long long v = (unsigned long long)__double_as_longlong(cs[lane].abp.t_ab);
-                redo = redo || v < tint || (v == tint && SRC_ABP + (uint32_t)lane < src);
-            }
+            if (f_abandon() && lane < (int)p.I) redo = redo || abandons_before(tint, src);
             // the non-local event happens in this round if it comes before anything a new iteration could bring
             const bool any_redo = __any_sync(FULL, redo);
             const bool do_event = !any_redo && first_here;
@@ -1953,7 +2092,7 @@ struct Sim {
             if (do_event) {
                 t = __longlong_as_double((long long)tint);
                 if (src >= SRC_SERVER) {
-                    on_server(src - SRC_SERVER, nd_ev);
+                    on_server(src - SRC_SERVER, nd_ev, SPL > 0 ? (uint32_t)nact[src - SRC_SERVER] : 0u, 0u, 0.0);
                 } else {
                     if (f_abandon() && src >= SRC_ABP) on_abandon((src - SRC_ABP) >> 3, (src - SRC_ABP) & 7u);
                     else if (src >= SRC_ARRIVAL) gate_dirty = true;
@@ -1985,14 +2124,14 @@ struct Sim {
 // shared-memory carve-up for one replication (one warp per block)
 struct SmemLayout {
     uint32_t off_tnext, off_tarr, off_it, off_nfin, off_pfrem, off_pfjob, off_K, off_Kpend, off_ndec, off_nact,
-        off_pfcur, off_sfin16, off_socc, img_sfin16, img_socc, srv_bytes, off_bkt, off_picked, off_touch, off_cs, off_ring, off_strec, off_stte, off_pqh, off_wcs, off_cmd, off_res, total;
+        off_pfcur, off_sfin16, off_socc, img_pfcur, img_pfrem, img_sfin16, img_socc, srv_bytes, off_head, off_next, off_picked, off_rows, off_left, off_cs, off_ring, off_ringpk, off_strec, off_stte, off_pqh, off_aim, off_wcs, off_cmd, off_res, total;
 };
 
 // tarr_global: the arrival times and the job words of the requests in prefill (read once per finished prefill) live in
 // global memory (large clusters: shared memory is what limits the resident replications there); I: classes (sizes the
 // class records and the ring of arrival draws)
 __host__ __device__ inline SmemLayout smem_layout(uint32_t N, uint32_t Npad, uint32_t B, uint32_t slots_smem, uint32_t nwarps, bool kappa,
-                                                  bool tarr_global, uint32_t I, bool cal)
+                                                  bool tarr_global, uint32_t I, uint32_t cal_nbk)
 {
     SmemLayout L;
     uint32_t o = 0;
@@ -2005,30 +2144,38 @@ __host__ __device__ inline SmemLayout smem_layout(uint32_t N, uint32_t Npad, uin
     L.off_Kpend = o; if (kappa) o += 4 * Npad;
     L.off_ndec = o; o += 2 * Npad;
     L.off_nact = o; o += 2 * Npad;
-    L.off_pfcur = o; o += 2 * Npad;
-    L.off_pfrem = o; o += 2 * Npad;
-    o = (o + 15u) & ~15u;
+    // (with the calendar the chunk of the running iteration follows from its batch word: the image has it, the chip does not)
+    const bool cal = cal_nbk > 0;
+    L.off_pfcur = L.img_pfcur = o;
+    L.img_pfrem = o + 2 * Npad;
+    L.off_pfrem = cal ? o : L.img_pfrem;
+    o = (o + 4 * Npad + 15u) & ~15u;
     // the slot arrays of the image cover the padded GPUs; on chip only the N real ones have any (N = 16, B = 256: 16 KB of shared
     // memory instead of 24, which is 12 resident replications per SM instead of 9)
     const uint32_t words = (B + 31u) >> 5;
     L.img_sfin16 = o;
-    L.img_socc = (o + (slots_smem ? 2 * Npad * B : 0u) + 15u) & ~15u;
+    if (cal) o = (L.off_pfrem + 2 * Npad + 15u) & ~15u;
+    L.img_socc = (L.img_sfin16 + (slots_smem ? 2 * Npad * B : 0u) + 15u) & ~15u;
     L.srv_bytes = (L.img_socc + (slots_smem ? 4 * Npad * words : 0u) + 15u) & ~15u;
     L.off_sfin16 = o; if (slots_smem) o += 2 * N * B;
     o = (o + 15u) & ~15u;
     L.off_socc = o; if (slots_smem) o += 4 * N * words;
     o = (o + 15u) & ~15u;
-    L.off_bkt = o; if (cal) o += (Npad + 127u) & ~127u;       // calendar of iteration ends
+    L.off_head = o; o += 4 * CAL_CHAINS * cal_nbk;       // calendar of iteration ends
+    L.off_next = o; if (cal) o += 2 * Npad;
     L.off_picked = o; if (cal) o += 2 * 32;
-    L.off_touch = o; o += 4 * TOUCH_CAP;
+    L.off_rows = o; if (cal) o += 3 * 4 * (Npad >> 5);
     o = (o + 15u) & ~15u;
+    L.off_left = o; if (cal) o += 16;
     L.off_cs = o; o += (uint32_t)sizeof(ClassState) * I;
     o = (o + 15u) & ~15u;
-    L.off_ring = o; o += (uint32_t)sizeof(ADraw) * 32 * I;
+    L.off_ring = o; o += 8 * 32 * I;
+    L.off_ringpk = o; o += 4 * 32 * I;
     const uint32_t stage = slots_smem ? STAGE_CAP : (nwarps == 1 ? ROW_STAGE_CAP : 0);
     L.off_strec = o; o += (uint32_t)sizeof(SlotRec) * stage;
     L.off_stte = o; o += 8 * stage;
-    L.off_pqh = o; o += (uint32_t)sizeof(QEntry) * MAXI;
+    L.off_pqh = o; o += (uint32_t)sizeof(QEntry) * I;
+    L.off_aim = o; o += (uint32_t)sizeof(ClassAim) * I;
     L.off_wcs = o; o += (uint32_t)sizeof(WarpClassStats) * I * nwarps;
     o = (o + 15u) & ~15u;
     L.off_cmd = o; if (nwarps > 1) o += (uint32_t)sizeof(MwCmd);        // master and helpers only
@@ -2054,20 +2201,28 @@ __device__ __forceinline__ void bind_pointers(Sim<SPL, F> &s, char *sm, const Sm
     s.pfcur = reinterpret_cast<uint16_t *>(sm + L.off_pfcur);
     s.sfin16 = reinterpret_cast<uint16_t *>(sm + L.off_sfin16);
     s.socc = reinterpret_cast<uint32_t *>(sm + L.off_socc);
-    s.bkt = reinterpret_cast<uint8_t *>(sm + L.off_bkt);
+    s.cal_head = reinterpret_cast<uint32_t *>(sm + L.off_head);
+    s.cal_next = reinterpret_cast<uint16_t *>(sm + L.off_next);
     s.picked = reinterpret_cast<uint16_t *>(sm + L.off_picked);
-    s.touch = reinterpret_cast<uint32_t *>(sm + L.off_touch);
+    s.row_key = reinterpret_cast<uint32_t *>(sm + L.off_rows);
+    s.left = reinterpret_cast<unsigned long long *>(sm + L.off_left);
     s.cs = reinterpret_cast<ClassState *>(sm + L.off_cs);
-    s.aring = reinterpret_cast<ADraw *>(sm + L.off_ring);
+    s.aring = reinterpret_cast<double *>(sm + L.off_ring);
+    s.aring_pk = reinterpret_cast<uint32_t *>(sm + L.off_ringpk);
     s.st_rec = reinterpret_cast<SlotRec *>(sm + L.off_strec);
     s.st_te = reinterpret_cast<double *>(sm + L.off_stte);
     s.pqh = reinterpret_cast<QEntry *>(sm + L.off_pqh);
+    s.aim = reinterpret_cast<ClassAim *>(sm + L.off_aim);
     s.wcs = reinterpret_cast<WarpClassStats *>(sm + L.off_wcs);
     s.cmd = reinterpret_cast<MwCmd *>(sm + L.off_cmd);
     s.res = reinterpret_cast<MwRes *>(sm + L.off_res);
-    s.n_pend = 0;
+    s.n_pend = 0; s.has_late = false;
+    s.late_tpf = 0.0; s.late_pk = 0;
     s.rec_after = 0;
-    s.ring_n = 0; s.ring_pos = 0; s.sched_pending = false; s.t0_pending = 0.0;
+    s.ring_n = 0; s.ring_pos = 0; s.sched_pending = false;
+    s.ring_blk = NONE32; s.ring_end = dinf();
+    s.stale = 0; s.pools = 0; s.pools_due = false;
+    s.place_base = ~0ull; s.place_w = 0;
     const Params &p = s.p;
     const size_t r = s.rep;
     s.s_fin = p.slot_fin + r * (size_t)p.N * p.B;
@@ -2085,7 +2240,7 @@ __global__ void __launch_bounds__(32) qsim_init_kernel(Params p)
     extern __shared__ __align__(16) char sm[];
     const int lane = threadIdx.x;
     for (uint32_t rep = blockIdx.x; rep < p.R; rep += gridDim.x) {
-        const SmemLayout L = smem_layout(p.Npad, p.Npad, p.B, p.slots_smem, 1, p.coef[5] != 0.0, p.tarr_global != 0, p.I, false);       // (laid out as the image)
+        const SmemLayout L = smem_layout(p.Npad, p.Npad, p.B, p.slots_smem, 1, p.coef[5] != 0.0, p.tarr_global != 0, p.I, 0);       // (laid out as the image)
         Sim<SPLT, FT> s(p, lane, rep);
         bind_pointers(s, sm, L);
         __syncwarp();
@@ -2113,9 +2268,10 @@ __global__ void __launch_bounds__(32) qsim_init_kernel(Params p)
         __syncwarp();
         // first arrival of every class: ask for draws, let the warp fill the rings, give the unused draws back
         s.sched_pending = lane < (int)p.I && p.n_inject == 0;
-        s.t0_pending = 0.0;
+        if (lane < (int)p.I) s.aring[lane * 32] = 0.0;
+        __syncwarp();
         if (p.n_inject > 0 && lane < (int)p.I) s.schedule_from(0.0);
-        for (int guard = 0; guard < 64; ++guard) {
+        for (uint32_t guard = 0; guard < 64u + p.nblk * p.I; ++guard) {
             uint32_t need = __ballot_sync(FULL, s.sched_pending);
             if (!need) break;
             for (; need; need &= need - 1) s.refill((uint32_t)__ffs((int)need) - 1u);
@@ -2160,10 +2316,30 @@ __device__ __forceinline__ void copy16(char *sm, char *img, uint32_t bytes, uint
         else    *reinterpret_cast<uint4 *>(img + o) = *reinterpret_cast<const uint4 *>(sm + o);
     }
 }
-template <bool IN>
+template <bool IN, bool CAL>
 __device__ __forceinline__ void stage_image(char *sm, char *img, const SmemLayout &L, const Params &p, uint32_t tid, uint32_t nthr)
 {
-    copy16<IN>(sm, img, L.img_sfin16, tid, nthr);
+    copy16<IN>(sm, img, CAL ? L.img_pfcur : L.img_sfin16, tid, nthr);
+    if (CAL) {
+        // the prompt remainders, and the chunk in progress from or to the batch word
+        __syncwarp();
+        uint16_t *na = reinterpret_cast<uint16_t *>(sm + L.off_nact), *rem = reinterpret_cast<uint16_t *>(sm + L.off_pfrem);
+        uint16_t *cur = reinterpret_cast<uint16_t *>(img + L.img_pfcur), *irem = reinterpret_cast<uint16_t *>(img + L.img_pfrem);
+        uint16_t *ina = reinterpret_cast<uint16_t *>(img + L.off_nact);
+        const double *tn = reinterpret_cast<const double *>(sm + L.off_tnext);
+#pragma unroll 1
+        for (uint32_t g = tid; g < p.Npad; g += nthr) {
+            if (IN) {
+                rem[g] = irem[g];
+                if (cur[g] != 0) na[g] |= (uint16_t)BATCH_MIXED;
+            } else {
+                const uint32_t w = na[g];
+                irem[g] = rem[g];
+                cur[g] = tn[g] < dinf() && (w & BATCH_MIXED) ? (uint16_t)min(p.C, (uint32_t)rem[g]) : (uint16_t)0;
+                ina[g] = (uint16_t)(w & ~BATCH_MIXED);
+            }
+        }
+    }
     if (p.slots_smem) {
         copy16<IN>(sm + L.off_sfin16, img + L.img_sfin16, 2 * p.N * p.B, tid, nthr);
         copy16<IN>(sm + L.off_socc, img + L.img_socc, 4 * p.N * ((p.B + 31u) >> 5), tid, nthr);
@@ -2195,6 +2371,7 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, (FT & F_MW) ? 
     // which K successive launches would end, so the result is theirs: that of one launch, up to the order in which the
     // fp64 sums of finished requests are added to the totals.
     __shared__ uint32_t sh_unit[2];
+    __shared__ double sh_T_reset;
     const uint32_t K = p.nchunk > 1 ? p.nchunk : 1u;
     const uint32_t n_units = p.R * K;
     for (uint32_t unit = blockIdx.x;; unit += gridDim.x) {
@@ -2245,7 +2422,7 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, (FT & F_MW) ? 
                 continue;
             }
         } else if (!p.advance && h.done) continue;
-        const SmemLayout L = smem_layout(p.N, p.Npad, p.B, p.slots_smem, nthr >> 5, p.coef[5] != 0.0, p.tarr_global != 0, p.I, Sim<SPLT, FT>::CAL);
+        const SmemLayout L = smem_layout(p.N, p.Npad, p.B, p.slots_smem, nthr >> 5, p.coef[5] != 0.0, p.tarr_global != 0, p.I, Sim<SPLT, FT>::CAL ? p.cal_nbk : 0u);
         Sim<SPLT, FT> s(p, lane, rep);
         s.warp = warp;
         s.nwarps = (int)(nthr >> 5);
@@ -2253,7 +2430,7 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, (FT & F_MW) ? 
         s.block_sync();
         // stage state: per-GPU arrays (coalesced 16-byte copies) and the class records; clear the per-warp accounting
         char *const img = p.srv + (size_t)rep * p.srv_bytes;
-        stage_image<true>(sm, img, L, p, (uint32_t)tid, nthr);
+        stage_image<true, Sim<SPLT, FT>::CAL>(sm, img, L, p, (uint32_t)tid, nthr);
         {
             const uint4 *src = reinterpret_cast<const uint4 *>(h.cs);
             uint4 *dst = reinterpret_cast<uint4 *>(s.cs);
@@ -2268,13 +2445,16 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, (FT & F_MW) ? 
         if (advance == 1) T_end = __dmul_rn((double)H_total, iter_time(p, 0, p.B, 0));
         if (advance == 2) T_end = p.T_abs;
         s.T_end = T_end;
-        s.T_reset = h.T_reset;
+        s.block_sync();       // (every thread has read the old times)
+        if (tid == 0) { h.T_end = T_end; h.H_total = H_total; }
+        if (tid == 0) sh_T_reset = h.T_reset;
+        s.T_reset_at = &sh_T_reset;
         s.tau_min = fmin(p.coef[0], p.coef[3]);
         s.t = 0.0;
         s.load_block(h.blk);
-        s.dq_head0 = h.dq_head0; s.dq_head1 = h.dq_head1; s.dq_n0 = h.dq_n0; s.dq_n1 = h.dq_n1;
-        s.place_ord = h.place_ord; s.events = h.events; s.rounds = h.rounds; s.sel_ord0 = h.sel_ord0; s.sel_ord1 = h.sel_ord1;
-        s.n_touch = 0; s.touch_all = false; s.need_start = 0; s.err = h.err; s.direct = false;
+        s.dq_head0 = h.dq_head0; s.dq_head1 = h.dq_head1; s.dq_n0 = h.dq_n0; s.dq_n1 = s.f_sli() ? h.dq_n1 : 0u;
+        s.place_ord = h.place_ord; s.events = 0; s.rounds = 0; s.touch_g = 0; s.sel_ord0 = h.sel_ord0; s.sel_ord1 = h.sel_ord1;
+        s.n_touch = 0; s.touch_all = false; s.need_start = 0; s.err = h.err; s.direct = false; s.handed = false;
         s.drain_dirty = true; s.gate_dirty = true;
         s.force_nonlocal = (p.force_dispatch != 0 && chunk == 0) || h.force != 0;
         s.n_idle_pf = 0;
@@ -2282,16 +2462,17 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, (FT & F_MW) ? 
         s.it_mixed = 0; s.it_solo = 0; s.busy_mixed = 0.0; s.busy_solo = 0.0;
         bool finished = true;
         if (warp == 0) {
+            if (lane < (int)p.I) s.derived_counters(false);
             s.n_idle_pf = s.count_idle_pf();
             if (lane < (int)p.I && s.cs[lane].pq_n > 0) s.pqh[lane] = s.pq[(size_t)lane * p.qcap + s.cs[lane].pq_head];
             __syncwarp();
-            s.it_mixed = h.iters_mixed[lane]; s.it_solo = h.iters_solo[lane];
             s.busy_mixed = h.busy_mixed[lane]; s.busy_solo = h.busy_solo[lane];
             if constexpr (Sim<SPLT, FT>::CAL) {
                 finished = s.err ? true : s.run_calendar();
             } else {
                 finished = s.err ? true : s.run();
             }
+            s.stage_late();
             s.flush_done();
             if (FT & F_MW) {
                 if (lane == 0) s.cmd->op = MW_EXIT;
@@ -2302,10 +2483,11 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, (FT & F_MW) ? 
         }
         s.block_sync();
         s.merge_warp_stats();
+        if (warp == 0 && lane < (int)p.I) s.derived_counters(true);
         if (warp == 0 && lane < (int)p.I) s.cs[lane].adraw -= s.ring_n;     // unused arrival draws are produced again next time
         s.block_sync();
         // stage back
-        stage_image<false>(sm, img, L, p, (uint32_t)tid, nthr);
+        stage_image<false, Sim<SPLT, FT>::CAL>(sm, img, L, p, (uint32_t)tid, nthr);
         {
             uint4 *dst = reinterpret_cast<uint4 *>(h.cs);
             const uint4 *src = reinterpret_cast<const uint4 *>(s.cs);
@@ -2315,7 +2497,7 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, (FT & F_MW) ? 
         for (int w = 0; w < s.nwarps; ++w) {
             if (warp == w) {
                 if (w == 0) {
-                    h.iters_mixed[lane] = s.it_mixed; h.iters_solo[lane] = s.it_solo;
+                    h.iters_mixed[lane] += s.it_mixed; h.iters_solo[lane] += s.it_solo;
                     h.busy_mixed[lane] = s.busy_mixed; h.busy_solo[lane] = s.busy_solo;
                 } else {
                     h.iters_mixed[lane] += s.it_mixed; h.iters_solo[lane] += s.it_solo;
@@ -2326,10 +2508,13 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, (FT & F_MW) ? 
             if (FT & F_MW) { __threadfence_block(); __syncthreads(); }
         }
         if (tid == 0) {
-            h.T_end = T_end; h.H_total = H_total; h.blk = s.blk;
-            h.dq_head0 = s.dq_head0; h.dq_head1 = s.dq_head1; h.dq_n0 = s.dq_n0; h.dq_n1 = s.dq_n1;
-            h.place_ord = s.place_ord; h.events = s.events; h.rounds = s.rounds; h.err = s.err;
-            h.sel_ord0 = s.sel_ord0; h.sel_ord1 = s.sel_ord1;
+            if (s.f_blocks()) h.blk = s.blk;
+            // (what an instance does not change is not written: it would be carried in registers through the whole run)
+            h.dq_head0 = s.dq_head0; h.dq_n0 = s.dq_n0;
+            if (s.f_sli()) { h.dq_head1 = s.dq_head1; h.dq_n1 = s.dq_n1; }
+            if (s.f_random()) h.place_ord = s.place_ord;
+            h.events += s.events; h.rounds += s.rounds; h.err = s.err;
+            if (s.f_slig()) { h.sel_ord0 = s.sel_ord0; h.sel_ord1 = s.sel_ord1; }
             h.done = finished ? 1u : 0u;
             h.force = s.force_nonlocal ? 1u : 0u;
             if (K > 1) {

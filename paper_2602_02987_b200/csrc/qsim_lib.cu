@@ -388,10 +388,11 @@ RunVariant pick_run_kernel(uint32_t N, uint32_t feat, bool scan)
 
 // Calendar of the one-warp kernels with a run-time row count.  Bucket width: about CAL_FILL iteration ends per bucket when
 // all GPUs are busy and iterations last (tau_min + tau_max) / 2 on average, but no wider than 0.45 of the shortest iteration.
-// More than 32 ends do not fit the lanes, fewer waste lanes and the pass over the ids (N = 512, R = 4096, per 250 iterations of
-// horizon: 708 ms at 12 and 16, 730 at 20, 783 with 10 in an earlier version of the pass).  Buckets: a power of two up to 256 that
-// spans the longest iteration; beyond about 2000 GPUs that limit sets the width.
+// More than 32 ends do not fit the lanes, fewer waste lanes and loads.  Buckets: a power of two that spans the longest iteration,
+// at most CAL_MAX (8 bytes of shared memory each; 4096 GPUs of the benchmark's kind need 424).  Beyond that the limit sets the
+// width; when the shortest iteration is shorter than a bucket (cal_K = 0) rounds read all GPUs instead.
 constexpr double CAL_FILL = 16.0;
+constexpr uint32_t CAL_MAX = 512;
 void calendar_shape(uint32_t N, uint32_t B, uint32_t C, const double *coef, Params &p)
 {
     const double tau_mix = coef[0] + coef[1] * (double)C + coef[2] * (double)B, tau_solo = coef[3] + coef[4] * (double)B;
@@ -400,12 +401,12 @@ void calendar_shape(uint32_t N, uint32_t B, uint32_t C, const double *coef, Para
     const double tau_min = coef[0] < coef[3] ? coef[0] : coef[3];
     double w = CAL_FILL * 0.5 * (tau_min + tau_batch) / (double)N;
     if (w > 0.45 * tau_min) w = 0.45 * tau_min;
-    if (w * 254.0 < 1.01 * tau_max) w = 1.01 * tau_max / 254.0;
+    if (w * (CAL_MAX - 2.0) < 1.01 * tau_max) w = 1.01 * tau_max / (CAL_MAX - 2.0);
     uint32_t nbk = 8;
-    while (nbk < 256u && w * (double)(nbk - 2u) < 1.01 * tau_max) nbk <<= 1;
+    while (nbk < CAL_MAX && w * (double)(nbk - 2u) < 1.01 * tau_max) nbk <<= 1;
     p.cal_nbk = nbk;
     p.cal_inv_w = 1.0 / w;
-    p.cal_K = (uint32_t)std::min(0.999 * tau_min / w, 254.0);        // (the margin is far above the rounding of a bucket index)
+    p.cal_K = (uint32_t)std::min(0.999 * tau_min / w, CAL_MAX - 2.0);        // (the margin is far above the rounding of a bucket index)
 }
 
 // More than 128 GPUs: do rounds read all GPUs, with how many warps, or work from the calendar of iteration ends?  Reading all
@@ -480,14 +481,17 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
     const bool kappa = coef[5] != 0.0;
     const uint32_t feat = features_of(cfg, classes, coef);
     h.feat = feat;
+    calendar_shape(cfg.N, cfg.B, cfg.C, coef, p);
+    if (p.cal_K == 0) h.plan.scan = true;       // (the longest iteration lasts hundreds of times as long as the shortest one)
     RunVariant v = pick_run_kernel(cfg.N, feat, h.plan.scan);
     // the per-GPU arrays are padded to the unrolled row count of the chosen instance
     if (v.spl > 0) p.Npad = (uint32_t)v.spl * 32u;
     // finish stamps + occupancy bits go to shared memory when the whole block state stays small
-    // (the limit of 40 KB counts MAXI accounting records and 160 bytes that the block no longer has: which configurations
+    // (the limit of 40 KB counts accounting records, copies of queue heads and draws that the block no longer has: which configurations
     // keep their stamps on chip fixes the layout of saved workspaces)
-    const uint32_t spared = 160u + (uint32_t)sizeof(WarpClassStats) * MAXI - (((uint32_t)sizeof(WarpClassStats) * cfg.I + 15u) & ~15u);
-    p.slots_smem = smem_layout(p.Npad, p.Npad, p.B, 1, 1, kappa, p.Npad > 128u, cfg.I, false).total + spared <= 40u * 1024u ? 1u : 0u;
+    const uint32_t spared = 160u + (uint32_t)sizeof(WarpClassStats) * MAXI - (((uint32_t)sizeof(WarpClassStats) * cfg.I + 15u) & ~15u) +
+                            ((320u + 72u * cfg.I) & ~15u);
+    p.slots_smem = smem_layout(p.Npad, p.Npad, p.B, 1, 1, kappa, p.Npad > 128u, cfg.I, 0).total + spared <= 40u * 1024u ? 1u : 0u;
     if (cfg.N > 992u) p.slots_smem = 0;     // (from 32 rows on the layout is that of several warps, which retire through the global lists)
     if (p.slots_smem) v = pick_run_kernel(cfg.N, feat | F_SLOTS, h.plan.scan);
     h.run_fn = v.fn;
@@ -497,9 +501,8 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
     // the requests in prefill (read once per finished prefill) move to global memory
     p.tarr_global = (p.Npad > 128u) ? 1u : 0u;
     const bool cal = cfg.N > 128u && h.nwarps == 1 && !h.plan.scan;      // run-time row count, one warp (Sim::CAL)
-    calendar_shape(cfg.N, cfg.B, cfg.C, coef, p);
-    h.lay = smem_layout(cfg.N, p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I, cal);
-    h.init_smem = smem_layout(p.Npad, p.Npad, p.B, p.slots_smem, 1, kappa, p.tarr_global != 0, cfg.I, false).total;
+    h.lay = smem_layout(cfg.N, p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I, cal ? p.cal_nbk : 0u);
+    h.init_smem = smem_layout(p.Npad, p.Npad, p.B, p.slots_smem, 1, kappa, p.tarr_global != 0, cfg.I, 0).total;
     p.srv_bytes = h.lay.srv_bytes;
     if (h.lay.total > 227u * 1024u - 64u)       // a few bytes of the block are the kernel's own
         return fail(QSIM_EINVAL, "N too large: per-replication GPU state does not fit shared memory");
@@ -1219,7 +1222,7 @@ int qsim_server_state(qsim_t *h, uint32_t r, uint32_t *n_dec, uint32_t *it, doub
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     const double *tn = reinterpret_cast<const double *>(img.data() + h->lay.off_tnext);
     const uint32_t *itv = reinterpret_cast<const uint32_t *>(img.data() + h->lay.off_it);
-    const uint16_t *rem = reinterpret_cast<const uint16_t *>(img.data() + h->lay.off_pfrem);
+    const uint16_t *rem = reinterpret_cast<const uint16_t *>(img.data() + h->lay.img_pfrem);
     const uint16_t *nd = reinterpret_cast<const uint16_t *>(img.data() + h->lay.off_ndec);
     for (uint32_t g = 0; g < h->cfg.N; ++g) {
         if (n_dec) n_dec[g] = nd[g];
