@@ -381,6 +381,7 @@ class QSimCTMC:
         self.cfg = qsim_ctmc_config(size=C.sizeof(qsim_ctmc_config), I=inp.I, N=inp.N, M=inp.M, B=inp.B, R=inp.R,
                                     qcap=inp.qcap, gate=inp.gate, router=inp.router, reserved=0, seed=inp.seed,
                                     rep_offset=inp.rep_offset)
+        self._records = None
         self.classes = (qsim_ctmc_class * inp.I)()
         for i in range(inp.I):
             self.classes[i] = qsim_ctmc_class(
@@ -409,11 +410,15 @@ class QSimCTMC:
     def stats(self) -> dict:
         import torch
         R, I = self.inp.R, self.inp.I
-        per = (qsim_ctmc_rep_stats * R)()
+        # the records (1.2 KB a replication) stay with the handle: new memory costs a page fault every 4 KB.  A second thread that
+        # reads at the same time takes memory of its own.
+        rec, self._records = self._records, None
+        if rec is None:
+            rec = np.empty(R, dtype=_CTMC_REP_STATS)
+        per = _ptr(rec)
         with torch.cuda.device(self.device):
             _check(self.L.qsim_ctmc_stats(C.byref(self.cfg), C.c_void_p(self.ptr), self.nbytes,
                                           C.c_void_p(self.stream.cuda_stream), per))
-        rec = np.frombuffer(per, dtype=_CTMC_REP_STATS)
         # the classes in use first, in one pass over the records, then one array per statistic
         cnt, state, area = (rec[n][:, :I].copy() for n in ("cnt", "state", "area"))
         out = {}
@@ -430,6 +435,7 @@ class QSimCTMC:
             _check(self.L.qsim_ctmc_revenue(C.byref(self.cfg), per, _ptr(P), _ptr(D), _ptr(prices),
                                             1 if self.inp.meta.get("separate", False) else 0, _ptr(rate)))
         out["_revenue_rate"] = rate
+        self._records = rec
         return out
 
     def close(self) -> None:
