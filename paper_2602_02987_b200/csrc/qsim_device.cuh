@@ -46,7 +46,7 @@ constexpr int LMAX = 8192;
 constexpr int NBIN = 1024;
 constexpr unsigned FULL = 0xffffffffu;
 constexpr uint32_t NONE32 = 0xffffffffu;
-constexpr uint32_t CAL_CHAINS = 2;       // lists per bucket of the calendar (by GPU index, odd or even)
+constexpr uint32_t CAL_CHAINS_NEAR = 4, CAL_CHAINS_FAR = 2;       // lists per bucket of the calendar (by GPU index); F_FAR: where memory on chip counts
 constexpr uint32_t CAL_NONE = 0xffffu;   // end of a list
 constexpr uint32_t BATCH_MASK = 0x1fffu, BATCH_MIXED = 0x2000u;   // nact: decodes in the batch (B <= 4096), the iteration processes prompt tokens (CAL)
 constexpr unsigned long long BUDGET_MAX = 1ull << 29;    // rounds per launch: per-lane counters of a launch have 32 bits
@@ -57,8 +57,10 @@ constexpr uint32_t CAL_FREE = 16;        // free lanes from which the calendar l
 // run time; otherwise the set bits say which features the instance contains and everything else is
 // compiled out.  SPL > 0 fixes the number of simulated GPUs per lane (N <= 32 SPL) so the per-GPU loops unroll.
 constexpr uint32_t F_GENERIC = 1, F_ABANDON = 2, F_SLI = 4, F_KAPPA = 8, F_HIST = 16, F_BLOCKS = 32, F_RANDOM = 64,
-                   F_OCC = 128, F_SLOTS = 256, F_MW = 512, F_FCFS = 1024, F_SLIG = 2048, F_IMM = 4096, F_SCAN = 8192, F_INJECT = 16384;
+                   F_OCC = 128, F_SLOTS = 256, F_MW = 512, F_FCFS = 1024, F_SLIG = 2048, F_IMM = 4096, F_SCAN = 8192, F_INJECT = 16384, F_FAR = 32768;
 // F_SCAN (run-time row count): rounds read all GPUs instead of working from the calendar of iteration ends.
+// F_FAR (calendar): the records of the GPUs stay in global memory (L2); on chip are only the calendar and what a choice among
+// the GPUs reads.  More replications are resident on an SM, each somewhat slower.
 // F_MW: several warps per replication.  Warp 0 (the master) runs the round loop and every event handler; the
 // other warps (helpers) wait at a block barrier for commands and take their share of the per-GPU work of a
 // round: rows r = warp, warp + W, ... of the candidate scan and of the local iteration ends / retirements.
@@ -371,6 +373,8 @@ struct Sim {
     // One warp and a run-time row count: iteration ends come from a calendar (load_bucket) instead of a scan of all GPUs,
     // except in the F_SCAN instances.
     static constexpr bool CAL = SPL == 0 && !(F & (F_MW | F_SCAN));
+    static constexpr bool FAR = CAL && (F & F_FAR) != 0;
+    static constexpr uint32_t CAL_CHAINS = FAR ? CAL_CHAINS_FAR : CAL_CHAINS_NEAR;
     static constexpr bool STAGED = !(F & F_MW);      // one warp: finished requests are accounted 32 at a time
     __device__ __forceinline__ bool f_abandon() const { return (F & F_GENERIC) ? p.any_theta != 0 : (F & F_ABANDON) != 0; }
     __device__ __forceinline__ bool f_sli() const { return (F & F_GENERIC) ? (p.router == 1 || p.router == 2) : (F & F_SLI) != 0; }
@@ -772,8 +776,10 @@ struct Sim {
                 const bool pf = tiers == WANT_PREFILL;
 #pragma unroll 1
                 for (uint32_t bits = __ballot_sync(FULL, (pf ? dirty_pf : dirty_dec) != 0); bits; bits = __ballot_sync(FULL, (pf ? dirty_pf : dirty_dec) != 0)) {
-                    const uint32_t l = (uint32_t)__ffs((int)bits) - 1u, m = __shfl_sync(FULL, pf ? dirty_pf : dirty_dec, (int)l);
-                    const uint32_t row = (((uint32_t)__ffs((int)m) - 1u) << 5) + l, g = (row << 5) + (uint32_t)lane;
+                    const uint32_t l = (uint32_t)__ffs((int)bits) - 1u;
+                    uint32_t row = l;
+                    if (rows > 32u) row += ((uint32_t)__ffs((int)__shfl_sync(FULL, pf ? dirty_pf : dirty_dec, (int)l)) - 1u) << 5;
+                    const uint32_t g = (row << 5) + (uint32_t)lane;
                     const uint32_t a = __reduce_min_sync(FULL, key_of(g, pf ? WANT_PREFILL : (f_sli() ? WANT_SOLO : (WANT_SOLO | WANT_MIX))));
                     if (f_sli() && !pf) {
                         const uint32_t b = __reduce_min_sync(FULL, key_of(g, WANT_MIX));
@@ -1605,7 +1611,7 @@ struct Sim {
     }
 
     // --- calendar of iteration ends (CAL) ---------------------------------------------------------------
-    // Time is cut into buckets of equal width.  The GPUs whose iterations end in a bucket form CAL_CHAINS linked lists (a new end is
+    // Time is cut into buckets of equal width.  The GPUs whose iterations end in a bucket form a few linked lists (a new end is
     // put at the front with one atomic exchange; a lane follows each list), and no iteration is longer than cal_nbk - 2
     // buckets, so a list holds the ends of one bucket only.  The warp works through the buckets in order: load_bucket gives
     // the GPUs of a bucket to lanes that hold none; rounds then look at the lanes only.  The next bucket is loaded as soon as
@@ -1643,8 +1649,8 @@ struct Sim {
         __syncwarp();
         return n;
     }
-    // This lane holds GPU g's pending end.  What the end will read from memory is asked for now, rounds before it is needed: the
-    // request whose prefill it finishes; the stamps of the decodes when one of them finishes.
+    // This lane holds GPU g's pending end.  The request whose prefill it finishes is read now, rounds before it is needed (N = 512,
+    // R = 4096: 569 -> 553 ms).  Asking for the stamps of the finishing decodes as well costs more than it saves (553 against 536).
     __device__ __forceinline__ void hold(uint32_t g)
     {
         held = true; held_g = g;
@@ -1652,13 +1658,6 @@ struct Sim {
         const uint32_t na = nact[g];
         held_na = na;
         if (na & 0x8000u) { held_pk = pfjob[g]; held_tarr = pf_tarr[g]; }
-        if ((na & 0x4000u) && !f_slots()) {
-            const uint32_t nd = ndec[g];
-            const char *a = reinterpret_cast<const char *>(s_fin + (size_t)g * p.B);
-#pragma unroll 1
-            for (uint32_t o = 0; o < nd * 4u; o += 128u) asm volatile("prefetch.global.L2 [%0];" :: "l"(a + o));
-            asm volatile("prefetch.global.L2 [%0];" :: "l"(s_rec + (size_t)g * p.B + (nd - 1u)));
-        }
     }
 
     // More ends in bucket `cur` than lanes (many GPUs that started together), or ends that are in no list: each lane gets the
@@ -1740,9 +1739,9 @@ struct Sim {
     // The round loop on the calendar: as run(), with the lanes' held ends in the place of all GPUs.
     // Bound: the chain of dependent instructions of each replication, about 1500 a round, and fetching them.  Measured at N = 512,
     // R = 4096, 250 iterations of horizon: 955 ms reading all rows in every round, 594 with a byte per GPU that names its bucket
-    // and is searched for every bucket, 563 with lists per bucket, one memory round trip per retirement and no registers
+    // and is searched for every bucket, 536 with lists per bucket (four; with two 2-3 % more), one memory round trip per retirement and no registers
     // spilled (8 bytes spilled in the loop cost 20 %: the L1 next to 200 KB of shared memory is too small for them).
-    // N = 4096, R = 1712: 698 -> 579 ms.  Cycles a warp waits for instructions, per instruction: 2.5 -> 1.2 of 9.1 -> 8.2.
+    // N = 4096, R = 1712: 702 -> 579 ms, 347 with the records in global memory.  Cycles a warp waits for instructions, per instruction: 2.5 -> 1.2 of 9.1 -> 8.2.
     __device__ bool run_calendar()
     {
         const uint32_t budget = (uint32_t)min(p.event_budget, BUDGET_MAX);
@@ -2124,14 +2123,14 @@ struct Sim {
 // shared-memory carve-up for one replication (one warp per block)
 struct SmemLayout {
     uint32_t off_tnext, off_tarr, off_it, off_nfin, off_pfrem, off_pfjob, off_K, off_Kpend, off_ndec, off_nact,
-        off_pfcur, off_sfin16, off_socc, img_pfcur, img_pfrem, img_sfin16, img_socc, srv_bytes, off_head, off_next, off_picked, off_rows, off_left, off_cs, off_ring, off_ringpk, off_strec, off_stte, off_pqh, off_aim, off_wcs, off_cmd, off_res, total;
+        off_pfcur, off_sfin16, off_socc, img_ndec, img_nact, img_pfcur, img_pfrem, img_sfin16, img_socc, srv_bytes, off_head, off_next, off_picked, off_rows, off_left, off_cs, off_ring, off_ringpk, off_strec, off_stte, off_pqh, off_aim, off_wcs, off_cmd, off_res, total;
 };
 
 // tarr_global: the arrival times and the job words of the requests in prefill (read once per finished prefill) live in
 // global memory (large clusters: shared memory is what limits the resident replications there); I: classes (sizes the
 // class records and the ring of arrival draws)
 __host__ __device__ inline SmemLayout smem_layout(uint32_t N, uint32_t Npad, uint32_t B, uint32_t slots_smem, uint32_t nwarps, bool kappa,
-                                                  bool tarr_global, uint32_t I, uint32_t cal_nbk)
+                                                  bool tarr_global, uint32_t I, uint32_t cal_nbk, bool far)
 {
     SmemLayout L;
     uint32_t o = 0;
@@ -2142,8 +2141,8 @@ __host__ __device__ inline SmemLayout smem_layout(uint32_t N, uint32_t Npad, uin
     L.off_pfjob = o; if (!tarr_global) o += 4 * Npad;
     L.off_K = o; if (kappa) o += 4 * Npad;        // KV-token counts exist only when the KV slope is on
     L.off_Kpend = o; if (kappa) o += 4 * Npad;
-    L.off_ndec = o; o += 2 * Npad;
-    L.off_nact = o; o += 2 * Npad;
+    L.off_ndec = L.img_ndec = o; o += 2 * Npad;
+    L.off_nact = L.img_nact = o; o += 2 * Npad;
     // (with the calendar the chunk of the running iteration follows from its batch word: the image has it, the chip does not)
     const bool cal = cal_nbk > 0;
     L.off_pfcur = L.img_pfcur = o;
@@ -2154,6 +2153,7 @@ __host__ __device__ inline SmemLayout smem_layout(uint32_t N, uint32_t Npad, uin
     // memory instead of 24, which is 12 resident replications per SM instead of 9)
     const uint32_t words = (B + 31u) >> 5;
     L.img_sfin16 = o;
+    if (far) { L.off_ndec = 0; L.off_pfrem = 2 * Npad; }       // (the other arrays are used where they are in the image)
     if (cal) o = (L.off_pfrem + 2 * Npad + 15u) & ~15u;
     L.img_socc = (L.img_sfin16 + (slots_smem ? 2 * Npad * B : 0u) + 15u) & ~15u;
     L.srv_bytes = (L.img_socc + (slots_smem ? 4 * Npad * words : 0u) + 15u) & ~15u;
@@ -2161,7 +2161,7 @@ __host__ __device__ inline SmemLayout smem_layout(uint32_t N, uint32_t Npad, uin
     o = (o + 15u) & ~15u;
     L.off_socc = o; if (slots_smem) o += 4 * N * words;
     o = (o + 15u) & ~15u;
-    L.off_head = o; o += 4 * CAL_CHAINS * cal_nbk;       // calendar of iteration ends
+    L.off_head = o; o += 4 * (far ? CAL_CHAINS_FAR : CAL_CHAINS_NEAR) * cal_nbk;       // calendar of iteration ends
     L.off_next = o; if (cal) o += 2 * Npad;
     L.off_picked = o; if (cal) o += 2 * 32;
     L.off_rows = o; if (cal) o += 3 * 4 * (Npad >> 5);
@@ -2188,16 +2188,17 @@ __host__ __device__ inline SmemLayout smem_layout(uint32_t N, uint32_t Npad, uin
 template <int SPL, uint32_t F>
 __device__ __forceinline__ void bind_pointers(Sim<SPL, F> &s, char *sm, const SmemLayout &L)
 {
-    s.tnext = reinterpret_cast<double *>(sm + L.off_tnext);
+    char *const rec = Sim<SPL, F>::FAR ? s.p.srv + (size_t)s.rep * s.p.srv_bytes : sm;
+    s.tnext = reinterpret_cast<double *>(rec + L.off_tnext);
     s.pf_tarr = s.p.tarr_global ? s.p.tarr_g + (size_t)s.rep * s.p.N : reinterpret_cast<double *>(sm + L.off_tarr);
-    s.it = reinterpret_cast<uint32_t *>(sm + L.off_it);
-    s.nfin = reinterpret_cast<uint32_t *>(sm + L.off_nfin);
+    s.it = reinterpret_cast<uint32_t *>(rec + L.off_it);
+    s.nfin = reinterpret_cast<uint32_t *>(rec + L.off_nfin);
     s.pfrem = reinterpret_cast<uint16_t *>(sm + L.off_pfrem);
     s.pfjob = s.p.tarr_global ? s.p.pfjob_g + (size_t)s.rep * s.p.N : reinterpret_cast<uint32_t *>(sm + L.off_pfjob);
-    s.K = reinterpret_cast<uint32_t *>(sm + L.off_K);
-    s.Kpend = reinterpret_cast<uint32_t *>(sm + L.off_Kpend);
+    s.K = reinterpret_cast<uint32_t *>(rec + L.off_K);
+    s.Kpend = reinterpret_cast<uint32_t *>(rec + L.off_Kpend);
     s.ndec = reinterpret_cast<uint16_t *>(sm + L.off_ndec);
-    s.nact = reinterpret_cast<uint16_t *>(sm + L.off_nact);
+    s.nact = reinterpret_cast<uint16_t *>(rec + L.off_nact);
     s.pfcur = reinterpret_cast<uint16_t *>(sm + L.off_pfcur);
     s.sfin16 = reinterpret_cast<uint16_t *>(sm + L.off_sfin16);
     s.socc = reinterpret_cast<uint32_t *>(sm + L.off_socc);
@@ -2233,14 +2234,14 @@ __device__ __forceinline__ void bind_pointers(Sim<SPL, F> &s, char *sm, const Sm
 }
 
 // Empty system at t = 0: idle GPUs, first arrival of every class scheduled, abandonment levels drawn.
-__global__ void __launch_bounds__(32) qsim_init_kernel(Params p)
+__global__ void __launch_bounds__(32, 1) qsim_init_kernel(Params p)
 {
     constexpr int SPLT = 0;
     constexpr uint32_t FT = F_GENERIC;
     extern __shared__ __align__(16) char sm[];
     const int lane = threadIdx.x;
     for (uint32_t rep = blockIdx.x; rep < p.R; rep += gridDim.x) {
-        const SmemLayout L = smem_layout(p.Npad, p.Npad, p.B, p.slots_smem, 1, p.coef[5] != 0.0, p.tarr_global != 0, p.I, 0);       // (laid out as the image)
+        const SmemLayout L = smem_layout(p.Npad, p.Npad, p.B, p.slots_smem, 1, p.coef[5] != 0.0, p.tarr_global != 0, p.I, 0, false);       // (laid out as the image)
         Sim<SPLT, FT> s(p, lane, rep);
         bind_pointers(s, sm, L);
         __syncwarp();
@@ -2271,11 +2272,10 @@ __global__ void __launch_bounds__(32) qsim_init_kernel(Params p)
         if (lane < (int)p.I) s.aring[lane * 32] = 0.0;
         __syncwarp();
         if (p.n_inject > 0 && lane < (int)p.I) s.schedule_from(0.0);
-        for (uint32_t guard = 0; guard < 64u + p.nblk * p.I; ++guard) {
-            uint32_t need = __ballot_sync(FULL, s.sched_pending);
-            if (!need) break;
-            for (; need; need &= need - 1) s.refill((uint32_t)__ffs((int)need) - 1u);
-        }
+#pragma unroll 1
+        for (uint32_t i = 0; i < p.I; ++i)
+#pragma unroll 1
+            for (uint32_t guard = 0; guard <= p.nblk && __shfl_sync(FULL, (int)s.sched_pending, (int)i) != 0; ++guard) s.refill(i);
         if (lane < (int)p.I) s.cs[lane].adraw -= s.ring_n;
         __syncwarp();
         // write everything out
@@ -2316,17 +2316,18 @@ __device__ __forceinline__ void copy16(char *sm, char *img, uint32_t bytes, uint
         else    *reinterpret_cast<uint4 *>(img + o) = *reinterpret_cast<const uint4 *>(sm + o);
     }
 }
-template <bool IN, bool CAL>
+template <bool IN, bool CAL, bool FAR>
 __device__ __forceinline__ void stage_image(char *sm, char *img, const SmemLayout &L, const Params &p, uint32_t tid, uint32_t nthr)
 {
-    copy16<IN>(sm, img, CAL ? L.img_pfcur : L.img_sfin16, tid, nthr);
+    if (!FAR) copy16<IN>(sm, img, CAL ? L.img_pfcur : L.img_sfin16, tid, nthr);
+    else copy16<IN>(sm + L.off_ndec, img + L.img_ndec, 2 * p.Npad, tid, nthr);
     if (CAL) {
         // the prompt remainders, and the chunk in progress from or to the batch word
         __syncwarp();
-        uint16_t *na = reinterpret_cast<uint16_t *>(sm + L.off_nact), *rem = reinterpret_cast<uint16_t *>(sm + L.off_pfrem);
+        uint16_t *na = reinterpret_cast<uint16_t *>((FAR ? img : sm) + L.off_nact), *rem = reinterpret_cast<uint16_t *>(sm + L.off_pfrem);
         uint16_t *cur = reinterpret_cast<uint16_t *>(img + L.img_pfcur), *irem = reinterpret_cast<uint16_t *>(img + L.img_pfrem);
-        uint16_t *ina = reinterpret_cast<uint16_t *>(img + L.off_nact);
-        const double *tn = reinterpret_cast<const double *>(sm + L.off_tnext);
+        uint16_t *ina = reinterpret_cast<uint16_t *>(img + L.img_nact);
+        const double *tn = reinterpret_cast<const double *>((FAR ? img : sm) + L.off_tnext);
 #pragma unroll 1
         for (uint32_t g = tid; g < p.Npad; g += nthr) {
             if (IN) {
@@ -2422,7 +2423,7 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, (FT & F_MW) ? 
                 continue;
             }
         } else if (!p.advance && h.done) continue;
-        const SmemLayout L = smem_layout(p.N, p.Npad, p.B, p.slots_smem, nthr >> 5, p.coef[5] != 0.0, p.tarr_global != 0, p.I, Sim<SPLT, FT>::CAL ? p.cal_nbk : 0u);
+        const SmemLayout L = smem_layout(p.N, p.Npad, p.B, p.slots_smem, nthr >> 5, p.coef[5] != 0.0, p.tarr_global != 0, p.I, Sim<SPLT, FT>::CAL ? p.cal_nbk : 0u, Sim<SPLT, FT>::FAR);
         Sim<SPLT, FT> s(p, lane, rep);
         s.warp = warp;
         s.nwarps = (int)(nthr >> 5);
@@ -2430,7 +2431,7 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, (FT & F_MW) ? 
         s.block_sync();
         // stage state: per-GPU arrays (coalesced 16-byte copies) and the class records; clear the per-warp accounting
         char *const img = p.srv + (size_t)rep * p.srv_bytes;
-        stage_image<true, Sim<SPLT, FT>::CAL>(sm, img, L, p, (uint32_t)tid, nthr);
+        stage_image<true, Sim<SPLT, FT>::CAL, Sim<SPLT, FT>::FAR>(sm, img, L, p, (uint32_t)tid, nthr);
         {
             const uint4 *src = reinterpret_cast<const uint4 *>(h.cs);
             uint4 *dst = reinterpret_cast<uint4 *>(s.cs);
@@ -2487,7 +2488,7 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, (FT & F_MW) ? 
         if (warp == 0 && lane < (int)p.I) s.cs[lane].adraw -= s.ring_n;     // unused arrival draws are produced again next time
         s.block_sync();
         // stage back
-        stage_image<false, Sim<SPLT, FT>::CAL>(sm, img, L, p, (uint32_t)tid, nthr);
+        stage_image<false, Sim<SPLT, FT>::CAL, Sim<SPLT, FT>::FAR>(sm, img, L, p, (uint32_t)tid, nthr);
         {
             uint4 *dst = reinterpret_cast<uint4 *>(h.cs);
             const uint4 *src = reinterpret_cast<const uint4 *>(s.cs);

@@ -77,6 +77,7 @@ struct qsim {
     int device = 0;
     void (*run_fn)(qsimdev::Params) = nullptr;
     uint32_t nwarps = 1;          // warps per replication (block size / 32)
+    bool far = false;             // calendar kernels: the GPU records stay in global memory
     RoundPlan plan;               // how the rounds of the warp family find what happens next on a large cluster
     void (*lane_fn)(qsimdev::Params) = nullptr;     // instance of the one-thread-per-replication run kernel
     bool allow_lane = true;       // the one-thread-per-replication family may run this handle
@@ -288,7 +289,7 @@ void add_row_variants(std::vector<RunVariant> &v)
     v.push_back({0, W | F_OCC | F_ABANDON, qsim_run_kernel<0, W | F_OCC | F_ABANDON>});
     v.push_back({0, W | F_OCC | F_ABANDON | F_SLI | F_HIST, qsim_run_kernel<0, W | F_OCC | F_ABANDON | F_SLI | F_HIST>});
     v.push_back({0, W | F_ABANDON | F_BLOCKS | F_HIST, qsim_run_kernel<0, W | F_ABANDON | F_BLOCKS | F_HIST>});
-    v.push_back({0, W | F_SLOTS | F_OCC | F_ABANDON | F_RANDOM, qsim_run_kernel<0, W | F_SLOTS | F_OCC | F_ABANDON | F_RANDOM>});
+    if constexpr ((W & F_FAR) == 0) v.push_back({0, W | F_SLOTS | F_OCC | F_ABANDON | F_RANDOM, qsim_run_kernel<0, W | F_SLOTS | F_OCC | F_ABANDON | F_RANDOM>});
     v.push_back({0, W | F_GENERIC, qsim_run_kernel<0, W | F_GENERIC>});
 }
 
@@ -302,6 +303,7 @@ const std::vector<RunVariant> &run_variants()
         // one warp, run-time row count (129 GPUs and more)
         add_row_variants<0u>(v);
         add_row_variants<F_SCAN>(v);
+        add_row_variants<F_FAR>(v);
         // several warps per replication (large clusters): instances for the occupancy gate with abandonment under
         // the solo-first and (with histograms) the SLI-aware router, the priority gate with blocks and histograms, and the generic one
         v.push_back({-1, F_MW | F_OCC | F_ABANDON, qsim_run_kernel<0, F_MW | F_OCC | F_ABANDON>});
@@ -364,12 +366,14 @@ RunVariant pick_run_kernel(uint32_t N, uint32_t feat, bool scan)
     const RunVariant *generic = nullptr, *best = nullptr;
     // QSIM_KERNEL=generic forces the run-time-configured instance (for cross-checking the specialised ones)
     const char *force = std::getenv("QSIM_KERNEL");
+    const uint32_t far = feat & F_FAR;
     if (force && std::strcmp(force, "generic") == 0) feat = ~0u;
     int best_bits = 99;
     for (const RunVariant &v : run_variants()) {
         if (v.spl < 0) continue;                            // the multi-warp instance is chosen by the caller
         if (v.spl != 0 && v.spl < rows) continue;          // too few GPUs per lane
         if (v.spl == 0 && ((v.feat & F_SCAN) != 0) != scan) continue;
+        if ((v.feat & F_FAR) != far) continue;
         if (v.spl == 0 && (v.feat & F_GENERIC)) { generic = &v; continue; }
         // smallest row count that fits (0 = run-time row count, beyond four rows); among those the feature set with
         // the fewest extras
@@ -450,6 +454,17 @@ RoundPlan round_plan(const qsim_config &c, double lambda, const double *coef)
     return plan;
 }
 
+// Calendar kernels: do the GPU records stay in global memory (F_FAR)?  Then more replications are resident, each of which waits for
+// L2 a few times a round.  Measured, near / far in ms: N = 512, R = 4096 253 / 259; N = 700, R = 2400 229 / 256; N = 1024, R = 2000 (seven
+// residents on chip) 291 / 346 and, SLI-aware, 304 / 372; N = 1500, R = 1300 (five) 269 / 198; N = 2048, R = 1500 (four) 385 / 213;
+// N = 4096, R = 1712 (two) 607 / 387.  QSIM_RECORDS=near|far overrides.
+bool far_records(const qsim_config &c, uint32_t near_bytes)
+{
+    if (const char *e = std::getenv("QSIM_RECORDS")) return std::strcmp(e, "far") == 0;
+    const uint32_t near = std::min(12u, 227u * 1024u / (near_bytes + 1024u));       // resident replications of an SM
+    return near < 6u && c.R > near * SMS;
+}
+
 double mean_rate(const qsim_config &c, const double *rates)      // requests per second and GPU, averaged over the blocks
 {
     double lam = 0.0;
@@ -491,7 +506,7 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
     // keep their stamps on chip fixes the layout of saved workspaces)
     const uint32_t spared = 160u + (uint32_t)sizeof(WarpClassStats) * MAXI - (((uint32_t)sizeof(WarpClassStats) * cfg.I + 15u) & ~15u) +
                             ((320u + 72u * cfg.I) & ~15u);
-    p.slots_smem = smem_layout(p.Npad, p.Npad, p.B, 1, 1, kappa, p.Npad > 128u, cfg.I, 0).total + spared <= 40u * 1024u ? 1u : 0u;
+    p.slots_smem = smem_layout(p.Npad, p.Npad, p.B, 1, 1, kappa, p.Npad > 128u, cfg.I, 0, false).total + spared <= 40u * 1024u ? 1u : 0u;
     if (cfg.N > 992u) p.slots_smem = 0;     // (from 32 rows on the layout is that of several warps, which retire through the global lists)
     if (p.slots_smem) v = pick_run_kernel(cfg.N, feat | F_SLOTS, h.plan.scan);
     h.run_fn = v.fn;
@@ -501,8 +516,13 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
     // the requests in prefill (read once per finished prefill) move to global memory
     p.tarr_global = (p.Npad > 128u) ? 1u : 0u;
     const bool cal = cfg.N > 128u && h.nwarps == 1 && !h.plan.scan;      // run-time row count, one warp (Sim::CAL)
-    h.lay = smem_layout(cfg.N, p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I, cal ? p.cal_nbk : 0u);
-    h.init_smem = smem_layout(p.Npad, p.Npad, p.B, p.slots_smem, 1, kappa, p.tarr_global != 0, cfg.I, 0).total;
+    h.lay = smem_layout(cfg.N, p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I, cal ? p.cal_nbk : 0u, false);
+    h.far = cal && p.slots_smem == 0 && far_records(cfg, h.lay.total);
+    if (h.far) {
+        h.run_fn = pick_run_kernel(cfg.N, feat | F_FAR, false).fn;
+        h.lay = smem_layout(cfg.N, p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I, p.cal_nbk, true);
+    }
+    h.init_smem = smem_layout(p.Npad, p.Npad, p.B, p.slots_smem, 1, kappa, p.tarr_global != 0, cfg.I, 0, false).total;
     p.srv_bytes = h.lay.srv_bytes;
     if (h.lay.total > 227u * 1024u - 64u)       // a few bytes of the block are the kernel's own
         return fail(QSIM_EINVAL, "N too large: per-replication GPU state does not fit shared memory");
@@ -998,7 +1018,7 @@ int qsim_set_injected(qsim_t *h, const double *t, const uint32_t *job, uint64_t 
     h->par.inject_job = h->d_inject_job;
     h->par.n_inject = (uint32_t)n;
     // the trace source lives in the instances built for it and in the run-time-configured ones
-    RunVariant v = pick_run_kernel(h->cfg.N, h->feat | F_INJECT | (h->par.slots_smem ? F_SLOTS : 0u), h->plan.scan);
+    RunVariant v = pick_run_kernel(h->cfg.N, h->feat | F_INJECT | (h->par.slots_smem ? F_SLOTS : 0u) | (h->far ? F_FAR : 0u), h->plan.scan);
     if (h->nwarps > 1)
         for (const RunVariant &mw : run_variants())
             if (mw.spl < 0 && (mw.feat & F_GENERIC)) v = mw;
@@ -1223,7 +1243,7 @@ int qsim_server_state(qsim_t *h, uint32_t r, uint32_t *n_dec, uint32_t *it, doub
     const double *tn = reinterpret_cast<const double *>(img.data() + h->lay.off_tnext);
     const uint32_t *itv = reinterpret_cast<const uint32_t *>(img.data() + h->lay.off_it);
     const uint16_t *rem = reinterpret_cast<const uint16_t *>(img.data() + h->lay.img_pfrem);
-    const uint16_t *nd = reinterpret_cast<const uint16_t *>(img.data() + h->lay.off_ndec);
+    const uint16_t *nd = reinterpret_cast<const uint16_t *>(img.data() + h->lay.img_ndec);
     for (uint32_t g = 0; g < h->cfg.N; ++g) {
         if (n_dec) n_dec[g] = nd[g];
         if (it) it[g] = itv[g];
