@@ -288,7 +288,8 @@ int qsim_simulate_static(const qsim_config *cfg, const qsim_class *classes, cons
  * which the tests use): QSIM_FAMILY=warp|lane picks the kernel family (a warp, or a few warps, per replication; one
  * thread per replication) where the configuration allows both; QSIM_WARPS=1..16 the warps per replication of the first
  * (two, four or sixteen by default on lightly loaded clusters of more than 992 GPUs, else one); QSIM_ROUNDS=scan|calendar how
- * its one-warp kernels find iteration ends on more than 128 GPUs;
+ * its one-warp kernels find iteration ends on more than 128 GPUs; QSIM_RECORDS=near|far whether those on the calendar keep the
+ * GPU records on chip or in global memory;
  * QSIM_LANE_LSH=2..5 the binary logarithm of the replications per warp of the second; QSIM_KERNEL=generic the kernel
  * instance that reads every feature from its parameters; QSIM_CHUNKS, see qsim_run.  Read when a handle is created
  * (QSIM_CHUNKS: at every qsim_run).
