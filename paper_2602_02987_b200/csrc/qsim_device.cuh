@@ -37,6 +37,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <type_traits>
 #include <cuda_runtime.h>
 
 namespace qsimdev {
@@ -49,7 +50,9 @@ constexpr uint32_t NONE32 = 0xffffffffu;
 constexpr uint32_t CAL_CHAINS_NEAR = 4, CAL_CHAINS_FAR = 2;       // lists per bucket of the calendar (by GPU index); F_FAR: where memory on chip counts
 constexpr uint32_t CAL_NONE = 0xffffu;   // end of a list
 constexpr uint32_t BATCH_MASK = 0x1fffu, BATCH_MIXED = 0x2000u;   // nact: decodes in the batch (B <= 4096), the iteration processes prompt tokens (CAL)
-constexpr unsigned long long BUDGET_MAX = 1ull << 29;    // rounds per launch: per-lane counters of a launch have 32 bits
+// Rounds per launch.  Counters of a launch have 32 bits where a lane ends at most four iterations of its own and one more in a round (the
+// calendar, unrolled rows); where it ends one for each of up to 128 rows, the iteration counters have 64 (Sim::IterCount).
+constexpr unsigned long long BUDGET_MAX = 1ull << 29;
 constexpr int ARRIVALS_PER_ROUND = 64;    // arrivals of a class that one round takes (a trace may bring any number at one time)
 constexpr uint32_t CAL_FREE = 16;        // free lanes from which the calendar loads another bucket
 
@@ -376,6 +379,7 @@ struct Sim {
     static constexpr bool FAR = CAL && (F & F_FAR) != 0;
     static constexpr uint32_t CAL_CHAINS = FAR ? CAL_CHAINS_FAR : CAL_CHAINS_NEAR;
     static constexpr bool STAGED = !(F & F_MW);      // one warp: finished requests are accounted 32 at a time
+    using IterCount = std::conditional_t<SPL == 0 && !CAL, unsigned long long, uint32_t>;      // (see BUDGET_MAX)
     __device__ __forceinline__ bool f_abandon() const { return (F & F_GENERIC) ? p.any_theta != 0 : (F & F_ABANDON) != 0; }
     __device__ __forceinline__ bool f_sli() const { return (F & F_GENERIC) ? (p.router == 1 || p.router == 2) : (F & F_SLI) != 0; }
     __device__ __forceinline__ bool f_slig() const { return (F & F_GENERIC) ? p.router == 2 : false; }
@@ -453,7 +457,7 @@ struct Sim {
     unsigned long long *left;    // crowded: earliest pending end of the bucket that no lane holds (time, source), in shared memory
     uint32_t dirty_dec, dirty_pf;   // bit k: the keys of row lane + 32 k are out of date (decode / prefill targets)
     // per-lane partial sums
-    uint32_t it_mixed, it_solo;
+    IterCount it_mixed, it_solo;
     double busy_mixed, busy_solo;
     // pre-generated arrival draws of this lane's class (ring in shared memory) and a pending scheduling request
     double *aring;
