@@ -440,3 +440,4 @@ class QSimCTMC:
 
     def close(self) -> None:
         self.ws = None
+        self._records = None
