@@ -1,6 +1,7 @@
 """ctypes binding of libqsim.so with the same names as include/qsim.h (argument marshalling only)."""
 from __future__ import annotations
 
+import collections
 import ctypes as C
 import os
 
@@ -381,7 +382,7 @@ class QSimCTMC:
         self.cfg = qsim_ctmc_config(size=C.sizeof(qsim_ctmc_config), I=inp.I, N=inp.N, M=inp.M, B=inp.B, R=inp.R,
                                     qcap=inp.qcap, gate=inp.gate, router=inp.router, reserved=0, seed=inp.seed,
                                     rep_offset=inp.rep_offset)
-        self._records = None
+        self._records = collections.deque(maxlen=1)
         self.classes = (qsim_ctmc_class * inp.I)()
         for i in range(inp.I):
             self.classes[i] = qsim_ctmc_class(
@@ -410,10 +411,11 @@ class QSimCTMC:
     def stats(self) -> dict:
         import torch
         R, I = self.inp.R, self.inp.I
-        # the records (1.2 KB a replication) stay with the handle: new memory costs a page fault every 4 KB.  A second thread that
-        # reads at the same time takes memory of its own.
-        rec, self._records = self._records, None
-        if rec is None:
+        # the records (1.2 KB a replication) stay with the handle: new memory costs a page fault every 4 KB.  They are taken out in
+        # one step, so a second thread that reads at the same time takes memory of its own.
+        try:
+            rec = self._records.pop()
+        except IndexError:
             rec = np.empty(R, dtype=_CTMC_REP_STATS)
         per = _ptr(rec)
         with torch.cuda.device(self.device):
@@ -435,9 +437,11 @@ class QSimCTMC:
             _check(self.L.qsim_ctmc_revenue(C.byref(self.cfg), per, _ptr(P), _ptr(D), _ptr(prices),
                                             1 if self.inp.meta.get("separate", False) else 0, _ptr(rate)))
         out["_revenue_rate"] = rate
-        self._records = rec
+        self._records.append(rec)
+        if self.ws is None:          # closed meanwhile
+            self._records.clear()
         return out
 
     def close(self) -> None:
         self.ws = None
-        self._records = None
+        self._records.clear()

@@ -2,6 +2,8 @@
 the records)."""
 import contextlib
 import gc
+import sys
+import threading
 import types
 import weakref
 
@@ -61,3 +63,55 @@ def test_a_closed_handle_keeps_no_records(handle, monkeypatch):
     sim.close()
     gc.collect()
     assert made[0]() is None
+
+
+def test_two_threads_that_read_at_the_same_time_share_no_records(handle):
+    """A second thread's read begins between any two steps of the first one's, and takes its numbers out of the records after the first one's
+    records were filled."""
+    sim, lib = handle
+    code = binding.QSimCTMC.stats.__code__
+    main = threading.get_ident()
+    step, steps = 0, 1
+    while step < steps:
+        sim.stats()
+        got, filled, begun, first_filled = {}, {}, threading.Event(), threading.Event()
+
+        def on_fill(k):
+            filled[threading.get_ident() == main] = k
+            if threading.get_ident() == main:
+                first_filled.set()
+            else:
+                begun.set()
+                assert first_filled.wait(10)
+
+        other = threading.Thread(target=lambda: got.update(other=sim.stats()["events"]))
+        count = 0
+
+        def trace(frame, event, arg):
+            nonlocal count
+            if frame.f_code is not code:
+                return None
+            if not frame.f_trace_opcodes:
+                frame.f_trace_opcodes = True
+                sys.settrace(trace)          # (takes note of it)
+            if event == "opcode":
+                if count == step:
+                    other.start()
+                    assert begun.wait(10)
+                count += 1
+            return trace
+
+        lib.filled = on_fill
+        before = sys.gettrace()
+        sys.settrace(trace)
+        try:
+            mine = sim.stats()["events"]
+        finally:
+            sys.settrace(before)
+        if not begun.is_set():          # (the first read had fewer steps this time)
+            break
+        other.join(10)
+        lib.filled = lambda k: None
+        assert (mine == filled[True]).all() and (got["other"] == filled[False]).all(), step
+        step, steps = step + 1, count
+    assert steps > 20
