@@ -80,6 +80,9 @@ def together(N):
     (lambda: presets.paper_instance(n=200, R=2), [700]),
     (lambda: short_iterations(140), [200]),
     (lambda: together(300), [40, 60]),
+    (lambda: together(1000), [40, 60]),
+    (lambda: light(presets.cfg2(N=700, R=2), 0.3), [70, 30]),             # 30 to 60 ends in a bucket
+    (lambda: light(presets.cfg4(N=1025, R=1), 0.1), [90]),
 ])
 def test_calendar_and_scan_against_the_oracle(make, calls, rounds):
     check(make(), calls, rounds)
