@@ -47,7 +47,7 @@ constexpr int LMAX = 8192;
 constexpr int NBIN = 1024;
 constexpr unsigned FULL = 0xffffffffu;
 constexpr uint32_t NONE32 = 0xffffffffu;
-constexpr uint32_t CAL_CHAINS_NEAR = 4, CAL_CHAINS_FAR = 2;       // lists per bucket of the calendar (by GPU index); F_FAR: where memory on chip counts
+constexpr uint32_t CAL_LSH_NEAR = 2, CAL_LSH_FAR = 1;       // lists per bucket of the calendar (by GPU index), binary logarithm; F_FAR: where memory on chip counts
 constexpr uint32_t CAL_NONE = 0xffffu;   // end of a list
 constexpr uint32_t BATCH_MASK = 0x1fffu, BATCH_MIXED = 0x2000u;   // nact: decodes in the batch (B <= 4096), the iteration processes prompt tokens (CAL)
 // Rounds per launch.  Counters of a launch have 32 bits where a lane ends at most four iterations of its own and one more in a round (the
@@ -60,10 +60,12 @@ constexpr uint32_t CAL_FREE = 16;        // free lanes from which the calendar l
 // run time; otherwise the set bits say which features the instance contains and everything else is
 // compiled out.  SPL > 0 fixes the number of simulated GPUs per lane (N <= 32 SPL) so the per-GPU loops unroll.
 constexpr uint32_t F_GENERIC = 1, F_ABANDON = 2, F_SLI = 4, F_KAPPA = 8, F_HIST = 16, F_BLOCKS = 32, F_RANDOM = 64,
-                   F_OCC = 128, F_SLOTS = 256, F_MW = 512, F_FCFS = 1024, F_SLIG = 2048, F_IMM = 4096, F_SCAN = 8192, F_INJECT = 16384, F_FAR = 32768;
+                   F_OCC = 128, F_SLOTS = 256, F_MW = 512, F_FCFS = 1024, F_SLIG = 2048, F_IMM = 4096, F_SCAN = 8192, F_INJECT = 16384, F_FAR = 32768,
+                   F_TIGHT = 65536;
 // F_SCAN (run-time row count): rounds read all GPUs instead of working from the calendar of iteration ends.
 // F_FAR (calendar): the records of the GPUs stay in global memory (L2); on chip are only the calendar and what a choice among
 // the GPUs reads.  More replications are resident on an SM, each somewhat slower.
+// F_TIGHT (calendar): the shortest iteration is shorter than a bucket.
 // F_MW: several warps per replication.  Warp 0 (the master) runs the round loop and every event handler; the
 // other warps (helpers) wait at a block barrier for commands and take their share of the per-GPU work of a
 // round: rows r = warp, warp + W, ... of the candidate scan and of the local iteration ends / retirements.
@@ -172,7 +174,8 @@ struct Params {
     double *tarr_g;              // [R][N]
     uint32_t *pfjob_g;           // [R][N] packed request in prefill, with tarr_g
     double cal_inv_w;            // calendar of iteration ends (run-time row count, one warp): buckets per second
-    uint32_t cal_nbk, cal_K;     // buckets (a power of two); buckets that the shortest iteration lasts at least (0: no calendar)
+    uint32_t cal_nbk, cal_K;     // buckets (a power of two); buckets that the shortest iteration lasts at least (0: F_TIGHT)
+    uint32_t cal_lsh;            // binary logarithm of the lists per bucket
     LanePar lane;
 };
 
@@ -377,7 +380,9 @@ struct Sim {
     // except in the F_SCAN instances.
     static constexpr bool CAL = SPL == 0 && !(F & (F_MW | F_SCAN));
     static constexpr bool FAR = CAL && (F & F_FAR) != 0;
-    static constexpr uint32_t CAL_CHAINS = FAR ? CAL_CHAINS_FAR : CAL_CHAINS_NEAR;
+    static constexpr bool TIGHT = CAL && (F & F_TIGHT) != 0;
+    __device__ __forceinline__ uint32_t cal_lsh() const { return (F & (F_GENERIC | F_TIGHT)) ? p.cal_lsh : (FAR ? CAL_LSH_FAR : CAL_LSH_NEAR); }
+    __device__ __forceinline__ uint32_t cal_lists() const { return p.cal_nbk << cal_lsh(); }
     static constexpr bool STAGED = !(F & F_MW);      // one warp: finished requests are accounted 32 at a time
     using IterCount = std::conditional_t<SPL == 0 && !CAL, unsigned long long, uint32_t>;      // (see BUDGET_MAX)
     __device__ __forceinline__ bool f_abandon() const { return (F & F_GENERIC) ? p.any_theta != 0 : (F & F_ABANDON) != 0; }
@@ -406,7 +411,7 @@ struct Sim {
     uint16_t *ndec, *nact, *pfcur;
     uint16_t *sfin16;            // [Npad][B]  low 16 bits of each slot's finish iteration (f_slots)
     uint32_t *socc;              // [Npad][ceil(B/32)]  slot occupancy bits; bits past B are set for good
-    uint32_t *cal_head;          // [buckets][CAL_CHAINS] first GPU of every list of the calendar (CAL)
+    uint32_t *cal_head;          // [buckets][1 << cal_lsh] first GPU of every list of the calendar (CAL)
     uint16_t *cal_next;          // [GPUs] the GPU after this one in its list (CAL)
     uint16_t *picked;            // [32] GPUs of the bucket being loaded (CAL)
     uint32_t *row_key;           // [3][rows] smallest key of every row of 32 GPUs (CAL, see choose())
@@ -1622,11 +1627,12 @@ struct Sim {
     // enough lanes are free, so that the next event that is not local is usually among the held ends.  Invariant: every pending
     // event lies in bucket cur - lead or later, so an iteration that starts now ends cal_K = floor(tau_min / width) >= 1
     // buckets after that one or later, and the bucket after `cur` may be loaded while lead + 1 < cal_K.
+    // F_TIGHT (cal_K = 0): one bucket at a time; every round loads what was filed in it meanwhile and ends before T_min + tau_min.
     __device__ __forceinline__ unsigned long long bucket_abs(double x) const { return __double2ull_rd(__dmul_rn(x, p.cal_inv_w)); }
     __device__ __forceinline__ void file_end(uint32_t g, double te)
     {
         const uint32_t b = (uint32_t)bucket_abs(te) & (p.cal_nbk - 1u);
-        cal_next[g] = (uint16_t)atomicExch(&cal_head[b * CAL_CHAINS + (g & (CAL_CHAINS - 1u))], g);
+        cal_next[g] = (uint16_t)atomicExch(&cal_head[(b << cal_lsh()) + (g & ((1u << cal_lsh()) - 1u))], g);
     }
 
     // Give the GPUs whose ends lie in bucket b to the free lanes (mine: this lane's, or NONE32); returns how many there are (nothing
@@ -1634,8 +1640,8 @@ struct Sim {
     __device__ __forceinline__ uint32_t load_bucket(unsigned long long b, uint32_t free_lanes, uint32_t &mine)
     {
         const uint32_t below = (1u << lane) - 1u;
-        uint32_t *head = cal_head + ((uint32_t)b & (p.cal_nbk - 1u)) * CAL_CHAINS + (uint32_t)lane;
-        uint32_t n = 0, g = (uint32_t)lane < CAL_CHAINS ? *head : CAL_NONE;
+        uint32_t *head = cal_head + (((uint32_t)b & (p.cal_nbk - 1u)) << cal_lsh()) + (uint32_t)lane;
+        uint32_t n = 0, g = ((uint32_t)lane >> cal_lsh()) == 0 ? *head : CAL_NONE;
 #pragma unroll 1
         for (uint32_t k = __ballot_sync(FULL, g != CAL_NONE); k && n <= 32u; k = __ballot_sync(FULL, g != CAL_NONE)) {
             const uint32_t pos = n + (uint32_t)__popc(k & below);
@@ -1646,7 +1652,7 @@ struct Sim {
             }
         }
         if (n == 0 || n > (uint32_t)__popc(free_lanes)) return n;
-        if ((uint32_t)lane < CAL_CHAINS) *head = CAL_NONE;
+        if (((uint32_t)lane >> cal_lsh()) == 0) *head = CAL_NONE;
         __syncwarp();
         const uint32_t rank = (uint32_t)__popc(free_lanes & below);
         if (!held && rank < n) mine = (uint32_t)picked[rank];
@@ -1675,8 +1681,8 @@ struct Sim {
         if (held) file_end(held_g, __longlong_as_double((long long)held_t));
         __syncwarp();
         uint32_t g = CAL_NONE;
-        if ((uint32_t)lane < CAL_CHAINS) {
-            uint32_t *head = cal_head + ((uint32_t)cur & (p.cal_nbk - 1u)) * CAL_CHAINS + (uint32_t)lane;
+        if (((uint32_t)lane >> cal_lsh()) == 0) {
+            uint32_t *head = cal_head + (((uint32_t)cur & (p.cal_nbk - 1u)) << cal_lsh()) + (uint32_t)lane;
             g = *head;
             *head = CAL_NONE;
         }
@@ -1725,8 +1731,8 @@ struct Sim {
     {
         uint32_t best = 0x7fffffffu;
 #pragma unroll 1
-        for (uint32_t c = (uint32_t)lane; c < p.cal_nbk * CAL_CHAINS; c += 32u)
-            if (cal_head[c] != CAL_NONE) best = min(best, (c / CAL_CHAINS - (uint32_t)cur) & (p.cal_nbk - 1u));
+        for (uint32_t c = (uint32_t)lane; c < cal_lists(); c += 32u)
+            if (cal_head[c] != CAL_NONE) best = min(best, ((c >> cal_lsh()) - (uint32_t)cur) & (p.cal_nbk - 1u));
         return __reduce_min_sync(FULL, best);
     }
 
@@ -1735,7 +1741,7 @@ struct Sim {
     {
         unsigned long long first = 0x7ff0000000000000ull;
 #pragma unroll 1
-        for (uint32_t c = (uint32_t)lane; c < p.cal_nbk * CAL_CHAINS; c += 32u) cal_head[c] = CAL_NONE;
+        for (uint32_t c = (uint32_t)lane; c < cal_lists(); c += 32u) cal_head[c] = CAL_NONE;
 #pragma unroll 1
         for (uint32_t g = (uint32_t)lane; g < p.N; g += 32u) first = min(first, (unsigned long long)__double_as_longlong(tnext[g]));
         if (lane < (int)p.I) first = min(first, class_first());
@@ -1804,7 +1810,7 @@ struct Sim {
             }
             // Load buckets (one copy of the code for every reason to): the current one again when it is crowded; the next one that
             // holds an event when no lane holds an end any more; the following one when enough lanes are free.
-            bool look = crowded;
+            bool look = crowded, again = TIGHT && !crowded;
             uint32_t turn = 0, d = 0;
 #pragma unroll 1
             for (;;) {
@@ -1814,6 +1820,8 @@ struct Sim {
                 look = false;
                 if (all) {
                     mine = load_crowded();
+                } else if (TIGHT && again) {
+                    again = false;       // (ends that were filed in the current bucket meanwhile)
                 } else if (free_lanes == FULL && !crowded) {
                     if (turn == 0) {
                         // buckets to the first class event or block end
@@ -1860,7 +1868,7 @@ struct Sim {
                     else want = min(n, 32u);            // (more than 32: it has to wait until no lane holds anything)
                     break;
                 }
-                look = n > 32u;
+                look = n > (TIGHT ? (uint32_t)__popc(free_lanes) : 32u);
             }
             const bool buffered = (dq_n0 | dq_n1) != 0;
             const uint32_t na = held_na, nd0 = ndec[held_g];
@@ -1886,6 +1894,17 @@ struct Sim {
             if (crowded) {
                 const uint32_t left_s = (uint32_t)left[1];
                 if (left_t < lim_t || (left_t == lim_t && left_s < lim_s)) { lim_t = left_t; lim_s = left_s; }
+            }
+            if (TIGHT) {
+                // no iteration that starts in this round can end before T_min + tau_min
+                unsigned long long tmin = held_t;
+                if (lane < (int)p.I) tmin = min(tmin, (unsigned long long)__double_as_longlong(cs[lane].ta));
+                const uint32_t hi = (uint32_t)(tmin >> 32), mhi = __reduce_min_sync(FULL, hi);
+                const uint32_t mlo = __reduce_min_sync(FULL, hi == mhi ? (uint32_t)tmin : NONE32);
+                if (mhi < 0x7ff00000u) {
+                    const unsigned long long wt = (unsigned long long)__double_as_longlong(__dadd_rn(__hiloint2double((int)mhi, (int)mlo), tau_min));
+                    if (wt <= lim_t) { lim_t = wt; lim_s = 0; }
+                }
             }
             const bool first_is_event = here && lim_t == tint && lim_s == src;      // nothing that is not held or could still start comes before it
             if (tend_bits < lim_t) { lim_t = tend_bits; lim_s = NONE32; }
@@ -2161,7 +2180,7 @@ struct SmemLayout {
 // global memory (large clusters: shared memory is what limits the resident replications there); I: classes (sizes the
 // class records and the ring of arrival draws)
 __host__ __device__ inline SmemLayout smem_layout(uint32_t N, uint32_t Npad, uint32_t B, uint32_t slots_smem, uint32_t nwarps, bool kappa,
-                                                  bool tarr_global, uint32_t I, uint32_t cal_nbk, bool far)
+                                                  bool tarr_global, uint32_t I, uint32_t cal_lists, bool far)
 {
     SmemLayout L;
     uint32_t o = 0;
@@ -2175,7 +2194,7 @@ __host__ __device__ inline SmemLayout smem_layout(uint32_t N, uint32_t Npad, uin
     L.off_ndec = L.img_ndec = o; o += 2 * Npad;
     L.off_nact = L.img_nact = o; o += 2 * Npad;
     // (with the calendar the chunk of the running iteration follows from its batch word: the image has it, the chip does not)
-    const bool cal = cal_nbk > 0;
+    const bool cal = cal_lists > 0;
     L.off_pfcur = L.img_pfcur = o;
     L.img_pfrem = o + 2 * Npad;
     L.off_pfrem = cal ? o : L.img_pfrem;
@@ -2192,7 +2211,7 @@ __host__ __device__ inline SmemLayout smem_layout(uint32_t N, uint32_t Npad, uin
     o = (o + 15u) & ~15u;
     L.off_socc = o; if (slots_smem) o += 4 * N * words;
     o = (o + 15u) & ~15u;
-    L.off_head = o; o += 4 * (far ? CAL_CHAINS_FAR : CAL_CHAINS_NEAR) * cal_nbk;       // calendar of iteration ends
+    L.off_head = o; o += 4 * cal_lists;       // calendar of iteration ends
     L.off_next = o; if (cal) o += 2 * Npad;
     L.off_picked = o; if (cal) o += 2 * 32;
     L.off_rows = o; if (cal) o += 3 * 4 * (Npad >> 5);
@@ -2454,8 +2473,8 @@ __global__ void __launch_bounds__((FT & F_MW) ? 32 * MW_MAX : 32, (FT & F_MW) ? 
                 continue;
             }
         } else if (!p.advance && h.done) continue;
-        const SmemLayout L = smem_layout(p.N, p.Npad, p.B, p.slots_smem, nthr >> 5, p.coef[5] != 0.0, p.tarr_global != 0, p.I, Sim<SPLT, FT>::CAL ? p.cal_nbk : 0u, Sim<SPLT, FT>::FAR);
         Sim<SPLT, FT> s(p, lane, rep);
+        const SmemLayout L = smem_layout(p.N, p.Npad, p.B, p.slots_smem, nthr >> 5, p.coef[5] != 0.0, p.tarr_global != 0, p.I, Sim<SPLT, FT>::CAL ? s.cal_lists() : 0u, Sim<SPLT, FT>::FAR);
         s.warp = warp;
         s.nwarps = (int)(nthr >> 5);
         bind_pointers(s, sm, L);

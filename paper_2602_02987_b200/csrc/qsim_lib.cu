@@ -78,6 +78,7 @@ struct qsim {
     void (*run_fn)(qsimdev::Params) = nullptr;
     uint32_t nwarps = 1;          // warps per replication (block size / 32)
     bool far = false;             // calendar kernels: the GPU records stay in global memory
+    bool tight = false;           // and: the shortest iteration is shorter than a bucket
     RoundPlan plan;               // how the rounds of the warp family find what happens next on a large cluster
     void (*lane_fn)(qsimdev::Params) = nullptr;     // instance of the one-thread-per-replication run kernel
     bool allow_lane = true;       // the one-thread-per-replication family may run this handle
@@ -304,6 +305,7 @@ const std::vector<RunVariant> &run_variants()
         add_row_variants<0u>(v);
         add_row_variants<F_SCAN>(v);
         add_row_variants<F_FAR>(v);
+        add_row_variants<F_TIGHT>(v);
         // several warps per replication (large clusters): instances for the occupancy gate with abandonment under
         // the solo-first and (with histograms) the SLI-aware router, the priority gate with blocks and histograms, and the generic one
         v.push_back({-1, F_MW | F_OCC | F_ABANDON, qsim_run_kernel<0, F_MW | F_OCC | F_ABANDON>});
@@ -366,14 +368,15 @@ RunVariant pick_run_kernel(uint32_t N, uint32_t feat, bool scan)
     const RunVariant *generic = nullptr, *best = nullptr;
     // QSIM_KERNEL=generic forces the run-time-configured instance (for cross-checking the specialised ones)
     const char *force = std::getenv("QSIM_KERNEL");
-    const uint32_t far = feat & F_FAR;
+    constexpr uint32_t KINDS = F_FAR | F_TIGHT;       // kinds of calendar kernels, chosen by the caller
+    const uint32_t kind = feat & KINDS;
     if (force && std::strcmp(force, "generic") == 0) feat = ~0u;
     int best_bits = 99;
     for (const RunVariant &v : run_variants()) {
         if (v.spl < 0) continue;                            // the multi-warp instance is chosen by the caller
         if (v.spl != 0 && v.spl < rows) continue;          // too few GPUs per lane
         if (v.spl == 0 && ((v.feat & F_SCAN) != 0) != scan) continue;
-        if ((v.feat & F_FAR) != far) continue;
+        if ((v.feat & KINDS) != kind) continue;
         if (v.spl == 0 && (v.feat & F_GENERIC)) { generic = &v; continue; }
         // smallest row count that fits (0 = run-time row count, beyond four rows); among those the feature set with
         // the fewest extras
@@ -393,10 +396,13 @@ RunVariant pick_run_kernel(uint32_t N, uint32_t feat, bool scan)
 // Calendar of the one-warp kernels with a run-time row count.  Bucket width: about CAL_FILL iteration ends per bucket when
 // all GPUs are busy and iterations last (tau_min + tau_max) / 2 on average, but no wider than 0.45 of the shortest iteration.
 // More than 32 ends do not fit the lanes, fewer waste lanes and loads.  Buckets: a power of two that spans the longest iteration,
-// at most CAL_MAX (8 bytes of shared memory each; 4096 GPUs of the benchmark's kind need 424).  Beyond that the limit sets the
-// width; when the shortest iteration is shorter than a bucket (cal_K = 0) rounds read all GPUs instead.
+// at most CAL_MAX (4 bytes of shared memory per list; 4096 GPUs of the benchmark's kind need 424).  Beyond that the limit sets the
+// width, and the shortest iteration may be shorter than a bucket (cal_K = 0, F_TIGHT).  Four lists per bucket, or two with the records in
+// global memory; with them on chip the run-time-configured instances, which may have the KV slope (whose longest iteration, a batch of
+// requests of the greatest lengths, takes 512 buckets), and the F_TIGHT ones keep no more than CAL_LISTS in all (KV slope, N = 200, R = 4000:
+// 43.9 ms with 2048 lists, 42.4 with 512).
 constexpr double CAL_FILL = 16.0;
-constexpr uint32_t CAL_MAX = 512;
+constexpr uint32_t CAL_MAX = 512, CAL_LISTS = 512;
 void calendar_shape(uint32_t N, uint32_t B, uint32_t C, const double *coef, Params &p)
 {
     const double tau_mix = coef[0] + coef[1] * (double)C + coef[2] * (double)B, tau_solo = coef[3] + coef[4] * (double)B;
@@ -411,6 +417,15 @@ void calendar_shape(uint32_t N, uint32_t B, uint32_t C, const double *coef, Para
     p.cal_nbk = nbk;
     p.cal_inv_w = 1.0 / w;
     p.cal_K = (uint32_t)std::min(0.999 * tau_min / w, CAL_MAX - 2.0);        // (the margin is far above the rounding of a bucket index)
+}
+
+// Lists per bucket (binary logarithm) for a calendar instance with the given features.
+uint32_t cal_lists_lsh(uint32_t nbk, uint32_t feat)
+{
+    uint32_t lsh = (feat & F_FAR) ? CAL_LSH_FAR : CAL_LSH_NEAR;
+    if ((feat & (F_GENERIC | F_TIGHT)) != 0 && (feat & F_FAR) == 0)
+        while (lsh > 0 && (nbk << lsh) > CAL_LISTS) --lsh;
+    return lsh;
 }
 
 // More than 128 GPUs: do rounds read all GPUs, with how many warps, or work from the calendar of iteration ends?  Reading all
@@ -497,8 +512,12 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
     const uint32_t feat = features_of(cfg, classes, coef);
     h.feat = feat;
     calendar_shape(cfg.N, cfg.B, cfg.C, coef, p);
-    if (p.cal_K == 0) h.plan.scan = true;       // (the longest iteration lasts hundreds of times as long as the shortest one)
-    RunVariant v = pick_run_kernel(cfg.N, feat, h.plan.scan);
+    // (the longest iteration lasts hundreds of times as long as the shortest one.  Reading all GPUs / calendar in ms, 3300 times: N = 140, R = 2000
+    // 11.6 / 15.8, N = 250, R = 2000 24.4 / 21.6, N = 300, R = 2000 32.9 / 25.3, N = 512, R = 1000 34.6 / 18.2, N = 2000, R = 400 101 / 20)
+    if (p.cal_K == 0 && cfg.N <= 200u) h.plan.scan = true;
+    h.tight = p.cal_K == 0 && cfg.N > 128u && !h.plan.scan;
+    const uint32_t kind = h.tight ? F_TIGHT : 0u;
+    RunVariant v = pick_run_kernel(cfg.N, feat | kind, h.plan.scan);
     // the per-GPU arrays are padded to the unrolled row count of the chosen instance
     if (v.spl > 0) p.Npad = (uint32_t)v.spl * 32u;
     // finish stamps + occupancy bits go to shared memory when the whole block state stays small
@@ -508,7 +527,7 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
                             ((320u + 72u * cfg.I) & ~15u);
     p.slots_smem = smem_layout(p.Npad, p.Npad, p.B, 1, 1, kappa, p.Npad > 128u, cfg.I, 0, false).total + spared <= 40u * 1024u ? 1u : 0u;
     if (cfg.N > 992u) p.slots_smem = 0;     // (from 32 rows on the layout is that of several warps, which retire through the global lists)
-    if (p.slots_smem) v = pick_run_kernel(cfg.N, feat | F_SLOTS, h.plan.scan);
+    if (p.slots_smem) v = pick_run_kernel(cfg.N, feat | F_SLOTS | kind, h.plan.scan);
     h.run_fn = v.fn;
     h.nwarps = 1;
     choose_multiwarp(cfg.N, feat, h.plan.warps, p, h.run_fn, h.nwarps);
@@ -516,11 +535,14 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
     // the requests in prefill (read once per finished prefill) move to global memory
     p.tarr_global = (p.Npad > 128u) ? 1u : 0u;
     const bool cal = cfg.N > 128u && h.nwarps == 1 && !h.plan.scan;      // run-time row count, one warp (Sim::CAL)
-    h.lay = smem_layout(cfg.N, p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I, cal ? p.cal_nbk : 0u, false);
-    h.far = cal && p.slots_smem == 0 && far_records(cfg, h.lay.total);
+    p.cal_lsh = cal_lists_lsh(p.cal_nbk, v.feat);
+    h.lay = smem_layout(cfg.N, p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I, cal ? p.cal_nbk << p.cal_lsh : 0u, false);
+    h.far = cal && p.slots_smem == 0 && !h.tight && far_records(cfg, h.lay.total);
     if (h.far) {
-        h.run_fn = pick_run_kernel(cfg.N, feat | F_FAR, false).fn;
-        h.lay = smem_layout(cfg.N, p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I, p.cal_nbk, true);
+        v = pick_run_kernel(cfg.N, feat | F_FAR, false);
+        h.run_fn = v.fn;
+        p.cal_lsh = cal_lists_lsh(p.cal_nbk, v.feat);
+        h.lay = smem_layout(cfg.N, p.Npad, p.B, p.slots_smem, h.nwarps, kappa, p.tarr_global != 0, cfg.I, p.cal_nbk << p.cal_lsh, true);
     }
     h.init_smem = smem_layout(p.Npad, p.Npad, p.B, p.slots_smem, 1, kappa, p.tarr_global != 0, cfg.I, 0, false).total;
     p.srv_bytes = h.lay.srv_bytes;
@@ -1018,7 +1040,7 @@ int qsim_set_injected(qsim_t *h, const double *t, const uint32_t *job, uint64_t 
     h->par.inject_job = h->d_inject_job;
     h->par.n_inject = (uint32_t)n;
     // the trace source lives in the instances built for it and in the run-time-configured ones
-    RunVariant v = pick_run_kernel(h->cfg.N, h->feat | F_INJECT | (h->par.slots_smem ? F_SLOTS : 0u) | (h->far ? F_FAR : 0u), h->plan.scan);
+    RunVariant v = pick_run_kernel(h->cfg.N, h->feat | F_INJECT | (h->par.slots_smem ? F_SLOTS : 0u) | (h->far ? F_FAR : 0u) | (h->tight ? F_TIGHT : 0u), h->plan.scan);
     if (h->nwarps > 1)
         for (const RunVariant &mw : run_variants())
             if (mw.spl < 0 && (mw.feat & F_GENERIC)) v = mw;

@@ -1,7 +1,8 @@
 """Clusters of more than 128 GPUs on one warp: rounds that work from the calendar of iteration ends and rounds that read all
 GPUs, both against the CPU oracle (integer statistics and per-GPU end state exact, fp64 statistics within 1e-9), at the edges
-of the calendar's shapes: sizes around its words and bucket counts, iterations shorter than a bucket, more iteration ends in
-a bucket than lanes, light load with empty buckets, a run cut into many short launches."""
+of the calendar's shapes: sizes around its rows and bucket counts, iterations that last a bucket and that are shorter (where small
+clusters read all GPUs instead), more iteration ends in a bucket than lanes, light load with empty buckets, a run cut into many
+short launches."""
 import contextlib
 import os
 
@@ -58,8 +59,23 @@ def light(inp, share):
 
 
 def short_iterations(N):
-    """Iteration times that differ by a factor of a thousand: the shortest is shorter than a bucket of the calendar."""
+    """Iteration times that differ by a factor of three thousand: the shortest is shorter than a bucket of the calendar."""
     return presets.cfg2(N=N, R=2).with_(coeffs=np.array([2e-5, 8e-5, 5e-5, 1e-5, 5e-5, 0.0]))
+
+
+def one_bucket(N):
+    """Iteration times that differ by a factor of 400: the shortest lasts one to two buckets, and no bucket is loaded ahead."""
+    return presets.cfg2(N=N, R=2).with_(coeffs=np.array([1.2e-4, 8e-5, 5e-5, 8.3e-5, 5e-5, 0.0]))
+
+
+def block_bytes(inp, **kw):
+    """Shared memory of a replication."""
+    from paper_2602_02987_b200 import QSim
+    with env(QSIM_FAMILY="warp", **kw):
+        sim = QSim(inp)
+    info = sim.layout_info()
+    sim.close()
+    return info["smem_bytes"]
 
 
 def together(N):
@@ -79,6 +95,13 @@ def together(N):
     (lambda: light(presets.cfg4(N=300, R=2), 0.0005), [900, 900]),
     (lambda: presets.paper_instance(n=200, R=2), [700]),
     (lambda: short_iterations(140), [200]),
+    (lambda: short_iterations(300), [60, 40]),
+    (lambda: short_iterations(300).with_(gate=1), [60]),                  # the run-time-configured instance
+    (lambda: presets.cfg3(N=220, R=2, block_len=0.2).with_(coeffs=short_iterations(1).coeffs), [150]),
+    (lambda: presets.cfg4(N=210, R=2).with_(coeffs=short_iterations(1).coeffs), [60]),
+    (lambda: presets.crowded("decode", N=260, R=2, placement=PLACE_RANDOM).with_(coeffs=np.array([2e-5, 8e-4, 5e-5, 1e-5, 5e-5, 0.0])), [6000, 2000]),
+    (lambda: one_bucket(140), [200]),
+    (lambda: one_bucket(600), [60]),
     (lambda: together(300), [40, 60]),
     (lambda: together(1000), [40, 60]),
     (lambda: light(presets.cfg2(N=700, R=2), 0.3), [70, 30]),             # 30 to 60 ends in a bucket
@@ -88,8 +111,26 @@ def test_calendar_and_scan_against_the_oracle(make, calls, rounds):
     check(make(), calls, rounds)
 
 
+@pytest.mark.parametrize("make,calendar", [(short_iterations, {200: False, 201: True, 300: True, 2000: True}), (one_bucket, {140: True, 300: True})])
+def test_iterations_shorter_than_a_bucket_keep_larger_clusters_on_the_calendar(make, calendar):
+    # (the calendar's lists take shared memory, 2 KB where iterations are shorter than a bucket)
+    for N, want in calendar.items():
+        lists = block_bytes(make(N), QSIM_ROUNDS="calendar", QSIM_WARPS="1") - block_bytes(make(N), QSIM_ROUNDS="scan")
+        assert (lists > 0) == want, N
+        if make is short_iterations:
+            assert lists < 2048 + 4 * N, N
+
+
+def test_the_kv_slope_takes_little_more_shared_memory():
+    """Its longest iteration asks for 512 buckets; their lists stay within 2 KB, next to the 8 bytes per GPU of the token counts."""
+    inp = presets.cfg2(N=224, R=2)
+    plain = block_bytes(inp, QSIM_ROUNDS="calendar", QSIM_WARPS="1", QSIM_KERNEL="generic")
+    slope = block_bytes(inp.with_(coeffs=presets.COEFFS_PAPER_KV), QSIM_ROUNDS="calendar", QSIM_WARPS="1")
+    assert 8 * 224 < slope - plain <= 8 * 224 + 2048
+
+
 @pytest.mark.parametrize("N", [1023, 2049, 4096])
-def test_calendar_on_large_clusters_with_as_many_buckets_as_ids(N):
+def test_calendar_on_large_clusters_with_many_buckets(N):
     check(presets.cfg2(N=N, R=1), [30, 30], "calendar")
 
 
