@@ -1329,7 +1329,8 @@ struct Sim {
         SlotRec *rec = s_rec + (size_t)g * p.B;
         if constexpr (SPL == 1) {
             // Up to 32 GPUs: the finished request's record and the tail entry that takes its place are read together, after the stamps, a
-            // second round trip, but less code (priority gate with blocks, N = 20, R = 4000, 24 blocks of 0.5 s: 9.5 ms, 10.5 the other way).
+            // second round trip, but less code, from which the run-time-configured instance gains most (priority gate with blocks, N = 20,
+            // R = 4000, 24 blocks of 0.5 s: 9.5 ms, 10.5 the other way).
 #pragma unroll 1
             for (int k0 = (int)((nd - 1u) & ~127u); k0 >= 0; k0 -= 128) {
                 uint32_t f[4], hit[4];
@@ -1829,9 +1830,10 @@ struct Sim {
     // The round loop on the calendar: as run(), with the lanes' held ends in the place of all GPUs.
     // Bound: the chain of dependent instructions of each replication, about 1500 a round, and fetching them.  Measured at N = 512,
     // R = 4096, 250 iterations of horizon: 955 ms reading all rows in every round, 594 with a byte per GPU that names its bucket
-    // and is searched for every bucket, 536 with lists per bucket (four; with two 2-3 % more), one memory round trip per retirement and no registers
-    // spilled (8 bytes spilled in the loop cost 20 %: the L1 next to 200 KB of shared memory is too small for them).
-    // N = 4096, R = 1712: 702 -> 579 ms, 347 with the records in global memory.  Cycles a warp waits for instructions, per instruction: 2.5 -> 1.2 of 9.1 -> 8.2.
+    // and is searched for every bucket, 556 with lists per bucket (four; with two 2-3 % more) and one memory round trip per retirement.  The
+    // instance of the occupancy gate spills no registers (8 bytes spilled in the loop cost 20 %: the L1 next to 200 KB of shared memory is too
+    // small for them), and any change of the loop moves its time by 1 to 10 % through the layout of the code.
+    // N = 4096, R = 1712: 702 -> 351 ms, 155 with the records in global memory.
     __device__ bool run_calendar()
     {
         const uint32_t budget = (uint32_t)min(p.event_budget, BUDGET_MAX);
@@ -2453,8 +2455,9 @@ __device__ __forceinline__ void stage_image(char *sm, char *img, const SmemLayou
 // Advance replications to their new end time (or until the per-launch event budget runs out).
 template <int SPLT, uint32_t FT>
 // One-warp instances whose slot records live in global memory need little shared memory, so registers decide how many
-// replications are resident on an SM: they are compiled for at least 12 blocks per SM (at most 168 registers, a few
-// bytes of spills; +16-24 % at N = 64 with thousands of replications).  Instances with the finish stamps on chip are
+// replications are resident on an SM: they are compiled for at least 12 blocks per SM (at most 168 registers; the specialised
+// instances spill nothing or 4 to 28 bytes, 44 in the SLI-aware one with the records in global memory, the run-time-configured ones 40 to 108; +16-24 % at
+// N = 64 with thousands of replications).  Instances with the finish stamps on chip are
 // limited by shared memory and keep all the registers they want (the cap cost them 13 %), but for those of up to 32 GPUs, whose
 // stamps take little (N = 16, R = 8192: 133 -> 98 ms).
 #ifndef QSIM_MIN_BLOCKS

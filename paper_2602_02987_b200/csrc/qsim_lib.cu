@@ -439,17 +439,17 @@ uint32_t cal_lists_lsh(uint32_t nbk, uint32_t feat)
 // for every choice either way): r = 2.6 rows (N = 600) 15.5 / 21.5, 1.95 rows (N = 300) 30.9 / 40.9, 1.95 rows (N = 150) 24.4 / 30.2, 1.0 rows
 // (N = 600) 35.6 / 42.1, 1.0 rows (N = 300) 58.5 / 62.5, 1.0 rows (N = 150) 41.8 / 41.0, 0.5 rows (N = 600) 65.0 / 64.8, 0.5 rows (N = 300) 98 / 85.  QSIM_ROUNDS=scan|calendar overrides (and means one warp).
 //
-// Several warps, from 32 rows on (two, from 64 rows four, from 128 rows sixteen: the best of sweeps).  The calendar's time hardly
-// depends on the load, being a pass over the ids per bucket, and that of several warps is proportional to the events.  Both sides
-// in ms for 20 iterations of horizon, several warps / calendar, at r = 49, 20, 10, 5 (cfg2 with 0.1, 0.25, 0.5, 0.95 of its load):
-//   N = 1024, R = 888   12 / 21    27 / 24    49 / 32    85 / 43
-//   N = 2048, R = 740   43 / 101   96 / 109   178 / 122  323 / 159
-//   N = 3000, R = 444   75 / 227   171 / 239  323 / 254  592 / 270
-//   N = 4096, R = 592   134 / 474  316 / 489  616 / 518  1143 / 531
-//   N = 4096, R = 148   34 / 237   80 / 245   156 / 258  287 / 266
-// The last two differ because a block of sixteen warps has an SM to itself, and two replications on the calendar share one.  The
-// lines below also hold for the priority gate with blocks (N = 1024, R = 585, r = 21: 55 / 62).  Uniform placement: N = 1024, R = 592, r = 49
-// and 20, 20 / 20 and 45 / 40; N = 2048, R = 444, r = 20 and 10, 90 / 95 and 171 / 140; N = 4096, R = 444, r = 20 and 10, 629 / 769 and 1238 / 1068.
+// Several warps, from 32 rows on (two, from 64 rows four, from 128 rows sixteen: the best of sweeps).  The time of several warps is
+// proportional to the events, that of the calendar grows more slowly: its lists are followed once per end.  Both sides in ms for 20 iterations of
+// horizon, several warps / calendar, at r = 49, 20, 10, 5 (cfg2 with 0.1, 0.25, 0.5, 0.95 of its load):
+//   N = 1024, R = 888   11.7 / 15.5    26 / 20     47 / 27     82 / 38
+//   N = 2048, R = 740   41 / 47        93 / 58     171 / 73    309 / 94
+//   N = 3000, R = 444   41 / 68        89 / 84     168 / 103   304 / 132
+//   N = 4096, R = 592   129 / 94       304 / 116   594 / 142   1120 / 185
+//   N = 4096, R = 148   33 / 61        78 / 79     150 / 105   281 / 146
+// The last two differ because a block of sixteen warps has an SM to itself, and six replications on the calendar share one.  Uniform
+// placement: N = 1024, R = 592, r = 49 and 20, 16.5 / 16.6 and 38 / 34; N = 2048, R = 444, r = 20 and 10, 78 / 75 and 146 / 118; N = 4096, R = 444, r = 20
+// and 10, 513 / 250 and 1002 / 389.
 constexpr uint32_t SMS = 148;
 RoundPlan round_plan(const qsim_config &c, double lambda, const double *coef)
 {
@@ -463,16 +463,18 @@ RoundPlan round_plan(const qsim_config &c, double lambda, const double *coef)
     const double per_end = lambda * 0.5 * (tau_min + tau_max);        // 1 / r
     plan.scan = 1.0 > per_end * from * rows;
     if (c.N > 992u) {
-        const double r_from = c.N <= 2016u ? (c.placement == QSIM_PLACE_RANDOM ? 45.0 : 20.5) : (c.N <= 4064u ? 19.0 : (c.R <= SMS ? 6.5 : 14.0));
+        const bool uniform = c.placement == QSIM_PLACE_RANDOM;
+        const double r_from = c.N <= 2016u ? (uniform ? 45.0 : 33.0) : c.N <= 2500u && c.R > 2u * SMS && !uniform ? 42.0 :
+                              c.N <= 4064u ? 21.0 : (c.R <= SMS ? 20.0 : 55.0);
         if (1.0 > per_end * r_from) plan.warps = c.N <= 2016u ? 2u : (c.N <= 4064u ? 4u : 16u);
     }
     return plan;
 }
 
 // Calendar kernels: do the GPU records stay in global memory (F_FAR)?  Then more replications are resident, each of which waits for
-// L2 a few times a round.  Measured, near / far in ms: N = 512, R = 4096 253 / 259; N = 700, R = 2400 229 / 256; N = 1024, R = 2000 (seven
-// residents on chip) 291 / 346 and, SLI-aware, 304 / 372; N = 1500, R = 1300 (five) 269 / 198; N = 2048, R = 1500 (four) 385 / 213;
-// N = 4096, R = 1712 (two) 607 / 387.  QSIM_RECORDS=near|far overrides.
+// L2 a few times a round.  Measured, near / far in ms: N = 700, R = 2400 95 / 109; N = 1024, R = 2000 (seven residents on chip) 128 / 156;
+// N = 1500, R = 754 and 1300 (five) 264 / 230 and 182 / 123; N = 2048, R = 603 and 1500 (four) 364 / 310 and 233 / 86; N = 4096, R = 301 and 1712
+// (two) 729 / 606 and 351 / 155 (the smaller R is 1.02 times what fits near).  QSIM_RECORDS=near|far overrides.
 bool far_records(const qsim_config &c, uint32_t near_bytes)
 {
     if (const char *e = std::getenv("QSIM_RECORDS")) return std::strcmp(e, "far") == 0;
@@ -550,18 +552,14 @@ int configure(qsim &h, const qsim_config &cfg, const qsim_class *classes, const 
         return fail(QSIM_EINVAL, "N too large: per-replication GPU state does not fit shared memory");
     h.sec = layout_sections(cfg, p.srv_bytes, p.tarr_global != 0);
     for (int k = 0; k < 6; ++k) h.coef[k] = coef[k];
-    // Kernel family.  A replication advances at about the same rate on one thread whatever its cluster size, while the
-    // warp-per-replication kernels are limited by the replications whose GPU state fits an SM (two or three beyond 2048
-    // GPUs) but advance each about seventy times as fast.  Measured (it/s, warp / thread): N = 4096, R = 1712: 1.72e8 / 1.41e8,
-    // R = 3800: 1.76e8 / 2.77e8; N = 3000, R = 2400: 2.30e8 / 1.83e8; N = 2048, R = 3456: 5.6e8 / 2.7e8.  Both lines cross at about 9.5
-    // million simulated GPUs (R x N); up to 2048 GPUs the warp kernels stay ahead for every R that fits in memory.
-    // QSIM_FAMILY=lane / warp overrides.
+    // Kernel family.  One thread per replication advances each at about the same rate whatever its cluster size, up to 4.6e8 server
+    // iterations a second; the warp-per-replication kernels are limited by the replications whose GPU state fits an SM (six to eight beyond
+    // 2048 GPUs, with the records in global memory) but advance each about seventy times as fast.  Measured (it/s, warp / thread): N = 4096, R = 1712:
+    // 8.0e8 / 1.6e8, R = 3800: 7.4e8 / 3.1e8; with B = 64 R = 6000: 9.5e8 / 4.6e8, R = 10000: 9.4e8 / 4.3e8; N = 3000, R = 4000: 9.6e8 / 3.3e8.  So a handle
+    // gets the warp kernels, unless QSIM_FAMILY=lane asks for the others or it resumes a state that they saved.
     std::memset(&p.lane, 0, sizeof p.lane);
-    bool lane = h.allow_lane && lane_supports(cfg, coef) && cfg.N > 2048u && (unsigned long long)cfg.R * cfg.N >= 9500000ull;
-    if (const char *e = std::getenv("QSIM_FAMILY")) {
-        if (std::strcmp(e, "lane") == 0) lane = h.allow_lane && lane_supports(cfg, coef);
-        else if (std::strcmp(e, "warp") == 0) lane = false;
-    }
+    bool lane = false;
+    if (const char *e = std::getenv("QSIM_FAMILY")) lane = std::strcmp(e, "lane") == 0 && h.allow_lane && lane_supports(cfg, coef);
     if (h.family >= 0) lane = h.family == 1 && h.allow_lane && lane_supports(cfg, coef);
     h.resident_blocks = 0;
     h.lane_fn = nullptr;

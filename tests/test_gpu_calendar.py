@@ -186,3 +186,18 @@ def test_several_warps_on_lightly_loaded_large_clusters(make, load, warps):
             sim.run(60)
             assert_parity(sim.stats(), run_oracle(inp, 60), what=f"{inp.name}, {want} warps")
         sim.close()
+
+
+@pytest.mark.parametrize("inp,load,warps", [
+    (lambda: presets.cfg2(N=1100, R=2), 0.2, 1),
+    (lambda: presets.cfg2(N=2200, R=297), 0.13, 1),
+    (lambda: presets.cfg2(N=2200, R=296), 0.13, 4),
+    (lambda: presets.cfg2(N=4096, R=148), 0.2, 16),
+    (lambda: presets.cfg2(N=4096, R=149), 0.1, 1),
+    (lambda: presets.cfg4(N=4096, R=2400).with_(B=16), 1.0, 1),          # (not one thread per replication)
+])
+def test_the_calendar_runs_medium_loads_and_many_replications_of_large_clusters(inp, load, warps):
+    from paper_2602_02987_b200 import QSim
+    sim = QSim(light(inp(), load))
+    assert sim.layout_info()["warps"] == warps
+    sim.close()
